@@ -3,10 +3,15 @@
 Every step of the decode path runs inside libonela.so; this module converts torch tensors to device
 pointers, checks shapes and dtypes, and raises on a negative status.  It fails loudly when the library
 is missing or cannot be loaded: there is no fallback of any kind.
+
+The calls a decode loop makes go through `_onela_pycall` first (csrc/onela_pycall.cpp), which makes the same checks on
+the tensors' C++ objects; whatever it does not take - an argument that is wrong, a dry run - goes through the checks
+here, which raise with the argument's name.
 """
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 from ctypes import POINTER, c_char_p, c_int32, c_int64, c_size_t, c_uint32, c_void_p
 from pathlib import Path
 
@@ -14,6 +19,7 @@ import torch
 
 _PKG = Path(__file__).resolve().parent
 LIB_PATH = _PKG / "libonela.so"
+PYCALL_PATH = _PKG / "_onela_pycall.so"
 
 OK, E_INVAL, E_CAPACITY, E_ORDER, E_CUDA, E_UNSUPPORTED, E_DEVICE_CHECK, E_TIMEOUT = 0, -1, -2, -3, -4, -5, -6, -7
 DTYPE_F32, DTYPE_BF16 = 0, 1
@@ -42,6 +48,7 @@ class OnelaError(RuntimeError):
 
 
 _lib = None
+_pycall = None
 
 # name -> (restype, argtypes); the ABI test checks this table against the header
 PROTOTYPES = {
@@ -88,6 +95,31 @@ def load_library() -> ctypes.CDLL:
             fn.restype, fn.argtypes = res, args
         _lib = lib
     return _lib
+
+
+# functions of the library in the order the native callers expect their addresses
+_CALLER_FUNCTIONS = ("onela_export_chains", "onela_init_shared_state", "onela_init_shared_states", "onela_prefill_shared_state",
+                     "onela_reorder_beams", "onela_select_beams", "onela_append_records", "onela_decode_step", "onela_append_decode_step",
+                     "onela_export_shared_state", "onela_release_request")
+_NATIVE_CALLS = ("init_state", "init_states", "prefill", "reorder", "select_beams", "append", "decode", "append_decode", "export_state",
+                 "release")
+
+
+def _native_caller(lib, handle, cfg):
+    """The native marshalling object of one context (see csrc/onela_pycall.cpp)."""
+    global _pycall
+    if _pycall is None:
+        if not PYCALL_PATH.exists():
+            raise RuntimeError(f"{PYCALL_PATH} is missing: run `python -m paper_2609_12399_b200.build` (or __graft_entry__.build()) first")
+        spec = importlib.util.spec_from_file_location("_onela_pycall", PYCALL_PATH)
+        _pycall = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(_pycall)
+    fns = tuple(ctypes.cast(getattr(lib, n), c_void_p).value for n in _CALLER_FUNCTIONS)
+    return _pycall.Caller(handle.value, ctypes.addressof(cfg), fns)
+
+
+def _no_native_call(*_):
+    return 1             # NOT_TAKEN: a dry run takes fake addresses, which only the checks below accept
 
 
 def status_string(status: int) -> str:
@@ -155,9 +187,14 @@ class Onela:
         self.handle = h
         self.rec_dtype = _TORCH_DTYPE[cfg.rec_dtype]
         self.out_dtype = _TORCH_DTYPE[cfg.out_dtype]
+        native = None if dry else _native_caller(self.lib, h, cfg)
+        for name in _NATIVE_CALLS:
+            setattr(self, "_" + name, getattr(native, name, _no_native_call))
 
     def close(self):
         if getattr(self, "handle", None):
+            for name in _NATIVE_CALLS:
+                setattr(self, "_" + name, _no_native_call)      # (a native caller keeps the raw handle)
             self.lib.onela_destroy(self.handle)
             self.handle = None
 
@@ -191,16 +228,25 @@ class Onela:
         _check(self.lib.onela_reset(self.handle, c_void_p(0 if self._dry() else _stream_ptr(stream))), "onela_reset")
 
     def onela_init_shared_state(self, request, layer, S0, stream=None):
+        st = self._init_state(request, layer, S0, stream)
+        if st <= 0:
+            return _check(st, "onela_init_shared_state")
         c = self.cfg
         p = self._ptr(S0, torch.float32, (c.value_heads, c.dv, c.dk), "S0")
         _check(self.lib.onela_init_shared_state(self.handle, request, layer, p, self._s(stream)), "onela_init_shared_state")
 
     def onela_init_shared_states(self, req_begin, req_count, S0, stream=None):
+        st = self._init_states(req_begin, req_count, S0, stream)
+        if st <= 0:
+            return _check(st, "onela_init_shared_states")
         c = self.cfg
         p = self._ptr(S0, torch.float32, (req_count, c.num_layers, c.value_heads, c.dv, c.dk), "S0")
         _check(self.lib.onela_init_shared_states(self.handle, req_begin, req_count, p, self._s(stream)), "onela_init_shared_states")
 
     def onela_prefill_shared_state(self, request, layer, k, v, alpha, beta, stream=None):
+        st = self._prefill(request, layer, k, v, alpha, beta, stream)
+        if st <= 0:
+            return _check(st, "onela_prefill_shared_state")
         c = self.cfg
         n = int(k.shape[0])
         _check(self.lib.onela_prefill_shared_state(
@@ -213,20 +259,33 @@ class Onela:
         """Returns the stored S_0 of (request, layer) as fp32 [H, dv, dk] on the device."""
         c = self.cfg
         out = torch.empty((c.value_heads, c.dv, c.dk), dtype=torch.float32, device=self.device)
+        st = self._export_state(request, layer, out, stream)
+        if st <= 0:
+            _check(st, "onela_export_shared_state")
+            return out
         _check(self.lib.onela_export_shared_state(self.handle, request, layer, c_void_p(out.data_ptr()),
                                                   self._s(stream)), "onela_export_shared_state")
         return out
 
     def onela_reorder_beams(self, req_begin, req_count, parents, W_new, stream=None):
+        st = self._reorder(req_begin, req_count, parents, W_new, stream)
+        if st <= 0:
+            return _check(st, "onela_reorder_beams")
         p = None if parents is None else self._ptr(parents, torch.int32, (req_count, W_new), "parents")
         _check(self.lib.onela_reorder_beams(self.handle, req_begin, req_count, p, W_new, self._s(stream)),
                "onela_reorder_beams")
 
     def onela_release_request(self, request):
+        st = self._release(request)
+        if st <= 0:
+            return _check(st, "onela_release_request")
         _check(self.lib.onela_release_request(self.handle, request), "onela_release_request")
 
     def onela_select_beams(self, req_begin, req_count, beam_scores, cand_logp, C, W_new, parents_out, codes_out, scores_out,
                            stream=None):
+        st = self._select_beams(req_begin, req_count, beam_scores, cand_logp, C, W_new, parents_out, codes_out, scores_out, stream)
+        if st <= 0:
+            return _check(st, "onela_select_beams")
         depth, W = self._width(req_begin)
         W_prev = W if depth >= 1 else 1
         _check(self.lib.onela_select_beams(
@@ -238,6 +297,9 @@ class Onela:
             self._ptr(scores_out, torch.float32, (req_count, W_new), "scores_out"), self._s(stream)), "onela_select_beams")
 
     def onela_append_records(self, req_begin, req_count, layer, k, v, alpha, beta, stream=None):
+        st = self._append(req_begin, req_count, layer, k, v, alpha, beta, stream)
+        if st <= 0:
+            return _check(st, "onela_append_records")
         c = self.cfg
         _, W = self._width(req_begin)
         _check(self.lib.onela_append_records(
@@ -248,6 +310,9 @@ class Onela:
             self._ptr(beta, torch.float32, (req_count, W, c.value_heads), "beta"), self._s(stream)), "onela_append_records")
 
     def onela_decode_step(self, req_begin, req_count, layer, q, out, stream=None):
+        st = self._decode(req_begin, req_count, layer, q, out, stream)
+        if st <= 0:
+            return _check(st, "onela_decode_step")
         c = self.cfg
         _, W = self._width(req_begin)
         _check(self.lib.onela_decode_step(
@@ -256,6 +321,9 @@ class Onela:
             self._ptr(out, self.out_dtype, (req_count, W, c.value_heads, c.dv), "out"), self._s(stream)), "onela_decode_step")
 
     def onela_append_decode_step(self, req_begin, req_count, layer, k, v, alpha, beta, q, out, stream=None):
+        st = self._append_decode(req_begin, req_count, layer, k, v, alpha, beta, q, out, stream)
+        if st <= 0:
+            return _check(st, "onela_append_decode_step")
         c = self.cfg
         _, W = self._width(req_begin)
         _check(self.lib.onela_append_decode_step(

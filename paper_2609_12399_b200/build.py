@@ -3,6 +3,7 @@ from __future__ import annotations
 
 import os
 import subprocess
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 from pathlib import Path
 
@@ -34,6 +35,30 @@ def _stale(target: Path, deps) -> bool:
         return True
     t = target.stat().st_mtime
     return any(d.stat().st_mtime > t for d in deps)
+
+
+# The binding's native argument marshalling: a CPython extension on torch's own headers and libraries (already in the
+# process when it is imported), host code only.
+PYCALL_SRC = CSRC / "onela_pycall.cpp"
+PYCALL_LIB = PKG / "_onela_pycall.so"
+
+
+def build_pycall(force: bool = False) -> Path:
+    header = ROOT / "include" / "onela.h"
+    if force or _stale(PYCALL_LIB, [PYCALL_SRC, header]):
+        import torch
+        from torch.utils import cpp_extension
+        nvcc = Path(_nvcc())
+        cuda_inc = nvcc.parent.parent / "include" if nvcc.is_absolute() else Path("/usr/local/cuda/include")
+        incs = [ROOT / "include", cuda_inc, sysconfig.get_paths()["include"], *cpp_extension.include_paths()]
+        libs = Path(torch.__file__).resolve().parent / "lib"
+        cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+               *(f"-I{i}" for i in incs), str(PYCALL_SRC), "-o", str(PYCALL_LIB), f"-L{libs}", "-lc10", "-lc10_cuda", "-ltorch_cpu",
+               "-ltorch_python"]
+        r = subprocess.run(cmd, capture_output=True, text=True)
+        if r.returncode != 0:
+            raise RuntimeError("g++ failed:\n" + " ".join(cmd) + "\n" + r.stdout + r.stderr)
+    return PYCALL_LIB
 
 
 # A second library for the tests of the bounded waits: the same sources with a short wait limit and a hook that
@@ -89,5 +114,6 @@ def build(force: bool = False, verbose: bool = False, lib: Path = LIB, obj_dir: 
 if __name__ == "__main__":
     import sys
     print(build(force="--force" in sys.argv, verbose="-v" in sys.argv))
+    print(build_pycall(force="--force" in sys.argv))
     if "--testhooks" in sys.argv:
         print(build_testhooks(force="--force" in sys.argv))
