@@ -321,12 +321,12 @@ onela_status onela_prefill_shared_state(onela_ctx* ctx, int32_t request, int32_t
     if (!ctx->dry()) {
         bool supported = true;
         const cudaError_t e = launch_prefill(k_dev, v_dev, alpha_dev, beta_dev, ctx->s0_slot(request, layer),
-                                             ctx->s0_scale_slot(request, layer), n_tokens, ctx->cfg.num_heads, ctx->cfg.dk,
-                                             ctx->cfg.dv, ctx->cfg.rec_dtype, &supported, s);
+                                             ctx->s0_scale_slot(request, layer), ctx->tiled_tc ? ctx->s0_f16_slot(request, layer) : nullptr,
+                                             ctx->lay.status, n_tokens, ctx->cfg.num_heads, ctx->cfg.dk, ctx->cfg.dv, ctx->cfg.rec_dtype,
+                                             &supported, s);
         if (!supported) return ONELA_E_UNSUPPORTED;
         if (e != cudaSuccess) return ONELA_E_CUDA;
         ctx->launches++;
-        if (ctx->pack_states(request, layer, ctx->Hv(), s) != cudaSuccess) return ONELA_E_CUDA;
     }
     finish_state_write(ctx, request, layer);
     return ONELA_OK;

@@ -180,9 +180,11 @@ cudaError_t launch_store_state(const float* S0_in, float* slot, float* scale_out
 cudaError_t launch_pack_state(const float* slot, const float* scale, uint16_t* dst, long long n_heads, int32_t dk, int32_t dv,
                               cudaStream_t stream);
 cudaError_t launch_export_state(const float* slot, float* S0_out, int32_t H, int32_t dk, int32_t dv, cudaStream_t stream);
-// returns cudaErrorInvalidValue with *supported = false when (dk, dv, dtype) has no instantiation
-cudaError_t launch_prefill(const void* k, const void* v, const float* alpha, const float* beta, float* slot,
-                           float* scale_out, int32_t n_tokens, int32_t H, int32_t dk, int32_t dv, int32_t rec_dtype,
+// Eq. 1 from the zero state over a prompt, into the store slot of one (request, layer), with the heads' operand scales and
+// (s0_f16 not null) the tiled kernel's operand copies (onela_prefill.cu).  Returns cudaErrorInvalidValue with *supported =
+// false when (dk, dv) has no instantiation.
+cudaError_t launch_prefill(const void* k, const void* v, const float* alpha, const float* beta, float* slot, float* scale_out,
+                           uint16_t* s0_f16, int32_t* status, int32_t n_tokens, int32_t H, int32_t dk, int32_t dv, int32_t rec_dtype,
                            bool* supported, cudaStream_t stream);
 
 // decode kernels

@@ -1,0 +1,911 @@
+// Prompt -> shared state on the tensor cores (sm_100a): S_T of Eq. 1 from the zero state, dk = dv in {32, 64, 128}.
+//
+// What bounded the kernel this one replaces: the recurrence itself.  One CTA per head walked the prompt token by token,
+// 1.1 us each on 32 of 148 SMs (16 384 tokens x 32 heads of 128 x 128 bf16: 17.9 ms).  Here a chunk of C = 64 tokens is
+// one step.  With g_i = prod_{l <= i} alpha_l inside the chunk, A_ij = beta_i (g_i / g_j) (k_i . k_j) for j < i (strictly
+// lower triangular; the ratios are running products, nothing is divided) and T = (I + A)^-1, Eq. 1 over the chunk is
+//      S_out = g_C S_in + Delta Y ,   Delta = V^T diag(beta) - S_in K^T diag(beta g) ,   Y = T^T diag(g_C / g) K
+// (the WY form of a product of Householder-like factors; Delta is dv x C, Y is C x dk).  T, Y and the coefficients depend
+// on the keys and gates alone, so they are prepared a chunk ahead of the state.
+//
+// Parallelism along the prompt.  The map of a run of chunks is affine, S -> S M + B, and M obeys the same recurrence as
+// S (from the identity, with V = 0).  A head's prompt is cut into segments, one per CTA of a cluster; every segment but
+// the first carries M as dk more state rows, and at the end the cluster folds the segments in order, S <- S M_p + B_p,
+// handing S from CTA to CTA through distributed shared memory.  Nothing goes through global memory but the inputs and
+// the result.
+//
+// One CTA: two TEAMS of 128 threads that prepare chunks in turn (keys -> operand tile, Gram product, inverse, Y) and 128
+// threads per CHAIN of 128 state rows (dk = 128: S and M are a chain each, and hide each other's latency; dk <= 64: one
+// chain holds both), coupled by mbarriers over a ring of key / value tiles and one of Y tiles.  A thread keeps one state row
+// in fp32 registers.  Products run as tcgen05.mma kind::f16 with fp32 accumulation, an operand being one fp16 number where
+// that is exact (bf16 keys, to 2^-28 of the row's largest) and otherwise the sum of two (22 to 23 significant bits); every
+// operand row carries its own power of two, exact to apply and to undo, so the range of the caller's data does not matter.
+// The tensor core's accumulator truncates, so the small products are accumulated first: with the large ones first the state
+// came out 3x less exact.  Relative error against fp64: 1.5e-7 at the usual gates, 2.9e-7 without decay (token by token in
+// fp32: 1.0e-7 and 3.5e-7).
+//   per chunk and chain:  [S_hi ; S_lo] K^T   2 x dk / 16 MMAs (M = 128, N = 64), A in tensor memory
+//                         Delta Y             3 x 4 MMAs (N = dk), A in tensor memory
+//   per chunk:            K K^T (dk / 16 MMAs), K^T T' (2 x 4 MMAs, A = the key tile read MN-major)
+// (fp32 records: keys in two parts as well, 3 products each.)
+// What bounds it now: the latency of a chain's step, about 10 000 cycles per chunk (28 MMAs at ~80 cycles, four conversions
+// between tensor memory, registers and tensor memory), beside two preparations in flight that take as long together; issue
+// slots are a third used, the tensor pipe a fifth.  16 384 tokens x 32 heads of 128 x 128 bf16: 18.2 ms -> 0.38 ms;
+// 1021 tokens x 16 heads of 64 x 64 fp32: 376 -> 32 us.
+//
+// Every wait is bounded: a thread that gives up keeps meeting its team's barriers, whose OR makes the team leave
+// together, and the cluster barriers; ONELA_E_TIMEOUT goes to the status word.
+#include <algorithm>
+#include <mutex>
+#include <type_traits>
+
+#include "onela_internal.h"
+#include "onela_layout.cuh"
+#include "onela_sm100.cuh"
+
+namespace onela {
+
+namespace {
+
+using sm100::bar_or;
+using sm100::idesc_f16;
+using sm100::mbar_init;
+using sm100::pack_f16x2;
+using sm100::pow2_scale;
+using sm100::smem_u32;
+using sm100::tmem_ld16;
+using sm100::tmem_st16;
+using sm100::umma_desc;
+
+constexpr int C = 64;              // tokens per chunk
+constexpr int TILE = C * 128;      // bytes of one K-major operand block: 64 rows of 64 fp16
+constexpr int KV_STAGES = 3, Y_STAGES = 2;
+constexpr int CTA_BARRIER = 9;     // named barrier of the whole CTA (1 - 4: the teams')
+constexpr int AP = C + 4;          // pitch (floats) of the C x C matrix: 16-byte rows
+constexpr int MAX_SEGMENTS = 8;    // portable cluster size
+// Largest elements of the scaled operand rows: keys and T' in [2^3, 2^4) (so |Y| < 64 * 2^8 = 2^14 stays inside fp16's
+// range unscaled), state rows and Delta rows in [2^12, 2^13).
+constexpr int NARROW = 3, WIDE = 12;
+
+struct PrefillArgs {
+    const void *k, *v;
+    const float *alpha, *beta;
+    float* slot;          // [H][dv][dk]
+    float* scale_out;     // [H]
+    uint16_t* s0_f16;     // the tiled decode kernel's operand copy (see Layout::s0_f16), or null
+    int32_t* status;
+    int32_t n_tokens, H;
+    int32_t first, rest;  // chunks of the first segment, of each other one (the last may hold fewer)
+};
+
+template <int D, typename T>
+struct Shape {
+    static constexpr int KB = D > 64 ? D / 64 : 1;                  // K blocks of 64 elements
+    static constexpr int PK = sizeof(T) == 4 ? 2 : 1;               // fp16 parts of a key
+    static constexpr int PREPS = 2, CHAINS = D == 128 ? 2 : 1;      // teams of 128 threads
+    static constexpr int THREADS = 128 * (PREPS + CHAINS);
+    static constexpr bool V_STAGED = sizeof(T) == 2;                // (fp32 values are read where they are: no room beside the keys)
+    static constexpr int K_BYTES = PK * KB * TILE;
+    static constexpr int KV_BYTES = K_BYTES + (V_STAGED ? C * D * (int)sizeof(T) : 0);
+    static constexpr int Y_BYTES = 2 * D * 128;                      // [hi, lo][dk rows][128 bytes]
+    static constexpr int RING = KV_STAGES * KV_BYTES + Y_STAGES * Y_BYTES;
+    // per preparing team: the C x C matrix, over it T' as an operand tile (hi, lo), and the scratch of its inversion
+    static constexpr int A_BYTES = (C * AP * 4 + 1023) / 1024 * 1024, X_BYTES = 5 * 1024;
+    static constexpr int TOK_BYTES = 4 * C * 4;                      // per token: alpha, 1 / key scale, weight in T', scratch
+    static constexpr int COEF_BYTES = 1024;                          // per Y stage: b[C], c[C], g_C
+    // (the Gram product reads 128 rows from a 64-row block and the MN-major tile a second block: what lies behind the key
+    // tile is read and the rows that come of it are ignored)
+    static constexpr int SMALL = PREPS * TOK_BYTES + Y_STAGES * COEF_BYTES + 128 * 4 + 256;
+    static constexpr int SMEM = RING + PREPS * (A_BYTES + X_BYTES) + SMALL + 1024;
+    static constexpr uint32_t CHAIN_COLS = D + C;                    // S operand (hi, lo) / Delta Y ; S K^T / Delta operand
+    static constexpr uint32_t PREP_COL = CHAINS * CHAIN_COLS;        // per preparing team: Gram product, then Y
+    static constexpr uint32_t TMEM_COLS = D == 128 ? 512 : 256;
+    static_assert(PREP_COL + PREPS * C <= TMEM_COLS && SMEM <= 232448 && RING >= D * 128 * 4 + 2 * KB * D * 128, "tensor and shared memory");
+    static_assert(32 * 36 * 4 <= X_BYTES && 2 * TILE <= A_BYTES, "scratch");
+    // registers: 512 threads start with 128 each; the state rows (dk floats per thread) take what the preparation leaves
+    static constexpr bool SPLIT_REGS = D == 128;
+    static constexpr int PREP_REGS = 80, CHAIN_REGS = 176;
+    static_assert(!SPLIT_REGS || PREPS * PREP_REGS + CHAINS * CHAIN_REGS <= 4 * 128, "a split beyond the launch's registers waits for ever");
+};
+
+// MN-major operand, 128-byte swizzle: rows (K index) of 64 elements, 8-row groups 1024 bytes apart, blocks of 64
+// elements along M or N `block` bytes apart.
+__device__ __forceinline__ uint64_t umma_desc_mn(uint32_t smem_addr, uint32_t block) {
+    return (uint64_t)((smem_addr & 0x3FFFF) >> 4) | ((uint64_t)(block >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) |
+           ((uint64_t)2 << 61);
+}
+constexpr uint32_t A_MN_MAJOR = 1u << 15, B_MN_MAJOR = 1u << 16;     // instruction descriptor: operand is MN-major
+
+__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void proxy_fence() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+__device__ __forceinline__ void arrive(uint32_t bar) { asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory"); }
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+// tcgen05.mma kind::f16 and its commit, reached by a whole converged warp and issued by one elected lane: the operands stay
+// in uniform registers (issued from inside a one-thread branch an MMA cost 113 cycles, mostly moving descriptors over).
+__device__ __forceinline__ void mma_ts(uint32_t d, uint32_t ta, uint64_t bdesc, uint32_t idesc, bool acc) {
+    asm volatile(
+        "{\n\t.reg .pred p, e;\n\telect.sync _|e, 0xffffffff;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d), "r"(ta), "l"(bdesc), "r"(idesc), "r"((uint32_t)acc)
+        : "memory");
+}
+__device__ __forceinline__ void mma_ss(uint32_t d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, bool acc) {
+    asm volatile(
+        "{\n\t.reg .pred p, e;\n\telect.sync _|e, 0xffffffff;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"((uint32_t)acc)
+        : "memory");
+}
+__device__ __forceinline__ void mma_commit(uint32_t bar) {
+    asm volatile(
+        "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+        "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar)
+        : "memory");
+}
+
+// Two numbers times a power of two as fp16 numbers hi + lo, packed.  (Rounding hi to a fixed grid instead would make sums
+// of hi x hi products exact, but leaves every lo as large as the row's largest element allows: 4x the error.)
+__device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t& lo) {
+    hi = pack_f16x2(a, b);
+    const float2 h = __half22float2(*reinterpret_cast<const __half2*>(&hi));
+    lo = pack_f16x2(a - h.x, b - h.y);
+}
+__device__ __forceinline__ void split16(const float* x, float scale, uint32_t* hi, uint32_t* lo) {
+    const float2 sc = make_float2(scale, scale);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        const float2 y = __fmul2_rn(make_float2(x[2 * e], x[2 * e + 1]), sc);
+        hi[e] = pack_f16x2(y.x, y.y);
+        const float2 h = __half22float2(*reinterpret_cast<const __half2*>(&hi[e]));
+        const float2 l = __fadd2_rn(y, make_float2(-h.x, -h.y));
+        lo[e] = pack_f16x2(l.x, l.y);
+    }
+}
+// ... as one K step of a tensor-memory A operand: columns [0, 8) hi, [8, 16) lo
+__device__ __forceinline__ void split_to_tmem(uint32_t taddr, const float* x, float scale) {
+    uint32_t w[16];
+    split16(x, scale, w, w + 8);
+    tmem_st16(taddr, w);
+}
+
+// acc[r] = sum over l < n of rows[r][l] cols[l]: eight rows (pitch AP, read as broadcast vectors) times this lane's column
+__device__ __forceinline__ void rows8(float* acc, const float* rows, const float* cols, int pitch, int n) {
+#pragma unroll
+    for (int r = 0; r < 8; ++r) acc[r] = 0.f;
+#pragma unroll 2
+    for (int l = 0; l < n; l += 4) {
+        const float t0 = cols[l * pitch], t1 = cols[(l + 1) * pitch], t2 = cols[(l + 2) * pitch], t3 = cols[(l + 3) * pitch];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            const float4 q = *reinterpret_cast<const float4*>(rows + r * AP + l);
+            acc[r] = fmaf(q.x, t0, fmaf(q.y, t1, fmaf(q.z, t2, fmaf(q.w, t3, acc[r]))));
+        }
+    }
+}
+
+template <int D, typename T>
+__global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(const PrefillArgs a) {
+    using Z = Shape<D, T>;
+    constexpr int KB = Z::KB, PK = Z::PK, KS = (D < 64 ? D : 64) / 16;        // K steps of 16 per block of 64
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+    uint8_t* y_ring = smem + KV_STAGES * Z::KV_BYTES;
+    uint8_t* prep_s = smem + Z::RING;                                         // per preparing team: matrix / T', scratch
+    float* tok_s = reinterpret_cast<float*>(prep_s + Z::PREPS * (Z::A_BYTES + Z::X_BYTES));
+    float* coef_s = tok_s + Z::PREPS * (Z::TOK_BYTES / 4);
+    float* hinv_s = coef_s + Y_STAGES * (Z::COEF_BYTES / 4);                  // [128] what undoes the scales of the rows handed on
+    uint64_t* bars = reinterpret_cast<uint64_t*>(hinv_s + 128);
+    auto bar_full = [&](int s) { return smem_u32(bars + s); };                // Y stage s prepared
+    auto bar_yfree = [&](int s) { return smem_u32(bars + 2 + s); };           // Y stage / key and value stage read out
+    auto bar_kvfree = [&](int s) { return smem_u32(bars + 4 + s); };
+    auto bar_prep = [&](int w) { return smem_u32(bars + 7 + w); };            // a preparing team's MMAs complete
+    auto bar_chain = [&](int c) { return smem_u32(bars + 9 + c); };           // a chain's
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 12);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+    const int rank = blockIdx.x, P = gridDim.x, h = blockIdx.y;               // segment of the prompt, segments, head
+    const int total = (a.n_tokens + C - 1) / C;
+    const int c_begin = rank == 0 ? 0 : a.first + (rank - 1) * a.rest;
+    const int n = max(0, min(total, rank == 0 ? a.first : c_begin + a.rest) - c_begin);   // chunks of this CTA
+    const bool has_m = rank > 0;
+
+    if (tid == 0) {
+        const int chains = D == 128 && has_m ? 2 : 1;
+        for (int s = 0; s < Y_STAGES; ++s) {
+            mbar_init(bar_full(s), 128);                                      // the preparing threads
+            mbar_init(bar_yfree(s), chains);                                  // the chains' commits
+        }
+        for (int s = 0; s < KV_STAGES; ++s) mbar_init(bar_kvfree(s), chains);
+        for (int w = 0; w < Z::PREPS; ++w) mbar_init(bar_prep(w), 1);
+        for (int c = 0; c < Z::CHAINS; ++c) mbar_init(bar_chain(c), 1);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(Z::TMEM_COLS) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+
+    bool fail = false;
+    // bounded wait that also gives up as soon as another role has
+    auto wait = [&](uint32_t bar, uint32_t parity) {
+        for (int i = 0; i < sm100::WAIT_LIMIT; ++i) {
+            if (sm100::mbar_try_wait(bar, parity)) return;
+            if ((i & 63) == 63 && *abort_flag) break;
+        }
+        fail = true;
+        *abort_flag = 1;
+    };
+
+    if (warp < 4 * Z::PREPS) {
+        // =============================== PREPARATION ===============================
+        // (two teams take the chunks in turn: each step of a chunk is bounded by the latency of its own dependent chain)
+        if constexpr (Z::SPLIT_REGS) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(Z::PREP_REGS));
+        const int team = warp >> 2, w4 = warp & 3, pt = tid & 127;
+        float* A_s = reinterpret_cast<float*>(prep_s + team * (Z::A_BYTES + Z::X_BYTES));       // [C][AP], later T'
+        uint8_t* T_s = reinterpret_cast<uint8_t*>(A_s);
+        float* X_s = reinterpret_cast<float*>(T_s + Z::A_BYTES);                                // [32][36]
+        float* alpha_s = tok_s + team * (Z::TOK_BYTES / 4);
+        float *kinv_s = alpha_s + C, *w_s = kinv_s + C, *max_s = w_s + C;
+        const uint32_t acc_at = tmem_base + Z::PREP_COL + team * C;
+        constexpr int VEC = Vec16<T>::N, CPR = D / VEC, LR = CPR < 8 ? CPR : 8;      // 16-byte chunks and lanes per key row
+        constexpr int ROWS = 128 / LR, PASSES = C / ROWS, NC = CPR / LR;
+        constexpr int BATCH = PASSES * NC > 8 ? 8 / NC : PASSES;                      // passes whose loads are in flight together
+        const T* kp = static_cast<const T*>(a.k) + (long long)h * D;
+        const T* vp = static_cast<const T*>(a.v) + (long long)h * D;
+        const long long row_stride = (long long)a.H * D;
+        auto gate_of = [&](const float* g, int t, float pad) { return t < a.n_tokens ? __ldg(g + (long long)t * a.H + h) : pad; };
+        float alpha_next = 1.f, beta_next = 0.f;
+        if (team < n && pt < C) {
+            alpha_next = gate_of(a.alpha, (c_begin + team) * C + pt, 1.f);
+            beta_next = gate_of(a.beta, (c_begin + team) * C + pt, 0.f);
+        }
+        uint32_t phase = 0;
+        for (int i = team; i < n; i += Z::PREPS) {
+            const int s = i % Y_STAGES, use = i / Y_STAGES, kvs = i % KV_STAGES, t0 = (c_begin + i) * C;
+            uint8_t *K_s = smem + kvs * Z::KV_BYTES, *Y_s = y_ring + s * Z::Y_BYTES;
+            float* co = coef_s + s * (Z::COEF_BYTES / 4);
+            if (i >= KV_STAGES) wait(bar_kvfree(kvs), (i / KV_STAGES - 1) & 1);
+            // values as they are ([token][dv]); tokens beyond the prompt are zeros with alpha = 1, beta = 0: they change nothing
+            if constexpr (Z::V_STAGED) for (int x = pt; x < C * CPR; x += 128) {
+                const int row = x / CPR, ch = x % CPR, t = t0 + row;
+                const uint32_t bytes = t < a.n_tokens ? 16u : 0u;
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(K_s + Z::K_BYTES + row * (D * (int)sizeof(T)) + ch * 16)),
+                             "l"(vp + min(t, a.n_tokens - 1) * row_stride + ch * VEC), "r"(bytes)
+                             : "memory");
+            }
+            // keys as the K-major operand tile, every row with its own power of two
+            const int lr = pt % LR, row0 = pt / LR;
+#pragma unroll
+            for (int p0 = 0; p0 < PASSES; p0 += BATCH) {
+                uint4 raw[BATCH][NC];
+#pragma unroll
+                for (int p = 0; p < BATCH; ++p) {
+                    const int t = t0 + (p0 + p) * ROWS + row0;
+#pragma unroll
+                    for (int c = 0; c < NC; ++c)
+                        raw[p][c] = t < a.n_tokens ? __ldg(reinterpret_cast<const uint4*>(kp + t * row_stride) + c * LR + lr) : make_uint4(0, 0, 0, 0);
+                }
+#pragma unroll
+                for (int p = 0; p < BATCH; ++p) {
+                    const int row = (p0 + p) * ROWS + row0;
+                    float x[NC * VEC], m = 0.f;
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) Vec16<T>::unpack(raw[p][c], x + c * VEC);
+#pragma unroll
+                    for (int e = 0; e < NC * VEC; ++e) m = fmaxf(m, fabsf(x[e]));
+#pragma unroll
+                    for (int o = LR / 2; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+                    float sc, inv;
+                    pow2_scale(m, NARROW, sc, inv);
+                    if (lr == 0) kinv_s[row] = inv;
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) {
+                        const int el = (c * LR + lr) * VEC;
+                        uint8_t* dst = K_s + (el >> 6) * TILE + row * 128 + ((((el & 63) >> 3) ^ (row & 7)) << 4) + (el & 7) * 2;
+                        const float* y = x + c * VEC;
+                        if constexpr (VEC == 8) {        // bf16 keys: exact in one fp16 number
+                            *reinterpret_cast<uint4*>(dst) = make_uint4(pack_f16x2(y[0] * sc, y[1] * sc), pack_f16x2(y[2] * sc, y[3] * sc),
+                                                                        pack_f16x2(y[4] * sc, y[5] * sc), pack_f16x2(y[6] * sc, y[7] * sc));
+                        } else {
+                            uint32_t hi[2], lo[2];
+#pragma unroll
+                            for (int e = 0; e < 2; ++e)
+                                split2(y[2 * e] * sc, y[2 * e + 1] * sc, hi[e], lo[e]);
+                            *reinterpret_cast<uint2*>(dst) = make_uint2(hi[0], hi[1]);
+                            *reinterpret_cast<uint2*>(dst + KB * TILE) = make_uint2(lo[0], lo[1]);
+                        }
+                    }
+                }
+            }
+            const float alpha = alpha_next, beta = beta_next;
+            if (pt < C) {
+                alpha_s[pt] = alpha;
+                if (i + Z::PREPS < n) {
+                    alpha_next = gate_of(a.alpha, t0 + Z::PREPS * C + pt, 1.f);
+                    beta_next = gate_of(a.beta, t0 + Z::PREPS * C + pt, 0.f);
+                }
+            }
+            proxy_fence();
+            tc_fence_before();
+            if (bar_or(1 + team, 128, fail ? 1 : 0)) { fail = true; break; }
+            if (w4 == 0) {          // Gram product of the (scaled) keys: rows 0 - 63 are wanted, 128 are computed
+                tc_fence_after();
+                const uint64_t kd = umma_desc(smem_u32(K_s));
+#pragma unroll 1
+                for (int t = PK == 2 ? 2 : 0; t >= 0; --t)                  // small terms first: (lo hi, hi lo,) hi hi
+#pragma unroll 1
+                    for (int kb = 0; kb < KB; ++kb)
+#pragma unroll
+                        for (int ks = 0; ks < KS; ++ks) {
+                            const int at = (kb * TILE + ks * 32) >> 4;
+                            mma_ss(acc_at, kd + (at + (t == 2 ? (KB * TILE) >> 4 : 0)), kd + (at + (t == 1 ? (KB * TILE) >> 4 : 0)), idesc_f16(C),
+                                   t != (PK == 2 ? 2 : 0) || kb || ks);
+                        }
+                mma_commit(bar_prep(team));
+            }
+            if (i + Z::PREPS < n) { // the lines of the team's next chunk into L2
+                constexpr int LINES = D * (int)sizeof(T) / 128 > 0 ? D * (int)sizeof(T) / 128 : 1;
+                for (int x = pt; x < 2 * C * LINES; x += 128) {
+                    const int row = (x >> 1) / LINES, ln = (x >> 1) % LINES, t = min(t0 + Z::PREPS * C + row, a.n_tokens - 1);
+                    const char* p = reinterpret_cast<const char*>(((x & 1) ? vp : kp) + t * row_stride) + ln * 128;
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+                }
+            }
+            wait(bar_prep(team), phase);
+            phase ^= 1;
+            tc_fence_after();
+            // A = beta_i (g_i / g_j) (k_i . k_j), row i by thread i; the gate products run from the right.  g = alpha_0 ...
+            // alpha_i; the other half of the threads takes the products of the gates behind the token.
+            float g = 1.f;
+            if (w4 >= 2) {
+                float gc = 1.f;
+#pragma unroll 2
+                for (int l = C - 4; l >= 0; l -= 4) {
+                    const float4 al = *reinterpret_cast<const float4*>(alpha_s + l);
+                    const int me = pt - C;
+                    if (l + 3 > me) gc *= al.w;
+                    if (l + 2 > me) gc *= al.z;
+                    if (l + 1 > me) gc *= al.y;
+                    if (l > me) gc *= al.x;
+                }
+                w_s[pt - C] = gc * kinv_s[pt - C];
+            } else {
+                const float coef = beta * kinv_s[pt];
+#pragma unroll 1
+                for (int cb = 3; cb >= 0; --cb) {
+                    uint32_t v[16];
+                    tmem_ld16(acc_at + cb * 16 + ((uint32_t)(w4 * 32) << 16), v);
+                    tc_wait_ld();
+#pragma unroll
+                    for (int e = 12; e >= 0; e -= 4) {
+                        const float4 al = *reinterpret_cast<const float4*>(alpha_s + cb * 16 + e), ki = *reinterpret_cast<const float4*>(kinv_s + cb * 16 + e);
+                        const float alv[4] = {al.x, al.y, al.z, al.w}, kiv[4] = {ki.x, ki.y, ki.z, ki.w};
+                        float row[4];
+#pragma unroll
+                        for (int f = 3; f >= 0; --f) {
+                            const int l = cb * 16 + e + f;
+                            row[f] = l < pt ? (coef * g) * (__uint_as_float(v[e + f]) * kiv[f]) : 0.f;
+                            g *= l <= pt ? alv[f] : 1.f;
+                        }
+                        *reinterpret_cast<float4*>(A_s + pt * AP + cb * 16 + e) = make_float4(row[0], row[1], row[2], row[3]);
+                    }
+                }
+                __syncwarp();
+                // T = (I + A)^-1 in place, from the diagonal out.  Blocks of 16, two per warp, one column per lane by forward
+                // substitution; then a warp's two blocks are joined, then the two warps': - T22 A21 T11 below the diagonal.
+                float* L = A_s + (w4 * 32) * (AP + 1) + (lane >> 4) * (16 * AP + 16);
+                const int col = lane & 15;
+                float x[16];
+#pragma unroll
+                for (int r = 0; r < 16; ++r) {
+                    float s0 = r == col ? 1.f : 0.f, s1 = 0.f;
+#pragma unroll
+                    for (int l = 0; l < r; l += 4) {
+                        const float4 q = *reinterpret_cast<const float4*>(L + r * AP + l);
+                        s0 = fmaf(-q.x, x[l], s0);
+                        if (l + 1 < r) s1 = fmaf(-q.y, x[l + 1], s1);
+                        if (l + 2 < r) s0 = fmaf(-q.z, x[l + 2], s0);
+                        if (l + 3 < r) s1 = fmaf(-q.w, x[l + 3], s1);
+                    }
+                    x[r] = s0 + s1;
+                }
+                __syncwarp();
+#pragma unroll
+                for (int r = 0; r < 16; ++r) L[r * AP + col] = x[r];
+                __syncwarp();
+                float* B21 = A_s + (w4 * 32) * (AP + 1) + (16 + (lane >> 4) * 8) * AP;       // eight rows of the lower block per half warp
+                float acc[8];
+                rows8(acc, B21, A_s + (w4 * 32) * (AP + 1) + col, AP, 16);
+#pragma unroll
+                for (int r = 0; r < 8; ++r) X_s[w4 * (16 * 20) + ((lane >> 4) * 8 + r) * 20 + col] = acc[r];
+                __syncwarp();
+                rows8(acc, B21 + 16, X_s + w4 * (16 * 20) + col, 20, 16);
+                __syncwarp();
+#pragma unroll
+                for (int r = 0; r < 8; ++r) B21[r * AP + col] = -acc[r];
+            }
+            tc_fence_before();
+            bar_or(1 + team, 128, 0);
+            {
+                float acc[8];
+                rows8(acc, A_s + (32 + 8 * w4) * AP, A_s + lane, AP, 32);
+#pragma unroll
+                for (int r = 0; r < 8; ++r) X_s[(8 * w4 + r) * 36 + lane] = acc[r];
+                bar_or(1 + team, 128, 0);
+                rows8(acc, A_s + (32 + 8 * w4) * AP + 32, X_s + lane, 36, 32);
+#pragma unroll
+                for (int r = 0; r < 8; ++r) A_s[(32 + 8 * w4 + r) * AP + lane] = -acc[r];
+            }
+            bar_or(1 + team, 128, 0);
+            if (i >= Y_STAGES) wait(bar_yfree(s), (use - 1) & 1);            // coefficients and Y go to the chunk's Y stage
+            // T'_ij = T_ji g_C / g_j (and the key's scale undone): row i by threads i and i + 64, as an operand tile (hi, lo)
+            {
+                const int ti = pt & 63, hf = pt >> 6;
+                const bool zero = hf == 0 && ti >= 32;
+                float t[32], m = 0.f;
+#pragma unroll
+                for (int j = 0; j < 32; ++j) {
+                    t[j] = zero ? 0.f : A_s[(32 * hf + j) * AP + ti] * w_s[32 * hf + j];
+                    m = fmaxf(m, fabsf(t[j]));
+                }
+                if (hf == 1) max_s[ti] = m;
+                bar_or(1 + team, 128, 0);
+                if (hf == 0) {
+                    m = fmaxf(m, max_s[ti]);
+                    float sc, inv;
+                    pow2_scale(m, NARROW, sc, inv);
+                    co[ti] = beta * inv;
+                    co[C + ti] = beta * g * kinv_s[ti] * inv;
+                    if (ti == C - 1) co[2 * C] = g;
+                    max_s[ti] = sc;
+                }
+                bar_or(1 + team, 128, 0);
+                const float sc = max_s[ti];
+#pragma unroll
+                for (int c = 0; c < 4; c += 2) {
+                    uint32_t hi[8], lo[8];
+                    split16(t + 8 * c, sc, hi, lo);
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        uint8_t* dst = T_s + ti * 128 + (((4 * hf + c + e) ^ (ti & 7)) << 4);
+                        *reinterpret_cast<uint4*>(dst) = make_uint4(hi[4 * e], hi[4 * e + 1], hi[4 * e + 2], hi[4 * e + 3]);
+                        *reinterpret_cast<uint4*>(dst + TILE) = make_uint4(lo[4 * e], lo[4 * e + 1], lo[4 * e + 2], lo[4 * e + 3]);
+                    }
+                }
+            }
+            proxy_fence();
+            bar_or(1 + team, 128, 0);
+            if (w4 == 0) {          // Y^T = K^T T'^T: lanes = dk, columns = tokens
+                tc_fence_after();
+                const uint64_t kd = umma_desc_mn(smem_u32(K_s), TILE), td = umma_desc(smem_u32(T_s));
+#pragma unroll 1
+                for (int t = PK; t >= 0; --t)                               // small terms first: (lo hi,) hi lo, hi hi
+#pragma unroll
+                    for (int ks = 0; ks < C / 16; ++ks)
+                        mma_ss(acc_at, kd + (t == 2 ? (KB * TILE) >> 4 : 0) + ((ks * 2048) >> 4), td + (t == 1 ? TILE >> 4 : 0) + ((ks * 32) >> 4),
+                               idesc_f16(C) | A_MN_MAJOR, t != PK || ks);
+                mma_commit(bar_prep(team));
+            }
+            wait(bar_prep(team), phase);
+            phase ^= 1;
+            tc_fence_after();
+#pragma unroll
+            for (int cb = 0; cb < 4; ++cb) {
+                uint32_t v[16], hi[8], lo[8];
+                tmem_ld16(acc_at + cb * 16 + ((uint32_t)(w4 * 32) << 16), v);
+                tc_wait_ld();
+#pragma unroll
+                for (int e = 0; e < 8; ++e) split2(__uint_as_float(v[2 * e]), __uint_as_float(v[2 * e + 1]), hi[e], lo[e]);
+                if (pt < D) {
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        uint8_t* dst = Y_s + pt * 128 + (((2 * cb + e) ^ (pt & 7)) << 4);
+                        *reinterpret_cast<uint4*>(dst) = make_uint4(hi[4 * e], hi[4 * e + 1], hi[4 * e + 2], hi[4 * e + 3]);
+                        *reinterpret_cast<uint4*>(dst + D * 128) = make_uint4(lo[4 * e], lo[4 * e + 1], lo[4 * e + 2], lo[4 * e + 3]);
+                    }
+                }
+            }
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            proxy_fence();
+            tc_fence_before();
+            arrive(bar_full(s));
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        bar_or(CTA_BARRIER, Z::THREADS, 0);                   // the chains take the rings' memory over
+        if (P > 1)
+            for (int p = 0; p < P; ++p) cluster_sync();       // (every thread of the cluster meets every one)
+    } else {
+
+    // =============================== STATE ROWS ===============================
+    // thread = one row: of S, of M (segments that do not start the prompt), or idle (dk <= 64)
+    if constexpr (Z::SPLIT_REGS) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(Z::CHAIN_REGS));
+    const int chain = (warp >> 2) - Z::PREPS, team = 1 + (warp >> 2);
+    const int r = (warp & 3) * 32 + lane;
+    const bool is_s = (D == 128 ? chain == 0 : r < D);
+    const bool is_m = has_m && (D == 128 ? chain == 1 : r >= D && r < 2 * D);
+    const int mrow = D == 128 ? r : r - D;
+    const uint32_t taddr = tmem_base + chain * Z::CHAIN_COLS + ((uint32_t)((warp & 3) * 32) << 16);
+    const uint32_t s_at = taddr, d_at = taddr + D;            // S operand / Delta Y ; S K^T / Delta operand
+    const uint32_t s_col = tmem_base + chain * Z::CHAIN_COLS, d_col = s_col + D;      // ... without the warp's lanes
+    const bool issuer = (warp & 3) == 0, leader = issuer && lane == 0;
+    uint32_t phase = 0;                                       // of the chain's barrier
+    float S[D];
+    float inv_row = 1.f;
+    auto store_operand = [&](float m) {                       // the row as the next product's A operand; m: its largest magnitude
+        float sc;
+        pow2_scale(m, WIDE, sc, inv_row);
+#pragma unroll
+        for (int b = 0; b < D / 16; ++b) split_to_tmem(s_at + 16 * b, S + 16 * b, sc);
+        tc_wait_st();
+        tc_fence_before();
+    };
+#pragma unroll
+    for (int d = 0; d < D; ++d) S[d] = is_m && d == mrow ? 1.f : 0.f;
+    if ((D < 128 || chain == 0 || has_m) && n > 0) {
+        store_operand(is_m ? 1.f : 0.f);
+        bar_or(team, 128, 0);
+        for (int i = 0; i < n; ++i) {
+            const int s = i % Y_STAGES, kvs = i % KV_STAGES;
+            const uint8_t *K_s = smem + kvs * Z::KV_BYTES, *Y_s = y_ring + s * Z::Y_BYTES;
+            const float* co = coef_s + s * (Z::COEF_BYTES / 4);
+            wait(bar_full(s), (i / Y_STAGES) & 1);
+            if (issuer) {                                     // S K^T, small terms first: (hi lo,) lo hi, hi hi
+                tc_fence_after();
+                const uint64_t kd = umma_desc(smem_u32(K_s));
+#pragma unroll 1
+                for (int t = PK; t >= 0; --t)
+#pragma unroll 1
+                    for (int kb = 0; kb < KB; ++kb)
+#pragma unroll
+                        for (int ks = 0; ks < KS; ++ks)
+                            mma_ts(d_col, s_col + (kb * 4 + ks) * 16 + (t == 1 ? 8 : 0), kd + (t == 2 ? (KB * TILE) >> 4 : 0) + ((kb * TILE + ks * 32) >> 4),
+                                   idesc_f16(C), t != PK || kb || ks);
+                mma_commit(bar_chain(chain));
+            }
+            wait(bar_chain(chain), phase);
+            phase ^= 1;
+            tc_fence_after();
+            // Delta (times what undoes Y's row scale), in place; S rows add beta v
+            const float neg = -inv_row, g_chunk = co[2 * C];
+            float m = 0.f;
+            auto delta = [&](auto with_v) {
+#pragma unroll 1
+                for (int b = 0; b < 4; ++b) {
+                    uint32_t v[16];
+                    tmem_ld16(d_at + 16 * b, v);
+                    float x[16];
+                    if constexpr (decltype(with_v)::value) {
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) {
+                            if constexpr (Z::V_STAGED) {
+                                const uint8_t* vp = K_s + Z::K_BYTES + ((16 * b + e) * D + r) * 2;
+                                x[e] = __uint_as_float((uint32_t)*reinterpret_cast<const uint16_t*>(vp) << 16);
+                            } else {
+                                const int t = min((c_begin + i) * C + 16 * b + e, a.n_tokens - 1);
+                                x[e] = __ldg(static_cast<const float*>(a.v) + ((long long)t * a.H + h) * D + r);
+                            }
+                        }
+                    }
+                    tc_wait_ld();
+#pragma unroll
+                    for (int e = 0; e < 16; e += 4) {
+                        const float4 cc = *reinterpret_cast<const float4*>(co + C + 16 * b + e);
+                        const float c4[4] = {cc.x, cc.y, cc.z, cc.w};
+                        float b4[4];
+                        if constexpr (decltype(with_v)::value) {
+                            const float4 bb = *reinterpret_cast<const float4*>(co + 16 * b + e);
+                            b4[0] = bb.x; b4[1] = bb.y; b4[2] = bb.z; b4[3] = bb.w;
+                        }
+#pragma unroll
+                        for (int f = 0; f < 4; f += 2) {
+                            float2 y = __fmul2_rn(make_float2(__uint_as_float(v[e + f]), __uint_as_float(v[e + f + 1])), make_float2(neg, neg));
+                            const float2 c2 = make_float2(c4[f], c4[f + 1]);
+                            if constexpr (decltype(with_v)::value)
+                                y = __ffma2_rn(c2, y, __fmul2_rn(make_float2(b4[f], b4[f + 1]), make_float2(x[e + f], x[e + f + 1])));
+                            else
+                                y = __fmul2_rn(c2, y);
+                            m = fmaxf(fmaxf(m, fabsf(y.x)), fabsf(y.y));
+                            v[e + f] = __float_as_uint(y.x);
+                            v[e + f + 1] = __float_as_uint(y.y);
+                        }
+                    }
+                    tmem_st16(d_at + 16 * b, v);
+                }
+            };
+            if (is_s) delta(std::true_type{});
+            else delta(std::false_type{});
+            tc_wait_st();
+            float sc, inv_d;
+            pow2_scale(m, WIDE, sc, inv_d);
+#pragma unroll 1
+            for (int b = 0; b < 4; ++b) {
+                uint32_t v[16];
+                tmem_ld16(d_at + 16 * b, v);
+                tc_wait_ld();
+                float x[16];
+#pragma unroll
+                for (int e = 0; e < 16; ++e) x[e] = __uint_as_float(v[e]);
+                split_to_tmem(d_at + 16 * b, x, sc);
+            }
+            tc_wait_st();
+            tc_fence_before();
+            if (bar_or(team, 128, fail ? 1 : 0)) { fail = true; break; }
+            if (issuer) {                                     // Delta Y: lo hi, hi lo, hi hi, over the S operand (read by now)
+                tc_fence_after();
+                const uint64_t yd = umma_desc(smem_u32(Y_s));
+#pragma unroll 1
+                for (int t = 2; t >= 0; --t)
+#pragma unroll
+                    for (int ks = 0; ks < C / 16; ++ks)
+                        mma_ts(s_col, d_col + ks * 16 + (t == 2 ? 8 : 0), yd + (t == 1 ? (D * 128) >> 4 : 0) + ((ks * 32) >> 4), idesc_f16(D), t != 2 || ks);
+                mma_commit(bar_chain(chain));
+                mma_commit(bar_yfree(s));                     // the stages' tiles are read; values and coefficients were before
+                mma_commit(bar_kvfree(kvs));
+            }
+            wait(bar_chain(chain), phase);
+            phase ^= 1;
+            tc_fence_after();
+            m = 0.f;
+#pragma unroll
+            for (int b = 0; b < D / 16; ++b) {
+                uint32_t v[16];
+                tmem_ld16(s_at + 16 * b, v);
+                tc_wait_ld();
+#pragma unroll
+                for (int e = 0; e < 16; e += 2) {
+                    S[16 * b + e] = fmaf(g_chunk, S[16 * b + e], __uint_as_float(v[e]) * inv_d);
+                    S[16 * b + e + 1] = fmaf(g_chunk, S[16 * b + e + 1], __uint_as_float(v[e + 1]) * inv_d);
+                    m = fmaxf(fmaxf(m, fabsf(S[16 * b + e])), fabsf(S[16 * b + e + 1]));
+                }
+            }
+            if (i + 1 < n) store_operand(m);
+            if (bar_or(team, 128, fail ? 1 : 0)) { fail = true; break; }
+        }
+    }
+    bar_or(CTA_BARRIER, Z::THREADS, 0);
+
+    // =============================== SEGMENTS IN ORDER ===============================
+    // S of the segments so far passes from CTA to CTA as the receiver's A operand (per row dk words in the order of the K
+    // steps, and what undoes the row's scale), written to the sender's shared memory and read over the cluster
+    uint4* hand_s = reinterpret_cast<uint4*>(smem);           // [dk / 4][128 rows]
+    uint8_t* M_s = smem + D * 128 * 4;                        // M_p as an MN-major B operand: [hi, lo][blocks of 64][dk rows][128 bytes]
+    auto hand_over = [&]() {
+        float m = 0.f, sc, inv;
+#pragma unroll
+        for (int d = 0; d < D; d += 2) m = fmaxf(fmaxf(m, fabsf(S[d])), fabsf(S[d + 1]));
+        pow2_scale(m, WIDE, sc, inv);
+        hinv_s[r] = inv;
+#pragma unroll
+        for (int b = 0; b < D / 16; ++b) {
+            uint32_t w[16];
+            split16(S + 16 * b, sc, w, w + 8);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) hand_s[(4 * b + q) * 128 + r] = make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+        }
+    };
+    if (P > 1) {
+        if (has_m && (D < 128 || chain == 1)) {               // M with one scale for all its rows (every warp of the team comes along)
+            float m = 0.f, sc, inv;
+            if (is_m) {
+#pragma unroll
+                for (int d = 0; d < D; d += 2) m = fmaxf(fmaxf(m, fabsf(S[d])), fabsf(S[d + 1]));
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+            if (lane == 0) tok_s[warp & 3] = m;
+            bar_or(team, 128, 0);
+            m = fmaxf(fmaxf(tok_s[0], tok_s[1]), fmaxf(tok_s[2], tok_s[3]));
+            pow2_scale(m, WIDE, sc, inv);
+            if (leader) tok_s[4] = inv;
+            if (is_m) {
+#pragma unroll
+                for (int b = 0; b < D / 16; ++b) {
+                    uint32_t hi[8], lo[8];
+                    split16(S + 16 * b, sc, hi, lo);
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const int ch = 2 * b + e;
+                        uint8_t* dst = M_s + (ch >> 3) * (D * 128) + mrow * 128 + (((ch & 7) ^ (mrow & 7)) << 4);
+                        *reinterpret_cast<uint4*>(dst) = make_uint4(hi[4 * e], hi[4 * e + 1], hi[4 * e + 2], hi[4 * e + 3]);
+                        *reinterpret_cast<uint4*>(dst + KB * D * 128) = make_uint4(lo[4 * e], lo[4 * e + 1], lo[4 * e + 2], lo[4 * e + 3]);
+                    }
+                }
+            }
+            proxy_fence();
+        }
+        if (rank == 0 && is_s) hand_over();
+        // (one chain holds the S operand; its product lands in the other chain's columns, or beside it)
+        const uint32_t o_at = D == 128 ? taddr + Z::CHAIN_COLS : d_at, o_col = D == 128 ? s_col + Z::CHAIN_COLS : d_col;
+        for (int p = 1; p < P; ++p) {
+            cluster_sync();
+            if (rank != p || chain != 0) continue;
+            const int row = is_s ? r : 0;                     // (rows that are none come along with row 0's data)
+            uint32_t peer, peer_inv;
+            asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer) : "r"(smem_u32(hand_s + row)), "r"(p - 1));
+            asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer_inv) : "r"(smem_u32(hinv_s + row)), "r"(p - 1));
+            float inv;
+            asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(inv) : "r"(peer_inv) : "memory");
+#pragma unroll 2
+            for (int b = 0; b < D / 16; ++b) {
+                uint32_t w[16];
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    asm volatile("ld.shared::cluster.v4.b32 {%0, %1, %2, %3}, [%4];"
+                                 : "=r"(w[4 * q]), "=r"(w[4 * q + 1]), "=r"(w[4 * q + 2]), "=r"(w[4 * q + 3])
+                                 : "r"(peer + (4 * b + q) * (128 * 16))
+                                 : "memory");
+                tmem_st16(s_at + 16 * b, w);
+            }
+            tc_wait_st();
+            tc_fence_before();
+            bar_or(team, 128, 0);
+            inv *= tok_s[4];
+            if (issuer) {
+                tc_fence_after();
+                const uint64_t md = umma_desc_mn(smem_u32(M_s), D * 128);
+#pragma unroll 1
+                for (int t = 2; t >= 0; --t)                  // lo hi, hi lo, hi hi
+#pragma unroll
+                    for (int ks = 0; ks < D / 16; ++ks)
+                        mma_ts(o_col, s_col + ks * 16 + (t == 2 ? 8 : 0), md + (t == 1 ? (KB * D * 128) >> 4 : 0) + ((ks * 2048) >> 4),
+                               idesc_f16(D) | B_MN_MAJOR, t != 2 || ks);
+                mma_commit(bar_chain(0));
+            }
+            wait(bar_chain(0), phase);
+            phase ^= 1;
+            tc_fence_after();
+#pragma unroll
+            for (int b = 0; b < D / 16; ++b) {
+                uint32_t v[16];
+                tmem_ld16(o_at + 16 * b, v);
+                tc_wait_ld();
+#pragma unroll
+                for (int e = 0; e < 16; ++e) S[16 * b + e] = fmaf(__uint_as_float(v[e]), inv, S[16 * b + e]);
+            }
+            tc_fence_before();
+            if (p + 1 < P && is_s) hand_over();
+        }
+        cluster_sync();                                       // nobody leaves while its shared memory may be read
+    }
+
+    // =============================== RESULT ===============================
+    if (rank == P - 1 && chain == 0) {
+        float m = 0.f;
+        if (is_s) {
+            float4* dst = reinterpret_cast<float4*>(a.slot + ((long long)h * D + r) * D);
+#pragma unroll
+            for (int d = 0; d < D; d += 4) dst[d / 4] = make_float4(S[d], S[d + 1], S[d + 2], S[d + 3]);
+#pragma unroll
+            for (int d = 0; d < D; ++d) m = fmaxf(m, fabsf(S[d]));
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        if (lane == 0) tok_s[warp & 3] = m;
+        bar_or(team, 128, 0);
+        m = fmaxf(fmaxf(tok_s[0], tok_s[1]), fmaxf(tok_s[2], tok_s[3]));
+        float sc, inv;
+        pow2_scale(m, 11, sc, inv);                           // the head's operand scale (see Layout::s0_scale)
+        if (leader) a.scale_out[h] = sc;
+        if (a.s0_f16) {                                       // the tiled kernel's operand: value rows padded to 128
+            char* dst = reinterpret_cast<char*>(a.s0_f16) + (long long)h * (128 * D * 2) + r * 128;
+#pragma unroll
+            for (int ch = 0; ch < D / 8; ++ch) {
+                uint4 w = make_uint4(0u, 0u, 0u, 0u);
+                if (is_s) {
+                    const float* x = S + 8 * ch;
+                    w = make_uint4(pack_f16x2(x[0] * sc, x[1] * sc), pack_f16x2(x[2] * sc, x[3] * sc), pack_f16x2(x[4] * sc, x[5] * sc),
+                                   pack_f16x2(x[6] * sc, x[7] * sc));
+                }
+                *reinterpret_cast<uint4*>(dst + (ch >> 3) * (128 * 128) + (((ch & 7) ^ (r & 7)) << 4)) = w;
+            }
+        }
+    }
+    }   // chains
+    if (fail && atomicCAS(a.status, ONELA_OK, ONELA_E_TIMEOUT) == ONELA_OK) a.status[1] = (int32_t)(blockIdx.x + gridDim.x * blockIdx.y);
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(Z::TMEM_COLS) : "memory");
+}
+
+// How a prompt of `chunks` chunks is cut: P segments (a cluster of P CTAs per head), the first of `first` chunks, the
+// others of `rest`.  Cost model, in chunk steps of a segment that carries M: a chunk of the first segment counts FIRST, one
+// fold at the end FOLD, and `resident[P]` clusters of P run at a time.
+struct Cut {
+    int P, first, rest;
+};
+Cut cut_prompt(int chunks, int H, bool two_chains, const int* resident) {
+    const double first_cost = two_chains ? 0.95 : 1.0, fold = 0.8;
+    Cut best{1, chunks, 0};
+    double best_cost = 1e30;
+    for (int P = 1; P <= MAX_SEGMENTS && P <= chunks; ++P) {
+        if (resident[P] < 1) continue;
+        int rest = 0, first = chunks;
+        if (P > 1) {
+            rest = std::max(1, (int)(chunks / (P - 1 + 1.0 / first_cost) + 0.5));
+            while (rest > 1 && (P - 1) * rest >= chunks) --rest;
+            first = chunks - (P - 1) * rest;
+            if (first < 1) continue;
+        }
+        const double waves = (double)((H + resident[P] - 1) / resident[P]);
+        const double cost = waves * (std::max(first * first_cost, (double)rest) + (P - 1) * fold + 2.0);
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = Cut{P, first, rest};
+        }
+    }
+    return best;
+}
+
+template <int D, typename T>
+cudaError_t launch_dt(const PrefillArgs& args, cudaStream_t stream) {
+    using Z = Shape<D, T>;
+    auto kern = prefill_chunk_kernel<D, T>;
+    // One-time set-up per instantiation and device: the shared-memory limit, and how many clusters of each size fit.
+    constexpr int MAX_DEVICES = 64;
+    static std::mutex setup_mutex;
+    static int resident_of[MAX_DEVICES][MAX_SEGMENTS + 1] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEVICES) return cudaErrorInvalidDevice;
+    cudaLaunchConfig_t cfg = {};
+    cfg.blockDim = dim3(Z::THREADS);
+    cfg.dynamicSmemBytes = Z::SMEM;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int* resident = resident_of[dev];
+    {
+        std::lock_guard<std::mutex> lock(setup_mutex);
+        if (resident[0] == 0) {
+            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Z::SMEM);
+            if (e != cudaSuccess) return e;
+            for (int P = 1; P <= MAX_SEGMENTS; ++P) {
+                attr[0].val.clusterDim.x = P;
+                cfg.gridDim = dim3(P, 1);
+                int clusters = 0;
+                e = cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg);
+                if (e != cudaSuccess) return e;
+                resident[P] = clusters;
+            }
+            resident[0] = 1;
+        }
+    }
+    PrefillArgs a = args;
+    const Cut cut = cut_prompt((a.n_tokens + C - 1) / C, a.H, Z::CHAINS == 2, resident);
+    a.first = cut.first;
+    a.rest = cut.rest;
+    attr[0].val.clusterDim.x = cut.P;
+    cfg.gridDim = dim3(cut.P, a.H);
+    return cudaLaunchKernelEx(&cfg, kern, a);
+}
+
+template <int D>
+cudaError_t launch_d(const PrefillArgs& a, int32_t rec_dtype, cudaStream_t stream) {
+    return rec_dtype == ONELA_DTYPE_BF16 ? launch_dt<D, __nv_bfloat16>(a, stream) : launch_dt<D, float>(a, stream);
+}
+
+}  // namespace
+
+cudaError_t launch_prefill(const void* k, const void* v, const float* alpha, const float* beta, float* slot, float* scale_out,
+                           uint16_t* s0_f16, int32_t* status, int32_t n_tokens, int32_t H, int32_t dk, int32_t dv, int32_t rec_dtype,
+                           bool* supported, cudaStream_t stream) {
+    const PrefillArgs a{k, v, alpha, beta, slot, scale_out, s0_f16, status, n_tokens, H, 0, 0};
+    *supported = true;
+    if (dk == 32 && dv == 32) return launch_d<32>(a, rec_dtype, stream);
+    if (dk == 64 && dv == 64) return launch_d<64>(a, rec_dtype, stream);
+    if (dk == 128 && dv == 128) return launch_d<128>(a, rec_dtype, stream);
+    *supported = false;
+    return cudaErrorInvalidValue;
+}
+
+}  // namespace onela

@@ -1,9 +1,8 @@
 // Shared-state store and record arena kernels.
 //  - append: copy one decode call's (k, v, alpha, beta) into the append-only arena (paper Section 3.3:
 //    records are written once to the slots of the current step and never relocated).
-//  - store_state / prefill: fill the store slot of one (request, layer) with S_0 (Section 3.2: the
-//    post-prefill state is stored once per request), either from a caller tensor or by running Eq. 1
-//    from the zero state over the prompt.
+//  - store_state: fill the store slot of one (request, layer) with S_0 (Section 3.2: the post-prefill state is
+//    stored once per request) from a caller tensor.
 #include <cuda_fp16.h>
 
 #include "onela_internal.h"
@@ -34,13 +33,6 @@ __global__ void __launch_bounds__(256) append_kernel(const char* __restrict__ k,
     for (int c = lane; c < nk + nv; c += 32) dst[c] = (c < nk) ? __ldg(ksrc + c) : __ldg(vsrc + (c - nk));
     if (lane == 0) gate_plane[dst_row] = make_float2(__ldg(alpha + row), __ldg(beta + row));
 }
-
-template <typename T>
-__device__ __forceinline__ float to_float(T x);
-template <>
-__device__ __forceinline__ float to_float<float>(float x) { return x; }
-template <>
-__device__ __forceinline__ float to_float<__nv_bfloat16>(__nv_bfloat16 x) { return __bfloat162float(x); }
 
 // The operand scale of a head (Layout::s0_scale) from the largest magnitude of its state.
 __device__ __forceinline__ float operand_scale(float peak) {
@@ -74,88 +66,6 @@ __global__ void __launch_bounds__(256) store_state_kernel(const float4* __restri
     }
     peak = block_max(peak);
     if (threadIdx.x == 0) scale_out[blockIdx.x] = operand_scale(peak);
-}
-
-// Eq. 1 from the zero state over the prompt, one CTA per head, thread i owns row i of S in registers.
-template <int DK, int DV, typename T>
-__global__ void __launch_bounds__(DV) prefill_kernel(const T* __restrict__ k, const T* __restrict__ v,
-                                                     const float* __restrict__ alpha, const float* __restrict__ beta,
-                                                     float* __restrict__ slot, float* __restrict__ scale_out,
-                                                     int32_t n_tokens, int32_t H) {
-    __shared__ __align__(16) float k_s[2][DK];
-    const int h = blockIdx.x, i = threadIdx.x;
-    float S[DK];
-#pragma unroll
-    for (int j = 0; j < DK; ++j) S[j] = 0.f;
-    constexpr int KPT = (DK + DV - 1) / DV;  // k elements each thread stages per token
-    float kn[KPT], vn = 0.f, an = 1.f, bn = 0.f;
-    auto fetch = [&](int t) {
-        const long long row = (long long)t * H + h;
-#pragma unroll
-        for (int c = 0; c < KPT; ++c) {
-            const int j = i + c * DV;
-            kn[c] = (j < DK) ? to_float(k[row * DK + j]) : 0.f;
-        }
-        vn = to_float(v[row * DV + i]);
-        an = __ldg(alpha + row);
-        bn = __ldg(beta + row);
-    };
-    auto stage = [&](int buf) {
-#pragma unroll
-        for (int c = 0; c < KPT; ++c) {
-            const int j = i + c * DV;
-            if (j < DK) k_s[buf][j] = kn[c];
-        }
-    };
-    if (n_tokens > 0) { fetch(0); stage(0); }
-    __syncthreads();
-    for (int t = 0; t < n_tokens; ++t) {
-        const float vt = vn, a = an, b = bn;
-        if (t + 1 < n_tokens) fetch(t + 1);
-        const float4* kk = reinterpret_cast<const float4*>(k_s[t & 1]);
-        float u0 = 0.f, u1 = 0.f, u2 = 0.f, u3 = 0.f;
-#pragma unroll
-        for (int j = 0; j < DK / 4; ++j) {
-            const float4 x = kk[j];
-            u0 = fmaf(S[4 * j + 0], x.x, u0);
-            u1 = fmaf(S[4 * j + 1], x.y, u1);
-            u2 = fmaf(S[4 * j + 2], x.z, u2);
-            u3 = fmaf(S[4 * j + 3], x.w, u3);
-        }
-        const float u = (u0 + u1) + (u2 + u3);
-        const float delta = b * (vt - a * u);   // Eq. 2's delta_t
-#pragma unroll
-        for (int j = 0; j < DK / 4; ++j) {
-            const float4 x = kk[j];
-            S[4 * j + 0] = fmaf(a, S[4 * j + 0], delta * x.x);
-            S[4 * j + 1] = fmaf(a, S[4 * j + 1], delta * x.y);
-            S[4 * j + 2] = fmaf(a, S[4 * j + 2], delta * x.z);
-            S[4 * j + 3] = fmaf(a, S[4 * j + 3], delta * x.w);
-        }
-        if (t + 1 < n_tokens) stage((t + 1) & 1);
-        __syncthreads();
-    }
-    float* dst = slot + (long long)h * DV * DK;
-    float peak = 0.f;
-#pragma unroll
-    for (int j = 0; j < DK; ++j) {
-        dst[(long long)i * DK + j] = S[j];
-        peak = fmaxf(peak, fabsf(S[j]));
-    }
-    peak = block_max(peak);
-    if (i == 0) scale_out[h] = operand_scale(peak);
-}
-
-template <int DK, int DV>
-cudaError_t prefill_dispatch(const void* k, const void* v, const float* alpha, const float* beta, float* slot,
-                             float* scale_out, int32_t n_tokens, int32_t H, int32_t rec_dtype, cudaStream_t stream) {
-    if (rec_dtype == ONELA_DTYPE_BF16)
-        prefill_kernel<DK, DV, __nv_bfloat16><<<H, DV, 0, stream>>>(
-            static_cast<const __nv_bfloat16*>(k), static_cast<const __nv_bfloat16*>(v), alpha, beta, slot, scale_out, n_tokens, H);
-    else
-        prefill_kernel<DK, DV, float><<<H, DV, 0, stream>>>(static_cast<const float*>(k), static_cast<const float*>(v),
-                                                           alpha, beta, slot, scale_out, n_tokens, H);
-    return cudaGetLastError();
 }
 
 }  // namespace
@@ -213,17 +123,6 @@ cudaError_t launch_store_state(const float* S0_in, float* slot, float* scale_out
 
 cudaError_t launch_export_state(const float* slot, float* S0_out, int32_t H, int32_t dk, int32_t dv, cudaStream_t stream) {
     return cudaMemcpyAsync(S0_out, slot, (size_t)H * dk * dv * sizeof(float), cudaMemcpyDeviceToDevice, stream);
-}
-
-cudaError_t launch_prefill(const void* k, const void* v, const float* alpha, const float* beta, float* slot,
-                           float* scale_out, int32_t n_tokens, int32_t H, int32_t dk, int32_t dv, int32_t rec_dtype,
-                           bool* supported, cudaStream_t stream) {
-    *supported = true;
-    if (dk == 32 && dv == 32) return prefill_dispatch<32, 32>(k, v, alpha, beta, slot, scale_out, n_tokens, H, rec_dtype, stream);
-    if (dk == 64 && dv == 64) return prefill_dispatch<64, 64>(k, v, alpha, beta, slot, scale_out, n_tokens, H, rec_dtype, stream);
-    if (dk == 128 && dv == 128) return prefill_dispatch<128, 128>(k, v, alpha, beta, slot, scale_out, n_tokens, H, rec_dtype, stream);
-    *supported = false;
-    return cudaErrorInvalidValue;
 }
 
 }  // namespace onela
