@@ -25,12 +25,11 @@
  *    host object released by onela_destroy(), which never touches the workspace.
  *  - `stream` is a cudaStream_t passed as void*.  Every call is asynchronous and ordered on that
  *    stream; inputs may be reused as soon as the stream has passed the call.  Only
- *    onela_poll_device_status() synchronises.  The warp-specialised tensor-core decode kernel is launched with programmatic
- *    stream serialisation: it may start while the previous kernel of the stream drains, but it reads only its
- *    own shared-state store before it has waited for that kernel's completion, so stream order holds for every
- *    tensor the caller passes.  A caller kernel that follows it AND is itself launched with programmatic stream
- *    serialisation must wait for its grid dependency before it reads the decode outputs, as that launch mode
- *    requires of any kernel.
+ *    onela_poll_device_status() synchronises.  Most kernels are launched with programmatic stream serialisation:
+ *    they may start while the previous kernel of the stream drains, but read only the library's own shared-state
+ *    store before they have waited for that kernel's completion, so stream order holds for every tensor the caller
+ *    passes.  A caller kernel that follows one AND is itself launched with programmatic stream serialisation must
+ *    wait for its grid dependency before it reads the outputs, as that launch mode requires of any kernel.
  *  - Tensors are dense, row-major, last index contiguous.  q, k, v use cfg.rec_dtype, outputs
  *    cfg.out_dtype, gates and S_0 are fp32.  All tensor pointers must be 16-byte aligned.
  *  - Errors the host can see return a negative status and launch nothing.  Errors only the device can
@@ -234,8 +233,8 @@ onela_status onela_decode_step(onela_ctx* ctx, int32_t req_begin, int32_t req_co
  * folded as each beam's newest record, and written to the arena by the same kernel, so they cross HBM
  * once instead of three times.  Same arguments, checks and call-order rules as the two calls it replaces
  * (it counts as the layer's one append of this decode call; decode_step may still be called afterwards).
- * One launch on both tensor-core kernels; where a CUDA-core kernel runs (dk = dv = 32, ONELA_FLAG_FORCE_GENERIC)
- * the call is the copy kernel followed by the decode kernel. */
+ * One launch on every kernel but one: grouped value heads on CUDA cores (ONELA_FLAG_FORCE_GENERIC) take the copy
+ * kernel followed by the decode kernel. */
 onela_status onela_append_decode_step(onela_ctx* ctx, int32_t req_begin, int32_t req_count, int32_t layer,
                                       const void* k_dev, const void* v_dev, const float* alpha_dev,
                                       const float* beta_dev, const void* q_dev, void* out_dev, void* stream);

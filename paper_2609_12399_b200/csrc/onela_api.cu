@@ -76,6 +76,7 @@ Layout carve(const onela_config& c, char* base) {
     l.unode = reinterpret_cast<uint8_t*>(take((size_t)c.num_requests * ONELA_UNODE_CAP * 16));
     if (uses_tiled_kernel(c))
         l.s0_f16 = reinterpret_cast<uint16_t*>(take((size_t)c.num_requests * c.num_layers * Hv * s0_f16_head_bytes(c.dk, c.dv)));
+    l.level_base = reinterpret_cast<int32_t*>(take((size_t)c.num_requests * c.max_steps * sizeof(int32_t)));
     l.total_bytes = off;
     return l;
 }
@@ -104,14 +105,8 @@ struct onela_ctx {
     long long s0_layer_floats() const { return (long long)Hv() * cfg.dv * cfg.dk; }
     float* s0_slot(int r, int l) const { return lay.s0 + ((long long)r * cfg.num_layers + l) * s0_layer_floats(); }
     float* s0_scale_slot(int r, int l) const { return lay.s0_scale + ((long long)r * cfg.num_layers + l) * Hv(); }
-    uint16_t* s0_f16_slot(int r, int l) const {       // tiled kernel's operand copy of (request, layer, head 0)
-        return lay.s0_f16 + ((long long)r * cfg.num_layers + l) * Hv() * (long long)(s0_f16_head_bytes(cfg.dk, cfg.dv) / 2);
-    }
-    // after a state write: the tiled kernel's operand copy of the n_heads states from (r, l) on
-    cudaError_t pack_states(int r, int l, long long n_heads, cudaStream_t s) {
-        if (!tiled_tc) return cudaSuccess;
-        launches++;
-        return launch_pack_state(s0_slot(r, l), s0_scale_slot(r, l), s0_f16_slot(r, l), n_heads, cfg.dk, cfg.dv, s);
+    uint16_t* s0_f16_slot(int r, int l) const {       // tiled kernel's operand copy of (request, layer, head 0), null without one
+        return !tiled_tc ? nullptr : lay.s0_f16 + ((long long)r * cfg.num_layers + l) * Hv() * (long long)(s0_f16_head_bytes(cfg.dk, cfg.dv) / 2);
     }
     int32_t* table_cur(int r) const {
         const int d = req[r].depth;
@@ -276,11 +271,10 @@ onela_status onela_init_shared_state(onela_ctx* ctx, int32_t request, int32_t la
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if ((st = ctx->prepare(s)) != ONELA_OK) return st;
     if (!ctx->dry()) {
-        if (launch_store_state(S0_dev, ctx->s0_slot(request, layer), ctx->s0_scale_slot(request, layer), ctx->Hv(),
-                               ctx->cfg.dk, ctx->cfg.dv, s) != cudaSuccess)
+        if (launch_store_state(S0_dev, ctx->s0_slot(request, layer), ctx->s0_scale_slot(request, layer), ctx->s0_f16_slot(request, layer),
+                               ctx->Hv(), ctx->cfg.dk, ctx->cfg.dv, s) != cudaSuccess)
             return ONELA_E_CUDA;
         ctx->launches++;
-        if (ctx->pack_states(request, layer, ctx->Hv(), s) != cudaSuccess) return ONELA_E_CUDA;
     }
     finish_state_write(ctx, request, layer);
     return ONELA_OK;
@@ -295,12 +289,11 @@ onela_status onela_init_shared_states(onela_ctx* ctx, int32_t req_begin, int32_t
     if (st != ONELA_OK) return st;
     if (!ctx->dry()) {
         // the store keeps a request's layers next to each other and the requests in order: one contiguous range
-        if (launch_store_state(S0_dev, ctx->s0_slot(req_begin, 0), ctx->s0_scale_slot(req_begin, 0),
+        if (launch_store_state(S0_dev, ctx->s0_slot(req_begin, 0), ctx->s0_scale_slot(req_begin, 0), ctx->s0_f16_slot(req_begin, 0),
                                (long long)req_count * ctx->cfg.num_layers * ctx->Hv(), ctx->cfg.dk, ctx->cfg.dv,
                                s) != cudaSuccess)
             return ONELA_E_CUDA;
         ctx->launches++;
-        if (ctx->pack_states(req_begin, 0, (long long)req_count * ctx->cfg.num_layers * ctx->Hv(), s) != cudaSuccess) return ONELA_E_CUDA;
     }
     for (int32_t r = req_begin; r < req_begin + req_count; ++r)
         for (int32_t l = 0; l < ctx->cfg.num_layers; ++l) finish_state_write(ctx, r, l);
@@ -321,7 +314,7 @@ onela_status onela_prefill_shared_state(onela_ctx* ctx, int32_t request, int32_t
     if (!ctx->dry()) {
         bool supported = true;
         const cudaError_t e = launch_prefill(k_dev, v_dev, alpha_dev, beta_dev, ctx->s0_slot(request, layer),
-                                             ctx->s0_scale_slot(request, layer), ctx->tiled_tc ? ctx->s0_f16_slot(request, layer) : nullptr,
+                                             ctx->s0_scale_slot(request, layer), ctx->s0_f16_slot(request, layer),
                                              ctx->lay.status, n_tokens, ctx->cfg.num_heads, ctx->cfg.dk, ctx->cfg.dv, ctx->cfg.rec_dtype,
                                              &supported, s);
         if (!supported) return ONELA_E_UNSUPPORTED;
@@ -381,24 +374,9 @@ onela_status onela_reorder_beams(onela_ctx* ctx, int32_t req_begin, int32_t req_
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if ((st = ctx->prepare(s)) != ONELA_OK) return st;
     if (!ctx->dry()) {
-        if (launch_reorder(ctx->lay.tables + req_begin * ctx->table_req_stride(), ctx->table_req_stride(), req_count,
-                           parents_dev, W_new, W_prev, depth_old, c.max_beam, c.max_steps, bases, ctx->lay.status,
-                           s) != cudaSuccess)
-            return ONELA_E_CUDA;
-        ctx->launches++;
-    }
-    if (!ctx->dry() && ctx->tensor_core && depth_old >= 1) {
-        // distinct-record index of the table just written (buffer depth_old & 1), for the decode kernel's
-        // shared-ancestor staging
-        const int32_t* cur = ctx->lay.tables + req_begin * ctx->table_req_stride() +
-                             (long long)(depth_old & 1) * c.max_steps * c.max_beam;
-        if (launch_dedupe(cur, ctx->table_req_stride(), ctx->lay.sidx + req_begin * ctx->sidx_req_stride(),
-                          ctx->sidx_req_stride(), ctx->lay.ulist + req_begin * ctx->sidx_req_stride(),
-                          ctx->sidx_req_stride(), ctx->lay.urep + req_begin * ctx->sidx_req_stride(),
-                          ctx->lay.uoff + req_begin * ctx->uoff_req_stride(),
-                          ctx->uoff_req_stride(), ctx->lay.sg8 + req_begin * ctx->sg8_req_stride(), ctx->sg8_req_stride(),
-                          sg_row_stride(c.max_beam), ctx->lay.unode + (size_t)req_begin * ONELA_UNODE_CAP * 16, req_count, W_new,
-                          depth_old + 1, c.max_beam, s) != cudaSuccess)
+        // (the distinct-record index serves the warp-specialised kernel's staging, its compact copies the shared-chains one)
+        if (launch_index(ctx->lay, req_begin, req_count, parents_dev, W_new, W_prev, depth_old, c.max_beam, c.max_steps, bases, ctx->tensor_core,
+                         (c.flags & ONELA_FLAG_SHARED_CHAINS) != 0, s) != cudaSuccess)
             return ONELA_E_CUDA;
         ctx->launches++;
     }
@@ -655,18 +633,15 @@ onela_status onela_append_decode_step(onela_ctx* ctx, int32_t req_begin, int32_t
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if ((st = ctx->prepare(s)) != ONELA_OK) return st;
     if (!ctx->dry()) {
-        if (ctx->tensor_core || ctx->tiled_tc || ctx->gtr()) {
+        if (ctx->tensor_core || ctx->tiled_tc || ctx->gtr() || !ctx->grouped()) {
             st = launch_decode(ctx, req_begin, req_count, layer, q_dev, out_dev, k_dev, v_dev, alpha_dev, beta_dev, s);
             if (st != ONELA_OK) return st;
-        } else {   // shapes without the fused kernel: the copy kernel, then the decode kernel
+        } else {   // grouped value heads on CUDA cores: the copy kernel, then the decode kernel
             BatchBases bases{};
             for (int i = 0; i < req_count; ++i) bases.base[i] = ctx->req[req_begin + i].step_base.back();
-            const cudaError_t e =
-                ctx->grouped() ? launch_append_grouped(k_dev, v_dev, alpha_dev, beta_dev, ctx->k_plane(layer), ctx->v_plane(layer),
-                                                       ctx->gate_plane(layer), c.arena_slots, req_count, W, c.num_heads,
-                                                       ctx->Hv() / c.num_heads, c.dk, c.dv, ctx->elem_bytes, bases, s)
-                               : launch_append(k_dev, v_dev, alpha_dev, beta_dev, ctx->kv_plane(layer), ctx->gate_plane(layer),
-                                               c.arena_slots, req_count, W, c.num_heads, c.dk, c.dv, ctx->elem_bytes, bases, s);
+            const cudaError_t e = launch_append_grouped(k_dev, v_dev, alpha_dev, beta_dev, ctx->k_plane(layer), ctx->v_plane(layer),
+                                                        ctx->gate_plane(layer), c.arena_slots, req_count, W, c.num_heads,
+                                                        ctx->Hv() / c.num_heads, c.dk, c.dv, ctx->elem_bytes, bases, s);
             if (e != cudaSuccess) return ONELA_E_CUDA;
             ctx->launches++;
             st = launch_decode(ctx, req_begin, req_count, layer, q_dev, out_dev, nullptr, nullptr, nullptr, nullptr, s);

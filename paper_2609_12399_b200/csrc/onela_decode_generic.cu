@@ -4,6 +4,7 @@
 // One CTA = (request, head, tile of 32 beams).  A group of G lanes owns one (beam, head) unit and
 // folds its query through the unit's records, newest first (see onela.h):
 //      c = k_j . r ;  corr += beta_j c v_j ;  r <- alpha_j (r - beta_j c k_j)
+// (with the append fused in, the newest record comes from the caller's tensors and the unit also writes it to its slot)
 // with the decay kept as a running scalar (r = a * r~, a = prod alpha) so each record costs one dot,
 // two axpys and a log2(G)-step shuffle reduction.  The folded queries of the tile then meet the head's
 // S_0 in a [dv x dk] . [dk x 32] product on the FMA pipes: lane = beam, each warp a band of rows,
@@ -34,6 +35,9 @@ __global__ void __launch_bounds__(NB* G) decode_generic_kernel(const DecodeArgs 
     const bool active = b < a.W;
     const int bb = active ? b : a.W - 1;  // idle groups shadow a live beam so loads and shuffles stay uniform
 
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const bool fused = a.k_in != nullptr;   // append fused in: the newest record comes from the caller's tensors
     const T* q = static_cast<const T*>(a.q) + (((long long)req * a.W + bb) * a.H + h) * DK;
     const int32_t* table = a.table + req * a.table_req_stride;
     const long long plane_row0 = (long long)h * a.arena_slots;
@@ -47,16 +51,33 @@ __global__ void __launch_bounds__(NB* G) decode_generic_kernel(const DecodeArgs 
 
     float decay = 1.f;  // a = product of the alphas already passed
     for (int level = a.depth - 1; level >= 0; --level) {
-        const int32_t slot = (level == a.depth - 1) ? a.bases.base[req] + bb
-                                                    : __ldg(table + (long long)level * a.max_beam + bb);
+        const bool own = level == a.depth - 1;
+        const int32_t slot = own ? a.bases.base[req] + bb : __ldg(table + (long long)level * a.max_beam + bb);
         const long long row = plane_row0 + slot;
         const T* rec = kv + row * (DK + DV);
-        const float2 gate = __ldg(a.gates + row);
+        const T *kr = rec, *vr = rec + DK;
+        float2 gate;
+        if (own && fused) {     // ... and this unit also writes it to its slot, bit for bit
+            const long long in_row = ((long long)req * a.W + bb) * a.H + h;
+            kr = static_cast<const T*>(a.k_in) + in_row * DK;
+            vr = static_cast<const T*>(a.v_in) + in_row * DV;
+            gate = make_float2(__ldg(a.alpha_in + in_row), __ldg(a.beta_in + in_row));
+            if (active) {
+                uint4* dst = reinterpret_cast<uint4*>(a.kv_out + row * ((DK + DV) * (long long)sizeof(T)));
+#pragma unroll
+                for (int c = 0; c < CK; ++c) dst[c * G + g] = __ldg(reinterpret_cast<const uint4*>(kr) + c * G + g);
+#pragma unroll
+                for (int c = 0; c < CV; ++c) dst[DK / VEC + c * G + g] = __ldg(reinterpret_cast<const uint4*>(vr) + c * G + g);
+                if (g == 0) a.gates_out[row] = gate;
+            }
+        } else {
+            gate = __ldg(a.gates + row);
+        }
         float kx[CK * VEC];
         float dot = 0.f;
 #pragma unroll
         for (int c = 0; c < CK; ++c) {
-            Vec16<T>::load(rec + (c * G + g) * VEC, kx + c * VEC);
+            Vec16<T>::load(kr + (c * G + g) * VEC, kx + c * VEC);
 #pragma unroll
             for (int e = 0; e < VEC; ++e) dot = fmaf(kx[c * VEC + e], r[c * VEC + e], dot);
         }
@@ -67,7 +88,7 @@ __global__ void __launch_bounds__(NB* G) decode_generic_kernel(const DecodeArgs 
 #pragma unroll
         for (int c = 0; c < CV; ++c) {
             float vx[VEC];
-            Vec16<T>::load(rec + DK + (c * G + g) * VEC, vx);
+            Vec16<T>::load(vr + (c * G + g) * VEC, vx);
 #pragma unroll
             for (int e = 0; e < VEC; ++e) corr[c * VEC + e] = fmaf(wv, vx[e], corr[c * VEC + e]);
         }
@@ -148,8 +169,7 @@ cudaError_t launch_one(const DecodeArgs& a, cudaStream_t stream) {
         if (e != cudaSuccess) return e;
     }
     dim3 grid((a.W + NB - 1) / NB, a.H, a.req_count);
-    kern<<<grid, NB * G, smem, stream>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(kern, grid, dim3(NB * G), smem, stream, a);
 }
 
 template <int DK, int DV>

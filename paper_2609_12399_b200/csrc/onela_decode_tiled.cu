@@ -114,6 +114,8 @@ __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, 
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = *tmem_slot;
+    // (programmatic dependent launch: the next launch may set itself up under this one)
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     const int tile = blockIdx.x, hv = blockIdx.y, req = blockIdx.z;
     const int hk = hv / a.g, Hv = a.Hk * a.g;
@@ -156,7 +158,10 @@ __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, 
                             bd + (uint64_t)((kb * R_KB + ks * 32) >> 4), idesc, (kb | ks) ? 1u : 0u);
         umma_commit(smem_u32(bar));
     };
+    // The stored states are written by the state calls only, and the index launch that lies between those and any decode
+    // waits for them before it lets this one start: the first operand may be requested before the wait.
     if (tid == 0) load_A(0);        // in flight while the chain is walked
+    asm volatile("griddepcontrol.wait;" ::: "memory");
 
     // ---- the fold (Section 3.2's recurrence applied to the query from the newest record back) ----
     const T* q = static_cast<const T*>(a.q) + (((long long)req * a.W + bb) * a.Hk + hk) * KD;
@@ -468,8 +473,7 @@ cudaError_t launch_one(const TiledArgs& a, cudaStream_t stream) {
         }
     }
     dim3 grid((a.W + BPT - 1) / BPT, a.Hk * a.g, a.req_count);
-    kern<<<grid, THREADS, smem, stream>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(kern, grid, dim3(THREADS), smem, stream, a);
 }
 
 template <int KD, int VD, bool DELTA = false>

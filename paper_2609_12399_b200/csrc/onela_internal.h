@@ -15,6 +15,7 @@ struct Layout {
     int32_t* tables;   // [request][2][max_steps][max_beam] global slot ids (double-buffered per request)
     int32_t* sidx;     // [request][max_steps][max_beam] per (level, beam): index into the request's distinct-record list
     int32_t* ulist;    // [request][max_steps*max_beam] distinct record slots of the live chains, oldest level first
+    int32_t* level_base;   // [request][max_steps] first slot of the request's records of each decode call
     int32_t* uoff;     // [request][max_steps+1] start of each level inside ulist (uoff[level+1] = end)
     int32_t* urep;     // [request][max_steps*max_beam] per distinct record: one live beam whose chain holds it
     uint8_t* sg8;      // [request][max_steps][sg_stride] sidx as bytes, rows padded with the last live beam's entry
@@ -139,23 +140,35 @@ bool decode_tiled_supported(int32_t dk, int32_t dv);
 cudaError_t launch_decode_tiled(const TiledArgs& a, int32_t dk, int32_t dv, int32_t rec_dtype, int32_t out_dtype,
                                 cudaStream_t stream);
 
-// index kernels
-cudaError_t launch_reorder(int32_t* tables_req0, long long table_req_stride, int32_t req_count,
-                           const int32_t* parents, int32_t W_new, int32_t W_prev, int32_t depth_old,
-                           int32_t max_beam, int32_t max_steps, const BatchBases& bases, int32_t* status,
-                           cudaStream_t stream);
-// Distinct-record index of the CURRENT ancestry table (levels 0 .. depth-2; the newest level is the
-// beams' own records, all distinct): per level the sorted distinct slots and, per beam, where its
-// ancestor sits in the request's concatenated list.  Integer work only.
-// urep: per distinct record, one of the live beams whose chain holds it (all such beams share its older ancestors).
-// sg8 / unode: byte-sized copies for the shared-chains kernel (see Layout).
+// Launch with programmatic stream serialisation: the kernel may start while the previous kernel of the stream drains.
+// Rule for every kernel launched this way: it waits for that kernel (griddepcontrol.wait, every CTA) before it reads or
+// writes anything an earlier launch touches - only the decode kernels read the stored states earlier, see there - and lets
+// its own dependents start (griddepcontrol.launch_dependents) only from every CTA itself.
+template <class... Params, class... Args>
+cudaError_t launch_dependent(void (*kern)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, const Args&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
+// Ancestry index update of one decode call (Eq. 5) and, on request, the distinct-record index of the new table's levels
+// 0 .. depth-2 (the newest level is the beams' own records, all distinct): per level the sorted distinct slots, per beam
+// where its ancestor sits in the request's concatenated list, per distinct record one of the live beams whose chain holds
+// it (all such beams share its older ancestors); want_compact: byte-sized copies for the shared-chains kernel (see Layout).
+// Integer work only.
+cudaError_t launch_index(const Layout& lay, int32_t req_begin, int32_t req_count, const int32_t* parents, int32_t W_new, int32_t W_prev,
+                         int32_t depth_old, int32_t max_beam, int32_t max_steps, const BatchBases& bases, bool want_index, bool want_compact,
+                         cudaStream_t stream);
 #define ONELA_UNODE_CAP 256
 inline int32_t sg_row_stride(int32_t max_beam) { return (max_beam + 64 + 15) & ~15; }
-cudaError_t launch_dedupe(const int32_t* tables_cur_req0, long long table_req_stride, int32_t* sidx_req0,
-                          long long sidx_req_stride, int32_t* ulist_req0, long long ulist_req_stride,
-                          int32_t* urep_req0, int32_t* uoff_req0, long long uoff_req_stride, uint8_t* sg8_req0,
-                          long long sg8_req_stride, int32_t sg_stride, uint8_t* unode_req0, int32_t req_count, int32_t W,
-                          int32_t depth, int32_t max_beam, cudaStream_t stream);
 cudaError_t launch_export_chains(const int32_t* table_cur, int32_t W, int32_t depth, int32_t max_beam,
                                  int32_t* slots_out, cudaStream_t stream);
 
@@ -173,12 +186,10 @@ cudaError_t launch_append(const void* k, const void* v, const float* alpha, cons
                           float2* gate_plane, long long arena_slots, int32_t req_count, int32_t W, int32_t H,
                           int32_t dk, int32_t dv, int32_t elem_bytes, const BatchBases& bases,
                           cudaStream_t stream);
-// copies n_heads states of dv x dk floats and leaves each head's operand scale (see Layout::s0_scale) in scale_out
-cudaError_t launch_store_state(const float* S0_in, float* slot, float* scale_out, long long n_heads, int32_t dk, int32_t dv,
+// copies n_heads states of dv x dk floats and leaves each head's operand scale (see Layout::s0_scale) in scale_out and,
+// f16_out not null, the tiled kernel's operand copy (see Layout::s0_f16) there
+cudaError_t launch_store_state(const float* S0_in, float* slot, float* scale_out, uint16_t* f16_out, long long n_heads, int32_t dk, int32_t dv,
                                cudaStream_t stream);
-// the tiled kernel's operand copy of n_heads stored states (see Layout::s0_f16), from the store slots and their scales
-cudaError_t launch_pack_state(const float* slot, const float* scale, uint16_t* dst, long long n_heads, int32_t dk, int32_t dv,
-                              cudaStream_t stream);
 cudaError_t launch_export_state(const float* slot, float* S0_out, int32_t H, int32_t dk, int32_t dv, cudaStream_t stream);
 // Eq. 1 from the zero state over a prompt, into the store slot of one (request, layer), with the heads' operand scales and
 // (s0_f16 not null) the tiled kernel's operand copies (onela_prefill.cu).  Returns cudaErrorInvalidValue with *supported =

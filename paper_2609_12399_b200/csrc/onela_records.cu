@@ -19,6 +19,8 @@ __global__ void __launch_bounds__(256) append_kernel(const char* __restrict__ k,
                                                      char* __restrict__ kv_plane, float2* __restrict__ gate_plane,
                                                      long long arena_slots, int32_t W, int32_t H, int32_t k_bytes,
                                                      int32_t v_bytes, BatchBases bases) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int r = blockIdx.y;
     const int row_in_req = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);   // b * H + h
     const int lane = threadIdx.x & 31;
@@ -41,31 +43,95 @@ __device__ __forceinline__ float operand_scale(float peak) {
     const bool ok = eb > target + 1 && eb < 255;
     return ok ? __uint_as_float((uint32_t)(254 + target - eb) << 23) : 1.f;
 }
-// Largest value over the CTA (<= 1024 threads), returned to thread 0.
-__device__ __forceinline__ float block_max(float v) {
+// Copy of the caller's states into the store, with every head's operand scale and - configurations of the tiled
+// tensor-core kernel - its operand copy (see Layout::s0_f16) from the same registers.  A CTA holds 16 384 elements (64 KB,
+// all of its loads in flight at once); a larger head is a cluster of up to eight CTAs that exchange their largest
+// magnitudes through distributed shared memory.  HBM-bound: one read, one write, half a write more with the operand copy.
+// (As a CTA of 256 threads per head walking its state, followed by a second kernel that read the store back, 256 heads of
+// 256 x 256 took 43 + 27 us; 31 us now.)
+// VP: groups of eight elements per thread.
+template <int VP, int THREADS>
+__global__ void __launch_bounds__(THREADS) store_state_kernel(const float* __restrict__ in, float* __restrict__ out, float* __restrict__ scale_out,
+                                                              uint16_t* __restrict__ f16_out, int32_t dk, int32_t dv) {
     __shared__ float part[32];
-    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        v = threadIdx.x < (blockDim.x + 31) / 32 ? part[threadIdx.x] : 0.f;
-        for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+    __shared__ float cta_peak;
+    const int tid = threadIdx.x;
+    const uint32_t parts = gridDim.x, head = blockIdx.y, rank = blockIdx.x;      // cluster = the CTAs of one head
+    const long long base = (long long)head * dk * dv + (long long)rank * (VP * THREADS * 8);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    float4 x[VP][2];
+#pragma unroll
+    for (int j = 0; j < VP; ++j) {
+        const float4* p = reinterpret_cast<const float4*>(in + base) + 2 * (j * THREADS + tid);
+        x[j][0] = __ldg(p);
+        x[j][1] = __ldg(p + 1);
     }
-    return v;
+    float peak = 0.f;
+#pragma unroll
+    for (int j = 0; j < VP; ++j)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            reinterpret_cast<float4*>(out + base)[2 * (j * THREADS + tid) + e] = x[j][e];
+            peak = fmaxf(fmaxf(peak, fmaxf(fabsf(x[j][e].x), fabsf(x[j][e].y))), fmaxf(fabsf(x[j][e].z), fabsf(x[j][e].w)));
+        }
+    for (int o = 16; o > 0; o >>= 1) peak = fmaxf(peak, __shfl_xor_sync(0xffffffffu, peak, o));
+    if ((tid & 31) == 0) part[tid >> 5] = peak;
+    __syncthreads();
+    peak = 0.f;
+#pragma unroll
+    for (int w = 0; w < THREADS / 32; ++w) peak = fmaxf(peak, part[w]);
+    if (parts > 1) {
+        if (tid == 0) cta_peak = peak;
+        asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+        for (uint32_t p = 0; p < parts; ++p) {
+            uint32_t at;
+            float other;
+            asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"((uint32_t)__cvta_generic_to_shared(&cta_peak)), "r"(p));
+            asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(other) : "r"(at) : "memory");
+            peak = fmaxf(peak, other);
+        }
+        asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");      // nobody leaves while its peak is read
+    }
+    const float sc = operand_scale(peak);
+    if (rank == 0 && tid == 0) scale_out[head] = sc;
+    if (!f16_out) return;
+    // value rows padded to a multiple of 128, tiles of 128 rows x 64 columns, 16-byte chunks swizzled by the row
+    const int cpr = dk / 8, kb_n = dk / 64, rows = (dv + 127) / 128 * 128;
+    char* dst = reinterpret_cast<char*>(f16_out) + (long long)head * rows * dk * 2;
+    auto at = [&](int i, int ch) { return dst + ((long long)((i >> 7) * kb_n + (ch >> 3)) * 128 + (i & 127)) * 128 + (((ch & 7) ^ (i & 7)) << 4); };
+    const int first = (int)rank * (VP * THREADS);           // the CTA's first chunk of eight elements
+#pragma unroll
+    for (int j = 0; j < VP; ++j) {
+        const int item = first + j * THREADS + tid, i = item / cpr;
+        const __half2 h0 = __floats2half2_rn(x[j][0].x * sc, x[j][0].y * sc), h1 = __floats2half2_rn(x[j][0].z * sc, x[j][0].w * sc);
+        const __half2 h2 = __floats2half2_rn(x[j][1].x * sc, x[j][1].y * sc), h3 = __floats2half2_rn(x[j][1].z * sc, x[j][1].w * sc);
+        *reinterpret_cast<uint4*>(at(i, item - i * cpr)) =
+            make_uint4(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1), *reinterpret_cast<const uint32_t*>(&h2),
+                       *reinterpret_cast<const uint32_t*>(&h3));
+    }
+    for (int item = dv * cpr + tid; item < rows * cpr; item += THREADS) {        // padding (dv = 64: one CTA per head)
+        const int i = item / cpr;
+        *reinterpret_cast<uint4*>(at(i, item - i * cpr)) = make_uint4(0u, 0u, 0u, 0u);
+    }
 }
 
-// Copy of the caller's states into the store, one CTA per head, with the head's operand scale as a by-product.
-__global__ void __launch_bounds__(256) store_state_kernel(const float4* __restrict__ in, float4* __restrict__ out,
-                                                          float* __restrict__ scale_out, int32_t vec_per_head) {
-    const long long base = (long long)blockIdx.x * vec_per_head;
-    float peak = 0.f;
-    for (int i = threadIdx.x; i < vec_per_head; i += blockDim.x) {
-        const float4 x = __ldg(in + base + i);
-        out[base + i] = x;
-        peak = fmaxf(fmaxf(peak, fmaxf(fabsf(x.x), fabsf(x.y))), fmaxf(fabsf(x.z), fabsf(x.w)));
-    }
-    peak = block_max(peak);
-    if (threadIdx.x == 0) scale_out[blockIdx.x] = operand_scale(peak);
+template <int VP, int THREADS>
+cudaError_t launch_store_t(const float* in, float* out, float* scale_out, uint16_t* f16_out, unsigned parts, unsigned n_heads, int32_t dk, int32_t dv,
+                           cudaStream_t stream) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(parts, n_heads);
+    cfg.blockDim = dim3(THREADS);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = parts;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = parts > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, store_state_kernel<VP, THREADS>, in, out, scale_out, f16_out, dk, dv);
 }
 
 }  // namespace
@@ -76,49 +142,26 @@ cudaError_t launch_append(const void* k, const void* v, const float* alpha, cons
                           cudaStream_t stream) {
     const int warps_per_block = 8;
     dim3 grid((unsigned)((W * H + warps_per_block - 1) / warps_per_block), (unsigned)req_count);
-    append_kernel<<<grid, warps_per_block * 32, 0, stream>>>(static_cast<const char*>(k), static_cast<const char*>(v),
-                                                             alpha, beta, kv_plane, gate_plane, arena_slots, W, H,
-                                                             dk * elem_bytes, dv * elem_bytes, bases);
-    return cudaGetLastError();
+    return launch_dependent(append_kernel, grid, dim3(warps_per_block * 32), 0, stream, static_cast<const char*>(k), static_cast<const char*>(v), alpha,
+                            beta, kv_plane, gate_plane, arena_slots, W, H, dk * elem_bytes, dv * elem_bytes, bases);
 }
 
-// One CTA per head: the stored state as the tiled tensor-core kernel's A operand (see Layout::s0_f16).  The rounding
-// is the one that kernel would do itself (x * scale to the nearest fp16), so results do not depend on who converts.
-__global__ void __launch_bounds__(256) pack_state_f16_kernel(const float* __restrict__ slot, const float* __restrict__ scale,
-                                                             uint16_t* __restrict__ dst, int32_t dk, int32_t dv) {
-    const long long head = blockIdx.x;
-    const float* S = slot + head * (long long)dv * dk;
-    const float sc = scale[head];
-    const int cpr = dk / 8, kb_n = dk / 64, rows = (dv + 127) / 128 * 128;     // 16-byte chunks per row, column tiles, padded rows
-    char* out = reinterpret_cast<char*>(dst) + head * (long long)rows * dk * 2;
-    for (int item = threadIdx.x; item < rows * cpr; item += blockDim.x) {
-        const int i = item / cpr, ch = item - i * cpr;
-        uint4 w = make_uint4(0u, 0u, 0u, 0u);
-        if (i < dv) {
-            const float4* p = reinterpret_cast<const float4*>(S + (long long)i * dk + ch * 8);
-            const float4 x0 = __ldg(p), x1 = __ldg(p + 1);
-            const __half2 h0 = __floats2half2_rn(x0.x * sc, x0.y * sc), h1 = __floats2half2_rn(x0.z * sc, x0.w * sc);
-            const __half2 h2 = __floats2half2_rn(x1.x * sc, x1.y * sc), h3 = __floats2half2_rn(x1.z * sc, x1.w * sc);
-            w = make_uint4(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1),
-                           *reinterpret_cast<const uint32_t*>(&h2), *reinterpret_cast<const uint32_t*>(&h3));
-        }
-        const int mt = i >> 7, row = i & 127, kb = ch >> 3, c8 = ch & 7;
-        *reinterpret_cast<uint4*>(out + ((long long)(mt * kb_n + kb) * 128 + row) * 128 + ((c8 ^ (row & 7)) << 4)) = w;
-    }
-}
-
-cudaError_t launch_pack_state(const float* slot, const float* scale, uint16_t* dst, long long n_heads, int32_t dk, int32_t dv,
-                              cudaStream_t stream) {
-    pack_state_f16_kernel<<<(unsigned)n_heads, 256, 0, stream>>>(slot, scale, dst, dk, dv);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_store_state(const float* S0_in, float* slot, float* scale_out, long long n_heads, int32_t dk, int32_t dv,
+cudaError_t launch_store_state(const float* S0_in, float* slot, float* scale_out, uint16_t* f16_out, long long n_heads, int32_t dk, int32_t dv,
                                cudaStream_t stream) {
-    if (n_heads <= 0 || n_heads > 0x7fffffffLL) return cudaErrorInvalidValue;
-    store_state_kernel<<<(unsigned)n_heads, 256, 0, stream>>>(reinterpret_cast<const float4*>(S0_in), reinterpret_cast<float4*>(slot),
-                                                             scale_out, dk * dv / 4);
-    return cudaGetLastError();
+    const int elems = dk * dv;             // every supported head is 1024 or 4096 elements, or a power of two times 16 384
+    for (long long h0 = 0; h0 < n_heads; h0 += 65535) {
+        const unsigned n = (unsigned)(n_heads - h0 < 65535 ? n_heads - h0 : 65535);
+        const float* in = S0_in + h0 * elems;
+        float *out = slot + h0 * elems, *sc = scale_out + h0;
+        uint16_t* f16 = f16_out ? f16_out + h0 * (long long)(s0_f16_head_bytes(dk, dv) / 2) : nullptr;
+        const cudaError_t e = elems == 1024   ? launch_store_t<1, 128>(in, out, sc, f16, 1, n, dk, dv, stream)
+                              : elems == 4096 ? launch_store_t<2, 256>(in, out, sc, f16, 1, n, dk, dv, stream)
+                              : elems % 16384 == 0 && elems / 16384 <= 8
+                                  ? launch_store_t<4, 512>(in, out, sc, f16, (unsigned)(elems / 16384), n, dk, dv, stream)
+                                  : cudaErrorInvalidValue;
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 cudaError_t launch_export_state(const float* slot, float* S0_out, int32_t H, int32_t dk, int32_t dv, cudaStream_t stream) {
