@@ -25,7 +25,7 @@ struct Layout {
     char* kv;          // [layer][head][arena_slots][dk + dv] in rec_dtype: one row = k | v of one record
                        // (grouped value heads: keys only, [layer][key head][arena_slots][dk])
     char* vv;          // grouped value heads only: values [layer][value head][arena_slots][dv]
-    unsigned long long* select_scratch;   // [request][ONELA_SELECT_PARTS][ONELA_SELECT_CAP]: partial results of beam selection
+    unsigned long long* select_scratch;   // [request][ONELA_SELECT_PARTS * ONELA_SELECT_CAP]: beam selection, candidates beyond its shared memory
     float* s0_scale;   // [request][layer][head]: the power of two that brings the head's largest |S_0| element into
                        // [2^11, 2^12) (1 for an all-zero or non-finite state); written with the state, read by the
                        // tensor-core kernel, whose fp16 operand it keeps in range
@@ -173,13 +173,14 @@ cudaError_t launch_export_chains(const int32_t* table_cur, int32_t W, int32_t de
                                  int32_t* slots_out, cudaStream_t stream);
 
 // global beam selection: the W_new best (parent, code) pairs per request, best first (see onela_select.cu).
-// `scratch` ([request][ONELA_SELECT_PARTS][ONELA_SELECT_CAP] 64-bit words) is used when a request has more than
-// 4096 candidates; at most ONELA_SELECT_PARTS * 4096 candidates per request.
+// At most ONELA_SELECT_PARTS * 4096 candidates per request.  `scratch` ([request][ONELA_SELECT_PARTS * ONELA_SELECT_CAP] 64-bit
+// words, or null) takes the candidates that the selection bound leaves where shared memory cannot hold them.
 #define ONELA_SELECT_CAP 1024
 #define ONELA_SELECT_PARTS 256
 cudaError_t launch_select(const float* beam_scores, const float* cand_logp, int32_t req_count, int32_t W_prev, int32_t C,
                           int32_t W_new, unsigned long long* scratch, int32_t* parents, int32_t* codes, float* scores,
                           cudaStream_t stream);
+int select_launches(long long candidates);      // kernels a call with a scratch launches
 
 // record / state kernels
 cudaError_t launch_append(const void* k, const void* v, const float* alpha, const float* beta, char* kv_plane,

@@ -5,12 +5,20 @@
 //
 // A candidate's rank is a 64-bit composite: its fp32 score (parent score + log-probability, mapped to
 // order-preserving bits; NaN lowest, -0 = +0) in the high word, 0xffffffff - flat index in the low word, so
-// composites are distinct and "larger" means "better, ties to the smaller flat index".  A CTA finds the k largest
-// composites of a range by an 8-bit radix select from the top byte down (the passes over the index bytes are
-// skipped when no tie straddles the cut) and gathers them in shared memory.
-// Two launches per call: `select_part_kernel` cuts a request's candidates into parts of 4096 and leaves each part's
-// own top-k (unordered) in a scratch area of the workspace; `select_merge_kernel` (one CTA per request) selects
-// among those and orders the survivors with a bitonic sort.  A request with a single part skips the scratch.
+// composites are distinct and "larger" means "better, ties to the smaller flat index".
+//
+// A cluster of up to eight CTAs of 1024 threads per request (`select_kernel`):
+//   1. every thread takes a strided share of the candidates and keeps its largest;
+//   2. the cluster's first CTA finds a bound that at least k of the threads' largest reach - so at least k candidates
+//      reach it, and with shares spread over all parents and codes hardly more do (1094 expected for k = 1024 of a million);
+//   3. the shares whose largest reaches the bound are looked into, what reaches it is gathered in the first CTA's shared
+//      memory (distributed shared memory, one remote atomic per CTA), ordered through a histogram of the scores and written
+//      out best first.
+// Requests beyond 131 072 candidates have the shares' largest found by a launch of its own over all SMs.
+// What bounds it: latency - the candidates are read once (512 KB for 512 x 256), then four cluster barriers and a dozen of a
+// CTA's; the code runs once per launch, so loops stay rolled.  (As two launches - every 4096 candidates by an eight-pass radix
+// select of their own, one CTA to merge the parts' lists - the 512 x 256 -> 512 selection took 36 - 43 us; 14 us now, and
+// 23 us for 4 requests of 1024 x 1000 -> 1024.)
 #include <mutex>
 
 #include "onela_internal.h"
@@ -21,8 +29,14 @@ namespace {
 
 constexpr int SEL_THREADS = 1024;
 constexpr int SEL_CAP = ONELA_SELECT_CAP;      // survivors per request (W_new <= SEL_CAP)
-constexpr int SEL_PART = 4096;                 // candidates per part: four per thread
-constexpr int SEL_PARTS_MAX = ONELA_SELECT_PARTS;
+constexpr int SEL_LIST = 4096;                 // candidates that reach the bound: room in shared memory
+constexpr int SEL_CTAS = 8;                    // CTAs per cluster at most
+constexpr int SEL_HELD = 16;                   // scores a thread keeps in registers
+constexpr int SEL_SHARES = ONELA_SELECT_PARTS * 4096 / SEL_HELD;      // shares of the largest request; the list behind them in the
+                                               // scratch takes all candidates of the k + k / 8 threads the bound may leave
+constexpr int SEL_BINS = 2048;
+constexpr int SEL_ROTATE = 977;                // a thread's place moves by this much from stripe to stripe, so that one code's
+                                               // candidates (a multiple of C apart) do not all fall to the same threads
 
 __device__ __forceinline__ uint32_t score_bits(float s) {
     if (s != s) return 0u;                              // NaN: below every number
@@ -30,22 +44,30 @@ __device__ __forceinline__ uint32_t score_bits(float s) {
     return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-struct ScoreSource {     // composites computed from the caller's scores; item i is flat index first + i
+struct ScoreSource {     // composites computed from the caller's scores; item i is flat index i
     const float* bs;
     const float* lp;
-    uint32_t first;
-    int C;
-    __device__ __forceinline__ unsigned long long operator()(uint32_t i) const {
-        const uint32_t idx = first + i;
-        const float s = __ldg(bs + idx / (uint32_t)C) + __ldg(lp + idx);
-        return ((unsigned long long)score_bits(s) << 32) | (unsigned long long)(0xffffffffu - idx);
+    uint32_t magic;      // i / C as (i magic / 2^32) >> shift, exactly (see divide_by)
+    int shift, C;
+    __device__ __forceinline__ uint32_t parent(uint32_t i) const { return magic ? __umulhi(i, magic) >> shift : i; }
+    __device__ __forceinline__ float score(uint32_t i) const { return __ldg(bs + parent(i)) + __ldg(lp + i); }
+    __device__ __forceinline__ unsigned long long join(uint32_t bits, uint32_t i) const {
+        return ((unsigned long long)bits << 32) | (unsigned long long)(0xffffffffu - i);
     }
+    __device__ __forceinline__ unsigned long long operator()(uint32_t i) const { return join(score_bits(score(i)), i); }
 };
+// i / C for i < 2^20: with m = ceil(2^t / C), i m / 2^t has the right integer part while i C < 2^t - t = 32 serves C <= 4096,
+// t = 40 (m below 2^32 then) the larger ones; C = 1 is no division.
+void divide_by(int32_t C, uint32_t& magic, int& shift) {
+    shift = C > 4096 ? 8 : 0;
+    magic = C == 1 ? 0u : (uint32_t)(((1ull << (32 + shift)) + (unsigned long long)C - 1ull) / (unsigned long long)C);
+}
 struct SelectShared {
-    unsigned int hist[256];
-    unsigned long long sel[SEL_CAP];
-    unsigned long long prefix;
-    unsigned int k, count, equal;
+    unsigned int hist[SEL_BINS];
+    unsigned long long sel[SEL_CAP];           // (the exhaustive selection's result)
+    unsigned long long prefix, lo, hi;
+    unsigned long long part_min[32], part_max[32];
+    unsigned int k, count, equal, part_sum[32];
 };
 
 // Leaves the k largest composites of item(0 .. n-1) in sh.sel[0 .. k) (unordered); k <= min(n, SEL_CAP).
@@ -136,9 +158,8 @@ __device__ void select_passes(const Item& item, uint32_t n, int k, SelectShared&
     }
     __syncthreads();
 }
-// The passes read every candidate four to eight times.  Up to ITEMS * SEL_THREADS candidates are fetched once, all
-// loads in flight together, and kept in registers (a pass then costs votes and shared-memory atomics only: the
-// merging CTA fell from 48 us to a fraction of that on 16 384 composites); longer lists are re-read from the source.
+// The exhaustive selection.  The passes read every candidate four to eight times: up to ITEMS * SEL_THREADS candidates are
+// fetched once, all loads in flight together, and kept in registers; longer lists are re-read from the source.
 template <int ITEMS, class Src>
 __device__ void select_topk(const Src& src, uint32_t n, int k, SelectShared& sh) {
     if (n <= (uint32_t)ITEMS * SEL_THREADS) {
@@ -156,159 +177,505 @@ __device__ void select_topk(const Src& src, uint32_t n, int k, SelectShared& sh)
     }
 }
 
-// Orders sh.sel[0 .. k) best first and writes the survivors out.
-__device__ void sort_and_emit(SelectShared& sh, int k, const float* bs, const float* lp, int C, int32_t* parents,
-                              int32_t* codes, float* scores) {
-    const int tid = threadIdx.x;
-    int n_sort = 2;
-    while (n_sort < k) n_sort <<= 1;                        // the sort runs over the next power of two
-    for (int i = tid; i < n_sort; i += SEL_THREADS)
-        if (i >= k) sh.sel[i] = 0ull;
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t in_first_cta(const void* p) {      // shared address in the cluster's first CTA
+    uint32_t at;
+    asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(at) : "r"((uint32_t)__cvta_generic_to_shared(p)));
+    return at;
+}
+__device__ __forceinline__ void st_cluster64(uint32_t at, unsigned long long x) { asm volatile("st.shared::cluster.b64 [%0], %1;" ::"r"(at), "l"(x) : "memory"); }
+__device__ __forceinline__ unsigned long long ld_cluster64(uint32_t at) {
+    unsigned long long x;
+    asm volatile("ld.shared::cluster.b64 %0, [%1];" : "=l"(x) : "r"(at) : "memory");
+    return x;
+}
+__device__ __forceinline__ unsigned add_cluster(uint32_t at, unsigned x) {
+    unsigned old;
+    asm volatile("atom.shared::cluster.add.u32 %0, [%1], %2;" : "=r"(old) : "r"(at), "r"(x) : "memory");
+    return old;
+}
+
+// The histogram step of bound_of: bins of the CTA's items counted in sh.hist, the bin that holds the want-th largest is
+// found; sh.equal = that bin, sh.count = items in it and above, sh.k = items above.  Ends with a barrier.
+__device__ __forceinline__ void bin_of_kth(unsigned want, SelectShared& sh) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     __syncthreads();
-    // Bitonic sort, descending.  Compare-exchange i of a step pairs elements inside the 64-element block i / 32 whenever
-    // the stride is below 64, and thread i (= pair i; n_sort / 2 <= 512 pairs) belongs to warp i / 32: those steps need
-    // the warp only, and a block-wide barrier stands just before and after each run of them.
-    auto exchange = [&](int i, int size, int stride) {
-        const int lo = 2 * i - (i & (stride - 1)), hi = lo + stride;
-        const bool desc = (lo & size) == 0;
-        const unsigned long long x = sh.sel[lo], y = sh.sel[hi];
-        if ((x < y) == desc) { sh.sel[lo] = y; sh.sel[hi] = x; }
-    };
-    static_assert(SEL_CAP / 2 <= SEL_THREADS, "one compare-exchange per thread and step");
-    const bool mine = tid < n_sort / 2;
-    for (int size = 2; size <= n_sort; size <<= 1) {
-        int stride = size >> 1;
-        for (; stride >= 64; stride >>= 1) {                // partners in different 64-element blocks
-            if (mine) exchange(tid, size, stride);
-            __syncthreads();
+    // counts of the bins from the top: thread t takes bins 2 t and 2 t + 1
+    const uint2 h = reinterpret_cast<const uint2*>(sh.hist)[tid];
+    unsigned incl = h.x + h.y;                                        // lanes >= this one
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned up = __shfl_down_sync(0xffffffffu, incl, o);
+        if (lane + o < 32) incl += up;
+    }
+    if (lane == 0) sh.part_sum[warp] = incl;
+    __syncthreads();
+    const unsigned above = __reduce_add_sync(0xffffffffu, lane > warp ? sh.part_sum[lane] : 0u);      // warps above this one
+    const unsigned ge0 = above + incl, ge1 = ge0 - h.x, gt1 = ge1 - h.y;
+    if (ge1 >= want && gt1 < want) {
+        sh.equal = 2 * tid + 1;
+        sh.count = ge1;
+        sh.k = gt1;
+    } else if (ge0 >= want && ge1 < want) {
+        sh.equal = 2 * tid;
+        sh.count = ge0;
+        sh.k = ge1;
+    }
+    __syncthreads();
+}
+
+// A bound that at least k, and as a rule little more, of the CTA's composites reach (COUNT per thread, 0 where there is
+// none; all threads call).  A histogram over the span of the scores at hand; where the bin that holds the k-th largest holds
+// too many more, further rounds look into that bin alone, on whole composites, down to single ones if they must.
+template <int COUNT>
+__device__ unsigned long long bound_of(const unsigned long long (&held)[COUNT], int k, SelectShared& sh) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    unsigned want = (unsigned)k;
+    const unsigned slack = max(32u, want / 8);
+    unsigned long long lo, hi;
+    {
+        uint32_t mn = 0xffffffffu, mx = 0u;
+#pragma unroll
+        for (int j = 0; j < COUNT; ++j)
+            if (held[j]) {
+                mn = min(mn, (uint32_t)(held[j] >> 32));
+                mx = max(mx, (uint32_t)(held[j] >> 32));
+            }
+        mn = __reduce_min_sync(0xffffffffu, mn);
+        mx = __reduce_max_sync(0xffffffffu, mx);
+        if (lane == 0) { sh.part_min[warp] = mn; sh.part_max[warp] = mx; }
+        reinterpret_cast<uint2*>(sh.hist)[tid] = make_uint2(0u, 0u);
+        __syncthreads();
+        mn = __reduce_min_sync(0xffffffffu, (uint32_t)sh.part_min[lane]);
+        mx = __reduce_max_sync(0xffffffffu, (uint32_t)sh.part_max[lane]);
+        const int shift = max(0, 32 - __clz(mx - mn) - 11);
+#pragma unroll
+        for (int j = 0; j < COUNT; ++j)
+            if (held[j]) atomicAdd(&sh.hist[((uint32_t)(held[j] >> 32) - mn) >> shift], 1u);
+        bin_of_kth(want, sh);
+        const uint32_t first = mn + (sh.equal << shift);
+        lo = (unsigned long long)first << 32;
+        hi = ((unsigned long long)(first + ((1u << shift) - 1u)) << 32) | 0xffffffffull;
+    }
+    while (sh.count - want > slack) {
+        want -= sh.k;
+        unsigned long long mn = ~0ull, mx = 0ull;
+#pragma unroll
+        for (int j = 0; j < COUNT; ++j)
+            if (held[j] >= lo && held[j] <= hi) {
+                mn = min(mn, held[j]);
+                mx = max(mx, held[j]);
+            }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            mn = min(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+            mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         }
-        for (; stride > 0; stride >>= 1) {                  // partners inside this warp's 64-element block
-            if (mine) exchange(tid, size, stride);
-            __syncwarp();
+        if (lane == 0) { sh.part_min[warp] = mn; sh.part_max[warp] = mx; }
+        reinterpret_cast<uint2*>(sh.hist)[tid] = make_uint2(0u, 0u);
+        __syncthreads();
+        mn = sh.part_min[lane];
+        mx = sh.part_max[lane];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            mn = min(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+            mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        }
+        const int shift = max(0, 64 - __clzll((long long)(mx - mn)) - 11);
+#pragma unroll
+        for (int j = 0; j < COUNT; ++j)
+            if (held[j] >= lo && held[j] <= hi) atomicAdd(&sh.hist[(unsigned)((held[j] - mn) >> shift)], 1u);
+        bin_of_kth(want, sh);
+        lo = mn + ((unsigned long long)sh.equal << shift);
+        hi = lo + (1ull << shift) - 1ull;
+        if (shift == 0) break;
+    }
+    return lo;
+}
+
+// Writes survivor x, which is the `rank`-th best, out.
+__device__ __forceinline__ void emit(unsigned long long x, int rank, const ScoreSource& src, int32_t* parents, int32_t* codes, float* scores) {
+    const uint32_t idx = 0xffffffffu - (uint32_t)(x & 0xffffffffull), par = src.parent(idx);
+    parents[rank] = (int)par;
+    codes[rank] = (int)(idx - par * (uint32_t)src.C);
+    scores[rank] = __ldg(src.bs + par) + __ldg(src.lp + idx);
+}
+
+// Orders list[0 .. n) best first (n <= 1024 E; `spare`: as much room again) and writes the k best out.  The scores at hand are
+// spread over SEL_BINS bins: an element's rank is the count of the bins before its own plus the number of larger ones in it,
+// as a rule one or two.  Where a bin holds many (equal scores): runs of 32 are sorted by their warp (shuffles), then merged
+// pairwise, an element's place being its own in its run plus the number of elements of the other run that come before it,
+// found by bisection.  (600 survivors: 2.5 us with bins; 6.7 us merged, whose scattered 64-bit reads conflict; 9.2 us as a
+// bitonic sort.)
+template <int E>
+__device__ void sort_and_emit(unsigned long long* list, unsigned long long* spare, int n, int k, SelectShared& sh, const ScoreSource& src,
+                              int32_t* parents, int32_t* codes, float* scores) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    unsigned long long x[E];
+    {
+        uint32_t mn = 0xffffffffu, mx = 0u;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const bool live = e * SEL_THREADS + tid < n;
+            x[e] = live ? list[e * SEL_THREADS + tid] : 0ull;
+            if (live) {
+                mn = min(mn, (uint32_t)(x[e] >> 32));
+                mx = max(mx, (uint32_t)(x[e] >> 32));
+            }
+        }
+        mn = __reduce_min_sync(0xffffffffu, mn);
+        mx = __reduce_max_sync(0xffffffffu, mx);
+        if (lane == 0) { sh.part_min[warp] = mn; sh.part_max[warp] = mx; }
+        reinterpret_cast<uint2*>(sh.hist)[tid] = make_uint2(0u, 0u);
+        __syncthreads();
+        mn = __reduce_min_sync(0xffffffffu, (uint32_t)sh.part_min[lane]);
+        mx = __reduce_max_sync(0xffffffffu, (uint32_t)sh.part_max[lane]);
+        const int shift = max(0, 32 - __clz(mx - mn) - 11);
+        unsigned at[E];
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+            if (e * SEL_THREADS + tid < n) at[e] = atomicAdd(&sh.hist[(mx - (uint32_t)(x[e] >> 32)) >> shift], 1u);
+        __syncthreads();
+        const uint2 h = reinterpret_cast<const uint2*>(sh.hist)[tid];
+        unsigned incl = h.x + h.y;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned up = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += up;
+        }
+        const unsigned most = __reduce_max_sync(0xffffffffu, max(h.x, h.y));
+        if (lane == 31) { sh.part_sum[warp] = incl; sh.part_min[warp] = most; }
+        __syncthreads();
+        const unsigned before = incl - h.x - h.y + __reduce_add_sync(0xffffffffu, lane < warp ? sh.part_sum[lane] : 0u);
+        const bool few = __reduce_max_sync(0xffffffffu, (uint32_t)sh.part_min[lane]) <= 32u;
+        reinterpret_cast<uint2*>(sh.hist)[tid] = make_uint2(before, before + h.x);       // where the bins start
+        __syncthreads();
+        if (few) {
+            unsigned bin[E];
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+                if (e * SEL_THREADS + tid < n) {
+                    bin[e] = (mx - (uint32_t)(x[e] >> 32)) >> shift;
+                    spare[sh.hist[bin[e]] + at[e]] = x[e];
+                }
+            __syncthreads();
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+                if (e * SEL_THREADS + tid < n) {
+                    const unsigned first = sh.hist[bin[e]], end = bin[e] + 1 < SEL_BINS ? sh.hist[bin[e] + 1] : (unsigned)n;
+                    unsigned rank = first;
+                    if (first < (unsigned)k) {
+                        for (unsigned q = first; q < end; ++q) rank += spare[q] > x[e];
+                        if (rank < (unsigned)k) emit(x[e], (int)rank, src, parents, codes, scores);
+                    }
+                }
+            return;
+        }
+    }
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        if (e * SEL_THREADS + (tid & ~31) >= n) continue;    // (the whole warp: nothing to sort)
+        // loops, not unrolled: the code runs once per launch, and fetching it is what it would cost
+#pragma unroll 1
+        for (int size = 2; size <= 32; size <<= 1)
+#pragma unroll 1
+            for (int stride = size >> 1; stride > 0; stride >>= 1) {
+                const unsigned long long y = __shfl_xor_sync(0xffffffffu, x[e], stride);
+                const bool keep_large = ((lane & size & 31) == 0) == ((lane & stride) == 0);      // (size 32: descending)
+                x[e] = (x[e] > y) == keep_large ? x[e] : y;
+            }
+    }
+    unsigned long long *from = spare, *to = list;
+    __syncthreads();                                         // the list has been read
+#pragma unroll
+    for (int e = 0; e < E; ++e) from[e * SEL_THREADS + tid] = x[e];
+    __syncthreads();
+    for (int run = 32; run < n; run <<= 1) {
+#pragma unroll 1
+        for (int e = 0; e < E; ++e) {
+            const int i = e * SEL_THREADS + tid, at = i & (run - 1), other = (i ^ run) & ~(run - 1);
+            const bool right = (i & run) != 0;               // equals (padding) keep their order: the left run's first
+            const unsigned long long me = from[i];
+            int lo = 0, len = run;                           // elements of the other run before this one: in [lo, lo + len]
+            while (len > 0) {
+                const int half = len >> 1;
+                const unsigned long long y = from[other + lo + half];
+                const bool before = right ? y >= me : y > me;
+                lo = before ? lo + half + 1 : lo;
+                len = before ? len - half - 1 : half;
+            }
+            to[(i & ~(2 * run - 1)) + at + lo] = me;
         }
         __syncthreads();
+        unsigned long long* t = from;
+        from = to;
+        to = t;
     }
-    for (int i = tid; i < k; i += SEL_THREADS) {
-        const uint32_t idx = 0xffffffffu - (uint32_t)(sh.sel[i] & 0xffffffffull);
-        const int par = (int)(idx / (uint32_t)C);
-        parents[i] = par;
-        codes[i] = (int)(idx - (uint32_t)par * (uint32_t)C);
-        scores[i] = __ldg(bs + par) + __ldg(lp + idx);
-    }
+#pragma unroll
+    for (int e = 0; e < E; ++e) x[e] = from[e * SEL_THREADS + tid];
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+        if (e * SEL_THREADS + tid < k) emit(x[e], e * SEL_THREADS + tid, src, parents, codes, scores);
 }
 
-// grid (parts, requests): the part's own top-k, unordered, to scratch[request][part][0 .. kp), kp = min(k, part size)
-__global__ void __launch_bounds__(SEL_THREADS) select_part_kernel(const float* __restrict__ beam_scores, const float* __restrict__ cand_logp,
-                                                                  int W_prev, int C, int k, unsigned long long* __restrict__ scratch) {
-    __shared__ SelectShared sh;
-    const int part = blockIdx.x, req = blockIdx.y;
-    const uint32_t N = (uint32_t)W_prev * (uint32_t)C, first = (uint32_t)part * SEL_PART;
-    const uint32_t n = min((uint32_t)SEL_PART, N - first);
-    const int kp = min((uint32_t)k, n);
-    const ScoreSource src{beam_scores + (long long)req * W_prev, cand_logp + (long long)req * W_prev * C, first, C};
-    select_topk<SEL_PART / SEL_THREADS>(src, n, kp, sh);
-    unsigned long long* out = scratch + ((long long)req * SEL_PARTS_MAX + part) * SEL_CAP;
-    for (int i = threadIdx.x; i < kp; i += SEL_THREADS) out[i] = sh.sel[i];
+// Running maximum of a thread's candidates in increasing index order: the larger score, the earlier one of equals, NaN below
+// every number (the order of the composites, on floats: a third of the instructions).
+struct Best {
+    float s = 0.f;
+    uint32_t i = 0xffffffffu;      // none
+    __device__ __forceinline__ void take(float x, uint32_t at) {
+        const bool better = x > s || i == 0xffffffffu || (s != s && x == x);
+        s = better ? x : s;
+        i = better ? at : i;
+    }
+    __device__ __forceinline__ unsigned long long composite(const ScoreSource& src) const { return i == 0xffffffffu ? 0ull : src.join(score_bits(s), i); }
+};
+
+// Where candidate j of place `me` lies when `span` (a power of two) threads share a range: consecutive threads take
+// consecutive candidates of a stripe, turned by SEL_ROTATE from stripe to stripe.
+__device__ __forceinline__ uint32_t place_of(int j, uint32_t me, uint32_t span) { return (uint32_t)j * span + ((me + (uint32_t)j * SEL_ROTATE) & (span - 1)); }
+
+// Requests of more candidates than a cluster's registers hold: the largest of every share of SEL_HELD, one CTA per 16 384
+// candidates, to scratch[request][share].
+__global__ void __launch_bounds__(SEL_THREADS) select_shares_kernel(const float* __restrict__ beam_scores, const float* __restrict__ cand_logp, int W_prev, int C,
+                                                                    uint32_t magic, int shift, unsigned long long* __restrict__ scratch) {
+    const int tid = threadIdx.x, req = blockIdx.y;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const uint32_t N = (uint32_t)W_prev * (uint32_t)C, first = blockIdx.x * (SEL_HELD * SEL_THREADS);
+    const ScoreSource src{beam_scores + (long long)req * W_prev, cand_logp + (long long)req * N, magic, shift, C};
+    Best best;
+#pragma unroll 8
+    for (int j = 0; j < SEL_HELD; ++j) {
+        const uint32_t i = first + place_of(j, tid, SEL_THREADS);
+        if (i < N) best.take(src.score(i), i);
+    }
+    scratch[(long long)req * (ONELA_SELECT_PARTS * SEL_CAP) + blockIdx.x * SEL_THREADS + tid] = best.composite(src);
 }
 
-// one CTA per request: the top-k of the parts' lists (parts > 1) or of the candidates themselves (parts == 1)
-__global__ void __launch_bounds__(SEL_THREADS) select_merge_kernel(const float* __restrict__ beam_scores, const float* __restrict__ cand_logp,
-                                                                   int W_prev, int C, int k, int parts,
-                                                                   const unsigned long long* __restrict__ scratch, int32_t* __restrict__ parents,
-                                                                   int32_t* __restrict__ codes, float* __restrict__ scores) {
+// grid (CTAs of a cluster, requests).  SHARES: the candidates' largest per share of SEL_HELD come from scratch
+// (select_shares_kernel), and only the shares that reach the bound are looked into.  `scratch` ([request][ONELA_SELECT_PARTS *
+// SEL_CAP], or null): also where the candidates that reach the bound go when they do not fit in shared memory (behind the shares).
+template <bool SHARES>
+__global__ void __launch_bounds__(SEL_THREADS) select_kernel(const float* __restrict__ beam_scores, const float* __restrict__ cand_logp, int W_prev, int C,
+                                                             uint32_t magic, int shift, int k, unsigned long long* __restrict__ scratch,
+                                                             int32_t* __restrict__ parents, int32_t* __restrict__ codes, float* __restrict__ scores) {
+    extern __shared__ unsigned long long room[];             // [8][1024]: the threads' largest; later list and sort
     __shared__ SelectShared sh;
-    const int req = blockIdx.x;
-    const float* bs = beam_scores + (long long)req * W_prev;
-    const float* lp = cand_logp + (long long)req * W_prev * C;
+    __shared__ unsigned n_list, n_mine, n_hits, s_at;
+    __shared__ unsigned long long s_bound;
+    const int tid = threadIdx.x;
+    const int ctas = gridDim.x, rank = blockIdx.x, req = blockIdx.y;
+    if (tid == 0) n_mine = n_hits = 0u;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const uint32_t N = (uint32_t)W_prev * (uint32_t)C;
-    if (parts == 1) {
-        select_topk<SEL_PART / SEL_THREADS>(ScoreSource{bs, lp, 0u, C}, N, k, sh);
+    const ScoreSource src{beam_scores + (long long)req * W_prev, cand_logp + (long long)req * N, magic, shift, C};
+    parents += (long long)req * k;
+    codes += (long long)req * k;
+    scores += (long long)req * k;
+    if (scratch) scratch += (long long)req * (ONELA_SELECT_PARTS * SEL_CAP);
+    const uint32_t span = (uint32_t)ctas * SEL_THREADS, me = (uint32_t)rank * SEL_THREADS + tid;
+    const uint32_t items = SHARES ? (N + SEL_HELD * SEL_THREADS - 1) / (SEL_HELD * SEL_THREADS) * SEL_THREADS : N;     // candidates, or shares
+    const int stripes = (int)((items + span - 1) / span);
+    // 1. this thread's candidates (shares)
+    unsigned long long best = 0ull;
+    if constexpr (SHARES) {
+#pragma unroll 8
+        for (int j = 0; j < stripes; ++j) {
+            const uint32_t i = place_of(j, me, span);
+            if (i < items) best = max(best, __ldcg(scratch + i));
+        }
     } else {
-        // every part but the last left min(k, SEL_PART) composites; read them as one list with gaps skipped
-        const uint32_t kp = min((uint32_t)k, (uint32_t)SEL_PART);
-        const uint32_t last_n = N - (uint32_t)(parts - 1) * SEL_PART, last_kp = min((uint32_t)k, last_n);
-        struct Gapped {
-            const unsigned long long* base;
-            uint32_t kp;
-            __device__ __forceinline__ unsigned long long operator()(uint32_t i) const {
-                return base[(long long)(i / kp) * SEL_CAP + (i % kp)];
-            }
-        };
-        const Gapped src{scratch + (long long)req * SEL_PARTS_MAX * SEL_CAP, kp};
-        select_topk<16>(src, (uint32_t)(parts - 1) * kp + last_kp, k, sh);
+        Best top;
+#pragma unroll 8
+        for (int j = 0; j < stripes; ++j) {
+            const uint32_t i = place_of(j, me, span);
+            if (i < N) top.take(src.score(i), i);
+        }
+        best = top.composite(src);
     }
-    sort_and_emit(sh, k, bs, lp, C, parents + (long long)req * k, codes + (long long)req * k, scores + (long long)req * k);
+    // 2. the bound
+    unsigned long long bound = 1ull;                         // (a composite is never 0: the index word of a candidate is not)
+    if (ctas > 1) {
+        st_cluster64(in_first_cta(room + rank * SEL_THREADS + tid), best);
+        cluster_barrier();
+        if (rank == 0) {
+            unsigned long long mine[SEL_CTAS];
+#pragma unroll
+            for (int c = 0; c < SEL_CTAS; ++c) mine[c] = c < ctas ? room[c * SEL_THREADS + tid] : 0ull;
+            bound = bound_of(mine, k, sh);
+            if (tid == 0) { s_bound = bound; n_list = 0u; }
+        }
+        cluster_barrier();
+        if (rank != 0) bound = ld_cluster64(in_first_cta(&s_bound));
+    } else {
+        if (stripes > 1) {
+            const unsigned long long mine[1] = {best};
+            bound = bound_of(mine, k, sh);
+        }
+        if (tid == 0) n_list = 0u;
+        __syncthreads();
+    }
+    // 3. the candidates that reach it: the shares whose largest does are listed, then all threads look into their members;
+    // what they find goes to a list of this CTA's, which is then appended to the first CTA's
+    uint16_t* hits = reinterpret_cast<uint16_t*>(room + 2 * SEL_LIST);      // thread (+ 1024 x stripe: share), of this CTA
+    if constexpr (SHARES) {
+        if (best >= bound)
+            for (int j = 0; j < stripes; ++j) {
+                const uint32_t i = place_of(j, me, span);
+                if (i < items && __ldcg(scratch + i) >= bound) hits[atomicAdd(&n_hits, 1u)] = (uint16_t)(j * SEL_THREADS + tid);
+            }
+    } else if (best >= bound) {
+        hits[atomicAdd(&n_hits, 1u)] = (uint16_t)tid;
+    }
+    __syncthreads();
+    const int members = SHARES ? SEL_HELD : stripes;
+    auto each = [&](auto&& put) {
+        const int todo = (int)n_hits * members;
+#pragma unroll 2
+        for (int x = tid; x < todo; x += SEL_THREADS) {
+            const int q = x / members, m = x - q * members;
+            uint32_t i = hits[q];
+            if constexpr (SHARES) {                          // share i of stripe j: member m among the 16 384 candidates of its CTA
+                i = place_of((int)(i / SEL_THREADS), (uint32_t)rank * SEL_THREADS + (i & (SEL_THREADS - 1)), span);
+                i = i / SEL_THREADS * (SEL_HELD * SEL_THREADS) + place_of(m, i & (SEL_THREADS - 1), SEL_THREADS);
+            } else {
+                i = place_of(m, (uint32_t)rank * SEL_THREADS + i, span);
+            }
+            if (i < N) {
+                const unsigned long long c = src(i);
+                if (c >= bound) put(c);
+            }
+        }
+    };
+    unsigned long long* mine = room + SEL_LIST;              // (beside the first CTA's list)
+    each([&](unsigned long long c) {
+        const unsigned at = atomicAdd(&n_mine, 1u);
+        if (at < SEL_LIST) mine[at] = c;
+    });
+    __syncthreads();
+    const unsigned cnt = n_mine;
+    if (tid == 0) s_at = add_cluster(in_first_cta(&n_list), cnt);
+    __syncthreads();
+    {
+        const unsigned at = s_at;
+        const uint32_t list_at = in_first_cta(room);
+        for (unsigned i = tid; i < min(cnt, (unsigned)SEL_LIST); i += SEL_THREADS)
+            if (at + i < SEL_LIST) st_cluster64(list_at + (at + i) * 8, mine[i]);
+    }
+    cluster_barrier();
+    unsigned n;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(n) : "r"(in_first_cta(&n_list)) : "memory");
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");       // this thread has read the first CTA's memory
+    if (n > SEL_LIST && scratch) {
+        // too many for shared memory (candidates that gather in few threads' shares): the list again, to global memory
+        asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+        if (rank == 0 && tid == 0) n_list = 0u;
+        cluster_barrier();
+        unsigned long long* out = scratch + SEL_SHARES;
+        each([&](unsigned long long c) { out[add_cluster(in_first_cta(&n_list), 1u)] = c; });
+        __threadfence();
+        asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    }
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    if (rank != 0) return;
+    if (n <= SEL_THREADS) {
+        sort_and_emit<1>(room, room + SEL_LIST, (int)n, k, sh, src, parents, codes, scores);
+    } else if (n <= 2 * SEL_THREADS) {
+        sort_and_emit<2>(room, room + SEL_LIST, (int)n, k, sh, src, parents, codes, scores);
+    } else if (n <= SEL_LIST) {
+        sort_and_emit<SEL_LIST / SEL_THREADS>(room, room + SEL_LIST, (int)n, k, sh, src, parents, codes, scores);
+    } else {                                                 // exhaustively, over the list or over all candidates
+        if (scratch) {
+            const unsigned long long* list = scratch + SEL_SHARES;
+            select_topk<SEL_HELD>([&](uint32_t i) { return __ldcg(list + i); }, n, k, sh);
+        } else {
+            select_topk<SEL_HELD>(src, N, k, sh);
+        }
+        sort_and_emit<1>(sh.sel, room, k, k, sh, src, parents, codes, scores);
+    }
 }
 
 }  // namespace
+
+int select_launches(long long candidates) { return candidates > (long long)SEL_CTAS * SEL_HELD * SEL_THREADS ? 2 : 1; }
 
 cudaError_t launch_select(const float* beam_scores, const float* cand_logp, int32_t req_count, int32_t W_prev, int32_t C,
                           int32_t W_new, unsigned long long* scratch, int32_t* parents, int32_t* codes, float* scores,
                           cudaStream_t stream) {
     const long long N = (long long)W_prev * C;
-    const int parts = (int)((N + SEL_PART - 1) / SEL_PART);
-    if (parts > SEL_PARTS_MAX) return cudaErrorInvalidValue;
-    if (parts > 1) {
-        select_part_kernel<<<dim3(parts, req_count), SEL_THREADS, 0, stream>>>(beam_scores, cand_logp, W_prev, C, W_new, scratch);
-        cudaError_t e = cudaGetLastError();
+    if (N > (long long)ONELA_SELECT_PARTS * 4096) return cudaErrorInvalidValue;
+    // CTAs per request: one while the candidates are at most four per thread (the exchange between CTAs costs more than the
+    // loads it shares out), then as many as keep them in registers, up to a portable cluster; beyond that the candidates are
+    // cut into shares first, on as many SMs as there are (one cluster alone read a million candidates at 31 us)
+    const int ctas = N <= 4 * SEL_THREADS ? 1 : N <= 2 * SEL_HELD * SEL_THREADS ? 2 : N <= 4 * SEL_HELD * SEL_THREADS ? 4 : SEL_CTAS;
+    const bool shares = scratch && select_launches(N) > 1;
+    // the threads' largest, later list and sort buffer: 64 KB; the shares that reach the bound: 16 KB
+    constexpr int SMEM = SEL_CTAS * SEL_THREADS * (int)sizeof(unsigned long long) + SEL_SHARES / SEL_CTAS * (int)sizeof(uint16_t);
+    static_assert(2 * SEL_LIST == SEL_CTAS * SEL_THREADS, "list and sort buffer");
+    static_assert(SEL_SHARES + (SEL_CAP + SEL_CAP / 8) * (ONELA_SELECT_PARTS * 4096 / (SEL_CTAS * SEL_THREADS)) <= ONELA_SELECT_PARTS * SEL_CAP, "scratch");
+    // one-time set-up per device (function attributes belong to a device's context)
+    constexpr int MAX_DEVICES = 64;
+    static std::mutex setup_mutex;
+    static bool ready[MAX_DEVICES] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEVICES) return cudaErrorInvalidDevice;
+    {
+        std::lock_guard<std::mutex> lock(setup_mutex);
+        if (!ready[dev]) {
+            cudaError_t e = cudaFuncSetAttribute(select_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(select_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+            if (e != cudaSuccess) return e;
+            ready[dev] = true;
+        }
+    }
+    uint32_t magic;
+    int shift;
+    divide_by(C, magic, shift);
+    if (shares) {
+        const unsigned parts = (unsigned)((N + SEL_HELD * SEL_THREADS - 1) / (SEL_HELD * SEL_THREADS));
+        const cudaError_t e = launch_dependent(select_shares_kernel, dim3(parts, req_count), dim3(SEL_THREADS), 0, stream, beam_scores, cand_logp, W_prev,
+                                               C, magic, shift, scratch);
         if (e != cudaSuccess) return e;
     }
-    select_merge_kernel<<<req_count, SEL_THREADS, 0, stream>>>(beam_scores, cand_logp, W_prev, C, W_new, parts, scratch, parents,
-                                                               codes, scores);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ctas, req_count);
+    cfg.blockDim = dim3(SEL_THREADS);
+    cfg.dynamicSmemBytes = SMEM;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = ctas;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    auto kern = shares ? select_kernel<true> : select_kernel<false>;
+    return cudaLaunchKernelEx(&cfg, kern, beam_scores, cand_logp, W_prev, C, magic, shift, W_new, scratch, parents, codes, scores);
 }
 
 }  // namespace onela
 
 // ---------------------------------------------------------------------------------------------------------------
-// Beam selection without a workspace (declared in onela.h as onela_select_beams_static).
-//
-// The partial lists go to an array that is part of the library image instead of the caller's workspace.  Its size is
-// fixed when the library is built: room for STATIC_REQUESTS requests of the same candidate count the workspace
-// version takes (ONELA_SELECT_PARTS parts of 4096 candidates, ONELA_SELECT_CAP survivors each) = 4 MiB, which
-// every GPU that loads the library holds until the process ends.  In host code the array's name is only a handle;
-// the device address comes from cudaGetSymbolAddress, asked for once per device on that device's first call.
-namespace onela {
-namespace {
-
-constexpr int STATIC_REQUESTS = 2;
-static __device__ __align__(256) unsigned long long g_static_select_scratch[(size_t)STATIC_REQUESTS * ONELA_SELECT_PARTS * ONELA_SELECT_CAP];
-
-constexpr int MAX_DEVICES = 64;
-std::mutex g_static_mutex;
-unsigned long long* g_static_ptr[MAX_DEVICES] = {};
-
-// device address of the array on the current device; nullptr when the runtime refuses
-unsigned long long* static_scratch_of_current_device() {
-    int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEVICES) return nullptr;
-    std::lock_guard<std::mutex> lock(g_static_mutex);
-    if (!g_static_ptr[dev]) {
-        void* p = nullptr;
-        if (cudaGetSymbolAddress(&p, g_static_select_scratch) != cudaSuccess) return nullptr;
-        g_static_ptr[dev] = static_cast<unsigned long long*>(p);
-    }
-    return g_static_ptr[dev];
-}
-
-}  // namespace
-}  // namespace onela
-
+// Beam selection without a workspace (declared in onela.h as onela_select_beams_static): the same launch, which needs no
+// device memory beyond the CTAs' own; where too many candidates reach the bound for shared memory, the exhaustive selection
+// runs over the candidates themselves.
 extern "C" onela_status onela_select_beams_static(const float* beam_scores_dev, const float* cand_logp_dev, int32_t req_count,
                                                   int32_t W_prev, int32_t C, int32_t W_new, int32_t* parents_out_dev,
                                                   int32_t* codes_out_dev, float* scores_out_dev, void* stream) {
     using namespace onela;
     if (!beam_scores_dev || !cand_logp_dev || !parents_out_dev || !codes_out_dev || !scores_out_dev) return ONELA_E_INVAL;
     if (req_count < 1 || W_prev < 1 || C < 1 || W_new < 1) return ONELA_E_INVAL;
-    // beyond what the built-in array holds: the caller has to use onela_select_beams with a workspace, or split the batch
+    // the call's documented limits: beyond them the caller has to use onela_select_beams, or split the batch
+    constexpr int STATIC_REQUESTS = 2;
     if (req_count > STATIC_REQUESTS) return ONELA_E_CAPACITY;
     if ((int64_t)W_prev * C > (int64_t)ONELA_SELECT_PARTS * 4096) return ONELA_E_CAPACITY;
     if (W_new > ONELA_SELECT_CAP || W_new > (int64_t)W_prev * C) return ONELA_E_CAPACITY;
-    unsigned long long* scratch = static_scratch_of_current_device();
-    if (!scratch) return ONELA_E_CUDA;
-    // nothing in the array has to start at zero: every word the merge step reads is written by the part step of
-    // the same call
-    if (launch_select(beam_scores_dev, cand_logp_dev, req_count, W_prev, C, W_new, scratch, parents_out_dev, codes_out_dev,
+    if (launch_select(beam_scores_dev, cand_logp_dev, req_count, W_prev, C, W_new, nullptr, parents_out_dev, codes_out_dev,
                       scores_out_dev, static_cast<cudaStream_t>(stream)) != cudaSuccess)
         return ONELA_E_CUDA;
     return ONELA_OK;
