@@ -1,6 +1,6 @@
 // Warp-specialised fused decode kernel for B200 (sm_100a): dk = dv = 128, bf16 records.
 //
-// One persistent CTA per SM, 16 warps in two roles coupled only by mbarriers:
+// One persistent CTA per SM, 17 warps in three roles coupled only by mbarriers:
 //   * 12 FOLD warps.  8 lanes own one (beam, head) unit; a warp folds 4 units at a time ("quad"): query
 //     folded through the unit's records newest -> oldest (c = k.r; corr += beta c v; r -= beta c k; decay a
 //     scalar; packed fp32x2 FMAs).  A quad's query and own record arrive through a per-warp stage of 16-byte
@@ -8,13 +8,12 @@
 //     warp also writes them to the arena.  Results go into a
 //     ring slot in shared memory: the folded query as a row of the K-major 128-byte-swizzled MMA operand
 //     (fp16, times a power of two that keeps the row inside fp16's range), corr as a row of the slot's corr tile.
-//   * 4 EPILOGUE warps (one per tensor-memory lane quadrant).  One lane of the first issues a group's 8 MMAs
-//     once all its rows are written - one group ahead of the epilogue, so neither the issuing nor the MMAs'
-//     latency lies between two epilogues.  When a group's MMAs have completed the four warps read the
-//     accumulator and transpose it, by plain stores, over the slot's operand rows (dead by then); the other
-//     three warps add that tile to the corr tile and store the outputs as coalesced 16-byte rows while the
-//     first issues the next group; then the slot is handed back.  They also prepare the next segment (below)
-//     while the fold warps work on the current one.
+//   * One MMA warp issues a group's 8 MMAs once all its rows are written.
+//   * 4 EPILOGUE warps (one per tensor-memory lane quadrant).  When a group's MMAs have completed they read the
+//     accumulators in a fragment layout (a thread has two neighbouring beams of an output), add the corr tile, transpose
+//     through matrix stores over the slot's operand rows (dead by then) and store the outputs as coalesced 16-byte
+//     rows; then the slot is handed back.  They also prepare the next segment (below) while the fold warps work on the
+//     current one.
 // Two ring slots (operand rows, corr tile, 48 accumulator columns each) keep the MMA and the epilogue of one
 // group under the folds of the next.  Work = groups of 48 consecutive beams of one (request, head), a
 // contiguous range per CTA chosen on the host; consecutive groups of one head form a segment.  Per segment the
@@ -54,22 +53,26 @@ constexpr int FOLD_WARPS = ONELA_FOLD_WARPS;
 constexpr int LPU = ONELA_LPU;                      // lanes per (beam, head) unit
 constexpr int UPW = 32 / LPU;                       // units a fold warp folds at a time (a "quad" when LPU = 8)
 constexpr int NCH = 16 / LPU;                       // 16-byte chunks per lane per 256-byte vector
-constexpr int THREADS = (FOLD_WARPS + 4) * 32;      // + 4 epilogue warps (16 warps: four per SM sub-partition)
+constexpr int THREADS = (FOLD_WARPS + 5) * 32;      // + 4 epilogue warps + the warp that issues the MMAs
+constexpr int MMA_WARP = FOLD_WARPS + 4;
 constexpr int GN = FOLD_WARPS * UPW;                // beams per group = MMA N (48)
 constexpr int R_KB_STRIDE = GN * 128;               // bytes between the two K blocks (64 fp16 each) of the operand
-constexpr int R_BYTES = 4 * R_KB_STRIDE;            // a slot's first tile: the group's operand rows (its first half),
-                                                    // later the transposed accumulators (all of it)
-constexpr int C_BYTES = GN * DV * 4;                // corr tile, row = beam
-constexpr int SLOT_BYTES = R_BYTES + C_BYTES;
+constexpr int OUT_PITCH = 256 + 16;                 // bytes between the rows of a group's bf16 outputs (bank-conflict-free)
+constexpr int R_BYTES = GN * OUT_PITCH;             // a slot's first tile: the group's operand rows, later its outputs as bf16
+constexpr int C_PITCH = DV + 4;                     // floats between the rows of the corr tile (bank-conflict-free)
+constexpr int C_BYTES = GN * C_PITCH * 4;           // corr tile, row = beam (fp32 outputs are formed in it)
+constexpr int SLOT_BYTES = (R_BYTES + C_BYTES + 1023) / 1024 * 1024;
+static_assert(R_BYTES >= 2 * R_KB_STRIDE && R_BYTES % 16 == 0, "the outputs lie over the operand rows");
 constexpr int SLOTS = 2;
 constexpr int HEAD_BYTES = UPW * (REC_BYTES + DK * 2);   // one quad's heads: own records + queries of its units
 constexpr int HEADS_TOTAL = FOLD_WARPS * HEAD_BYTES;     // one stage per fold warp (a deeper ring measured slower)
 #ifndef ONELA_STAGE_BUF
-#define ONELA_STAGE_BUF 58
+#define ONELA_STAGE_BUF 64
 #endif
 // Two staging buffers of STAGE_BUF distinct ancestor records each (segment s uses buffer s & 1); a CTA whose whole
 // range is one segment uses them as one.  Sized so that the CTA stays within the 196 KiB shared-memory carve-out
 // (what is left of the SM's 256 KiB serves the gathered records as L1).
+// (58 -> 64 records: beam-512 stack at depth 8 46 -> 42.5 us, its parents' level then fits more often.)
 constexpr int STAGE_BUF = ONELA_STAGE_BUF;
 constexpr int STAGE_BYTES = 2 * STAGE_BUF * REC_BYTES;
 constexpr int GATE_BYTES = (2 * STAGE_BUF * 8 + 127) & ~127;   // padded: the heads' stages behind it stay 128-byte aligned (measured: 1.5 % faster)
@@ -84,19 +87,17 @@ constexpr int SMEM_BYTES = SLOTS * SLOT_BYTES + STAGE_BYTES + GATE_BYTES + HEADS
 // query and its own key, both projected through the parent state - so a group holds GN / 2 beams; per ring slot the
 // beams' own value rows (raw) and three scalars each (alpha_t, beta_t, k_t . q_t) wait for the epilogue.
 constexpr int DELTA_BEAMS = GN / 2;
-constexpr int DELTA_SLOT_BYTES = DELTA_BEAMS * (DV * 2) + DELTA_BEAMS * 16;
+constexpr int DELTA_V_PITCH = DV * 2 + 16;       // (bank-conflict-free)
+constexpr int DELTA_SLOT_BYTES = DELTA_BEAMS * DELTA_V_PITCH + DELTA_BEAMS * 16;
 constexpr int SMEM_BYTES_DELTA = SMEM_BYTES + SLOTS * DELTA_SLOT_BYTES;
 static_assert(SMEM_BYTES_DELTA <= 232448, "shared memory per CTA (delta records)");
-static_assert((DELTA_BEAMS * 16) % 96 == 0, "three storing warps share a delta group's 16-byte chunks evenly");
 constexpr uint32_t S0_COL = 128;                 // accumulators of the ring slots in [0, SLOTS * GN); S_0 buffers (64 columns) at 128 and 256
 constexpr int R_TARGET = 8;                      // a scaled operand row's largest element lies in [2^8, 2^9) x (decay in [1, 2)): far inside fp16's range
 constexpr uint32_t TMEM_COLS = 512;
-static_assert(SLOTS * GN <= 128, "accumulator columns");
-static_assert(R_BYTES >= C_BYTES, "the accumulators are transposed over the operand rows");
+static_assert(SLOTS * GN <= 128 && GN == 48, "accumulator columns");
 static_assert(2 * STAGE_BUF <= 128, "one staged record per epilogue lane");
 static_assert(SMEM_BYTES <= 232448, "shared memory per CTA");
 static_assert(GN % 16 == 0 && GN >= 16 && GN <= 256, "MMA N");
-static_assert((GN * 16) % 96 == 0, "three storing warps share a group's 16-byte chunks evenly");
 using L = Lanes<LPU>;
 using RecT = L::R;
 
@@ -149,7 +150,9 @@ struct Head {           // what a unit's fold needs first
 
 // Contiguous ranges of groups, one per CTA, balanced on the host with the cost of starting a segment counted in.
 constexpr int MAX_CTAS = DECODE_MAX_CTAS;
-using Partition = DecodePartition;
+struct Partition {
+    int4 cta[MAX_CTAS + 1];      // first group; its place within its (request, head) pair; request | segments << 8; head
+};
 
 // GROUPED: value head h reads the queries and keys of key head h / g; a.H counts VALUE heads, the record's k lives in
 // the key heads' plane (a.kv) and its v in the value heads' plane (a.vv), 256 bytes each.
@@ -164,7 +167,7 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
     const uint32_t base = (raw + 1023u) & ~1023u;            // swizzle atoms need 1024-byte alignment
     uint8_t* smem = smem_raw + (base - raw);
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // (warp: uniform for the compiler too)
     uint8_t* ring = smem;
     uint8_t* stage = ring + SLOTS * SLOT_BYTES;
     float2* gates_s = reinterpret_cast<float2*>(stage + STAGE_BYTES);
@@ -179,7 +182,7 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
     uint8_t* delta_s = heads + HEADS_TOTAL + 256 + INV_BYTES;                // DELTA: [SLOTS][value rows | scalars]
 #ifdef ONELA_WS_TL
     unsigned long long* tl_s = reinterpret_cast<unsigned long long*>(delta_s + (DELTA ? SLOTS * DELTA_SLOT_BYTES : 0));
-    const int tl_role = (int)blockIdx.x != g_ws_tl_cta ? -1 : warp == 0 ? 0 : warp == FOLD_WARPS ? 1 : warp == FOLD_WARPS + 1 ? 2 : -1;
+    const int tl_role = (int)blockIdx.x != g_ws_tl_cta ? -1 : warp == 0 ? 0 : warp == MMA_WARP ? 1 : warp == FOLD_WARPS ? 2 : -1;
     int tl_n = 0;
 #endif
     constexpr int BPG = DELTA ? DELTA_BEAMS : GN;                            // beams per group
@@ -215,13 +218,18 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the next launch may set itself up under this one
     TL(1, 0);   // tensor memory allocated, barriers ready
 
-    const int g_begin = part.begin[blockIdx.x], g_end = part.begin[blockIdx.x + 1];
-    const int pair_begin = g_begin / groups_per_pair;
-    const int n_segs = g_begin < g_end ? (g_end - 1) / groups_per_pair - pair_begin + 1 : 0;
+    const int4 mine = part.cta[blockIdx.x];
+    const int g_begin = mine.x, g_end = part.cta[blockIdx.x + 1].x, gip_begin = mine.y, n_segs = mine.z >> 8;
+    const int req_begin = mine.z & 255, h_begin = mine.w;
+    // request and head of segment `seg` of this CTA (host-made starting point: divisions here delayed every launch)
+    auto pair_of = [&](int seg, int& req, int& h) {
+        req = req_begin;
+        for (h = h_begin + seg; h >= a.H; h -= a.H) ++req;
+    };
     const bool single = n_segs == 1;                       // one segment: the two staging buffers serve as one
     const int stage_cap = single ? 2 * STAGE_BUF : STAGE_BUF;
     const int old = a.depth - 1;          // records older than a beam's own: levels old-1 .. 0
@@ -252,23 +260,41 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
     // Row-major fp32 in the store; lane i of tensor memory holds row i, two elements per column; the 64 columns of
     // buffer `buf` start at S0_COL + 128 buf.  A warp takes the 32 rows of its lane quadrant and the 32-element blocks
     // kb0, kb0 + step, ...; the S_0 after this one is requested into L2 on the way.
-    auto load_s0 = [&](int pair_now, int buf, int kb0, int step, bool has_next) {
+    // A block goes over in the 16 x 256-bit fragment layout: four threads share 64 consecutive bytes of a row, so a load
+    // touches 8 lines.  (With a row per thread - the 32 x 32-bit layout - it touched 32, and the 128 loads of a state kept
+    // the load unit busy for 4096 cycles: 2.4 us of every launch passed between a CTA's set-up and its dependency wait.)
+    auto s0_fragment = [&](int quad) { return (long long)(quad * 32 + (lane >> 2)) * DK + (lane & 3) * 4; };
+    auto request_s0 = [&](const float* p, float4* x) {
+#pragma unroll
+        for (int c = 0; c < 8; ++c)          // rows + 8 (c & 3), columns + 16 (c >> 2) of the 32 x 32 block
+            x[c] = __ldg(reinterpret_cast<const float4*>(p + (c & 3) * (8 * DK) + (c >> 2) * 16));
+    };
+    auto store_s0 = [&](uint32_t taddr, const float4* x, float sc) {
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            uint32_t v[8];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const float4 y = x[(c >> 1) * 4 + half * 2 + (c & 1)];
+                v[2 * c] = pack_f16x2(y.x * sc, y.y * sc);
+                v[2 * c + 1] = pack_f16x2(y.z * sc, y.w * sc);
+            }
+            tmem_st_16x16(taddr + ((uint32_t)(half * 16) << 16), v);
+        }
+    };
+    auto load_s0 = [&](int seg, int buf, int kb0, int step, bool has_next) {
         const int quad = warp & 3, i = quad * 32 + lane;
-        const int req = pair_now / a.H, h = pair_now - req * a.H;
-        const float* row = a.s0 + req * a.s0_req_stride + (long long)h * (DV * DK) + (long long)i * DK;
+        int req, h, nreq = 0, nh = 0;
+        pair_of(seg, req, h);
+        if (has_next) pair_of(seg + 1, nreq, nh);
+        const float* block = a.s0 + req * a.s0_req_stride + (long long)h * (DV * DK) + s0_fragment(quad);
         const float sc = __ldg(a.s0_scale + req * a.s0_scale_req_stride + value_head(h));
 #pragma unroll 1
         for (int kb = kb0; kb < 4; kb += step) {
-            uint32_t v[16];
-#pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                const float4 x = __ldg(reinterpret_cast<const float4*>(row + kb * 32) + c);
-                v[2 * c] = pack_f16x2(x.x * sc, x.y * sc);
-                v[2 * c + 1] = pack_f16x2(x.z * sc, x.w * sc);
-            }
-            tmem_st16(tmem_base + S0_COL + buf * 128 + kb * 16 + ((uint32_t)(quad * 32) << 16), v);
+            float4 x[8];
+            request_s0(block + kb * 32, x);
+            store_s0(tmem_base + S0_COL + buf * 128 + kb * 16 + ((uint32_t)(quad * 32) << 16), x, sc);
             if (has_next) {
-                const int nreq = (pair_now + 1) / a.H, nh = (pair_now + 1) - nreq * a.H;
                 const float* nrow = a.s0 + nreq * a.s0_req_stride + (long long)nh * (DV * DK) + (long long)i * DK + kb * 32;
                 asm volatile("prefetch.global.L2 [%0];" ::"l"(nrow));
             }
@@ -284,27 +310,19 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
     float4 s0_first[8];
     float s0_first_scale = 1.f;
     if (n_segs > 0 && s0_mine) {
-        const int req = pair_begin / a.H, h = pair_begin - req * a.H;
+        const int req = req_begin, h = h_begin;
         s0_first_scale = __ldg(a.s0_scale + req * a.s0_scale_req_stride + value_head(h));
-        const float* row = a.s0 + req * a.s0_req_stride + (long long)h * (DV * DK) + (long long)((warp & 3) * 32 + lane) * DK + (warp >> 2) * 32;
-#pragma unroll
-        for (int c = 0; c < 8; ++c) s0_first[c] = __ldg(reinterpret_cast<const float4*>(row) + c);
+        request_s0(a.s0 + req * a.s0_req_stride + (long long)h * (DV * DK) + s0_fragment(warp & 3) + (warp >> 2) * 32, s0_first);
         if (n_segs > 1) {
-            const int nreq = (pair_begin + 1) / a.H, nh = (pair_begin + 1) - nreq * a.H;
+            int nreq, nh;
+            pair_of(1, nreq, nh);
             asm volatile("prefetch.global.L2 [%0];" ::"l"(a.s0 + nreq * a.s0_req_stride + (long long)nh * (DV * DK) +
                                                           (long long)((warp & 3) * 32 + lane) * DK + (warp >> 2) * 32));
         }
     }
     auto put_first_s0 = [&]() {
         if (n_segs == 0 || !s0_mine) return;
-        const float sc = s0_first_scale;
-        uint32_t v[16];
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            v[2 * c] = pack_f16x2(s0_first[c].x * sc, s0_first[c].y * sc);
-            v[2 * c + 1] = pack_f16x2(s0_first[c].z * sc, s0_first[c].w * sc);
-        }
-        tmem_st16(tmem_base + S0_COL + (warp >> 2) * 16 + ((uint32_t)((warp & 3) * 32) << 16), v);
+        store_s0(tmem_base + S0_COL + (warp >> 2) * 16 + ((uint32_t)((warp & 3) * 32) << 16), s0_first, s0_first_scale);
         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncwarp();
@@ -355,11 +373,10 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
         };
         Unit u0;                                         // this warp's current quad; u1, u2: the next two
         {
-            const int pair = g_begin / groups_per_pair;
             u0.seg = 0;
-            u0.req = pair / a.H;
-            u0.h = pair - u0.req * a.H;
-            u0.gip = g_begin - pair * groups_per_pair;
+            u0.req = req_begin;
+            u0.h = h_begin;
+            u0.gip = gip_begin;
         }
         // The heads of a quad (own record and query of its units) arrive by 16-byte async copies into the warp's
         // stage, one quad ahead of their use (each lane copies exactly the chunks it reads back); the gates ride in
@@ -693,7 +710,7 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
                         *reinterpret_cast<uint4*>(row + (((ci & 7) ^ sw) << 4)) =
                             make_uint4(pack_f16x2(x[0].x, x[0].y), pack_f16x2(x[1].x, x[1].y), pack_f16x2(x[2].x, x[2].y),
                                        pack_f16x2(x[3].x, x[3].y));
-                        float* crow = C_s + u * DV;
+                        float* crow = C_s + u * C_PITCH;
                         *reinterpret_cast<float4*>(crow + corr_chunk(2 * ci) * 4) =
                             make_float4(corr[4 * c].x, corr[4 * c].y, corr[4 * c + 1].x, corr[4 * c + 1].y);
                         *reinterpret_cast<float4*>(crow + corr_chunk(2 * ci + 1) * 4) =
@@ -704,8 +721,8 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
                     uint8_t* ds = delta_s + s * DELTA_SLOT_BYTES;
                     const int bq = u >> 1;
 #pragma unroll
-                    for (int c = 0; c < NCH; ++c) *reinterpret_cast<uint4*>(ds + bq * (DV * 2) + (c * LPU + g) * 16) = cur.own.v[c];
-                    if (g == 0) *reinterpret_cast<float4*>(ds + DELTA_BEAMS * (DV * 2) + bq * 16) = make_float4(cur.own.gate.x, cur.own.gate.y, kq, 0.f);
+                    for (int c = 0; c < NCH; ++c) *reinterpret_cast<uint4*>(ds + bq * DELTA_V_PITCH + (c * LPU + g) * 16) = cur.own.v[c];
+                    if (g == 0) *reinterpret_cast<float4*>(ds + DELTA_BEAMS * DELTA_V_PITCH + bq * 16) = make_float4(cur.own.gate.x, cur.own.gate.y, kq, 0.f);
                 }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy writes -> visible to the MMA
                 __syncwarp();
@@ -750,17 +767,46 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
         }
         if (ahead) fold_quads(std::true_type{});
         else fold_quads(std::false_type{});
+    } else if (warp == MMA_WARP) {
+        // =============================== MMA ISSUE ===============================
+        // A group's 8 MMAs go out as soon as its rows are written and its segment's S_0 is in place (complete rows imply that
+        // the epilogue has read the accumulators of two groups ago: a slot's rows are written after it was handed back).
+        int seg = 0, gip = gip_begin;
+        bool seg_first = true;
+        for (int gcount = 0; gcount < g_end - g_begin; ++gcount) {
+            const int s = gcount % SLOTS, use = gcount / SLOTS;
+            TL(20, gcount);  // issue: waiting for the rows
+            bool ok = wait_or_abort(bar_full(s), use & 1, abort_flag);
+            TL(21, gcount);  // issue: rows complete
+            // segment 0's S_0 has a barrier of its own; segment seg >= 1 is use ((seg + 1) >> 1) - 1 of its buffer's barrier
+            if (ok && seg_first) ok = seg == 0 ? wait_or_abort(bar_s0_first, 0, abort_flag) : wait_or_abort(bar_s0(seg & 1), (((seg + 1) >> 1) - 1) & 1, abort_flag);
+            if (!__all_sync(0xffffffffu, ok)) { dead = true; break; }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            constexpr uint32_t idesc = idesc_f16(GN);
+            const uint64_t bd = umma_desc(smem_u32(ring + s * SLOT_BYTES));
+            const uint32_t s0_at = tmem_base + S0_COL + (seg & 1) * 128;
+#pragma unroll
+            for (int kb = 0; kb < 2; ++kb)          // K block of 64 elements; 16 elements (32 bytes, 8 columns) per MMA
+#pragma unroll
+                for (int ks = 0; ks < 4; ++ks)
+                    mma_ts(tmem_base + s * GN, s0_at + (kb * 4 + ks) * 8, bd + (uint64_t)((kb * R_KB_STRIDE + ks * 32) >> 4), idesc, (kb | ks) != 0);
+            mma_commit(bar_done(s));   // arrives when the MMAs above have completed
+            TL(22, gcount);  // issue: MMAs out
+            seg_first = ++gip == groups_per_pair;
+            if (seg_first) { gip = 0; ++seg; }
+        }
+        if (dead && lane == 0) *abort_flag = 1;
     } else {
-        // =============================== EPILOGUE (+ MMA issue, + preparation of the next segments) ===============================
+        // =============================== EPILOGUE (+ preparation of the next segments) ===============================
         dependency_wait();
         const int quad = warp & 3;                    // tensor-memory lane quadrant of this warp
-        const int i = quad * 32 + lane;               // output element (dv index) of this thread
         int staged_issued[2] = {0, 0};                // stagings requested per buffer (what teardown must wait for)
         // Stage the distinct records of segment `seg`: one 512-byte bulk copy per record, its gates by a plain load, one
         // record per lane.  Every lane arrives once, announcing the bytes it requested; its gate store is ordered
         // before the arrival.  The barrier completes even when nothing is staged.
         auto stage_segment = [&](int seg) {
-            const int pair = pair_begin + seg, req = pair / a.H, h = pair - req * a.H;
+            int req, h;
+            pair_of(seg, req, h);
             const int b = single ? 0 : (seg & 1);
             int levels, count;
             staging_of(req, levels, count);
@@ -782,7 +828,7 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
         };
         // S_0 of segment `seg` (>= 1) into its tensor-memory buffer, by the four epilogue warps alone.
         auto prepare_s0 = [&](int seg) {
-            load_s0(pair_begin + seg, seg & 1, 0, 1, seg + 1 < n_segs);
+            load_s0(seg, seg & 1, 0, 1, seg + 1 < n_segs);
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_s0(seg & 1));
         };
@@ -793,43 +839,8 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
             prepare_s0(1);
         }
 
-        // The first epilogue warp issues a group's 8 MMAs as soon as all its rows are written (never a fold warp:
-        // whichever fold warp issued would be the last to finish its next quad).  It does so one group AHEAD: once
-        // the tile of group k is complete (the named barrier below) it issues group k + 1 while the other three
-        // warps store group k, so neither the issuing nor the MMAs' latency lies between two epilogues.
-        auto issue_mma = [&](int gcount, int seg, bool seg_first) -> bool {     // warp FOLD_WARPS only; true: gave up
-            const int s = gcount % SLOTS, use = gcount / SLOTS;
-            int mma_failed = 0;
-            if (lane == 0) {
-                TL(20, gcount);  // issue: waiting for the rows
-                bool ok = wait_or_abort(bar_full(s), use & 1, abort_flag);
-                TL(21, gcount);  // issue: rows complete
-                // segment 0's S_0 has a barrier of its own; segment seg >= 1 is use ((seg + 1) >> 1) - 1 of its
-                // buffer's barrier
-                if (ok && seg_first && seg >= 1) ok = wait_or_abort(bar_s0(seg & 1), (((seg + 1) >> 1) - 1) & 1, abort_flag);
-                if (ok && gcount == 0) ok = wait_or_abort(bar_s0_first, 0, abort_flag);
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                if (ok) {
-                    constexpr uint32_t idesc = idesc_f16(GN);
-                    const uint64_t bd = umma_desc(smem_u32(ring + s * SLOT_BYTES));
-                    const uint32_t s0_at = tmem_base + S0_COL + (seg & 1) * 128;
-#pragma unroll
-                    for (int kb = 0; kb < 2; ++kb)          // K block of 64 elements; 16 elements (32 bytes, 8 columns) per MMA
-#pragma unroll
-                        for (int ks = 0; ks < 4; ++ks)
-                            umma_f16_ts(tmem_base + s * GN, s0_at + (kb * 4 + ks) * 8,
-                                        bd + (uint64_t)((kb * R_KB_STRIDE + ks * 32) >> 4), idesc, (kb | ks) ? 1u : 0u);
-                } else {
-                    mma_failed = 1;
-                }
-                umma_commit(bar_done(s));   // arrives when the MMAs above have completed
-                TL(22, gcount);  // issue: MMAs out
-            }
-            return __shfl_sync(0xffffffffu, mma_failed, 0) != 0;
-        };
-        // (request, head, group within the pair) of the group at hand, advanced without divisions
-        int pair = pair_begin, req = pair / a.H, h = pair - req * a.H, gip = g_begin - pair * groups_per_pair;
-        int issued = 0;                               // groups whose MMAs have been issued (first epilogue warp)
+        // (request, head, group within the pair, segment) of the group at hand, advanced without divisions
+        int req = req_begin, h = h_begin, gip = gip_begin, seg = 0;
         // A warp that gives up (`fail`) never leaves on its own: it skips its work, raises the abort flag and keeps
         // arriving at the iteration's named barrier, whose OR makes all four warps leave in the same iteration.
         bool fail = false;
@@ -837,113 +848,110 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
             fail = true;
             if (lane == 0) *abort_flag = 1;
         };
+        const int et = (warp - FOLD_WARPS) * 32 + lane;
+        const int fr = lane >> 2, fc = (lane & 3) * 2;        // this thread's place in the accumulators' fragments: output, beam
         for (int gcount = 0; gcount < g_end - g_begin; ++gcount) {
             const int s = gcount % SLOTS, use = gcount / SLOTS;
-            const int seg = pair - pair_begin;
             const bool seg_first = gcount == 0 || gip == 0;
-            const bool has_next = gcount + 1 < g_end - g_begin;
-            const bool next_first = gip + 1 == groups_per_pair;      // the next group opens a segment
-            if (!fail && warp == FOLD_WARPS && issued == gcount) {
-                if (issue_mma(gcount, seg, seg_first)) give_up();
-                ++issued;
-            }
             TL(30, gcount);  // epilogue: waiting for the accumulators
             if (!fail && !wait_or_abort(bar_done(s), use & 1, abort_flag)) give_up();
             TL(31, gcount);  // epilogue: accumulators complete
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            float* C_s = reinterpret_cast<float*>(ring + s * SLOT_BYTES + R_BYTES);
+            uint8_t* O_s = ring + s * SLOT_BYTES;             // bf16 outputs, over the operand rows (dead once the MMAs have completed)
+            float* C_s = reinterpret_cast<float*>(O_s + R_BYTES);
+            const uint8_t* ds = delta_s + s * DELTA_SLOT_BYTES;
             const int b0 = gip * BPG;
-            const uint32_t taddr = tmem_base + s * GN + ((uint32_t)(quad * 32) << 16);
-            float* A_s = reinterpret_cast<float*>(ring + s * SLOT_BYTES);   // the operand rows are dead once the MMAs have completed
             if (!fail) {
-                // accumulator rows (dv) of this thread, all beams of the group, transposed into a tile laid out like
-                // the corr tile, over the slot's operand rows (plain stores: nothing here waits for a shared-memory read)
-                uint32_t v[GN];
+                // The accumulators (lane = output, column = beam) come in the 16 x 256-bit fragment layout: a thread has two
+                // neighbouring beams of an output, adds its corr elements, and the pair - packed to bf16 - goes out through
+                // a transposing matrix store, eight outputs of a beam per 16-byte row.  (As 32 x 32-bit rows written
+                // transposed in fp32, read back beside the corr tile and stored by three warps, a group took 1.75 us of
+                // these warps at every depth; 0.8 us now.)
+                float2 w[GN / 8];                             // what undoes the scales of each beam's row
 #pragma unroll
-                for (int c0 = 0; c0 < GN; c0 += 16) tmem_ld16(taddr + c0, v + c0);
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                const int ip = corr_chunk(i >> 2) * 4 + (i & 3);   // where the corr tile keeps element i of a row
+                for (int nb = 0; nb < GN / 8; ++nb) w[nb] = *reinterpret_cast<const float2*>(inv_s + s * GN + nb * 8 + fc);
+                uint32_t packed[4][GN / 8];
 #pragma unroll
-                for (int j = 0; j < GN; ++j) A_s[j * DV + ip] = __uint_as_float(v[j]);
-            }
-            // the four epilogue warps: tile complete - or somebody gave up, and then all four leave here together
-            if (bar_or(1, 128, fail ? 1 : 0)) { dead = true; break; }
-            TL(32, gcount);  // epilogue: tile transposed
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            if (warp == FOLD_WARPS) {
-                // This warp's part of the slot is read out; the next group's MMAs go out now - unless that group
-                // opens a segment whose S_0 this very iteration prepares below (a one-group segment).
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bar_free(s));
-                if (has_next && !(next_first && seg_first && seg >= 1)) {
-                    if (issue_mma(gcount + 1, seg + (next_first ? 1 : 0), next_first)) give_up();   // carried to the next barrier
-                    ++issued;
-                }
-            } else if constexpr (DELTA) {
-                // Eq. 2 and 4 on the two projections of each beam (rows 2 j and 2 j + 1 of the tile):
-                //   delta_t = beta_t (v_t - alpha_t S_{t-1} k_t) ,  o_t = alpha_t S_{t-1} q_t + delta_t (k_t . q_t) ;
-                // the output row and the record's delta half (in the record dtype) leave as 16-byte stores
-                const int et = (warp - FOLD_WARPS - 1) * 32 + lane;
-                const uint8_t* ds = delta_s + s * DELTA_SLOT_BYTES;
-                OutT* out0 = static_cast<OutT*>(a.out) + (((long long)req * a.W + b0) * a.H + h) * DV;
-                char* rec0 = a.kv_out + ((long long)h * a.arena_slots + a.bases.base[req] + b0) * REC_BYTES + DK * 2;
+                for (int half = 0; half < 2; ++half) {
+                    uint32_t v[GN / 2];
+                    const uint32_t taddr = tmem_base + s * GN + ((uint32_t)(quad * 32 + half * 16) << 16);
+                    tmem_ld_16x32(taddr, v);
+                    tmem_ld_16x16(taddr + 32, v + 16);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    const int dv0 = quad * 32 + half * 16 + fr;
+                    // where the corr tile keeps outputs dv0 and dv0 + 8 of a row
+                    const int p0 = corr_chunk(dv0 >> 2) * 4 + (dv0 & 3), p1 = corr_chunk((dv0 + 8) >> 2) * 4 + (dv0 & 3);
 #pragma unroll
-                for (int it = 0; it < DELTA_BEAMS * 16 / 96; ++it) {
-                    const int idx = it * 96 + et, j = idx >> 4, ch = idx & 15;
-                    if (b0 + j < a.W) {
-                        const int c0 = corr_chunk(2 * ch) * 4, c1 = corr_chunk(2 * ch + 1) * 4;
-                        const float wq = inv_s[s * GN + 2 * j], wk = inv_s[s * GN + 2 * j + 1];
-                        const float* Aq = A_s + (2 * j) * DV;
-                        const float* Cq = C_s + (2 * j) * DV;
-                        const float4 aq0 = *reinterpret_cast<const float4*>(Aq + c0), aq1 = *reinterpret_cast<const float4*>(Aq + c1);
-                        const float4 cq0 = *reinterpret_cast<const float4*>(Cq + c0), cq1 = *reinterpret_cast<const float4*>(Cq + c1);
-                        const float4 ak0 = *reinterpret_cast<const float4*>(Aq + DV + c0), ak1 = *reinterpret_cast<const float4*>(Aq + DV + c1);
-                        const float4 ck0 = *reinterpret_cast<const float4*>(Cq + DV + c0), ck1 = *reinterpret_cast<const float4*>(Cq + DV + c1);
-                        const float uq[8] = {fmaf(aq0.x, wq, cq0.x), fmaf(aq0.y, wq, cq0.y), fmaf(aq0.z, wq, cq0.z), fmaf(aq0.w, wq, cq0.w),
-                                             fmaf(aq1.x, wq, cq1.x), fmaf(aq1.y, wq, cq1.y), fmaf(aq1.z, wq, cq1.z), fmaf(aq1.w, wq, cq1.w)};
-                        const float uk[8] = {fmaf(ak0.x, wk, ck0.x), fmaf(ak0.y, wk, ck0.y), fmaf(ak0.z, wk, ck0.z), fmaf(ak0.w, wk, ck0.w),
-                                             fmaf(ak1.x, wk, ck1.x), fmaf(ak1.y, wk, ck1.y), fmaf(ak1.z, wk, ck1.z), fmaf(ak1.w, wk, ck1.w)};
-                        const float4 sc = *reinterpret_cast<const float4*>(ds + DELTA_BEAMS * (DV * 2) + j * 16);     // alpha_t, beta_t, k_t . q_t
-                        float2 vx[4];
-                        unpack8(*reinterpret_cast<const uint4*>(ds + j * (DV * 2) + ch * 16), vx);
-                        const float vv[8] = {vx[0].x, vx[0].y, vx[1].x, vx[1].y, vx[2].x, vx[2].y, vx[3].x, vx[3].y};
-                        float dl[8], o[8];
+                    for (int nb = 0; nb < GN / 8; ++nb) {
+                        float* c = C_s + (nb * 8 + fc) * C_PITCH;
+                        float o[4] = {fmaf(__uint_as_float(v[4 * nb]), w[nb].x, c[p0]), fmaf(__uint_as_float(v[4 * nb + 1]), w[nb].y, c[C_PITCH + p0]),
+                                      fmaf(__uint_as_float(v[4 * nb + 2]), w[nb].x, c[p1]), fmaf(__uint_as_float(v[4 * nb + 3]), w[nb].y, c[C_PITCH + p1])};
+                        if constexpr (DELTA) {
+                            // Eq. 2 and 4 on the two projections of a beam (its rows of the group are neighbours):
+                            //   delta_t = beta_t (v_t - alpha_t S_{t-1} k_t) ,  o_t = alpha_t S_{t-1} q_t + delta_t (k_t . q_t)
+                            const int j = nb * 4 + (fc >> 1);
+                            const float4 sc = *reinterpret_cast<const float4*>(ds + DELTA_BEAMS * DELTA_V_PITCH + j * 16);     // alpha_t, beta_t, k_t . q_t
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) {
-                            dl[e] = sc.y * fmaf(-sc.x, uk[e], vv[e]);
-                            o[e] = fmaf(dl[e], sc.z, sc.x * uq[e]);
+                            for (int e = 0; e < 2; ++e) {
+                                const uint32_t vb = *reinterpret_cast<const uint16_t*>(ds + j * DELTA_V_PITCH + (dv0 + 8 * e) * 2);
+                                const float dl = sc.y * fmaf(-sc.x, o[2 * e + 1], __uint_as_float(vb << 16));
+                                o[2 * e] = fmaf(dl, sc.z, sc.x * o[2 * e]);
+                                o[2 * e + 1] = dl;
+                            }
                         }
-                        store8<OutT>(out0 + (long long)j * a.H * DV + ch * 8, o);
-                        store8<__nv_bfloat16>(reinterpret_cast<__nv_bfloat16*>(rec0 + (long long)j * REC_BYTES + ch * 16), dl);
+                        if constexpr (sizeof(OutT) == 2) {
+                            packed[2 * half][nb] = pack_bf16x2(o[0], o[1]);
+                            packed[2 * half + 1][nb] = pack_bf16x2(o[2], o[3]);
+                        } else {                              // fp32 outputs: in place of the corr elements
+                            c[p0] = o[0];
+                            c[C_PITCH + p0] = o[1];
+                            c[p1] = o[2];
+                            c[C_PITCH + p1] = o[3];
+                        }
                     }
                 }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bar_free(s));
-            } else {
-                // coalesced stores by the other three warps: 16 lanes cover one beam's 128 outputs, 8 elements each
-                const int et = (warp - FOLD_WARPS - 1) * 32 + lane;
+                if constexpr (sizeof(OutT) == 2) {
+                    const uint32_t at = smem_u32(O_s) + (lane & 7) * OUT_PITCH + quad * 64 + (lane >> 3) * 16;
+#pragma unroll
+                    for (int nb = 0; nb < GN / 8; ++nb)
+                        asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(at + nb * 8 * OUT_PITCH),
+                                     "r"(packed[0][nb]), "r"(packed[1][nb]), "r"(packed[2][nb]), "r"(packed[3][nb])
+                                     : "memory");
+                }
+            }
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            // the four epilogue warps: tile complete - or somebody gave up, and then all four leave here together
+            if (bar_or(1, 128, fail ? 1 : 0)) { dead = true; break; }
+            TL(32, gcount);  // epilogue: outputs formed
+            {
+                // rows of 256 bytes (bf16) or 512 (fp32) to global memory as 16-byte vectors, a row by 16 or 32 lanes
                 OutT* out0 = static_cast<OutT*>(a.out) + (((long long)req * a.W + b0) * a.H + h) * DV;
-                float w8[GN * 16 / 96];                        // what undoes the scales of each row this thread stores
+                char* rec0 = nullptr;                         // DELTA: the odd rows are the records' delta halves
+                if constexpr (DELTA) rec0 = a.kv_out + ((long long)h * a.arena_slots + a.bases.base[req] + b0) * REC_BYTES + DK * 2;
+                constexpr int CH = sizeof(OutT) == 2 ? 16 : 32;
 #pragma unroll
-                for (int it = 0; it < GN * 16 / 96; ++it) w8[it] = inv_s[s * GN + ((it * 96 + et) >> 4)];
-#pragma unroll
-                for (int it = 0; it < GN * 16 / 96; ++it) {    // GN * 16 chunks of 16 bytes over 96 threads
-                    const int idx = it * 96 + et, j = idx >> 4, ch = idx & 15;
-                    if (b0 + j < a.W) {
-                        const int o0 = j * DV + corr_chunk(2 * ch) * 4, o1 = j * DV + corr_chunk(2 * ch + 1) * 4;
-                        const float4 x0 = *reinterpret_cast<const float4*>(C_s + o0), y0 = *reinterpret_cast<const float4*>(A_s + o0);
-                        const float4 x1 = *reinterpret_cast<const float4*>(C_s + o1), y1 = *reinterpret_cast<const float4*>(A_s + o1);
-                        const float w = w8[it];
-                        const float o[8] = {fmaf(y0.x, w, x0.x), fmaf(y0.y, w, x0.y), fmaf(y0.z, w, x0.z), fmaf(y0.w, w, x0.w),
-                                            fmaf(y1.x, w, x1.x), fmaf(y1.y, w, x1.y), fmaf(y1.z, w, x1.z), fmaf(y1.w, w, x1.w)};
-                        store8<OutT>(out0 + (long long)j * a.H * DV + ch * 8, o);
+                for (int it = 0; it < GN * CH / 128; ++it) {
+                    const int j = it * (128 / CH) + et / CH, ch = et % CH;
+                    if (b0 + (DELTA ? j >> 1 : j) >= a.W) continue;
+                    if constexpr (sizeof(OutT) == 2) {
+                        const uint4 x = *reinterpret_cast<const uint4*>(O_s + j * OUT_PITCH + ch * 16);
+                        char* dst = !DELTA     ? reinterpret_cast<char*>(out0 + (long long)j * a.H * DV)
+                                    : (j & 1) ? rec0 + (long long)(j >> 1) * REC_BYTES
+                                              : reinterpret_cast<char*>(out0 + (long long)(j >> 1) * a.H * DV);
+                        *reinterpret_cast<uint4*>(dst + ch * 16) = x;
+                    } else {
+                        const float4 x = *reinterpret_cast<const float4*>(C_s + j * C_PITCH + corr_chunk(ch) * 4);
+                        if (DELTA && (j & 1))
+                            *reinterpret_cast<uint2*>(rec0 + (long long)(j >> 1) * REC_BYTES + ch * 8) = make_uint2(pack_bf16x2(x.x, x.y), pack_bf16x2(x.z, x.w));
+                        else
+                            *reinterpret_cast<float4*>(out0 + (long long)(DELTA ? j >> 1 : j) * a.H * DV + ch * 4) = x;
                     }
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar_free(s));
             }
 
-            TL(33, gcount);  // epilogue: group stored / next group issued
+            TL(33, gcount);  // epilogue: group stored
             // Past the first group of segment seg >= 1 every MMA of segment seg - 1 has completed and the fold warps
             // have read its staging buffer out (they signal that): both are free for segment seg + 1.  (More groups
             // follow, so a warp that gives up here meets the others at the next iteration's barrier.)
@@ -957,7 +965,7 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
             }
             if (++gip == groups_per_pair) {
                 gip = 0;
-                ++pair;
+                ++seg;
                 if (++h == a.H) { h = 0; ++req; }
             }
         }
@@ -1020,7 +1028,8 @@ struct PartitionCost {
 PartitionCost partition_cost(int depth) {
     return {8 + (depth > 1 ? depth - 1 : 0), depth <= ONELA_SHALLOW_DEPTH ? ONELA_SEG_SHALLOW : ONELA_SEG_DEEP};
 }
-int greedy_fill(int total_groups, int gpp, int limit, int max_ctas, PartitionCost c, int32_t* begin) {
+template <class Begin>
+int greedy_fill(int total_groups, int gpp, int limit, int max_ctas, PartitionCost c, Begin* begin) {
     int n = 0, gi = 0;
     while (gi < total_groups) {
         if (n == max_ctas) return max_ctas + 1;
@@ -1043,14 +1052,15 @@ int greedy_fill(int total_groups, int gpp, int limit, int max_ctas, PartitionCos
     if (begin) begin[n] = total_groups;
     return n;
 }
-int make_partition(int total_groups, int gpp, int sms, PartitionCost c, Partition* part) {
+template <class Begin>
+int make_partition(int total_groups, int gpp, int sms, PartitionCost c, Begin* begin) {
     int lo = c.seg + c.group, hi = c.seg * (total_groups / gpp + 2) + c.group * total_groups;
     while (lo < hi) {
         const int mid = (lo + hi) / 2;
-        if (greedy_fill(total_groups, gpp, mid, sms, c, nullptr) <= sms) hi = mid;
+        if (greedy_fill<Begin>(total_groups, gpp, mid, sms, c, nullptr) <= sms) hi = mid;
         else lo = mid + 1;
     }
-    return greedy_fill(total_groups, gpp, lo, sms, c, part->begin);
+    return greedy_fill(total_groups, gpp, lo, sms, c, begin);
 }
 
 template <typename OutT, bool GROUPED, bool FUSED, bool DELTA = false>
@@ -1078,12 +1088,18 @@ cudaError_t launch_ws_t(const DecodeArgs& a, cudaStream_t stream) {
     const int groups_per_pair = (a.W + GN - 1) / GN;
     const int total_groups = a.req_count * a.H * groups_per_pair;
     static thread_local Partition part;          // the last launch's partition, reused while the shape stays
-    static thread_local int part_total = -1, part_gpp = -1, part_sms = -1, part_group = -1, part_seg = -1, part_ctas = 0;
+    static thread_local int part_total = -1, part_gpp = -1, part_h = -1, part_sms = -1, part_group = -1, part_seg = -1, part_ctas = 0;
     const PartitionCost cost = partition_cost(a.depth);
-    if (part_total != total_groups || part_gpp != groups_per_pair || part_sms != sms || part_group != cost.group ||
+    if (part_total != total_groups || part_h != a.H || part_gpp != groups_per_pair || part_sms != sms || part_group != cost.group ||
         part_seg != cost.seg) {
-        part_ctas = make_partition(total_groups, groups_per_pair, sms, cost, &part);
-        part_total = total_groups; part_gpp = groups_per_pair; part_sms = sms;
+        int32_t begin[MAX_CTAS + 1];
+        part_ctas = make_partition(total_groups, groups_per_pair, sms, cost, begin);
+        for (int i = 0; i < part_ctas; ++i) {
+            const int pair = begin[i] / groups_per_pair, segs = (begin[i + 1] - 1) / groups_per_pair - pair + 1;
+            part.cta[i] = make_int4(begin[i], begin[i] - pair * groups_per_pair, pair / a.H | segs << 8, pair % a.H);
+        }
+        part.cta[part_ctas].x = total_groups;
+        part_total = total_groups; part_h = a.H; part_gpp = groups_per_pair; part_sms = sms;
         part_group = cost.group; part_seg = cost.seg;
     }
     // Programmatic dependent launch: this launch's CTAs may start, allocate and read S_0 while the previous
@@ -1122,7 +1138,7 @@ extern "C" int onela_testhook_drop_full_arrival(int on) {
 #endif
 
 int make_decode_partition(int total_groups, int groups_per_pair, int sms, int group_cost, int seg_cost, DecodePartition* part) {
-    return make_partition(total_groups, groups_per_pair, sms > MAX_CTAS ? MAX_CTAS : sms, PartitionCost{group_cost, seg_cost}, part);
+    return make_partition(total_groups, groups_per_pair, sms > MAX_CTAS ? MAX_CTAS : sms, PartitionCost{group_cost, seg_cost}, part->begin);
 }
 int decode_sm_count() { return sm_count_ws(); }
 

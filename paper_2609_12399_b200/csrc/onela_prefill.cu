@@ -48,6 +48,9 @@ namespace {
 
 using sm100::bar_or;
 using sm100::idesc_f16;
+using sm100::mma_commit;
+using sm100::mma_ss;
+using sm100::mma_ts;
 using sm100::mbar_init;
 using sm100::pack_f16x2;
 using sm100::pow2_scale;
@@ -124,27 +127,6 @@ __device__ __forceinline__ void arrive(uint32_t bar) { asm volatile("mbarrier.ar
 __device__ __forceinline__ void cluster_sync() {
     asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
-// tcgen05.mma kind::f16 and its commit, reached by a whole converged warp and issued by one elected lane: the operands stay
-// in uniform registers (issued from inside a one-thread branch an MMA cost 113 cycles, mostly moving descriptors over).
-__device__ __forceinline__ void mma_ts(uint32_t d, uint32_t ta, uint64_t bdesc, uint32_t idesc, bool acc) {
-    asm volatile(
-        "{\n\t.reg .pred p, e;\n\telect.sync _|e, 0xffffffff;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d), "r"(ta), "l"(bdesc), "r"(idesc), "r"((uint32_t)acc)
-        : "memory");
-}
-__device__ __forceinline__ void mma_ss(uint32_t d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, bool acc) {
-    asm volatile(
-        "{\n\t.reg .pred p, e;\n\telect.sync _|e, 0xffffffff;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"((uint32_t)acc)
-        : "memory");
-}
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-    asm volatile(
-        "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
-        "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar)
-        : "memory");
-}
-
 // Two numbers times a power of two as fp16 numbers hi + lo, packed.  (Rounding hi to a fixed grid instead would make sums
 // of hi x hi products exact, but leaves every lo as large as the row's largest element allows: 4x the error.)
 __device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t& lo) {

@@ -59,7 +59,7 @@ def main() -> None:
     for r in range(wl.R):
         for l in range(wl.L):
             ctx.onela_init_shared_state(r, l, S0[r * wl.H:(r + 1) * wl.H].contiguous())
-    buf = (ctypes.c_ulonglong * 800)()
+    buf = (ctypes.c_ulonglong * 900)()
     cnt = (ctypes.c_int * 4)()
     flush = torch.empty(256 << 20, dtype=torch.uint8, device=dev)
     for t in range(wl.D):
