@@ -547,6 +547,7 @@ onela_status launch_decode(onela_ctx* ctx, int32_t req_begin, int32_t req_count,
     a.kv = a.kv_out;
     a.vv = a.vv_out;
     a.Hk = c.num_heads;
+    a.Hv = ctx->Hv();
     a.g = ctx->Hv() / c.num_heads * tiles;
     a.tiles = tiles;
     a.k_stride = (long long)(ctx->grouped() ? c.dk : c.dk + c.dv) * ctx->elem_bytes;

@@ -360,23 +360,42 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
         // Quad k of this warp belongs to group g_begin + k: rows UPW * warp .. + UPW - 1 of the group.
         const int n_quads = g_end - g_begin;
         uint8_t* my_heads = heads + warp * HEAD_BYTES;
-        struct Unit { int seg, req, h, gip; };           // segment, request, head, group within the (request, head) pair
+        // segment, request, head, group within the (request, head) pair; GROUPED: the head's key head and its place among that
+        // key head's heads, its value head and its place among that one's tiles - carried along, not divided out for every quad
+        // (the divisions were a sixth of the grouped launches' time: 128 x 256 on 16 value heads 24.2 -> 20.8 us)
+        struct Unit { int seg, req, h, gip, kh, ki, vh, vi; };
         auto beam_of = [&](const Unit& u) { return u.gip * BPG + (DELTA ? (UPW * warp + grp) >> 1 : UPW * warp + grp); };
         auto live_beam = [&](const Unit& u) { return min(beam_of(u), a.W - 1); };   // idle units shadow a live beam
         auto next_unit = [&](Unit u) {                   // the quad after u's, without divisions
             if (++u.gip == groups_per_pair) {
                 u.gip = 0;
                 ++u.seg;
-                if (++u.h == a.H) { u.h = 0; ++u.req; }
+                if (GROUPED && ++u.ki == a.g) { u.ki = 0; ++u.kh; }
+                if (GROUPED && ++u.vi == a.tiles) { u.vi = 0; ++u.vh; }
+                if (++u.h == a.H) { u.h = u.kh = u.vh = 0; ++u.req; }
             }
             return u;
         };
+        // rows of the caller's tensors and of the arena for a unit (see krow_in, vrow_in, k_at, v_at)
+        auto krow_of = [&](const Unit& n, int bb) { return ((long long)n.req * a.W + bb) * (GROUPED ? a.Hk : a.H) + (GROUPED ? n.kh : n.h); };
+        auto k_of = [&](const Unit& n, long long slot) { return GROUPED ? kv + (n.kh * a.arena_slots + slot) * a.k_stride : k_at(n.h, slot); };
+        auto v_of = [&](const Unit& n, long long slot) {
+            return GROUPED ? a.vv + (n.vh * a.arena_slots + slot) * a.v_stride + n.vi * (DV * 2) : v_at(n.h, slot);
+        };
+        auto value_head_of = [&](const Unit& n) { return GROUPED ? n.vh : n.h; };
         Unit u0;                                         // this warp's current quad; u1, u2: the next two
         {
             u0.seg = 0;
             u0.req = req_begin;
             u0.h = h_begin;
             u0.gip = gip_begin;
+            u0.kh = u0.ki = u0.vh = u0.vi = 0;
+            if (GROUPED) {
+                u0.kh = key_head(h_begin);
+                u0.ki = h_begin - u0.kh * a.g;
+                u0.vh = value_head(h_begin);
+                u0.vi = h_begin - u0.vh * a.tiles;
+            }
         }
         // The heads of a quad (own record and query of its units) arrive by 16-byte async copies into the warp's
         // stage, one quad ahead of their use (each lane copies exactly the chunks it reads back); the gates ride in
@@ -386,19 +405,19 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
             if (lane < UPW * 6) {
                 const int un = lane / 6, item = lane % 6;
                 const int b2 = min(n.gip * BPG + (DELTA ? (UPW * warp + un) >> 1 : UPW * warp + un), a.W - 1);
-                const long long krow2 = krow_in(n.req, b2, n.h), vrow2 = vrow_in(n.req, b2, n.h);
+                const long long krow2 = krow_of(n, b2), vrow2 = vrow_in(n.req, b2, n.h);
                 const long long slot2 = a.bases.base[n.req] + b2;
                 const char* p2 = item < 2 ? reinterpret_cast<const char*>(qbase) + krow2 * (DK * 2)
                                  : fused  ? (item < 4 ? static_cast<const char*>(a.k_in) + krow2 * (DK * 2)
                                                       : static_cast<const char*>(a.v_in) + vrow2 * (DV * 2))
-                                          : (item < 4 ? k_at(n.h, slot2) : v_at(n.h, slot2));
+                                          : (item < 4 ? k_of(n, slot2) : v_of(n, slot2));
                 asm volatile("prefetch.global.L2 [%0];" ::"l"(p2 + (item & 1) * 128));
             }
         };
         auto issue_head = [&](const Unit& u) {
             const uint32_t dst = smem_u32(my_heads);
             const int bb = live_beam(u);
-            const long long krow = krow_in(u.req, bb, u.h);
+            const long long krow = krow_of(u, bb);
             const char* qr = reinterpret_cast<const char*>(qbase + krow * DK) + g * 16;
             if (fused) {   // the call's records come straight from the caller's k and v tensors
                 const char* kr = static_cast<const char*>(a.k_in) + krow * (DK * 2) + g * 16;
@@ -410,8 +429,8 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
                 }
             } else {
                 const long long slot = a.bases.base[u.req] + bb;
-                const char* kr = k_at(u.h, slot) + g * 16;
-                const char* vr = v_at(u.h, slot) + g * 16;
+                const char* kr = k_of(u, slot) + g * 16;
+                const char* vr = v_of(u, slot) + g * 16;
 #pragma unroll
                 for (int c = 0; c < NCH; ++c) {
                     cp_async16(dst + grp * REC_BYTES + (c * LPU + g) * 16, kr + c * LPU * 16);
@@ -424,8 +443,8 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
         };
         auto load_gate = [&](const Unit& u) {
             const int bb = live_beam(u);
-            if (!fused) return __ldg(a.gates + (long long)value_head(u.h) * a.arena_slots + a.bases.base[u.req] + bb);
-            const long long in_row = GROUPED ? ((long long)u.req * a.W + bb) * (a.H / a.tiles) + value_head(u.h) : vrow_in(u.req, bb, u.h);
+            if (!fused) return __ldg(a.gates + (long long)value_head_of(u) * a.arena_slots + a.bases.base[u.req] + bb);
+            const long long in_row = GROUPED ? ((long long)u.req * a.W + bb) * a.Hv + value_head_of(u) : vrow_in(u.req, bb, u.h);
             return make_float2(__ldg(a.alpha_in + in_row), __ldg(a.beta_in + in_row));
         };
         // staging layout of the request whose quads are being looked at (the same for all heads of a request)
@@ -483,8 +502,8 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
                     staged_levels = staged_levels_of(u0.req);
                     // levels gathered from global memory whose lines are worth requesting ahead (end of the loop)
                     if (AHEAD) n_ahead = (info_sparse >> staged_levels) ? min(old - staged_levels, NIDX * LPU - staged_levels) : 0;
-                    seg_inv_s0 = 1.f / __ldg(a.s0_scale + u0.req * a.s0_scale_req_stride + value_head(u0.h));   // a power of two
-                    plane_row0 = (long long)value_head(u0.h) * a.arena_slots;      // row 0 of the head's gate plane
+                    seg_inv_s0 = 1.f / __ldg(a.s0_scale + u0.req * a.s0_scale_req_stride + value_head_of(u0));   // a power of two
+                    plane_row0 = (long long)value_head_of(u0) * a.arena_slots;      // row 0 of the head's gate plane
                     own_row0 = plane_row0 + a.bases.base[u0.req];
                     table_r = a.table + u0.req * a.table_req_stride;
                     sidx_r = a.sidx + u0.req * a.sidx_req_stride;
@@ -521,11 +540,11 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
                     } else if (fused && beam_of(u0) < a.W) {   // the append: this beam's record goes to its arena slot, bit for bit
                         if constexpr (GROUPED) {
                             const long long slot = a.bases.base[u0.req] + bb;
-                            uint4* vdst = reinterpret_cast<uint4*>(a.vv_out + (v_at(u0.h, slot) - a.vv)) + g;
+                            uint4* vdst = reinterpret_cast<uint4*>(a.vv_out + (v_of(u0, slot) - a.vv)) + g;
 #pragma unroll
                             for (int c = 0; c < NCH; ++c) vdst[c * LPU] = cur.own.v[c];
-                            if (u0.h % a.g == 0) {     // the key is stored once per key head: by its first value head
-                                uint4* kdst = reinterpret_cast<uint4*>(a.kv_out + (k_at(u0.h, slot) - kv)) + g;
+                            if (u0.ki == 0) {     // the key is stored once per key head: by its first value head
+                                uint4* kdst = reinterpret_cast<uint4*>(a.kv_out + (k_of(u0, slot) - kv)) + g;
 #pragma unroll
                                 for (int c = 0; c < NCH; ++c) kdst[c * LPU] = cur.own.k[c];
                             }
@@ -537,7 +556,7 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
                                 dst[16 + c * LPU] = cur.own.v[c];
                             }
                         }
-                        if (g == 0 && (!GROUPED || u0.h % a.tiles == 0)) a.gates_out[own_row0 + bb] = gate0;
+                        if (g == 0 && (!GROUPED || u0.vi == 0)) a.gates_out[own_row0 + bb] = gate0;
                     }
                 }
                 gate0 = gate1;
@@ -620,8 +639,8 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
                                   const long long slot = idx_of(level);
                                   if constexpr (GROUPED) {
                                       RecT rec;
-                                      const uint4* kp = reinterpret_cast<const uint4*>(k_at(u0.h, slot)) + g;
-                                      const uint4* vp = reinterpret_cast<const uint4*>(v_at(u0.h, slot)) + g;
+                                      const uint4* kp = reinterpret_cast<const uint4*>(k_of(u0, slot)) + g;
+                                      const uint4* vp = reinterpret_cast<const uint4*>(v_of(u0, slot)) + g;
 #pragma unroll
                                       for (int c = 0; c < NCH; ++c) {
                                           rec.k[c] = __ldg(kp + c * LPU);
@@ -751,7 +770,7 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
                             if (j == src / LPU) slot = x;
                         }
                         if (level >= staged_levels && level < NIDX * LPU && ((info_sparse >> level) & 1)) {
-                            const char* line = (g & 2) ? v_at(u1.h, slot) + (g & 1) * 128 : k_at(u1.h, slot) + (g & 1) * 128;
+                            const char* line = (g & 2) ? v_of(u1, slot) + (g & 1) * 128 : k_of(u1, slot) + (g & 1) * 128;
                             asm volatile("prefetch.global.L2 [%0];" ::"l"(line));
                         }
                     }

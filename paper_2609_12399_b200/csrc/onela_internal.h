@@ -75,7 +75,7 @@ struct DecodeArgs {
     // layer's key plane [Hk][arena_slots][dk], vv / vv_out its value plane [H][arena_slots][dv]; q and k_in have Hk heads
     const char* vv;
     char* vv_out;
-    int32_t Hk, g;
+    int32_t Hk, g, Hv;      // key heads, value tiles per key head, value heads (before they are cut into tiles)
     // ... and value widths of 256 / 512 (grouped or not): every value head is cut into `tiles` heads of 128 outputs, so
     // H = tiles * (value heads) and g = tiles * (value heads per key head); k_stride / v_stride: bytes between
     // consecutive slots of a key head's keys and of a value head's values (from kv and vv: one interleaved plane or two)
