@@ -95,6 +95,9 @@ constexpr uint32_t S0_COL = 128;                 // accumulators of the ring slo
 constexpr int R_TARGET = 8;                      // a scaled operand row's largest element lies in [2^8, 2^9) x (decay in [1, 2)): far inside fp16's range
 constexpr uint32_t TMEM_COLS = 512;
 static_assert(SLOTS * GN <= 128 && GN == 48, "accumulator columns");
+// Where chains share too little to be staged (see gather_queued) the staging area holds two gathered records per unit instead.
+constexpr int QUEUE_SLOT = UPW * REC_BYTES + 64;     // a quad's records of one level, then their gates
+static_assert(FOLD_WARPS * 2 * QUEUE_SLOT <= STAGE_BYTES && LPU >= 8, "gather queues");
 static_assert(2 * STAGE_BUF <= 128, "one staged record per epilogue lane");
 static_assert(SMEM_BYTES <= 232448, "shared memory per CTA");
 static_assert(GN % 16 == 0 && GN >= 16 && GN <= 256, "MMA N");
@@ -355,6 +358,23 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
         }
     };
 
+    // Chains that share little - fewer than half of the first request's older levels can be staged, and the beams' parents are
+    // more than a quarter as many as there are beams - are gathered through a queue: nothing is staged, and every fold warp
+    // keeps two levels' records on their way by async copies, across quads.  (A decision per CTA, which both roles make alike;
+    // the requests of a batch follow one parent law as a rule.)  A gather into registers waits out L2's latency at every
+    // level: 8 x 1024 beams with uniform parents 24 us per level that way, 15 us through the queue (depth 6: 202 -> 165 us).
+    // Where the line lies, measured on 4 x 300 beams, uniform parents, depth 4 - 7: staging what can be staged 22.6 us, the
+    // queue as soon as one level cannot be staged 21.8 us, but on 2 x 200 beams, Zipf(1.2), 21 us against 18 us with the rule.
+    auto gather_queued = [&](int& levels, int& count) {
+        levels = count = 0;
+        if (n_segs == 0 || old == 0) return false;
+        uint32_t sparse;
+        staging_of(req_begin, levels, count, &sparse);
+        if (2 * levels >= old || !((sparse >> (min(old, 32) - 1)) & 1)) return false;
+        levels = count = 0;
+        return true;
+    };
+
     if (warp < FOLD_WARPS) {
         // =============================== FOLD ===============================
         // Quad k of this warp belongs to group g_begin + k: rows UPW * warp .. + UPW - 1 of the group.
@@ -449,9 +469,9 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
         };
         // staging layout of the request whose quads are being looked at (the same for all heads of a request)
         int info_req = -1, info_levels = 0, info_count = 0;
-        uint32_t info_sparse = 0;
+        bool queued = false;
         auto staged_levels_of = [&](int req) {
-            if (req != info_req) { staging_of(req, info_levels, info_count, &info_sparse); info_req = req; }
+            if (req != info_req && !queued) { staging_of(req, info_levels, info_count); info_req = req; }
             return info_levels;
         };
         constexpr int NIDX = LPU >= 8 ? 1 : 8 / LPU;     // the unit's lanes hold the indices of its first 8 levels
@@ -480,28 +500,57 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
             issue_head(u0);
             gate0 = load_gate(u0);
             if (1 < n_quads) gate1 = load_gate(u1);
+            queued = gather_queued(info_levels, info_count);
+            info_req = req_begin;
             idx_next = load_idx(u0);
         }
         TL(2, 0);   // dependencies waited for, first heads requested
         put_first_s0();
         TL(3, 0);   // first S_0 in tensor memory
-        int cur_seg = -1, buf = 0, staged_levels = 0, n_ahead = 0;
+        int cur_seg = -1, buf = 0, staged_levels = 0;
         float seg_inv_s0 = 1.f;
         bool staged_ready = false;
         long long plane_row0 = 0, own_row0 = 0;
         const int32_t *table_r = nullptr, *sidx_r = nullptr;
-        // The loop exists twice, with and without the requests ahead of the gathered records (at its end): where
-        // they are not wanted the loop is exactly the one without them (their mere presence measured 0.7 % slower).
-        auto fold_quads = [&](auto ahead_tag) {
-            constexpr bool AHEAD = decltype(ahead_tag)::value;
+        // The loop exists twice, with the gather queue and without.
+        auto fold_quads = [&](auto queue_tag) {
+            constexpr bool QUEUE = decltype(queue_tag)::value;
+            const bool two = old >= 2;               // gathers in flight: two, or the one older level there is
+            uint8_t* my_queue = stage + warp * (2 * QUEUE_SLOT);
+            const uint32_t queue_at = smem_u32(my_queue);
+            int q_in = 0, q_out = 0;                 // place in the queue of the next request / the next record
+            auto queue_record = [&](const Unit& n, const Idx& ix, int item) {      // the item-th older record, newest first, of quad n's units
+                const int level = old - 1 - item;
+                const int32_t near = __shfl_sync(0xffffffffu, ix.v[0], level & (LPU - 1), LPU);
+                const int32_t slot = level < LPU ? near : __ldg(a.table + n.req * a.table_req_stride + (long long)level * a.max_beam + live_beam(n));
+                const char *kp = k_of(n, slot) + g * 16, *vp = v_of(n, slot) + g * 16;
+                const uint32_t dst = queue_at + q_in * QUEUE_SLOT + grp * REC_BYTES + g * 16;
+#pragma unroll
+                for (int c = 0; c < NCH; ++c) {
+                    cp_async16(dst + c * LPU * 16, kp + c * LPU * 16);
+                    cp_async16(dst + DK * 2 + c * LPU * 16, vp + c * LPU * 16);
+                }
+                if (g == 0) cp_async8(queue_at + q_in * QUEUE_SLOT + UPW * REC_BYTES + grp * 8, a.gates + (long long)value_head_of(n) * a.arena_slots + slot);
+                q_in ^= two ? 1 : 0;
+            };
+            auto commit = [&]() { asm volatile("cp.async.commit_group;" ::: "memory"); };
+            // all but the `two ? x + 1 : x` youngest groups of copies have landed
+            auto wait_but = [&](auto x) {
+                if (two) asm volatile("cp.async.wait_group %0;" ::"n"(decltype(x)::value + 1) : "memory");
+                else asm volatile("cp.async.wait_group %0;" ::"n"(decltype(x)::value) : "memory");
+            };
+            if (QUEUE) {
+                for (int item = 0; item < (two ? 2 : 1); ++item) {
+                    if (n_quads > 0) queue_record(u0, idx_next, item);
+                    commit();
+                }
+            }
             for (int k = 0; k < n_quads && !dead; ++k, u0 = u1, u1 = u2, u2 = next_unit(u2)) {
                 if (u0.seg != cur_seg) {          // entering a segment: nothing to wait for here
                     cur_seg = u0.seg;
                     buf = single ? 0 : (cur_seg & 1);
                     staged_ready = false;
                     staged_levels = staged_levels_of(u0.req);
-                    // levels gathered from global memory whose lines are worth requesting ahead (end of the loop)
-                    if (AHEAD) n_ahead = (info_sparse >> staged_levels) ? min(old - staged_levels, NIDX * LPU - staged_levels) : 0;
                     seg_inv_s0 = 1.f / __ldg(a.s0_scale + u0.req * a.s0_scale_req_stride + value_head_of(u0));   // a power of two
                     plane_row0 = (long long)value_head_of(u0) * a.arena_slots;      // row 0 of the head's gate plane
                     own_row0 = plane_row0 + a.bases.base[u0.req];
@@ -515,7 +564,8 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
                 Head cur;
                 {
                     TL(10, k);  // fold: quad start
-                    asm volatile("cp.async.wait_group 0;" ::: "memory");
+                    if (QUEUE) wait_but(std::integral_constant<int, 1>{});      // (younger: the first gathers of this quad)
+                    else asm volatile("cp.async.wait_group 0;" ::: "memory");
                     TL(11, k);  // fold: heads landed
                     const uint4* rec = reinterpret_cast<const uint4*>(my_heads + grp * REC_BYTES) + g;
                     const uint4* qv = reinterpret_cast<const uint4*>(my_heads + UPW * REC_BYTES + grp * (DK * 2)) + g;
@@ -529,6 +579,7 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
                     // the next quad's copies go out before this quad's stores (each lane overwrites only the chunks it
                     // has just read)
                     if (k + 1 < n_quads) issue_head(u1);
+                    else if (QUEUE) commit();
                     if (DELTA) {
                         // the key half of the record and the gates; delta_t follows from the epilogue
                         if ((grp & 1) == 0 && beam_of(u0) < a.W) {
@@ -652,7 +703,32 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
                                       return L::load_global(kv, a.gates, plane_row0 + slot, g);
                                   }
                               };
-                if (DELTA) {     // the replay runs over the older records only; the beam's own is formed in the epilogue
+                if constexpr (QUEUE) {
+                    if (!DELTA) L::template fold_step<false>(cur.own, r, corr, decay);
+                    for (int item = 0; item < old; ++item) {
+                        // younger than the wanted record: the other gather in flight, and the next quad's heads while the
+                        // records requested before them last
+                        if (item < (two ? 2 : 1)) wait_but(std::integral_constant<int, 1>{});
+                        else wait_but(std::integral_constant<int, 0>{});
+                        __syncwarp();                        // (the gates were copied by the unit's first lane)
+                        const uint8_t* slot_s = my_queue + q_out * QUEUE_SLOT;
+                        const uint4* p = reinterpret_cast<const uint4*>(slot_s + grp * REC_BYTES) + g;
+                        RecT rec;
+#pragma unroll
+                        for (int c = 0; c < NCH; ++c) {
+                            rec.k[c] = p[c * LPU];
+                            rec.v[c] = p[16 + c * LPU];
+                        }
+                        rec.gate = *reinterpret_cast<const float2*>(slot_s + UPW * REC_BYTES + grp * 8);
+                        q_out ^= two ? 1 : 0;
+                        __syncwarp();                        // the place is read out: the record after the next (the next) takes it
+                        const int next = item + (two ? 2 : 1);
+                        if (next < old) queue_record(u0, my_idx, next);
+                        else if (k + 1 < n_quads) queue_record(u1, idx_next, next - old);
+                        commit();
+                        L::template fold_step<DELTA>(rec, r, corr, decay);
+                    }
+                } else if (DELTA) {     // the replay runs over the older records only; the beam's own is formed in the epilogue
                     if (old - 1 >= staged_levels) {
                         const RecT first = gather(old - 1);
                         L::template fold_chain_simple<true>(first, old - 2, staged_levels, gather, r, corr, decay);
@@ -750,41 +826,9 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
 #endif
                 if (lane == 0) mbar_arrive(bar_full(s));
                 TL(14, k);  // fold: rows written
-
-                // The next quad's records of the levels that are NOT staged are gathered from global memory in the middle
-                // of its dependent chain.  Where a level has little sharing (most of its records are used by one or two
-                // beams: uniform parents) their lines are requested now, a whole quad ahead - the slot ids have arrived
-                // by now; where many beams share few records the gathers hit L1/L2 anyway and the requests only cost
-                // (measured: +6 % on 8 x 1024 beams with uniform parents, -3 % on the Zipf(1.5) stack if done always).
-                // One request per lane: lane g of a unit asks for line g & 3 of the record of level
-                // old - 1 - 2 p - (g >> 2), newest levels first.  (The segment's own staging layout is used for the
-                // next quad: it differs only across a change of request, and a request is a hint.)
-                if (AHEAD && n_ahead > 0 && k + 1 < n_quads) {
-                    for (int p = 0; 2 * p < n_ahead; ++p) {
-                        const int level = old - 1 - 2 * p - (g >> 2);
-                        const int src = max(level, 0);
-                        int32_t slot = 0;
-#pragma unroll
-                        for (int j = 0; j < NIDX; ++j) {
-                            const int32_t x = __shfl_sync(0xffffffffu, idx_next.v[j], src & (LPU - 1), LPU);
-                            if (j == src / LPU) slot = x;
-                        }
-                        if (level >= staged_levels && level < NIDX * LPU && ((info_sparse >> level) & 1)) {
-                            const char* line = (g & 2) ? v_of(u1, slot) + (g & 1) * 128 : k_of(u1, slot) + (g & 1) * 128;
-                            asm volatile("prefetch.global.L2 [%0];" ::"l"(line));
-                        }
-                    }
-                }
             }
         };
-        // little sharing somewhere in the first request's gathered levels: take the loop that requests lines ahead
-        // (the requests of a batch follow one parent law as a rule; it is a hint either way)
-        bool ahead = false;
-        if (n_quads > 0) {
-            const int sl0 = staged_levels_of(u0.req);
-            ahead = old > sl0 && (info_sparse >> sl0) != 0;
-        }
-        if (ahead) fold_quads(std::true_type{});
+        if (queued) fold_quads(std::true_type{});
         else fold_quads(std::false_type{});
     } else if (warp == MMA_WARP) {
         // =============================== MMA ISSUE ===============================
@@ -819,6 +863,8 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
         // =============================== EPILOGUE (+ preparation of the next segments) ===============================
         dependency_wait();
         const int quad = warp & 3;                    // tensor-memory lane quadrant of this warp
+        int first_levels, first_count;
+        const bool queued = gather_queued(first_levels, first_count);          // nothing is staged then
         int staged_issued[2] = {0, 0};                // stagings requested per buffer (what teardown must wait for)
         // Stage the distinct records of segment `seg`: one 512-byte bulk copy per record, its gates by a plain load, one
         // record per lane.  Every lane arrives once, announcing the bytes it requested; its gate store is ordered
@@ -827,8 +873,8 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
             int req, h;
             pair_of(seg, req, h);
             const int b = single ? 0 : (seg & 1);
-            int levels, count;
-            staging_of(req, levels, count);
+            int levels = first_levels, count = first_count;      // (of the first request; zero with a gather queue)
+            if (!queued && req != req_begin) staging_of(req, levels, count);
             const long long plane_row0 = (long long)value_head(h) * a.arena_slots;
             const int li = (warp - FOLD_WARPS) * 32 + lane;
             if (li < count) {
