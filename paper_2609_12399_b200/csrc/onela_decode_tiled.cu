@@ -9,11 +9,16 @@
 //      the caller's tensors and the unit also writes it to its arena slot.
 //   2. The folded queries go to shared memory as rows of the MMA's B operand: fp16, K-major, 128-byte swizzle, each row
 //      times the power of two that brings its largest element into [2^8, 2^9) (exact; undone after the product).
-//   3. Per tile of 128 value rows: the S_0 rows become the A operand the same way (fp16, times the head's power of two
-//      kept with the state), dk / 16 MMAs (M = 128, N = beams, K = 16) accumulate S_0 . r~ in tensor memory, and while
-//      they run the next tile's A operand is built and the previous tile's accumulator is read back (lane = value
-//      row), scaled and added to corr in a shared-memory tile whose rows the units then store as 16-byte vectors.  Two
-//      A operands and two accumulators alternate.
+//   3. Per tile of 128 value rows the A operand (the state's stored fp16 copy, by bulk copies) meets the rows: dk / 16 MMAs
+//      (M = 128, N = beams, K = 16) accumulate S_0 . r~ in tensor memory; the accumulators go through a shared-memory tile
+//      (lane = value row in, a beam's row out) to the units' lanes, which undo the scales, add corr from their registers
+//      and store 16-byte vectors.  Where there is room two A operands and two accumulators alternate.
+// What bounds it: the phases of a CTA in sequence (inputs from HBM, dependent gathers, MMAs, accumulators through shared
+// memory), overlapped only by the other CTAs of the SM - one at the widest shapes.  us per launch on the beam-512 stack
+// before / after corr was left in registers, the MMAs issued by an elected lane of a converged warp and the loads moved ahead
+// of the first barrier: 64 x 64 bf16 29.8 / 24.0 (depth 1 - 8), 256 x 256 bf16 79.9 / 70.9, 256 x 512 bf16 (600 beams x 16
+// heads) 36.6 / 32.0, 128 x 256 fp32 23.5 / 21.5.  Requests of the next wave's inputs into L2 made it 3 % slower; a persistent
+// loop over the tiles of beams spills (the invariants of every pointer stay live): 64 x 64 40 us.
 // The only wait is for the MMAs' completion; it is bounded, and all threads agree on its outcome before going on
 // (ONELA_E_TIMEOUT in the status word otherwise).
 #include <mutex>
@@ -31,16 +36,18 @@ using sm100::idesc_f16;
 using sm100::mbar_expect_tx;
 using sm100::mbar_init;
 using sm100::mbar_wait;
+using sm100::mma_commit;
+using sm100::mma_ss;
 using sm100::pack_f16x2;
 using sm100::pow2_scale;
 using sm100::smem_u32;
 using sm100::tmem_ld16;
-using sm100::umma_commit;
 using sm100::umma_desc;
-using sm100::umma_f16_ss;
 
 constexpr int G = 8;                   // lanes per unit
-constexpr int CP = 128 + 4;            // pitch (floats) of the output tile: conflict-free for both access patterns
+// pitch (floats) of the output tile: conflict-free for both access patterns
+template <int VD>
+__host__ __device__ constexpr int tile_pitch() { return (VD < 128 ? VD : 128) + 4; }
 constexpr int ROW_TARGET = 8;          // a scaled operand row's largest element lies in [2^8, 2^9)
 
 // Beams per CTA (= MMA N; 8 threads each).  Key width 256 takes 64: every CTA turns the whole head's S_0 into its A
@@ -59,13 +66,15 @@ __host__ __device__ constexpr size_t tiled_smem_bytes() {
     // two A operands where there is a next tile to prepare and the key is narrow (at key width 256 the second buffer
     // leaves the fold's record loads 34 KB of L1: 89 -> 106 us at 256 x 256)
     constexpr int NB = tiled_beams<KD, VD>(), ABUF = (VD > 128 && KD <= 128) ? 2 : 1;
-    return 1024 + (size_t)ABUF * (KD / 64) * 128 * 128 + (size_t)(KD / 64) * NB * 128 + (size_t)NB * CP * 4 + NB * 4 + 64;
+    return 1024 + (size_t)ABUF * (KD / 64) * 128 * 128 + (size_t)(KD / 64) * NB * 128 + (size_t)NB * tile_pitch<VD>() * 4 + 64;
 }
 
 // CTAs per SM the registers are capped for: small CTAs are latency-bound (a string of dependent loads per level, one MMA
-// round trip), so the narrowest shape gets four.
-template <int KD, int VD>
-__host__ __device__ constexpr int tiled_min_ctas() { return KD + VD <= 128 ? 4 : tiled_beams<KD, VD>() == 64 ? 1 : 2; }
+// round trip), so the narrowest shape gets four, with bf16 records - half the registers - five (64 x 64 on the beam-512
+// stack: 30 -> 27 us; six: 28.5; fp32 records, five: 16 -> 17 us).  (64 beams of 256 threads at two per SM, or 16 lanes per
+// unit, were 5 - 10 % slower at 256 x 256.)
+template <int KD, int VD, typename T>
+__host__ __device__ constexpr int tiled_min_ctas() { return KD + VD <= 128 ? (sizeof(T) == 2 ? 5 : 4) : tiled_beams<KD, VD>() == 64 ? 1 : 2; }
 
 // DELTA: the arena keeps (alpha_t, delta_t, k_t) (Section 3.2, Eq. 2-4).  A beam owns TWO rows of the tile - its query
 // and its own key, both projected through the parent state: S_{t-1} x = D S_0 x + sum_j d_j (k_j . x) delta_j, the
@@ -73,8 +82,8 @@ __host__ __device__ constexpr int tiled_min_ctas() { return KD + VD <= 128 ? 4 :
 // o_t = alpha_t S_{t-1} q_t + delta_t (k_t . q_t) are formed from the two rows and the record is written; always with
 // the append fused in, dk = dv <= 128.
 template <int KD, int VD, typename T, typename OutT, bool DELTA = false>
-__global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, VD>()) decode_tiled_kernel(const TiledArgs a) {
-    constexpr int NB = tiled_beams<KD, VD>(), THREADS = NB * G;
+__global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, VD, T>()) decode_tiled_kernel(const TiledArgs a) {
+    constexpr int NB = tiled_beams<KD, VD>(), CP = tile_pitch<VD>();
     constexpr int BPT = DELTA ? NB / 2 : NB;          // beams per tile
     static_assert(!DELTA || (KD == VD && VD <= 128), "delta records: square heads, one tile of value rows");
     constexpr uint32_t ACC_COLS = 2 * NB;      // two accumulators of NB columns (a power of two >= 32)
@@ -93,12 +102,11 @@ __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, 
     uint8_t* A_s = smem;                                               // [ABUF][KB][128 rows][128 bytes]: tile mt in buffer mt & 1
     uint8_t* R_s = A_s + ABUF * KB * A_KB;                             // [KB][NB rows][128 bytes]
     float* C_s = reinterpret_cast<float*>(R_s + KB * R_KB);            // [NB][CP]
-    float* inv_s = C_s + NB * CP;                                      // [NB] what undoes a row's scales
-    uint64_t* bar = reinterpret_cast<uint64_t*>(inv_s + NB);          // a tile's MMAs complete
+    uint64_t* bar = reinterpret_cast<uint64_t*>(C_s + NB * CP);        // a tile's MMAs complete
     uint64_t* abar = bar + 1;                                          // [2] an A operand has landed
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(abar + 2);
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // (warp: uniform for the compiler too)
     if (tid == 0) {
         mbar_init(smem_u32(bar), 1);
         mbar_init(smem_u32(abar), 1);
@@ -110,10 +118,9 @@ __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, 
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    // (barriers and tensor memory are first used by others than the threads above after the barrier that ends the fold: no
+    // barrier stands between a CTA's start and its first loads)
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem_base = *tmem_slot;
     // (programmatic dependent launch: the next launch may set itself up under this one)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
@@ -140,13 +147,14 @@ __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, 
             bulk_load(smem_u32(A_s + (mt & (ABUF - 1)) * (KB * A_KB) + kb * A_KB), A_src + ((long long)mt * KB + kb) * A_KB, A_KB, ab);
         ++a_loads;
     };
-    // one thread: once the tile's A operand has landed, its dk / 16 MMAs into accumulator mt & 1 and the commit that
+    // the first warp: once the tile's A operand has landed, its dk / 16 MMAs into accumulator mt & 1 and the commit that
     // completes the barrier's phase (if the operand does not land in time nothing is issued, and the CTA's wait for the
-    // MMAs runs out in turn)
+    // MMAs runs out in turn); issued by one elected lane of the converged warp (see mma_ss)
+    uint32_t tmem_base = 0;
     auto issue = [&](int mt) {
         const bool landed = mbar_wait(smem_u32(abar + (mt & (ABUF - 1))), (ABUF == 2 ? mt >> 1 : mt) & 1);
         ++a_waits;
-        if (!landed) return;
+        if (!__all_sync(0xffffffffu, landed)) return;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint64_t ad = umma_desc(smem_u32(A_s + (mt & (ABUF - 1)) * (KB * A_KB))), bd = umma_desc(smem_u32(R_s));
         constexpr uint32_t idesc = idesc_f16(NB);
@@ -154,9 +162,9 @@ __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, 
         for (int kb = 0; kb < KB; ++kb)
 #pragma unroll
             for (int ks = 0; ks < 4; ++ks)
-                umma_f16_ss(tmem_base + (mt & 1) * NB, ad + (uint64_t)((kb * A_KB + ks * 32) >> 4),
-                            bd + (uint64_t)((kb * R_KB + ks * 32) >> 4), idesc, (kb | ks) ? 1u : 0u);
-        umma_commit(smem_u32(bar));
+                mma_ss(tmem_base + (mt & 1) * NB, ad + (uint64_t)((kb * A_KB + ks * 32) >> 4), bd + (uint64_t)((kb * R_KB + ks * 32) >> 4), idesc,
+                       (kb | ks) != 0);
+        mma_commit(smem_u32(bar));
     };
     // The stored states are written by the state calls only, and the index launch that lies between those and any decode
     // waits for them before it lets this one start: the first operand may be requested before the wait.
@@ -198,14 +206,40 @@ __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, 
         x.gate = __ldg(gates + slot);
         return x;
     };
+    // (narrow heads: packed fp32x2 multiply-adds; wide ones do not have the registers for aligned pairs: 256 x 512 37 -> 50 us)
+    constexpr bool PACKED = KD + VD <= 128;
+    auto pair_fma = [&](float w, const float* x, float* acc) {
+        if constexpr (PACKED) {
+            const float2 y = __ffma2_rn(make_float2(w, w), make_float2(x[0], x[1]), make_float2(acc[0], acc[1]));
+            acc[0] = y.x;
+            acc[1] = y.y;
+        } else {
+            acc[0] = fmaf(w, x[0], acc[0]);
+            acc[1] = fmaf(w, x[1], acc[1]);
+        }
+    };
     auto fold = [&](const Raw& x) {       // c = k . r~ ;  corr += decay beta c v ;  r~ -= beta c k ;  decay *= alpha
         float kx[CK * VEC];
         float dot = 0.f;
+        if constexpr (PACKED) {
+            float2 d0 = make_float2(0.f, 0.f), d1 = d0;
 #pragma unroll
-        for (int c = 0; c < CK; ++c) {
-            Vec16<T>::unpack(x.k[c], kx + c * VEC);
+            for (int c = 0; c < CK; ++c) {
+                Vec16<T>::unpack(x.k[c], kx + c * VEC);
 #pragma unroll
-            for (int e = 0; e < VEC; ++e) dot = fmaf(kx[c * VEC + e], r[c * VEC + e], dot);
+                for (int e = c * VEC; e < (c + 1) * VEC; e += 4) {
+                    d0 = __ffma2_rn(make_float2(kx[e], kx[e + 1]), make_float2(r[e], r[e + 1]), d0);
+                    d1 = __ffma2_rn(make_float2(kx[e + 2], kx[e + 3]), make_float2(r[e + 2], r[e + 3]), d1);
+                }
+            }
+            dot = (d0.x + d0.y) + (d1.x + d1.y);
+        } else {
+#pragma unroll
+            for (int c = 0; c < CK; ++c) {
+                Vec16<T>::unpack(x.k[c], kx + c * VEC);
+#pragma unroll
+                for (int e = 0; e < VEC; ++e) dot = fmaf(kx[c * VEC + e], r[c * VEC + e], dot);
+            }
         }
 #pragma unroll
         for (int off = G / 2; off > 0; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
@@ -218,11 +252,11 @@ __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, 
             float vx[VEC];
             Vec16<T>::unpack(x.v[c], vx);
 #pragma unroll
-            for (int e = 0; e < VEC; ++e) corr[c * VEC + e] = fmaf(wv, vx[e], corr[c * VEC + e]);
+            for (int e = 0; e < VEC; e += 2) pair_fma(wv, vx + e, corr + c * VEC + e);
         }
         if constexpr (!DELTA) {
 #pragma unroll
-            for (int e = 0; e < CK * VEC; ++e) r[e] = fmaf(-bc, kx[e], r[e]);
+            for (int e = 0; e < CK * VEC; e += 2) pair_fma(-bc, kx + e, r + e);
         }
         decay *= x.gate.x;
     };
@@ -319,6 +353,7 @@ __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, 
     }
 
     // ---- the folded query decay * r~ as the unit's operand row ----
+    float inv_row;               // what undoes the row's scales
     {
         float m = 0.f;
 #pragma unroll
@@ -328,7 +363,7 @@ __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, 
         float sc, inv;
         pow2_scale(m * fabsf(decay), ROW_TARGET, sc, inv);
         const float f = decay * sc;
-        if (g == 0) inv_s[grp] = inv / sc0;      // both powers of two
+        inv_row = inv / sc0;                     // both powers of two
 #pragma unroll
         for (int c = 0; c < CK; ++c) {
             const int el0 = (c * G + g) * VEC;   // first element of the chunk
@@ -345,10 +380,12 @@ __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, 
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy writes -> visible to the MMA
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 #ifdef ONELA_TEST_HOOKS
-    if (tid == 0 && !(g_hook_tiled_skip_issue && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0)) issue(0);
+    if (warp == 0 && !(g_hook_tiled_skip_issue && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0)) issue(0);
 #else
-    if (tid == 0) issue(0);
+    if (warp == 0) issue(0);
 #endif
 
     OutT* out = static_cast<OutT*>(a.out) + (((long long)req * a.W + b) * Hv + hv) * VD;
@@ -356,15 +393,6 @@ __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, 
     bool failed = false;
 #pragma unroll
     for (int mt = 0; mt < MT; ++mt) {
-        // this tile's part of corr, one row per unit
-#pragma unroll
-        for (int c = 0; c < CV; ++c) {
-            if ((c * G * VEC) / 128 != mt) continue;
-            float* dst = C_s + grp * CP + (c * G + g) * VEC - mt * 128;
-#pragma unroll
-            for (int e = 0; e < VEC; e += 4)
-                *reinterpret_cast<float4*>(dst + e) = make_float4(corr[c * VEC + e], corr[c * VEC + e + 1], corr[c * VEC + e + 2], corr[c * VEC + e + 3]);
-        }
         if (ABUF == 2 && mt + 1 < MT && tid == 0) {
             // the next tile's A operand, under this tile's MMAs: its buffer was last read by tile mt - 1, whose
             // completion this thread has waited for
@@ -377,7 +405,7 @@ __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, 
         if (ABUF == 2) {
             // ... and its MMAs, under this tile's epilogue: their accumulator was read out before the barrier that
             // ended the previous iteration
-            if (mt + 1 < MT && tid == 0) issue(mt + 1);
+            if (mt + 1 < MT && warp == 0) issue(mt + 1);
         } else if (mt + 1 < MT && tid == 0) {        // one A operand: free now; its MMAs go out after the barrier below
             load_A(mt + 1);
         }
@@ -388,29 +416,56 @@ __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, 
             const int i = quad * 32 + lane;          // value row within the tile
             if (mt * 128 + i < VD) {
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    float* cell = C_s + (half * 16 + j) * CP + i;
-                    *cell = fmaf(__uint_as_float(v[j]), inv_s[half * 16 + j], *cell);
-                }
+                for (int j = 0; j < 16; ++j) C_s[(half * 16 + j) * CP + i] = __uint_as_float(v[j]);
             }
         }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
-        if (ABUF == 1 && mt + 1 < MT && tid == 0) issue(mt + 1);
+        if (ABUF == 1 && mt + 1 < MT && warp == 0) issue(mt + 1);
+        // A unit's lanes read their elements of its row back, undo the scales and add corr, which never left their registers.
+        // (Corr added in the tile - written there before, read and written again under the accumulator - cost twice the
+        // shared-memory accesses.)
+        auto output = [&](int c, float* x) {
+            // (a chunk of eight elements by two 16-byte reads: lanes 4 - 7 take theirs in the other order, off the banks of lanes 0 - 3)
+            const float* src = C_s + grp * CP + (c * G + g) * VEC - mt * 128;
+            const int first = VEC == 8 ? (g >> 2) * 4 : 0;
+            const float4 t = *reinterpret_cast<const float4*>(src + first);
+            float y[VEC];
+            y[0] = t.x; y[1] = t.y; y[2] = t.z; y[3] = t.w;
+            if constexpr (VEC == 8) {
+                const float4 w = *reinterpret_cast<const float4*>(src + (first ^ 4));
+                y[0] = first ? w.x : t.x; y[1] = first ? w.y : t.y; y[2] = first ? w.z : t.z; y[3] = first ? w.w : t.w;
+                y[4] = first ? t.x : w.x; y[5] = first ? t.y : w.y; y[6] = first ? t.z : w.z; y[7] = first ? t.w : w.w;
+            }
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) x[e] = fmaf(y[e], inv_row, corr[c * VEC + e]);
+        };
         if constexpr (DELTA) {
             // Eq. 2 and 4 on the beam's two rows (even: S_{t-1} q_t, odd: S_{t-1} k_t), by the even row's lanes:
             //   delta_t = beta_t (v_t - alpha_t S_{t-1} k_t) ,  o_t = alpha_t S_{t-1} q_t + delta_t (k_t . q_t)
+            float own[CV][VEC];
+#pragma unroll
+            for (int c = 0; c < CV; ++c) output(c, own[c]);
+            __syncwarp();
+            if (key_row) {
+#pragma unroll
+                for (int c = 0; c < CV; ++c)
+#pragma unroll
+                    for (int e = 0; e < VEC; e += 4)
+                        *reinterpret_cast<float4*>(C_s + grp * CP + (c * G + g) * VEC + e) = make_float4(own[c][e], own[c][e + 1], own[c][e + 2], own[c][e + 3]);
+            }
+            __syncwarp();
             if (active && !key_row) {
                 T* ddst = vplane + (long long)(a.bases.base[req] + bb) * a.v_stride;
 #pragma unroll
                 for (int c = 0; c < CV; ++c) {
-                    const float* uq = C_s + grp * CP + (c * G + g) * VEC;
+                    const float* uk = C_s + (grp + 1) * CP + (c * G + g) * VEC;
                     float vx[VEC], dl[VEC], o[VEC];
                     Vec16<T>::unpack(cur.v[c], vx);
 #pragma unroll
                     for (int e = 0; e < VEC; ++e) {
-                        dl[e] = cur.gate.y * fmaf(-cur.gate.x, uq[CP + e], vx[e]);
-                        o[e] = fmaf(dl[e], kq, cur.gate.x * uq[e]);
+                        dl[e] = cur.gate.y * fmaf(-cur.gate.x, uk[e], vx[e]);
+                        o[e] = fmaf(dl[e], kq, cur.gate.x * own[c][e]);
                     }
                     store_out<OutT, VEC>(out + (c * G + g) * VEC, o);
                     store_out<T, VEC>(ddst + (c * G + g) * VEC, dl);
@@ -420,17 +475,12 @@ __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, 
 #pragma unroll
             for (int c = 0; c < CV; ++c) {
                 if ((c * G * VEC) / 128 != mt) continue;
-                const float* src = C_s + grp * CP + (c * G + g) * VEC - mt * 128;
                 float x[VEC];
-#pragma unroll
-                for (int e = 0; e < VEC; e += 4) {
-                    const float4 t = *reinterpret_cast<const float4*>(src + e);
-                    x[e] = t.x; x[e + 1] = t.y; x[e + 2] = t.z; x[e + 3] = t.w;
-                }
+                output(c, x);
                 store_out<OutT, VEC>(out + (c * G + g) * VEC, x);
             }
         }
-        if (mt + 1 < MT) __syncthreads();      // the tile is read out before the next corr rows overwrite it
+        if (mt + 1 < MT) __syncthreads();      // the tile is read out before the next accumulators overwrite it
     }
     if (tid == 0) {
         // a CTA must not exit with bulk copies still landing in its shared memory: after a wait ran out nobody may
@@ -466,7 +516,7 @@ cudaError_t launch_one(const TiledArgs& a, cudaStream_t stream) {
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             // shared memory for the CTAs the registers allow and no more: what is left of the SM's 228 KB serves the
             // fold's record loads as L1 (asking for all of it made 128 x 128 fp32 14 % slower)
-            constexpr int pct = (int)((tiled_min_ctas<KD, VD>() * (smem + 1024) * 100 + 228 * 1024 - 1) / (228 * 1024));
+            constexpr int pct = (int)((tiled_min_ctas<KD, VD, T>() * (smem + 1024) * 100 + 228 * 1024 - 1) / (228 * 1024));
             if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, pct > 100 ? 100 : pct);
             if (e != cudaSuccess) return e;
             ready[dev] = true;
