@@ -16,7 +16,11 @@ namespace {
 // The slots of one level of one request are consecutive (level_base keeps the first), so a level's records are a bitmap of
 // max_beam bits: marks are atomic ORs into shared memory, a warp per level turns them into running counts, and a position
 // is a count plus the bits below - three barriers for all levels.  (As two kernels, with one prefix sum over max_beam marks
-// and seven barriers per level, the pair took 5.5 us at depth 2 and 19 us at depth 8 for 4 x 512 beams; 2.9 - 4.1 us now.)
+// and seven barriers per level, the pair took 5.5 us at depth 2 and 19 us at depth 8 for 4 x 512 beams; 2.9 - 4.1 us here.)
+// What is left is latency: parents, then the old table's slots beside their levels' first slots, two barriers, the stores.  The
+// parents are asked for before anything else, nothing stands between them and the table, a thread has its beam's slots in
+// registers for the positions, and there are no more threads than beams: 0.9 us less per launch at 128 beams and depth 2 - 4,
+// 2.1 us less at 4 x 512 beams and depth 2 - 8 than with a barrier before the parents, slots read back and 1024 threads.
 // Levels beyond `chunk` are taken in further rounds of the same three steps.
 struct IndexArgs {
     int32_t* tables;            // [request][2][max_steps][max_beam]
@@ -32,7 +36,7 @@ struct IndexArgs {
 __global__ void __launch_bounds__(1024) index_kernel(const __grid_constant__ IndexArgs a) {
     extern __shared__ uint32_t bits[];                     // [chunk][words] marks, then [chunk][words] running counts
     __shared__ int32_t s_count[32], s_base[32], s_off;
-    const int r = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int r = blockIdx.x, tid = threadIdx.x, threads = blockDim.x, lane = tid & 31, warp = tid >> 5;
     const int words = (a.max_beam + 31) / 32, levels = a.depth_old, chunk = a.chunk;
     uint32_t* counts = bits + chunk * words;
     const long long buf = (long long)a.max_steps * a.max_beam;
@@ -42,13 +46,15 @@ __global__ void __launch_bounds__(1024) index_kernel(const __grid_constant__ Ind
     int32_t *sidx = a.sidx + r * a.sidx_req_stride, *ulist = a.ulist + r * a.sidx_req_stride, *urep = a.urep + r * a.sidx_req_stride;
     int32_t* uoff = a.uoff + r * a.uoff_req_stride;
     if (a.want_index)
-        for (int i = tid; i < min(chunk, levels) * words; i += 1024) bits[i] = 0u;
+        for (int i = tid; i < min(chunk, levels) * words; i += threads) bits[i] = 0u;
     if (tid == 0) s_off = 0;
+    __syncthreads();
     // the caller's parents, the old table and every array written here belong to earlier launches of the stream
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // h_t(b, t): the record a beam is about to append lives at base(req, t) + b
-    for (int b = tid; b < a.W_new; b += 1024) newt[(long long)a.depth_old * a.max_beam + b] = a.bases.base[r] + b;
+    const int p_first = levels > 0 && tid < a.W_new ? a.parents[(long long)r * a.W_new + tid] : 0;
+    for (int b = tid; b < a.W_new; b += threads) newt[(long long)a.depth_old * a.max_beam + b] = a.bases.base[r] + b;
     if (tid == 0) {
         lbase[a.depth_old] = a.bases.base[r];
         if (a.want_index) uoff[0] = 0;
@@ -57,30 +63,34 @@ __global__ void __launch_bounds__(1024) index_kernel(const __grid_constant__ Ind
         const int n = min(chunk, levels - l0);
         if (a.want_index && l0 > 0) {
             __syncthreads();
-            for (int i = tid; i < n * words; i += 1024) bits[i] = 0u;
+            for (int i = tid; i < n * words; i += threads) bits[i] = 0u;
+            __syncthreads();
         }
-        if (tid < n) s_base[tid] = lbase[l0 + tid];
-        __syncthreads();
+        if (tid < n) s_base[tid] = lbase[l0 + tid];            // (for the positions; the marks read it beside the old table)
+        int32_t slot[8];
         // Eq. 5: the child inherits its parent's row (levels < t-1) and, at level t-1, the parent's own slot, which is the
         // last entry of the parent's row - one gather covers both cases.
-        for (int b = tid; b < a.W_new; b += 1024) {
-            int p = a.parents[(long long)r * a.W_new + b];
+        for (int b = tid; b < a.W_new; b += threads) {
+            int p = b == tid ? p_first : a.parents[(long long)r * a.W_new + b];
             if ((unsigned)p >= (unsigned)a.W_prev) {
                 if (atomicCAS(a.status, ONELA_OK, ONELA_E_DEVICE_CHECK) == ONELA_OK) a.status[1] = p;
                 p = 0;
             }
             for (int l1 = 0; l1 < n; l1 += 8) {             // eight gathers in flight
-                int32_t slot[8];
+                int32_t first[8];
 #pragma unroll
                 for (int e = 0; e < 8; ++e)
-                    if (l1 + e < n) slot[e] = oldt[(long long)(l0 + l1 + e) * a.max_beam + p];
+                    if (l1 + e < n) {
+                        slot[e] = oldt[(long long)(l0 + l1 + e) * a.max_beam + p];
+                        first[e] = lbase[l0 + l1 + e];
+                    }
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
                     const int l = l1 + e;
                     if (l >= n) break;
                     newt[(long long)(l0 + l) * a.max_beam + b] = slot[e];
                     if (a.want_index) {
-                        const int key = slot[e] - s_base[l];
+                        const int key = slot[e] - first[e];
                         atomicOr(&bits[l * words + (key >> 5)], 1u << (key & 31));
                     }
                 }
@@ -89,7 +99,7 @@ __global__ void __launch_bounds__(1024) index_kernel(const __grid_constant__ Ind
         if (!a.want_index) continue;
         __syncthreads();
         // counts of the records before each word, level by level (one warp each); then the levels' offsets in the list
-        for (int l = warp; l < n; l += 32) {
+        for (int l = warp; l < n; l += threads / 32) {
             int32_t run = 0;
             for (int w0 = 0; w0 < words; w0 += 32) {
                 const int w = w0 + lane;
@@ -115,13 +125,13 @@ __global__ void __launch_bounds__(1024) index_kernel(const __grid_constant__ Ind
             if (lane >= o) c_incl += t;
         }
         if (warp == 0 && lane < n) uoff[l0 + lane + 1] = off + c_incl;
-        for (int b0 = 0; b0 < a.W_new; b0 += 1024) {       // (whole warps stay in the loop for the shuffles)
+        const bool kept = a.W_new <= threads && n <= 8;   // this thread's slots are still in its registers
+        for (int b0 = 0; b0 < a.W_new; b0 += threads) {       // (whole warps stay in the loop for the shuffles)
             const int b = b0 + tid;
             for (int l1 = 0; l1 < n; l1 += 8) {
-                int32_t slot[8];
 #pragma unroll
                 for (int e = 0; e < 8; ++e)                // (written by this thread)
-                    slot[e] = l1 + e < n && b < a.W_new ? newt[(long long)(l0 + l1 + e) * a.max_beam + b] : 0;
+                    if (!kept) slot[e] = l1 + e < n && b < a.W_new ? newt[(long long)(l0 + l1 + e) * a.max_beam + b] : 0;
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
                     const int l = l1 + e;
@@ -150,12 +160,12 @@ __global__ void __launch_bounds__(1024) index_kernel(const __grid_constant__ Ind
     __syncthreads();
     const int32_t total = s_off;
     uint8_t* sg8 = a.sg8 + r * a.sg8_req_stride;
-    for (int i = tid; i < levels * a.sg_stride; i += 1024) {
+    for (int i = tid; i < levels * a.sg_stride; i += threads) {
         const int level = i / a.sg_stride, b = i - level * a.sg_stride;
         sg8[i] = (uint8_t)sidx[(long long)level * a.max_beam + min(b, a.W_new - 1)];
     }
     uint8_t* unode = a.unode + (long long)r * (ONELA_UNODE_CAP * 16);
-    for (int j = tid; j < min(total, ONELA_UNODE_CAP); j += 1024) {
+    for (int j = tid; j < min(total, ONELA_UNODE_CAP); j += threads) {
         int lv = 0;
         for (int l = 1; l < levels; ++l) lv += (j >= uoff[l]) ? 1 : 0;
         const int rp = urep[j];
@@ -216,7 +226,9 @@ cudaError_t launch_index(const Layout& lay, int32_t req_begin, int32_t req_count
         cudaError_t e = cudaFuncSetAttribute(index_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    return launch_dependent(index_kernel, dim3(req_count), dim3(1024), smem, stream, a);
+    // a thread per beam; at least eight warps (one counts a level)
+    const int threads = W_new > 1024 ? 1024 : W_new < 256 ? 256 : (W_new + 31) / 32 * 32;
+    return launch_dependent(index_kernel, dim3(req_count), dim3(threads), smem, stream, a);
 }
 
 cudaError_t launch_export_chains(const int32_t* table_cur, int32_t W, int32_t depth, int32_t max_beam,
