@@ -46,11 +46,8 @@ using namespace sm100;
 #ifndef ONELA_FOLD_WARPS
 #define ONELA_FOLD_WARPS 12
 #endif
-#ifndef ONELA_LPU
-#define ONELA_LPU 8
-#endif
 constexpr int FOLD_WARPS = ONELA_FOLD_WARPS;
-constexpr int LPU = ONELA_LPU;                      // lanes per (beam, head) unit
+constexpr int LPU = 8;                              // lanes per (beam, head) unit
 constexpr int UPW = 32 / LPU;                       // units a fold warp folds at a time (a "quad" when LPU = 8)
 constexpr int NCH = 16 / LPU;                       // 16-byte chunks per lane per 256-byte vector
 constexpr int THREADS = (FOLD_WARPS + 5) * 32;      // + 4 epilogue warps + the warp that issues the MMAs
@@ -305,9 +302,10 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     };
-    // The first segment's S_0 is requested by all warps (one 32-column block each) before the launch's dependencies are
-    // waited for, and put into tensor memory after the first heads have been requested: the store is written only by
-    // the state calls (a copy or a prefill kernel), and a reorder launch always separates those from a decode.
+    // The first segment's S_0 is requested by all warps (one 32-column block each) and put into tensor memory before the
+    // launch's dependencies are waited for: the store is written only by the state calls (a copy or a prefill kernel), and
+    // a reorder launch always separates those from a decode.  (Put there after the first heads had been requested, it stood
+    // between them and the fold: 0.4 us of a launch of 128 x 16 to 512 x 32 units, 1 - 1.5 %; large launches are the same.)
     static_assert(THREADS >= 512, "the first sixteen warps take one 32-column block of the first S_0 each");
     const bool s0_mine = warp < 16;
     float4 s0_first[8];
@@ -338,15 +336,15 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
         asm volatile("griddepcontrol.wait;" ::: "memory");
     };
 
-    // How many of the oldest levels of a request's chains fit in `stage_cap` staged records (whole levels only), and
-    // how many records that is.  Lane l looks at level l (one load latency for the whole chain); warp-uniform.
+    // Where the levels of a request's distinct records end in its list: lane l has level l's (`ends_of`).  From these,
+    // how many of the oldest levels of a request's chains fit in `stage_cap` staged records (whole levels only), and
+    // how many records that is; warp-uniform.
     // `sparse` (optional): bit l set when level l has more than W / 4 distinct records, i.e. little sharing - the
     // levels whose gathered records are worth requesting ahead.
-    auto staging_of = [&](int req, int& levels, int& count, uint32_t* sparse = nullptr) {
-        const int32_t* uoff = a.uoff + req * a.uoff_req_stride;
+    auto ends_of = [&](int req) { return lane < old ? __ldg(a.uoff + req * a.uoff_req_stride + lane + 1) : 0x7fffffff; };
+    auto staging_from = [&](int e_all, int& levels, int& count, uint32_t* sparse = nullptr) {
         // (at most the eight oldest levels, whose list positions a unit's lanes hold: the staged fold then never has to
         // look an index up in memory)
-        const int e_all = (lane < old) ? __ldg(uoff + lane + 1) : 0x7fffffff;
         const int e = lane < 8 ? e_all : 0x7fffffff;
         levels = __popc(__ballot_sync(0xffffffffu, e <= stage_cap));
         count = __shfl_sync(0xffffffffu, e, levels > 0 ? levels - 1 : 0);
@@ -357,6 +355,7 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
             *sparse = __ballot_sync(0xffffffffu, lane < old && (e_all - prev) * 4 > a.W);
         }
     };
+    auto staging_of = [&](int req, int& levels, int& count) { staging_from(ends_of(req), levels, count); };
 
     // Chains that share little - fewer than half of the first request's older levels can be staged, and the beams' parents are
     // more than a quarter as many as there are beams - are gathered through a queue: nothing is staged, and every fold warp
@@ -365,11 +364,11 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
     // level: 8 x 1024 beams with uniform parents 24 us per level that way, 15 us through the queue (depth 6: 202 -> 165 us).
     // Where the line lies, measured on 4 x 300 beams, uniform parents, depth 4 - 7: staging what can be staged 22.6 us, the
     // queue as soon as one level cannot be staged 21.8 us, but on 2 x 200 beams, Zipf(1.2), 21 us against 18 us with the rule.
-    auto gather_queued = [&](int& levels, int& count) {
+    auto gather_queued = [&](int ends, int& levels, int& count) {        // (ends: those of the first request)
         levels = count = 0;
         if (n_segs == 0 || old == 0) return false;
         uint32_t sparse;
-        staging_of(req_begin, levels, count, &sparse);
+        staging_from(ends, levels, count, &sparse);
         if (2 * levels >= old || !((sparse >> (min(old, 32) - 1)) & 1)) return false;
         levels = count = 0;
         return true;
@@ -495,20 +494,35 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
         Idx idx_next{};
         Unit u1 = next_unit(u0), u2 = next_unit(u1);
         if (n_quads > 0) request_heads(u0);
+        put_first_s0();
         dependency_wait();
         if (n_quads > 0) {
             issue_head(u0);
             gate0 = load_gate(u0);
             if (1 < n_quads) gate1 = load_gate(u1);
-            queued = gather_queued(info_levels, info_count);
-            info_req = req_begin;
-            idx_next = load_idx(u0);
+        }
+        // The first quad's indices, asked for in both places where they may stand, beside the levels' ends that tell which
+        // of the two counts: one latency instead of two.  (With the same for the first staging list and no wait for the
+        // segment's scale: 8 layers x 128 beams x 16 heads, depth 4, 209 -> 201 us a generation; 4 x 512 x 32, 1.5 %.)
+        int32_t in_table = 0, in_list = 0;
+        int ends = 0x7fffffff;
+        if (n_quads > 0) {
+            ends = ends_of(req_begin);
+            if (g < old) {
+                const long long at = (long long)g * a.max_beam + live_beam(u0);
+                in_table = __ldg(a.table + u0.req * a.table_req_stride + at);
+                in_list = __ldg(a.sidx + u0.req * a.sidx_req_stride + at);
+            }
         }
         TL(2, 0);   // dependencies waited for, first heads requested
-        put_first_s0();
-        TL(3, 0);   // first S_0 in tensor memory
+        if (n_quads > 0) {
+            queued = gather_queued(ends, info_levels, info_count);
+            info_req = req_begin;
+            idx_next.v[0] = g < info_levels ? in_list : in_table;
+        }
+        TL(3, 0);   // first indices there
         int cur_seg = -1, buf = 0, staged_levels = 0;
-        float seg_inv_s0 = 1.f;
+        float seg_scale = 1.f;                   // the segment's S_0 scale, a power of two
         bool staged_ready = false;
         long long plane_row0 = 0, own_row0 = 0;
         const int32_t *table_r = nullptr, *sidx_r = nullptr;
@@ -551,7 +565,7 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
                     buf = single ? 0 : (cur_seg & 1);
                     staged_ready = false;
                     staged_levels = staged_levels_of(u0.req);
-                    seg_inv_s0 = 1.f / __ldg(a.s0_scale + u0.req * a.s0_scale_req_stride + value_head_of(u0));   // a power of two
+                    seg_scale = __ldg(a.s0_scale + u0.req * a.s0_scale_req_stride + value_head_of(u0));   // (used when the quad is folded: no wait here)
                     plane_row0 = (long long)value_head_of(u0) * a.arena_slots;      // row 0 of the head's gate plane
                     own_row0 = plane_row0 + a.bases.base[u0.req];
                     table_r = a.table + u0.req * a.table_req_stride;
@@ -790,7 +804,7 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
                     }
                     float d_scale, d_inv;
                     pow2_scale(decay, 0, d_scale, d_inv);
-                    if (g == 0) inv_s[s * GN + u] = (q_inv * d_inv) * seg_inv_s0;
+                    if (g == 0) inv_s[s * GN + u] = (q_inv * d_inv) * __uint_as_float(0x7f000000u - __float_as_uint(seg_scale));   // 1 / seg_scale
                     const float dcs = (decay * d_scale) * q_scale;
                     const float2 dc = make_float2(dcs, dcs);
 #pragma unroll
@@ -861,24 +875,31 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
         if (dead && lane == 0) *abort_flag = 1;
     } else {
         // =============================== EPILOGUE (+ preparation of the next segments) ===============================
+        put_first_s0();
         dependency_wait();
         const int quad = warp & 3;                    // tensor-memory lane quadrant of this warp
+        // the first request's levels and its list, asked for together (beyond the list's end: not used)
+        const int li = (warp - FOLD_WARPS) * 32 + lane;
+        int ends = 0x7fffffff, first_slot = 0;
+        if (n_segs > 0) {
+            ends = ends_of(req_begin);
+            first_slot = __ldg(a.ulist + req_begin * a.ulist_req_stride + min((long long)li, a.ulist_req_stride - 1));
+        }
         int first_levels, first_count;
-        const bool queued = gather_queued(first_levels, first_count);          // nothing is staged then
+        const bool queued = gather_queued(ends, first_levels, first_count);          // nothing is staged then
         int staged_issued[2] = {0, 0};                // stagings requested per buffer (what teardown must wait for)
         // Stage the distinct records of segment `seg`: one 512-byte bulk copy per record, its gates by a plain load, one
         // record per lane.  Every lane arrives once, announcing the bytes it requested; its gate store is ordered
         // before the arrival.  The barrier completes even when nothing is staged.
-        auto stage_segment = [&](int seg) {
+        auto stage_segment = [&](int seg, const int* known) {        // known: this lane's entry of the list, where it has been read already
             int req, h;
             pair_of(seg, req, h);
             const int b = single ? 0 : (seg & 1);
             int levels = first_levels, count = first_count;      // (of the first request; zero with a gather queue)
             if (!queued && req != req_begin) staging_of(req, levels, count);
             const long long plane_row0 = (long long)value_head(h) * a.arena_slots;
-            const int li = (warp - FOLD_WARPS) * 32 + lane;
             if (li < count) {
-                const long long slot = __ldg(a.ulist + req * a.ulist_req_stride + li), row = plane_row0 + slot;
+                const long long slot = known ? *known : __ldg(a.ulist + req * a.ulist_req_stride + li), row = plane_row0 + slot;
                 const uint32_t dst = smem_u32(stage + (b * STAGE_BUF + li) * REC_BYTES);
                 if constexpr (GROUPED) {      // the two halves of the staged row come from the two planes
                     bulk_load(dst, k_at(h, slot), DK * 2, bar_stage(b));
@@ -897,10 +918,9 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_s0(seg & 1));
         };
-        if (n_segs > 0) stage_segment(0);
-        put_first_s0();
+        if (n_segs > 0) stage_segment(0, &first_slot);
         if (n_segs > 1) {          // (doing this part later, or before the dependency wait with all warps, measured slower)
-            stage_segment(1);
+            stage_segment(1, nullptr);
             prepare_s0(1);
         }
 
@@ -1024,7 +1044,7 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
                 if (!wait_or_abort(bar_sfree((seg + 1) & 1), ((seg - 1) >> 1) & 1, abort_flag)) {
                     give_up();
                 } else {
-                    stage_segment(seg + 1);
+                    stage_segment(seg + 1, nullptr);
                     prepare_s0(seg + 1);
                 }
             }
