@@ -9,6 +9,11 @@
 // two axpys and a log2(G)-step shuffle reduction.  The folded queries of the tile then meet the head's
 // S_0 in a [dv x dk] . [dk x 32] product on the FMA pipes: lane = beam, each warp a band of rows,
 // S_0 rows read as warp-uniform (broadcast) 16-byte loads, R from padded shared memory.
+// What bounds it at 32 x 32: a chain of latencies, not bytes - the slots, the records, then the state's rows out of L2.  The
+// unit's lanes hold the slots of the chain's levels, a record is on its way while the one before it is folded, and the
+// state waits in shared memory, fetched before the launch's dependencies are waited for.  Generations before / after (each
+// level's slot and record looked up in turn, the state read through L1): 4 x 200 beams x 24 heads, 4 layers, depth 4 163 / 116
+// us; 8 x 1024 x 32, depth 8 865 / 747 us; bf16 4 x 512 x 32, 2 layers, depth 8 384 / 342 us; 8 beams, 2 heads 14.2 / 12.3 us.
 #include "onela_internal.h"
 #include "onela_layout.cuh"
 
@@ -17,6 +22,10 @@ namespace onela {
 namespace {
 
 constexpr int NB = 32;  // beams per tile
+// The state fits beside the tile's rows (4 KB) and a lane's part of a record in eight registers: dk = dv = 32, the shape
+// that this kernel serves as the product path.
+template <int DK, int DV>
+__host__ __device__ constexpr bool generic_small() { return DK * DV <= 1024; }
 
 template <int DK, int DV, typename T, typename OutT, int G>
 __global__ void __launch_bounds__(NB* G) decode_generic_kernel(const DecodeArgs a) {
@@ -28,6 +37,8 @@ __global__ void __launch_bounds__(NB* G) decode_generic_kernel(const DecodeArgs 
     extern __shared__ __align__(16) float smem[];
     float* R_s = smem;             // [NB][RP]  folded queries
     float* C_s = smem + NB * RP;   // [NB][CP]  corr, then the finished outputs
+    constexpr bool SMALL = generic_small<DK, DV>();
+    float* S_s = C_s + NB * CP;    // SMALL: [DV][DK]  the head's S_0
 
     const int tile = blockIdx.x, h = blockIdx.y, req = blockIdx.z;
     const int grp = threadIdx.x / G, g = threadIdx.x % G;
@@ -35,6 +46,11 @@ __global__ void __launch_bounds__(NB* G) decode_generic_kernel(const DecodeArgs 
     const bool active = b < a.W;
     const int bb = active ? b : a.W - 1;  // idle groups shadow a live beam so loads and shuffles stay uniform
 
+    // (the store is written only by the state calls, and a reorder launch always lies between those and a decode)
+    const float* S0h = a.s0 + req * a.s0_req_stride + (long long)h * DV * DK;
+    if constexpr (SMALL) {
+        for (int i = threadIdx.x; i < DV * DK / 4; i += NB * G) reinterpret_cast<float4*>(S_s)[i] = __ldg(reinterpret_cast<const float4*>(S0h) + i);
+    }
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const bool fused = a.k_in != nullptr;   // append fused in: the newest record comes from the caller's tensors
@@ -43,6 +59,29 @@ __global__ void __launch_bounds__(NB* G) decode_generic_kernel(const DecodeArgs 
     const long long plane_row0 = (long long)h * a.arena_slots;
     const T* kv = reinterpret_cast<const T*>(a.kv);
 
+    const int old = a.depth - 1;           // records older than the beam's own: levels old - 1 .. 0
+    // lane l of a unit has the slot of its ancestor at level l: one latency for the chain (deeper levels are looked up)
+    const int32_t my_slot = g < old ? __ldg(table + (long long)g * a.max_beam + bb) : 0;
+    auto row_of = [&](int level) {
+        const int32_t near = __shfl_sync(0xffffffffu, my_slot, level & (G - 1), G);
+        return plane_row0 + (level < G ? near : __ldg(table + (long long)level * a.max_beam + bb));
+    };
+    struct Rec {
+        float k[CK * VEC], v[CV * VEC];
+        float2 gate;
+    };
+    auto load_halves = [&](const T* kr, const T* vr, Rec& x) {
+#pragma unroll
+        for (int c = 0; c < CK; ++c) Vec16<T>::load(kr + (c * G + g) * VEC, x.k + c * VEC);
+#pragma unroll
+        for (int c = 0; c < CV; ++c) Vec16<T>::load(vr + (c * G + g) * VEC, x.v + c * VEC);
+    };
+    auto load_record = [&](int level, Rec& x) {
+        const long long row = row_of(level);
+        const T* rec = kv + row * (DK + DV);
+        load_halves(rec, rec + DK, x);
+        x.gate = __ldg(a.gates + row);
+    };
     float r[CK * VEC], corr[CV * VEC];
 #pragma unroll
     for (int c = 0; c < CK; ++c) Vec16<T>::load(q + (c * G + g) * VEC, r + c * VEC);
@@ -50,51 +89,57 @@ __global__ void __launch_bounds__(NB* G) decode_generic_kernel(const DecodeArgs 
     for (int e = 0; e < CV * VEC; ++e) corr[e] = 0.f;
 
     float decay = 1.f;  // a = product of the alphas already passed
-    for (int level = a.depth - 1; level >= 0; --level) {
-        const bool own = level == a.depth - 1;
-        const int32_t slot = own ? a.bases.base[req] + bb : __ldg(table + (long long)level * a.max_beam + bb);
-        const long long row = plane_row0 + slot;
-        const T* rec = kv + row * (DK + DV);
-        const T *kr = rec, *vr = rec + DK;
-        float2 gate;
-        if (own && fused) {     // ... and this unit also writes it to its slot, bit for bit
+    auto fold = [&](const Rec& x) {
+        float dot = 0.f;
+#pragma unroll
+        for (int e = 0; e < CK * VEC; ++e) dot = fmaf(x.k[e], r[e], dot);
+#pragma unroll
+        for (int off = G / 2; off > 0; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
+        const float bc = x.gate.y * dot;      // beta_j * (k_j . r~_j)
+        const float wv = decay * bc;          // beta_j * c_j with c_j = a_j (k_j . r~_j)
+#pragma unroll
+        for (int e = 0; e < CV * VEC; ++e) corr[e] = fmaf(wv, x.v[e], corr[e]);
+#pragma unroll
+        for (int e = 0; e < CK * VEC; ++e) r[e] = fmaf(-bc, x.k[e], r[e]);
+        decay *= x.gate.x;
+    };
+    Rec cur;
+    {
+        const long long row = plane_row0 + a.bases.base[req] + bb;
+        if (fused) {     // ... and this unit also writes it to its slot, bit for bit
             const long long in_row = ((long long)req * a.W + bb) * a.H + h;
-            kr = static_cast<const T*>(a.k_in) + in_row * DK;
-            vr = static_cast<const T*>(a.v_in) + in_row * DV;
-            gate = make_float2(__ldg(a.alpha_in + in_row), __ldg(a.beta_in + in_row));
+            const T *kr = static_cast<const T*>(a.k_in) + in_row * DK, *vr = static_cast<const T*>(a.v_in) + in_row * DV;
+            load_halves(kr, vr, cur);
+            cur.gate = make_float2(__ldg(a.alpha_in + in_row), __ldg(a.beta_in + in_row));
             if (active) {
                 uint4* dst = reinterpret_cast<uint4*>(a.kv_out + row * ((DK + DV) * (long long)sizeof(T)));
 #pragma unroll
                 for (int c = 0; c < CK; ++c) dst[c * G + g] = __ldg(reinterpret_cast<const uint4*>(kr) + c * G + g);
 #pragma unroll
                 for (int c = 0; c < CV; ++c) dst[DK / VEC + c * G + g] = __ldg(reinterpret_cast<const uint4*>(vr) + c * G + g);
-                if (g == 0) a.gates_out[row] = gate;
+                if (g == 0) a.gates_out[row] = cur.gate;
             }
         } else {
-            gate = __ldg(a.gates + row);
+            const T* rec = kv + row * (DK + DV);
+            load_halves(rec, rec + DK, cur);
+            cur.gate = __ldg(a.gates + row);
         }
-        float kx[CK * VEC];
-        float dot = 0.f;
-#pragma unroll
-        for (int c = 0; c < CK; ++c) {
-            Vec16<T>::load(kr + (c * G + g) * VEC, kx + c * VEC);
-#pragma unroll
-            for (int e = 0; e < VEC; ++e) dot = fmaf(kx[c * VEC + e], r[c * VEC + e], dot);
+    }
+    if constexpr (SMALL) {       // a record is on its way while the one before it is folded
+        Rec next;
+        if (old > 0) load_record(old - 1, next);
+        for (int level = old; level > 0; --level) {
+            fold(cur);
+            cur = next;
+            if (level > 1) load_record(level - 2, next);
         }
-#pragma unroll
-        for (int off = G / 2; off > 0; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
-        const float bc = gate.y * dot;        // beta_j * (k_j . r~_j)
-        const float wv = decay * bc;          // beta_j * c_j with c_j = a_j (k_j . r~_j)
-#pragma unroll
-        for (int c = 0; c < CV; ++c) {
-            float vx[VEC];
-            Vec16<T>::load(vr + (c * G + g) * VEC, vx);
-#pragma unroll
-            for (int e = 0; e < VEC; ++e) corr[c * VEC + e] = fmaf(wv, vx[e], corr[c * VEC + e]);
+        fold(cur);
+    } else {
+        fold(cur);
+        for (int level = old - 1; level >= 0; --level) {
+            load_record(level, cur);
+            fold(cur);
         }
-#pragma unroll
-        for (int e = 0; e < CK * VEC; ++e) r[e] = fmaf(-bc, kx[e], r[e]);
-        decay *= gate.x;
     }
 
 #pragma unroll
@@ -118,7 +163,6 @@ __global__ void __launch_bounds__(NB* G) decode_generic_kernel(const DecodeArgs 
     // out[beam][i] = sum_k S0[i][k] R[beam][k] + corr[beam][i]; lane = beam, warp = band of DV/G rows
     {
         const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        const float* S0h = a.s0 + req * a.s0_req_stride + (long long)h * DV * DK;
         const float* Rl = R_s + lane * RP;
         constexpr int ROWS = DV / G;
         for (int i0 = warp * ROWS; i0 < (warp + 1) * ROWS; i0 += 4) {
@@ -128,7 +172,8 @@ __global__ void __launch_bounds__(NB* G) decode_generic_kernel(const DecodeArgs 
                 const float4 rv = *reinterpret_cast<const float4*>(Rl + k);
 #pragma unroll
                 for (int rr = 0; rr < 4; ++rr) {
-                    const float4 sv = __ldg(reinterpret_cast<const float4*>(S0h + (long long)(i0 + rr) * DK + k));
+                    const float* sp = (SMALL ? S_s : S0h) + (long long)(i0 + rr) * DK + k;
+                    const float4 sv = SMALL ? *reinterpret_cast<const float4*>(sp) : __ldg(reinterpret_cast<const float4*>(sp));
                     acc[rr] = fmaf(sv.x, rv.x, acc[rr]);
                     acc[rr] = fmaf(sv.y, rv.y, acc[rr]);
                     acc[rr] = fmaf(sv.z, rv.z, acc[rr]);
@@ -163,7 +208,7 @@ cudaError_t launch_one(const DecodeArgs& a, cudaStream_t stream) {
     constexpr int VEC = Vec16<T>::N;
     constexpr int G = (DK / VEC >= 8 && DV / VEC >= 8) ? 8 : 4;
     auto kern = decode_generic_kernel<DK, DV, T, OutT, G>;
-    const size_t smem = sizeof(float) * NB * ((DK + 4) + (DV + 4));
+    const size_t smem = sizeof(float) * (NB * ((DK + 4) + (DV + 4)) + (generic_small<DK, DV>() ? DK * DV : 0));
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
