@@ -71,10 +71,11 @@ __host__ __device__ constexpr size_t tiled_smem_bytes() {
 
 // CTAs per SM the registers are capped for: small CTAs are latency-bound (a string of dependent loads per level, one MMA
 // round trip), so the narrowest shape gets four, with bf16 records - half the registers - five (64 x 64 on the beam-512
-// stack: 30 -> 27 us; six: 28.5; fp32 records, five: 16 -> 17 us).  (64 beams of 256 threads at two per SM, or 16 lanes per
-// unit, were 5 - 10 % slower at 256 x 256.)
-template <int KD, int VD, typename T>
-__host__ __device__ constexpr int tiled_min_ctas() { return KD + VD <= 128 ? (sizeof(T) == 2 ? 5 : 4) : tiled_beams<KD, VD>() == 64 ? 1 : 2; }
+// stack: 30 -> 27 us; six: 28.5; fp32 records, five: 16 -> 17 us, three: 4 - 7 % slower at 65 536 units), unless a beam has two
+// rows, where five spill (4 x 300 beams x 16 heads, 6 calls, a generation: 185 -> 177 us).  (64 beams of 256 threads at two per
+// SM, or 16 lanes per unit, were 5 - 10 % slower at 256 x 256.)
+template <int KD, int VD, typename T, bool DELTA>
+__host__ __device__ constexpr int tiled_min_ctas() { return KD + VD <= 128 ? (sizeof(T) == 4 || DELTA ? 4 : 5) : tiled_beams<KD, VD>() == 64 ? 1 : 2; }
 
 // DELTA: the arena keeps (alpha_t, delta_t, k_t) (Section 3.2, Eq. 2-4).  A beam owns TWO rows of the tile - its query
 // and its own key, both projected through the parent state: S_{t-1} x = D S_0 x + sum_j d_j (k_j . x) delta_j, the
@@ -82,7 +83,7 @@ __host__ __device__ constexpr int tiled_min_ctas() { return KD + VD <= 128 ? (si
 // o_t = alpha_t S_{t-1} q_t + delta_t (k_t . q_t) are formed from the two rows and the record is written; always with
 // the append fused in, dk = dv <= 128.
 template <int KD, int VD, typename T, typename OutT, bool DELTA = false>
-__global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, VD, T>()) decode_tiled_kernel(const TiledArgs a) {
+__global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, VD, T, DELTA>()) decode_tiled_kernel(const TiledArgs a) {
     constexpr int NB = tiled_beams<KD, VD>(), CP = tile_pitch<VD>();
     constexpr int BPT = DELTA ? NB / 2 : NB;          // beams per tile
     static_assert(!DELTA || (KD == VD && VD <= 128), "delta records: square heads, one tile of value rows");
@@ -263,7 +264,11 @@ __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, 
     // The beam's own record: from its arena slot, or - append fused in - from the caller's tensors, in which case this
     // unit also writes it to the slot, bit for bit (16-byte vectors; the key once per key head, by its first value
     // head).  The fold reads the caller's copy, so nothing in this launch reads what another CTA of it writes.
-    Raw cur;
+    // 64 x 64 with fp32 records asks for the newest older record before the append's stores, which wait for the own one, and keeps
+    // the own fold out of the loop: no spills, 4 x 300 beams x 16 heads 168 -> 159 us a generation, 4 x 512 x 32 1038 -> 988 us.
+    // (bf16 records: 1.4 % faster on the stack, 2 - 3 % slower on 60 - 128 beams; 128 x 128: 1 % slower.  They keep the loop.)
+    constexpr bool EARLY = !DELTA && KD + VD <= 128 && sizeof(T) == 4;
+    Raw cur, first;
     {
         const long long slot = a.bases.base[req] + bb;
         T* kdst = kplane + slot * a.k_stride;
@@ -281,6 +286,7 @@ __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, 
         for (int c = 0; c < CK; ++c) cur.k[c] = __ldg(reinterpret_cast<const uint4*>(ksrc) + c * G + g);
 #pragma unroll
         for (int c = 0; c < CV; ++c) cur.v[c] = __ldg(reinterpret_cast<const uint4*>(vsrc) + c * G + g);
+        if (EARLY && old > 0) first = fetch_slot(old > G ? slot_far(old - 1) : slot_near(old - 1));
         if (fused && active && !key_row) {
             if constexpr (!DELTA) {      // (the delta half of a delta record is written after the contraction)
 #pragma unroll
@@ -327,6 +333,22 @@ __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, 
                 x = next;
             }
             fold(x);
+        }
+    } else if constexpr (EARLY) {
+        fold(cur);
+        if (old > 0) {
+            cur = first;
+            for (int level = old - 2; level >= G; --level) {
+                const Raw next = fetch_slot(slot_far(level));
+                fold(cur);
+                cur = next;
+            }
+            for (int level = min(old - 2, near_top); level >= 0; --level) {
+                const Raw next = fetch_slot(slot_near(level));
+                fold(cur);
+                cur = next;
+            }
+            fold(cur);
         }
     } else if constexpr (AHEAD) {
         for (int level = old - 1; level >= G; --level) {
@@ -516,7 +538,7 @@ cudaError_t launch_one(const TiledArgs& a, cudaStream_t stream) {
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             // shared memory for the CTAs the registers allow and no more: what is left of the SM's 228 KB serves the
             // fold's record loads as L1 (asking for all of it made 128 x 128 fp32 14 % slower)
-            constexpr int pct = (int)((tiled_min_ctas<KD, VD, T>() * (smem + 1024) * 100 + 228 * 1024 - 1) / (228 * 1024));
+            constexpr int pct = (int)((tiled_min_ctas<KD, VD, T, DELTA>() * (smem + 1024) * 100 + 228 * 1024 - 1) / (228 * 1024));
             if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, pct > 100 ? 100 : pct);
             if (e != cudaSuccess) return e;
             ready[dev] = true;
