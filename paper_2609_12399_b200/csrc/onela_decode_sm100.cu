@@ -1094,44 +1094,35 @@ int sm_count_ws() {
 // Contiguous group ranges for the CTAs.  A CTA's cost is counted as group_cost * groups + seg_cost * segments (starting
 // a segment: S_0 reloaded, staging refilled, the ring's overlap lost for a moment) and the smallest bound T is searched
 // for which a greedy fill needs no more CTAs than there are SMs.  Returns the number of CTAs used.
-// The costs, in units of ~500 cycles, follow what the kernel measures on the beam-512 stack: a group takes ~4000
-// cycles plus ~500 per chain level beyond the first; starting a segment ~6000 at depth <= 3 (where whole (request,
-// head) pairs per CTA, 128 x 11 groups, beat 141 x 10 groups over two segments by 0.6-1.5 us) and ~3000 deeper (where
-// the shorter CTA wins by 0.6-2.5 us).
+// The costs, in units of ~500 cycles, follow what the kernel measures: a group takes ~4000 cycles plus ~500 per chain level
+// beyond the first; a CTA's first two segments ~3000 each (the second is set up beside the first), every further one ~6000 at
+// depth <= 3, where the epilogue warps that prepare it set the pace, and ~3000 deeper.  (All segments at 6000 up to depth 3:
+// 2 x 512 beams x 32 heads in whole pairs of 11 groups, cut 6 + 5, instead of fives, 116 against 108 us a generation of
+// three calls; 4 x 400 beams, 16 key and 32 value heads 161 / 152; delta records 2 x 200 beams 384 / 375; the beam-512 stack
+// 1092 / 1089.  All at 3000: 7 x 333 beams as three segments of 11 groups, 228, instead of two of 12, 218.)
 struct PartitionCost {
-    int group, seg;
+    int group, seg, more;        // more: the third segment and on
 };
-#ifndef ONELA_SEG_SHALLOW
-#define ONELA_SEG_SHALLOW 12
-#endif
-#ifndef ONELA_SEG_DEEP
-#define ONELA_SEG_DEEP 6
-#endif
-#ifndef ONELA_SHALLOW_DEPTH
-#define ONELA_SHALLOW_DEPTH 3
-#endif
-PartitionCost partition_cost(int depth) {
-    return {8 + (depth > 1 ? depth - 1 : 0), depth <= ONELA_SHALLOW_DEPTH ? ONELA_SEG_SHALLOW : ONELA_SEG_DEEP};
-}
+PartitionCost partition_cost(int depth) { return {8 + (depth > 1 ? depth - 1 : 0), 6, depth <= 3 ? 12 : 6}; }
 template <class Begin>
 int greedy_fill(int total_groups, int gpp, int limit, int max_ctas, PartitionCost c, Begin* begin) {
     int n = 0, gi = 0;
     while (gi < total_groups) {
         if (n == max_ctas) return max_ctas + 1;
         if (begin) begin[n] = gi;
-        int cost = 0;
-        bool any = false;
+        int cost = 0, segs = 0;
         while (gi < total_groups) {
             const int pair_end = (gi / gpp + 1) * gpp;
-            const int room = (limit - cost - c.seg) / c.group;     // groups of this segment that still fit
+            const int start = segs < 2 ? c.seg : c.more;
+            const int room = (limit - cost - start) / c.group;     // groups of this segment that still fit
             if (room <= 0) break;
             const int take = room < pair_end - gi ? room : pair_end - gi;
             gi += take;
-            cost += c.seg + take * c.group;
-            any = true;
+            cost += start + take * c.group;
+            ++segs;
             if (gi < pair_end) break;
         }
-        if (!any) return max_ctas + 1;   // the bound does not admit a single group
+        if (segs == 0) return max_ctas + 1;   // the bound does not admit a single group
         ++n;
     }
     if (begin) begin[n] = total_groups;
@@ -1139,7 +1130,7 @@ int greedy_fill(int total_groups, int gpp, int limit, int max_ctas, PartitionCos
 }
 template <class Begin>
 int make_partition(int total_groups, int gpp, int sms, PartitionCost c, Begin* begin) {
-    int lo = c.seg + c.group, hi = c.seg * (total_groups / gpp + 2) + c.group * total_groups;
+    int lo = c.seg + c.group, hi = (c.seg > c.more ? c.seg : c.more) * (total_groups / gpp + 2) + c.group * total_groups;
     while (lo < hi) {
         const int mid = (lo + hi) / 2;
         if (greedy_fill<Begin>(total_groups, gpp, mid, sms, c, nullptr) <= sms) hi = mid;
@@ -1223,7 +1214,7 @@ extern "C" int onela_testhook_drop_full_arrival(int on) {
 #endif
 
 int make_decode_partition(int total_groups, int groups_per_pair, int sms, int group_cost, int seg_cost, DecodePartition* part) {
-    return make_partition(total_groups, groups_per_pair, sms > MAX_CTAS ? MAX_CTAS : sms, PartitionCost{group_cost, seg_cost}, part->begin);
+    return make_partition(total_groups, groups_per_pair, sms > MAX_CTAS ? MAX_CTAS : sms, PartitionCost{group_cost, seg_cost, seg_cost}, part->begin);
 }
 int decode_sm_count() { return sm_count_ws(); }
 
