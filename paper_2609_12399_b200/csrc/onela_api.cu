@@ -89,7 +89,6 @@ struct onela_ctx {
     std::vector<ReqState> req;
     int64_t cursor = 0;        // next free arena slot
     int64_t launches = 0;
-    int64_t decode_mark = -1;  // value of `launches` right after the last decode launch
     bool status_cleared = false;
     bool tensor_core = false;  // decode_step runs the warp-specialised tcgen05 kernel
     bool tiled_tc = false;     // decode_step runs the tiled tcgen05 kernel (the other shapes from 64 x 64 up)
@@ -577,7 +576,6 @@ onela_status launch_decode(onela_ctx* ctx, int32_t req_begin, int32_t req_count,
     a.depth = depth;
     a.max_beam = c.max_beam;
     for (int i = 0; i < req_count; ++i) a.bases.base[i] = ctx->req[req_begin + i].step_base.back();
-    a.early_ok = ctx->launches == ctx->decode_mark ? 1 : 0;
     bool supported = true;
     const bool wy = ctx->tensor_core && !ctx->gtr() && (c.flags & ONELA_FLAG_SHARED_CHAINS) && !ctx->grouped() && tiles == 1 && depth >= 2 &&
                     depth <= WY_MAX_LEVELS + 1;
@@ -588,7 +586,6 @@ onela_status launch_decode(onela_ctx* ctx, int32_t req_begin, int32_t req_count,
     if (!supported) return ONELA_E_UNSUPPORTED;
     if (e != cudaSuccess) return ONELA_E_CUDA;
     ctx->launches++;
-    ctx->decode_mark = ctx->launches;
     return ONELA_OK;
 }
 

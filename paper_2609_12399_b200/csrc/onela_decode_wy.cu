@@ -431,9 +431,10 @@ __global__ void __launch_bounds__(THREADS, 1) decode_wy_kernel(const __grid_cons
         }
     } else {
         // =============================== BACK SIDE: epilogue team and solver team ===============================
-        // What the set-up reads (index arrays, S_0, records of earlier decode calls) was written at least two launches
-        // ago when the host says so; the epilogue team still waits for the predecessor before its first store.
-        if (!a.early_ok) dependency_wait();
+        // The index arrays and the older records may still be in the making when this launch starts, whatever came before it:
+        // the index kernel lets its dependents start before it has written anything, and so does a decode launch between
+        // the two.  Only the wait says that they are there.
+        dependency_wait();
         const bool epi = warp < SOL_WARP0;
         const int quad = warp & 3;                    // tensor-memory lane quadrant of this warp
         const int row_i = quad * 32 + lane;           // tensor-memory lane of this thread
@@ -696,7 +697,6 @@ __global__ void __launch_bounds__(THREADS, 1) decode_wy_kernel(const __grid_cons
             if (epi) {
                 const int te = tid - EPI_WARP0 * 32;          // 0 .. 127
                 float* T_s = reinterpret_cast<float*>(T_raw);
-                dependency_wait();
                 for (int gi = seg_g0; gi < seg_g1; ++gi, ++gcount) {
                     const int s = gcount % SLOTS, vs = gcount % VSLOTS;
                     const int b0 = (gi - pair * groups_per_pair) * GN;

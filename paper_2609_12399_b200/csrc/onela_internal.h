@@ -84,10 +84,6 @@ struct DecodeArgs {
     // tensor-core kernel: per-head operand scale of S_0 (see Layout), entry of (req_begin, layer, head 0)
     const float* s0_scale;
     long long s0_scale_req_stride;
-    // 1 when the launch that precedes this one on the context was a decode launch as well (of another layer or of
-    // this one): nothing that launch wrote is read here except the caller's tensors, so a programmatic dependent
-    // launch may read the index arrays, S_0 and the older records before it waits for its predecessor
-    int32_t early_ok;
 };
 
 // Grouped value heads (Hv = g * Hk): what the grouped decode kernel needs.

@@ -78,3 +78,55 @@ def test_more_pairs_than_sms_several_segments_per_cta():
     wl = CFG4.scaled(R=5, L=1, H=34, W=60, D=4, prompt_len=32, seed=77)
     worst, _ = _check(wl, "fp32", True)
     assert worst < 1.5e-3
+
+
+def test_layers_back_to_back_in_a_replayed_graph():
+    """Reorder, layer, layer, ... of a grid that leaves most SMs free, replayed as a graph: every launch may start as soon as
+    the one before it has let it, so a layer that did not wait would read the index arrays while they are written.  Two
+    replays on different inputs (other parents, so other arrays: what the first left behind is wrong for the second)."""
+    wl = CFG4.scaled(R=1, L=4, H=4, W=96, D=6, prompt_len=32)
+    cases = [make_case(wl), make_case(wl.scaled(seed=wl.seed + 1))]
+    for case in cases:
+        counts = distinct_counts(case)
+        assert max(c[0] for c in counts.values()) <= 160 and max(c[1] for c in counts.values()) <= 64, counts
+
+    def tensors(case):
+        calls = []
+        for t in range(wl.D):
+            par = torch.zeros((1, wl.W), dtype=torch.int32) if t == 0 else case["parents"][(0, t)][None]
+            lay = [[case["tok"][(0, l, t)][n][None] for n in ("k", "v", "alpha", "beta")] + [case["q"][(0, l, t)][None]] for l in range(wl.L)]
+            calls.append([par] + [x for one in lay for x in one])
+        return [torch.stack([case["S0"][(0, l)] for l in range(wl.L)])[None]] + [x for c in calls for x in c]
+
+    held = [x.contiguous().cuda() for x in tensors(cases[0])]
+    outs = [[torch.empty((1, wl.W, wl.H, wl.dv), device="cuda") for _ in range(wl.L)] for _ in range(wl.D)]
+    ctx = P.Onela(P.make_config(1, wl.L, wl.H, wl.dk, wl.dv, wl.W, wl.D, wl.dtype, "fp32", wl.W * wl.D, P.FLAG_SHARED_CHAINS))
+
+    def generation():
+        ctx.onela_init_shared_states(0, 1, held[0])
+        at = 1
+        for t in range(wl.D):
+            ctx.onela_reorder_beams(0, 1, held[at] if t else None, wl.W)
+            at += 1
+            for l in range(wl.L):
+                ctx.onela_append_decode_step(0, 1, l, *held[at:at + 5], outs[t][l])
+                at += 5
+        ctx.onela_release_request(0)
+
+    generation()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        generation()
+    for case in cases:
+        for dst, src in zip(held, tensors(case)):
+            dst.copy_(src)
+        for per_layer in outs:
+            for o in per_layer:
+                o.fill_(float("nan"))
+        graph.replay()
+        torch.cuda.synchronize()
+        assert ctx.onela_poll_device_status() == (0, 0)
+        ref, _ = run_oracle(case)
+        got = {(0, l, t): outs[t][l][0].cpu() for t in range(wl.D) for l in range(wl.L)}
+        assert check_parity(case, got, ref, label="shared-chains kernel, graph") < 1.5e-3
