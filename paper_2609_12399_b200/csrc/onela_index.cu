@@ -214,15 +214,16 @@ cudaError_t launch_index(const Layout& lay, int32_t req_begin, int32_t req_count
     a.max_steps = max_steps;
     a.want_index = want_index && depth_old >= 1;
     a.bases = bases;
-    // levels per round: two words per 32 beams and level, at most 32 levels (one per lane) and 48 KB - one level's bitmap
-    // always fits up to 190 000 beams
+    // levels per round: two words per 32 beams and level, at most 32 levels (one per lane) and what a launch gets without
+    // asking, 48 KB less the kernel's static shared memory - one level's bitmap fits up to 192 000 beams
+    constexpr size_t ROOM = 47 * 1024;
     const size_t per_level = 2 * sizeof(uint32_t) * (size_t)((max_beam + 31) / 32);
-    int chunk = (int)(48 * 1024 / per_level);
+    int chunk = (int)(ROOM / per_level);
     chunk = chunk < 1 ? 1 : chunk > 32 ? 32 : chunk;
     if (chunk > depth_old) chunk = depth_old > 0 ? depth_old : 1;
     a.chunk = chunk;
     const size_t smem = a.want_index ? per_level * chunk : 0;
-    if (smem > 48 * 1024) {
+    if (smem > ROOM) {
         cudaError_t e = cudaFuncSetAttribute(index_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
