@@ -1102,6 +1102,7 @@ int sm_count_ws() {
 // 1092 / 1089.  All at 3000: 7 x 333 beams as three segments of 11 groups, 228, instead of two of 12, 218.)
 struct PartitionCost {
     int group, seg, more;        // more: the third segment and on
+    bool operator==(const PartitionCost& o) const { return group == o.group && seg == o.seg && more == o.more; }
 };
 PartitionCost partition_cost(int depth) { return {8 + (depth > 1 ? depth - 1 : 0), 6, depth <= 3 ? 12 : 6}; }
 template <class Begin>
@@ -1164,10 +1165,10 @@ cudaError_t launch_ws_t(const DecodeArgs& a, cudaStream_t stream) {
     const int groups_per_pair = (a.W + GN - 1) / GN;
     const int total_groups = a.req_count * a.H * groups_per_pair;
     static thread_local Partition part;          // the last launch's partition, reused while the shape stays
-    static thread_local int part_total = -1, part_gpp = -1, part_h = -1, part_sms = -1, part_group = -1, part_seg = -1, part_ctas = 0;
+    static thread_local int part_total = -1, part_gpp = -1, part_h = -1, part_sms = -1, part_ctas = 0;
+    static thread_local PartitionCost part_cost{};
     const PartitionCost cost = partition_cost(a.depth);
-    if (part_total != total_groups || part_h != a.H || part_gpp != groups_per_pair || part_sms != sms || part_group != cost.group ||
-        part_seg != cost.seg) {
+    if (part_total != total_groups || part_h != a.H || part_gpp != groups_per_pair || part_sms != sms || !(part_cost == cost)) {
         int32_t begin[MAX_CTAS + 1];
         part_ctas = make_partition(total_groups, groups_per_pair, sms, cost, begin);
         for (int i = 0; i < part_ctas; ++i) {
@@ -1176,7 +1177,7 @@ cudaError_t launch_ws_t(const DecodeArgs& a, cudaStream_t stream) {
         }
         part.cta[part_ctas].x = total_groups;
         part_total = total_groups; part_h = a.H; part_gpp = groups_per_pair; part_sms = sms;
-        part_group = cost.group; part_seg = cost.seg;
+        part_cost = cost;
     }
     // Programmatic dependent launch: this launch's CTAs may start, allocate and read S_0 while the previous
     // kernel of the stream drains; the kernel waits for that kernel's completion before it reads anything else.
