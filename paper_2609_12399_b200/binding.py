@@ -12,6 +12,7 @@ from __future__ import annotations
 
 import ctypes
 import importlib.util
+import sysconfig
 from ctypes import POINTER, c_char_p, c_int32, c_int64, c_size_t, c_uint32, c_void_p
 from pathlib import Path
 
@@ -19,7 +20,13 @@ import torch
 
 _PKG = Path(__file__).resolve().parent
 LIB_PATH = _PKG / "libonela.so"
-PYCALL_PATH = _PKG / "_onela_pycall.so"
+
+
+def pycall_path() -> Path:
+    """The native marshalling module inlines torch's and CPython's object layouts, so it fits the two versions it was compiled
+    against and no others: they are part of its file name, and a build for others is not found."""
+    return _PKG / f"_onela_pycall.{sysconfig.get_config_var('SOABI')}.torch-{torch.__version__}.so"
+
 
 OK, E_INVAL, E_CAPACITY, E_ORDER, E_CUDA, E_UNSUPPORTED, E_DEVICE_CHECK, E_TIMEOUT = 0, -1, -2, -3, -4, -5, -6, -7
 DTYPE_F32, DTYPE_BF16 = 0, 1
@@ -109,9 +116,11 @@ def _native_caller(lib, handle, cfg):
     """The native marshalling object of one context (see csrc/onela_pycall.cpp)."""
     global _pycall
     if _pycall is None:
-        if not PYCALL_PATH.exists():
-            raise RuntimeError(f"{PYCALL_PATH} is missing: run `python -m paper_2609_12399_b200.build` (or __graft_entry__.build()) first")
-        spec = importlib.util.spec_from_file_location("_onela_pycall", PYCALL_PATH)
+        path = pycall_path()
+        if not path.exists():
+            raise RuntimeError(f"{path} is missing: run `python -m paper_2609_12399_b200.build` (or __graft_entry__.build()) first, "
+                               "under the torch and Python that load it")
+        spec = importlib.util.spec_from_file_location("_onela_pycall", path)
         _pycall = importlib.util.module_from_spec(spec)
         spec.loader.exec_module(_pycall)
     fns = tuple(ctypes.cast(getattr(lib, n), c_void_p).value for n in _CALLER_FUNCTIONS)

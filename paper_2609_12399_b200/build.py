@@ -40,25 +40,27 @@ def _stale(target: Path, deps) -> bool:
 # The binding's native argument marshalling: a CPython extension on torch's own headers and libraries (already in the
 # process when it is imported), host code only.
 PYCALL_SRC = CSRC / "onela_pycall.cpp"
-PYCALL_LIB = PKG / "_onela_pycall.so"
 
 
 def build_pycall(force: bool = False) -> Path:
-    header = ROOT / "include" / "onela.h"
-    if force or _stale(PYCALL_LIB, [PYCALL_SRC, header]):
+    from paper_2609_12399_b200.binding import pycall_path
+    header, target = ROOT / "include" / "onela.h", pycall_path()
+    if force or _stale(target, [PYCALL_SRC, header]):
         import torch
         from torch.utils import cpp_extension
+        for old in PKG.glob("_onela_pycall*.so"):
+            old.unlink()
         nvcc = Path(_nvcc())
         cuda_inc = nvcc.parent.parent / "include" if nvcc.is_absolute() else Path("/usr/local/cuda/include")
         incs = [ROOT / "include", cuda_inc, sysconfig.get_paths()["include"], *cpp_extension.include_paths()]
         libs = Path(torch.__file__).resolve().parent / "lib"
         cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
-               *(f"-I{i}" for i in incs), str(PYCALL_SRC), "-o", str(PYCALL_LIB), f"-L{libs}", "-lc10", "-lc10_cuda", "-ltorch_cpu",
+               *(f"-I{i}" for i in incs), str(PYCALL_SRC), "-o", str(target), f"-L{libs}", "-lc10", "-lc10_cuda", "-ltorch_cpu",
                "-ltorch_python"]
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError("g++ failed:\n" + " ".join(cmd) + "\n" + r.stdout + r.stderr)
-    return PYCALL_LIB
+    return target
 
 
 # A second library for the tests of the bounded waits: the same sources with a short wait limit and a hook that

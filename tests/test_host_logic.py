@@ -404,3 +404,15 @@ def test_distinct_record_count():
                                 distinct_per_request=[8])
     assert b["algorithmic"] == 2 * 128 * 128 * 4 + 4 * 2 * 512 + 4 * 3 * 4 + 8 * 2 * 520
     assert b["undeduplicated"] == 2 * 128 * 128 * 4 + 4 * 2 * 512 + 4 * 3 * 4 + 12 * 2 * 520
+
+
+def test_native_calls_built_for_another_torch_are_not_loaded(monkeypatch):
+    """The native marshalling inlines torch's object layouts: a build for another version is stale, and is not imported."""
+    import torch
+    built = build.build_pycall()
+    assert built.exists() and not build._stale(built, [build.PYCALL_SRC])
+    monkeypatch.setattr(torch, "__version__", "0.0.0")
+    monkeypatch.setattr(binding, "_pycall", None)
+    assert binding.pycall_path() != built and build._stale(binding.pycall_path(), [build.PYCALL_SRC])
+    with pytest.raises(RuntimeError, match="is missing"):
+        binding._native_caller(binding.load_library(), None, None)
