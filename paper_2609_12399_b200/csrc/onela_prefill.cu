@@ -1,36 +1,44 @@
 // Prompt -> shared state on the tensor cores (sm_100a): S_T of Eq. 1 from the zero state, dk = dv in {32, 64, 128}.
 //
-// What bounded the kernel this one replaces: the recurrence itself.  One CTA per head walked the prompt token by token,
-// 1.1 us each on 32 of 148 SMs (16 384 tokens x 32 heads of 128 x 128 bf16: 17.9 ms).  Here a chunk of C = 64 tokens is
-// one step.  With g_i = prod_{l <= i} alpha_l inside the chunk, A_ij = beta_i (g_i / g_j) (k_i . k_j) for j < i (strictly
-// lower triangular; the ratios are running products, nothing is divided) and T = (I + A)^-1, Eq. 1 over the chunk is
-//      S_out = g_C S_in + Delta Y ,   Delta = V^T diag(beta) - S_in K^T diag(beta g) ,   Y = T^T diag(g_C / g) K
-// (the WY form of a product of Householder-like factors; Delta is dv x C, Y is C x dk).  T, Y and the coefficients depend
-// on the keys and gates alone, so they are prepared a chunk ahead of the state.
+// Token by token (one CTA per head, the recurrence in fp32) a prompt costs 1.1 us per token on as many SMs as there are
+// heads.  Here a chunk of C = 64 tokens is one step, in the chunked form of the delta rule (the WY representation of a product
+// of Householder-like factors, Bischof and Van Loan 1987; with gates, Gated DeltaNet, Yang et al. 2024).  With g_i =
+// prod_{l <= i} alpha_l inside the chunk, A_ij = beta_i (g_i / g_j) (k_i . k_j) for j < i (strictly lower triangular; the
+// ratios are running products, nothing is divided) and T = (I + A)^-1, Eq. 1 over the chunk is
+//      S_out = g_C S_in + Delta K ,   Delta = U - S_in W^T ,
+//      U^T = diag(g_C / g) T diag(beta) V (C x dv) ,   W = diag(g_C / g) T diag(beta g) K (C x dk) .
+// T, U and W depend on the tokens alone, so they are prepared a chunk ahead of the state.  (The other grouping, T applied to
+// the keys behind Delta, costs the state the rounding of that product; here what the newest tokens contribute - the greater
+// part of the state at the usual gates - is U, in fp32, times the keys as they were given.)
 //
 // Parallelism along the prompt.  The map of a run of chunks is affine, S -> S M + B, and M obeys the same recurrence as
-// S (from the identity, with V = 0).  A head's prompt is cut into segments, one per CTA of a cluster; every segment but
+// S (from the identity, with U = 0).  A head's prompt is cut into segments, one per CTA of a cluster; every segment but
 // the first carries M as dk more state rows, and at the end the cluster folds the segments in order, S <- S M_p + B_p,
 // handing S from CTA to CTA through distributed shared memory.  Nothing goes through global memory but the inputs and
 // the result.
 //
-// One CTA: two TEAMS of 128 threads that prepare chunks in turn (keys -> operand tile, Gram product, inverse, Y) and 128
+// One CTA: two TEAMS of 128 threads that prepare chunks in turn (keys -> operand tile, Gram product, inverse, W, U) and 128
 // threads per CHAIN of 128 state rows (dk = 128: S and M are a chain each, and hide each other's latency; dk <= 64: one
-// chain holds both), coupled by mbarriers over a ring of key / value tiles and one of Y tiles.  A thread keeps one state row
-// in fp32 registers.  Products run as tcgen05.mma kind::f16 with fp32 accumulation, an operand being one fp16 number where
-// that is exact (bf16 keys, to 2^-28 of the row's largest) and otherwise the sum of two (22 to 23 significant bits); every
-// operand row carries its own power of two, exact to apply and to undo, so the range of the caller's data does not matter.
-// The tensor core's accumulator truncates, so the small products are accumulated first: with the large ones first the state
-// came out 3x less exact.  Relative error against fp64: 1.5e-7 at the usual gates, 2.9e-7 without decay (token by token in
-// fp32: 1.0e-7 and 3.5e-7).
-//   per chunk and chain:  [S_hi ; S_lo] K^T   2 x dk / 16 MMAs (M = 128, N = 64), A in tensor memory
-//                         Delta Y             3 x 4 MMAs (N = dk), A in tensor memory
-//   per chunk:            K K^T (dk / 16 MMAs), K^T T' (2 x 4 MMAs, A = the key tile read MN-major)
-// (fp32 records: keys in two parts as well, 3 products each.)
-// What bounds it now: the latency of a chain's step, about 10 000 cycles per chunk (28 MMAs at ~80 cycles, four conversions
-// between tensor memory, registers and tensor memory), beside two preparations in flight that take as long together; issue
-// slots are a third used, the tensor pipe a fifth.  16 384 tokens x 32 heads of 128 x 128 bf16: 18.2 ms -> 0.38 ms;
-// 1021 tokens x 16 heads of 64 x 64 fp32: 376 -> 32 us.
+// chain holds both), coupled by mbarriers over rings of key, W and U tiles.  A thread keeps one state row in fp32 registers.
+// Products run as tcgen05.mma kind::f16 with fp32 accumulation, an operand being one fp16 number where that is exact (bf16
+// keys, to 2^-28 of the row's largest), otherwise the sum of two (22 to 23 significant bits) or, fp32 records, three where
+// that shows (Delta of the S rows, the keys at dk <= 64); U's operands are bf16, the values as they are or in three parts, T
+// diag(beta) in three.  Every fp16 row carries its own power of two, exact to apply and to undo, so the range of the caller's
+// data does not matter.
+//
+// Precision.  The tensor core's accumulator truncates towards zero at every MMA.  So the small products are accumulated
+// first, and half a unit of the last place per step that counts (KEEP, below) is given back with an operand's low part.  The
+// running products of the gates carry their rounding errors along (two more FMAs each), which was the largest single error of
+// the preparation.  Relative error against 64 bits, 24 to 16 384 tokens, gates in [0.9, 1]: 0.7 - 0.9e-7; token by token in
+// fp32 0.83 - 0.98e-7 (1.25 - 1.81e-7 in the other grouping, uncompensated).  Without decay 0.7 - 2.0e-7 against 1.0 -
+// 3.6e-7; gates spread over [0, 1] 0.5 - 0.75e-7 against 0.5 - 0.6e-7.
+//   per chunk and chain:  S W^T               3 x dk / 16 MMAs (M = 128, N = 64), A in tensor memory
+//                         Delta K             2 x 4 MMAs (N = dk), A in tensor memory
+//   per chunk:            K K^T (dk / 16 MMAs), K^T T'^T (2 x 4), V^T (T diag(beta))^T (3 x 4), A = the tile read MN-major
+// (fp32 records: Delta K 5 or 6 products, the lowest part of Delta in shared memory; K K^T three, K^T T'^T three, U six.)
+// What bounds it now: the latency of a chain's step and, as long, the two preparations in flight, about 11 000 cycles per
+// chunk.  16 384 tokens x 32 heads of 128 x 128 bf16: 18.2 ms token by token, 0.44 ms (0.38 ms in the other grouping, whose
+// errors were larger); 1021 tokens x 16 heads of 64 x 64 fp32: 376 -> 39 us (35).
 //
 // Every wait is bounded: a thread that gives up keeps meeting its team's barriers, whose OR makes the team leave
 // together, and the cluster barriers; ONELA_E_TIMEOUT goes to the status word.
@@ -61,13 +69,17 @@ using sm100::umma_desc;
 
 constexpr int C = 64;              // tokens per chunk
 constexpr int TILE = C * 128;      // bytes of one K-major operand block: 64 rows of 64 fp16
-constexpr int KV_STAGES = 3, Y_STAGES = 2;
+constexpr int K_STAGES = 3;
 constexpr int CTA_BARRIER = 9;     // named barrier of the whole CTA (1 - 4: the teams')
 constexpr int AP = C + 4;          // pitch (floats) of the C x C matrix: 16-byte rows
 constexpr int MAX_SEGMENTS = 8;    // portable cluster size
-// Largest elements of the scaled operand rows: keys and T' in [2^3, 2^4) (so |Y| < 64 * 2^8 = 2^14 stays inside fp16's
+// Largest elements of the scaled operand rows: keys and T' in [2^3, 2^4) (so |W| < 64 * 2^8 = 2^14 stays inside fp16's
 // range unscaled), state rows and Delta rows in [2^12, 2^13).
 constexpr int NARROW = 3, WIDE = 12;
+// What the accumulators' truncation takes on average, given back by the operand that goes into the next product: an MMA drops
+// half a unit of the last place of a partial sum, 0.72 x 2^-24 of it, and of the partial sums of a product's last steps (the
+// large terms) the final one and a part of those before it count.  Delta: U's and its own product's; W: its own and S W^T's.
+constexpr float KEEP_DELTA = 1.5f * 0x1p-24f, KEEP_W = 2.f * 0x1p-24f;
 
 struct PrefillArgs {
     const void *k, *v;
@@ -83,27 +95,30 @@ struct PrefillArgs {
 template <int D, typename T>
 struct Shape {
     static constexpr int KB = D > 64 ? D / 64 : 1;                  // K blocks of 64 elements
-    static constexpr int PK = sizeof(T) == 4 ? 2 : 1;               // fp16 parts of a key
+    static constexpr int PK = sizeof(T) == 2 ? 1 : D == 128 ? 2 : 3;      // fp16 parts of a key
+    static constexpr int DP = PK == 1 ? 2 : 3;                       // ... of the S rows' Delta
     static constexpr int PREPS = 2, CHAINS = D == 128 ? 2 : 1;      // teams of 128 threads
     static constexpr int THREADS = 128 * (PREPS + CHAINS);
-    static constexpr bool V_STAGED = sizeof(T) == 2;                // (fp32 values are read where they are: no room beside the keys)
     static constexpr int K_BYTES = PK * KB * TILE;
-    static constexpr int KV_BYTES = K_BYTES + (V_STAGED ? C * D * (int)sizeof(T) : 0);
-    static constexpr int Y_BYTES = 2 * D * 128;                      // [hi, lo][dk rows][128 bytes]
-    static constexpr int RING = KV_STAGES * KV_BYTES + Y_STAGES * Y_BYTES;
-    // per preparing team: the C x C matrix, over it T' as an operand tile (hi, lo), and the scratch of its inversion
+    static constexpr int W_BYTES = D * 256 > 2 * TILE ? D * 256 : 2 * TILE;    // [hi, lo][dk rows][128 bytes]; before that T' (hi, lo)
+    static constexpr int U_BYTES = C * D * 4 > 3 * TILE ? C * D * 4 : 3 * TILE;       // [token][dv]; before that T diag(beta) in three parts
+    static constexpr int L_BYTES = DP == 3 ? 128 * 128 : 0;          // lowest part of the Delta operand
+    // (fp32 at dk = 128: a tile of each is what there is room for; the preparation waits for the chain once per chunk more)
+    static constexpr int W_STAGES = D == 128 && PK == 2 ? 1 : 2, U_STAGES = W_STAGES;
+    static constexpr int RING = K_STAGES * K_BYTES + W_STAGES * W_BYTES + U_STAGES * U_BYTES + L_BYTES;
+    // per preparing team: the C x C matrix, over it the values as an operand tile, and the scratch of the inversion
     static constexpr int A_BYTES = (C * AP * 4 + 1023) / 1024 * 1024, X_BYTES = 5 * 1024;
-    static constexpr int TOK_BYTES = 4 * C * 4;                      // per token: alpha, 1 / key scale, weight in T', scratch
-    static constexpr int COEF_BYTES = 1024;                          // per Y stage: b[C], c[C], g_C
+    static constexpr int TOK_BYTES = 5 * C * 4;                      // per token: alpha, beta, 1 / key scale, row and column weights in T'
+    static constexpr int COEF_BYTES = 1024;                          // per U stage: weight of U[C], what undoes W's scale[C], g_C
     // (the Gram product reads 128 rows from a 64-row block and the MN-major tile a second block: what lies behind the key
     // tile is read and the rows that come of it are ignored)
-    static constexpr int SMALL = PREPS * TOK_BYTES + Y_STAGES * COEF_BYTES + 128 * 4 + 256;
+    static constexpr int SMALL = PREPS * TOK_BYTES + U_STAGES * COEF_BYTES + 128 * 4 + 256;
     static constexpr int SMEM = RING + PREPS * (A_BYTES + X_BYTES) + SMALL + 1024;
-    static constexpr uint32_t CHAIN_COLS = D + C;                    // S operand (hi, lo) / Delta Y ; S K^T / Delta operand
-    static constexpr uint32_t PREP_COL = CHAINS * CHAIN_COLS;        // per preparing team: Gram product, then Y
+    static constexpr uint32_t CHAIN_COLS = D + C;                    // S operand (hi, lo) / Delta K ; S W^T / Delta operand (hi, lo)
+    static constexpr uint32_t PREP_COL = CHAINS * CHAIN_COLS;        // per preparing team: Gram product, then W, then U
     static constexpr uint32_t TMEM_COLS = D == 128 ? 512 : 256;
     static_assert(PREP_COL + PREPS * C <= TMEM_COLS && SMEM <= 232448 && RING >= D * 128 * 4 + 2 * KB * D * 128, "tensor and shared memory");
-    static_assert(32 * 36 * 4 <= X_BYTES && 2 * TILE <= A_BYTES, "scratch");
+    static_assert(32 * 36 * 4 <= X_BYTES && (A_BYTES + X_BYTES) % 1024 == 0 && 2 * TILE <= A_BYTES, "scratch; a tile's swizzle atoms");
     // registers: 512 threads start with 128 each; the state rows (dk floats per thread) take what the preparation leaves
     static constexpr bool SPLIT_REGS = D == 128;
     static constexpr int PREP_REGS = 80, CHAIN_REGS = 176;
@@ -117,6 +132,7 @@ __device__ __forceinline__ uint64_t umma_desc_mn(uint32_t smem_addr, uint32_t bl
            ((uint64_t)2 << 61);
 }
 constexpr uint32_t A_MN_MAJOR = 1u << 15, B_MN_MAJOR = 1u << 16;     // instruction descriptor: operand is MN-major
+constexpr uint32_t BF16_OPERANDS = (1u << 7) | (1u << 10);           // ... both are bf16
 
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -127,23 +143,49 @@ __device__ __forceinline__ void arrive(uint32_t bar) { asm volatile("mbarrier.ar
 __device__ __forceinline__ void cluster_sync() {
     asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
-// Two numbers times a power of two as fp16 numbers hi + lo, packed.  (Rounding hi to a fixed grid instead would make sums
-// of hi x hi products exact, but leaves every lo as large as the row's largest element allows: 4x the error.)
+// Two numbers times a power of two as fp16 numbers hi + lo (+ low), packed.  (Rounding hi to a fixed grid instead would make
+// sums of hi x hi products exact, but leaves every lo as large as the row's largest element allows.)
 __device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t& lo) {
     hi = pack_f16x2(a, b);
     const float2 h = __half22float2(*reinterpret_cast<const __half2*>(&hi));
     lo = pack_f16x2(a - h.x, b - h.y);
 }
-__device__ __forceinline__ void split16(const float* x, float scale, uint32_t* hi, uint32_t* lo) {
-    const float2 sc = make_float2(scale, scale);
+__device__ __forceinline__ void split3(float a, float b, uint32_t& hi, uint32_t& lo, uint32_t& low) {
+    hi = pack_f16x2(a, b);
+    const float2 h = __half22float2(*reinterpret_cast<const __half2*>(&hi));
+    const float ra = a - h.x, rb = b - h.y;
+    lo = pack_f16x2(ra, rb);
+    const float2 l = __half22float2(*reinterpret_cast<const __half2*>(&lo));
+    low = pack_f16x2(ra - l.x, rb - l.y);
+}
+// Sixteen numbers times `scale` in two parts or (low not null) three; `keep`: what the low part gives on top (see KEEP_DELTA).
+__device__ __forceinline__ void split16(const float* x, float scale, uint32_t* hi, uint32_t* lo, float keep = 0.f, uint32_t* low = nullptr) {
+    const float2 sc = make_float2(scale, scale), kp = make_float2(keep, keep);
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
         const float2 y = __fmul2_rn(make_float2(x[2 * e], x[2 * e + 1]), sc);
         hi[e] = pack_f16x2(y.x, y.y);
         const float2 h = __half22float2(*reinterpret_cast<const __half2*>(&hi[e]));
-        const float2 l = __fadd2_rn(y, make_float2(-h.x, -h.y));
+        float2 l = __fadd2_rn(y, make_float2(-h.x, -h.y));
+        if (keep != 0.f) l = __ffma2_rn(y, kp, l);
         lo[e] = pack_f16x2(l.x, l.y);
+        if (low) {
+            const float2 q = __half22float2(*reinterpret_cast<const __half2*>(&lo[e]));
+            const float2 r = __fadd2_rn(l, make_float2(-q.x, -q.y));
+            low[e] = pack_f16x2(r.x, r.y);
+        }
     }
+}
+// Two fp32 numbers as the sum of three bf16 ones each, packed: eight bits at a time, exact.  (The first is cut off, so that the
+// largest numbers stay finite, the second rounded, so that the third has either sign and products left out have no bias.)
+__device__ __forceinline__ void split_bf16(float a, float b, uint32_t (&part)[3]) {
+    const uint32_t ua = __float_as_uint(a), ub = __float_as_uint(b);
+    part[0] = __byte_perm(ua, ub, 0x7632);
+    const float ra = a - __uint_as_float(ua & 0xffff0000u), rb = b - __uint_as_float(ub & 0xffff0000u);
+    part[1] = sm100::pack_bf16x2(ra, rb);
+    float ma, mb;
+    unpack_bf16x2(part[1], ma, mb);
+    part[2] = sm100::pack_bf16x2(ra - ma, rb - mb);
 }
 // ... as one K step of a tensor-memory A operand: columns [0, 8) hi, [8, 16) lo
 __device__ __forceinline__ void split_to_tmem(uint32_t taddr, const float* x, float scale) {
@@ -173,18 +215,25 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
     constexpr int KB = Z::KB, PK = Z::PK, KS = (D < 64 ? D : 64) / 16;        // K steps of 16 per block of 64
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-    uint8_t* y_ring = smem + KV_STAGES * Z::KV_BYTES;
-    uint8_t* prep_s = smem + Z::RING;                                         // per preparing team: matrix / T', scratch
+    uint8_t* w_ring = smem + K_STAGES * Z::K_BYTES;
+    float* u_ring = reinterpret_cast<float*>(w_ring + Z::W_STAGES * Z::W_BYTES);
+    uint8_t* low_s = reinterpret_cast<uint8_t*>(u_ring) + Z::U_STAGES * Z::U_BYTES;      // the Delta operand's lowest part
+    uint8_t* prep_s = smem + Z::RING;                                         // per preparing team: matrix / values, scratch
     float* tok_s = reinterpret_cast<float*>(prep_s + Z::PREPS * (Z::A_BYTES + Z::X_BYTES));
     float* coef_s = tok_s + Z::PREPS * (Z::TOK_BYTES / 4);
-    float* hinv_s = coef_s + Y_STAGES * (Z::COEF_BYTES / 4);                  // [128] what undoes the scales of the rows handed on
+    float* hinv_s = coef_s + Z::U_STAGES * (Z::COEF_BYTES / 4);               // [128] what undoes the scales of the rows handed on
     uint64_t* bars = reinterpret_cast<uint64_t*>(hinv_s + 128);
-    auto bar_full = [&](int s) { return smem_u32(bars + s); };                // Y stage s prepared
-    auto bar_yfree = [&](int s) { return smem_u32(bars + 2 + s); };           // Y stage / key and value stage read out
-    auto bar_kvfree = [&](int s) { return smem_u32(bars + 4 + s); };
-    auto bar_prep = [&](int w) { return smem_u32(bars + 7 + w); };            // a preparing team's MMAs complete
-    auto bar_chain = [&](int c) { return smem_u32(bars + 9 + c); };           // a chain's
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 12);
+    // W and U: the barriers of even and odd chunks, however many tiles there are (a wait by parity does not tell a chunk's turn
+    // from the one after next, and a team that comes late may find both past)
+    auto bar_w = [&](int i) { return smem_u32(bars + (i & 1)); };             // W prepared
+    auto bar_u = [&](int i) { return smem_u32(bars + 2 + (i & 1)); };         // U (and its coefficients)
+    auto bar_wfree = [&](int i) { return smem_u32(bars + 4 + (i & 1)); };     // W, U read out
+    auto bar_ufree = [&](int i) { return smem_u32(bars + 6 + (i & 1)); };
+    auto bar_kfree = [&](int s) { return smem_u32(bars + 8 + s); };           // key stage s read out
+    auto bar_prep = [&](int w) { return smem_u32(bars + 11 + w); };           // a preparing team's MMAs complete
+    auto bar_chain = [&](int c) { return smem_u32(bars + 13 + c); };          // a chain's
+    auto turn = [](int i) { return (uint32_t)(i >> 1) & 1; };                 // chunk i's parity on its pair of barriers
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 15);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
@@ -196,11 +245,13 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
 
     if (tid == 0) {
         const int chains = D == 128 && has_m ? 2 : 1;
-        for (int s = 0; s < Y_STAGES; ++s) {
-            mbar_init(bar_full(s), 128);                                      // the preparing threads
-            mbar_init(bar_yfree(s), chains);                                  // the chains' commits
+        for (int s = 0; s < 2; ++s) {
+            mbar_init(bar_w(s), 128);                                         // the preparing threads
+            mbar_init(bar_u(s), 128);
+            mbar_init(bar_wfree(s), chains);                                  // the chains' commits
+            mbar_init(bar_ufree(s), chains);                                  // ... their leaders
         }
-        for (int s = 0; s < KV_STAGES; ++s) mbar_init(bar_kvfree(s), chains);
+        for (int s = 0; s < K_STAGES; ++s) mbar_init(bar_kfree(s), chains);
         for (int w = 0; w < Z::PREPS; ++w) mbar_init(bar_prep(w), 1);
         for (int c = 0; c < Z::CHAINS; ++c) mbar_init(bar_chain(c), 1);
         *abort_flag = 0;
@@ -231,11 +282,12 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
         // (two teams take the chunks in turn: each step of a chunk is bounded by the latency of its own dependent chain)
         if constexpr (Z::SPLIT_REGS) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(Z::PREP_REGS));
         const int team = warp >> 2, w4 = warp & 3, pt = tid & 127;
-        float* A_s = reinterpret_cast<float*>(prep_s + team * (Z::A_BYTES + Z::X_BYTES));       // [C][AP], later T'
-        uint8_t* T_s = reinterpret_cast<uint8_t*>(A_s);
-        float* X_s = reinterpret_cast<float*>(T_s + Z::A_BYTES);                                // [32][36]
+        float* A_s = reinterpret_cast<float*>(prep_s + team * (Z::A_BYTES + Z::X_BYTES));       // [C][AP], later the values
+        uint8_t* V_s = reinterpret_cast<uint8_t*>(A_s);
+        float* X_s = A_s + Z::A_BYTES / 4;                                                      // [32][36]
         float* alpha_s = tok_s + team * (Z::TOK_BYTES / 4);
-        float *kinv_s = alpha_s + C, *w_s = kinv_s + C, *max_s = w_s + C;
+        float *beta_s = alpha_s + C, *kinv_s = beta_s + C, *row_s = kinv_s + C, *col_s = row_s + C;
+        constexpr int VR = sizeof(T) == 2 ? 1 : 3;                            // bf16 parts of a value
         const uint32_t acc_at = tmem_base + Z::PREP_COL + team * C;
         constexpr int VEC = Vec16<T>::N, CPR = D / VEC, LR = CPR < 8 ? CPR : 8;      // 16-byte chunks and lanes per key row
         constexpr int ROWS = 128 / LR, PASSES = C / ROWS, NC = CPR / LR;
@@ -251,19 +303,14 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
         }
         uint32_t phase = 0;
         for (int i = team; i < n; i += Z::PREPS) {
-            const int s = i % Y_STAGES, use = i / Y_STAGES, kvs = i % KV_STAGES, t0 = (c_begin + i) * C;
-            uint8_t *K_s = smem + kvs * Z::KV_BYTES, *Y_s = y_ring + s * Z::Y_BYTES;
-            float* co = coef_s + s * (Z::COEF_BYTES / 4);
-            if (i >= KV_STAGES) wait(bar_kvfree(kvs), (i / KV_STAGES - 1) & 1);
-            // values as they are ([token][dv]); tokens beyond the prompt are zeros with alpha = 1, beta = 0: they change nothing
-            if constexpr (Z::V_STAGED) for (int x = pt; x < C * CPR; x += 128) {
-                const int row = x / CPR, ch = x % CPR, t = t0 + row;
-                const uint32_t bytes = t < a.n_tokens ? 16u : 0u;
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(K_s + Z::K_BYTES + row * (D * (int)sizeof(T)) + ch * 16)),
-                             "l"(vp + min(t, a.n_tokens - 1) * row_stride + ch * VEC), "r"(bytes)
-                             : "memory");
-            }
-            // keys as the K-major operand tile, every row with its own power of two
+            const int ks_n = i % K_STAGES, ws = i % Z::W_STAGES, us = i % Z::U_STAGES, t0 = (c_begin + i) * C;
+            uint8_t *K_s = smem + ks_n * Z::K_BYTES, *W_s = w_ring + ws * Z::W_BYTES;
+            float *U_s = u_ring + us * (Z::U_BYTES / 4), *co = coef_s + us * (Z::COEF_BYTES / 4);
+            uint8_t* T_s = reinterpret_cast<uint8_t*>(U_s);                  // T diag(beta), later U
+            if (i >= K_STAGES) wait(bar_kfree(ks_n), (i / K_STAGES - 1) & 1);
+            // keys as the K-major operand tile, every row with its own power of two; tokens beyond the prompt are zeros with
+            // alpha = 1, beta = 0: they change nothing.  (First loads on their way since the chunk before, the state's update on
+            // packed pairs: dk = 128 bf16 438 -> 485 us at 16 384 tokens, by spills.)
             const int lr = pt % LR, row0 = pt / LR;
 #pragma unroll
             for (int p0 = 0; p0 < PASSES; p0 += BATCH) {
@@ -297,12 +344,13 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
                             *reinterpret_cast<uint4*>(dst) = make_uint4(pack_f16x2(y[0] * sc, y[1] * sc), pack_f16x2(y[2] * sc, y[3] * sc),
                                                                         pack_f16x2(y[4] * sc, y[5] * sc), pack_f16x2(y[6] * sc, y[7] * sc));
                         } else {
-                            uint32_t hi[2], lo[2];
+                            uint32_t hi[2], lo[2], low[2];
 #pragma unroll
                             for (int e = 0; e < 2; ++e)
-                                split2(y[2 * e] * sc, y[2 * e + 1] * sc, hi[e], lo[e]);
+                                split3(y[2 * e] * sc, y[2 * e + 1] * sc, hi[e], lo[e], low[e]);
                             *reinterpret_cast<uint2*>(dst) = make_uint2(hi[0], hi[1]);
                             *reinterpret_cast<uint2*>(dst + KB * TILE) = make_uint2(lo[0], lo[1]);
+                            if constexpr (PK == 3) *reinterpret_cast<uint2*>(dst + 2 * KB * TILE) = make_uint2(low[0], low[1]);
                         }
                     }
                 }
@@ -310,6 +358,7 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
             const float alpha = alpha_next, beta = beta_next;
             if (pt < C) {
                 alpha_s[pt] = alpha;
+                beta_s[pt] = beta;
                 if (i + Z::PREPS < n) {
                     alpha_next = gate_of(a.alpha, t0 + Z::PREPS * C + pt, 1.f);
                     beta_next = gate_of(a.beta, t0 + Z::PREPS * C + pt, 0.f);
@@ -322,14 +371,14 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
                 tc_fence_after();
                 const uint64_t kd = umma_desc(smem_u32(K_s));
 #pragma unroll 1
-                for (int t = PK == 2 ? 2 : 0; t >= 0; --t)                  // small terms first: (lo hi, hi lo,) hi hi
+                for (int t = PK > 1 ? 2 : 0; t >= 0; --t)                   // small terms first: (lo hi, hi lo,) hi hi
 #pragma unroll 1
                     for (int kb = 0; kb < KB; ++kb)
 #pragma unroll
                         for (int ks = 0; ks < KS; ++ks) {
                             const int at = (kb * TILE + ks * 32) >> 4;
                             mma_ss(acc_at, kd + (at + (t == 2 ? (KB * TILE) >> 4 : 0)), kd + (at + (t == 1 ? (KB * TILE) >> 4 : 0)), idesc_f16(C),
-                                   t != (PK == 2 ? 2 : 0) || kb || ks);
+                                   t != (PK > 1 ? 2 : 0) || kb || ks);
                         }
                 mma_commit(bar_prep(team));
             }
@@ -344,21 +393,26 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
             wait(bar_prep(team), phase);
             phase ^= 1;
             tc_fence_after();
-            // A = beta_i (g_i / g_j) (k_i . k_j), row i by thread i; the gate products run from the right.  g = alpha_0 ...
-            // alpha_i; the other half of the threads takes the products of the gates behind the token.
-            float g = 1.f;
+            // A = beta_i (g_i / g_j) (k_i . k_j), row i by thread i; the gate products run from the right, each as a sum of two
+            // numbers (the product and what its roundings have left out).  g = alpha_0 ... alpha_i; the other half of the
+            // threads takes the products of the gates behind the token.
+            float g = 1.f, g_rest = 0.f;
+            auto times = [&](float x) {
+                const float p = g * x;
+                g_rest = fmaf(g_rest, x, fmaf(g, x, -p));
+                g = p;
+            };
             if (w4 >= 2) {
-                float gc = 1.f;
 #pragma unroll 2
                 for (int l = C - 4; l >= 0; l -= 4) {
                     const float4 al = *reinterpret_cast<const float4*>(alpha_s + l);
                     const int me = pt - C;
-                    if (l + 3 > me) gc *= al.w;
-                    if (l + 2 > me) gc *= al.z;
-                    if (l + 1 > me) gc *= al.y;
-                    if (l > me) gc *= al.x;
+                    times(l + 3 > me ? al.w : 1.f);
+                    times(l + 2 > me ? al.z : 1.f);
+                    times(l + 1 > me ? al.y : 1.f);
+                    times(l > me ? al.x : 1.f);
                 }
-                w_s[pt - C] = gc * kinv_s[pt - C];
+                row_s[pt - C] = (g + g_rest) * kinv_s[pt - C];
             } else {
                 const float coef = beta * kinv_s[pt];
 #pragma unroll 1
@@ -374,12 +428,13 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
 #pragma unroll
                         for (int f = 3; f >= 0; --f) {
                             const int l = cb * 16 + e + f;
-                            row[f] = l < pt ? (coef * g) * (__uint_as_float(v[e + f]) * kiv[f]) : 0.f;
-                            g *= l <= pt ? alv[f] : 1.f;
+                            row[f] = l < pt ? (coef * (g + g_rest)) * (__uint_as_float(v[e + f]) * kiv[f]) : 0.f;
+                            times(l <= pt ? alv[f] : 1.f);
                         }
                         *reinterpret_cast<float4*>(A_s + pt * AP + cb * 16 + e) = make_float4(row[0], row[1], row[2], row[3]);
                     }
                 }
+                col_s[pt] = (g + g_rest) * kinv_s[pt];
                 __syncwarp();
                 // T = (I + A)^-1 in place, from the diagonal out.  Blocks of 16, two per warp, one column per lane by forward
                 // substitution; then a warp's two blocks are joined, then the two warps': - T22 A21 T11 below the diagonal.
@@ -427,80 +482,175 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
                 for (int r = 0; r < 8; ++r) A_s[(32 + 8 * w4 + r) * AP + lane] = -acc[r];
             }
             bar_or(1 + team, 128, 0);
-            if (i >= Y_STAGES) wait(bar_yfree(s), (use - 1) & 1);            // coefficients and Y go to the chunk's Y stage
-            // T'_ij = T_ji g_C / g_j (and the key's scale undone): row i by threads i and i + 64, as an operand tile (hi, lo)
+            // T' = diag(g_C / g) T diag(beta g), the keys' scales undone on both sides, as an operand tile (fp16 hi, lo) where W
+            // will be, and T diag(beta) as one (bf16, three parts) where U will be.  Row pt / 2 by threads pt and pt + 1, columns
+            // 16 h .. and 32 + 16 h .. (conflict-free reads)
+            if (i >= Z::W_STAGES) wait(bar_wfree(i - Z::W_STAGES), turn(i - Z::W_STAGES));
+            if (i >= Z::U_STAGES) wait(bar_ufree(i - Z::U_STAGES), turn(i - Z::U_STAGES));
             {
-                const int ti = pt & 63, hf = pt >> 6;
-                const bool zero = hf == 0 && ti >= 32;
+                const int ti = pt >> 1, hf = pt & 1;
+                const float weight = row_s[ti];
                 float t[32], m = 0.f;
 #pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    t[j] = zero ? 0.f : A_s[(32 * hf + j) * AP + ti] * w_s[32 * hf + j];
-                    m = fmaxf(m, fabsf(t[j]));
+                for (int q = 0; q < 8; ++q) {
+                    const int at = 16 * hf + (q >> 2) * 32 + (q & 3) * 4;
+                    const float4 x = *reinterpret_cast<const float4*>(A_s + ti * AP + at), be = *reinterpret_cast<const float4*>(beta_s + at);
+                    const float4 c4 = *reinterpret_cast<const float4*>(col_s + at);
+                    t[4 * q] = x.x * be.x;
+                    t[4 * q + 1] = x.y * be.y;
+                    t[4 * q + 2] = x.z * be.z;
+                    t[4 * q + 3] = x.w * be.w;
+                    m = fmaxf(fmaxf(m, fabsf((t[4 * q] * c4.x) * weight)), fabsf((t[4 * q + 1] * c4.y) * weight));
+                    m = fmaxf(fmaxf(m, fabsf((t[4 * q + 2] * c4.z) * weight)), fabsf((t[4 * q + 3] * c4.w) * weight));
                 }
-                if (hf == 1) max_s[ti] = m;
-                bar_or(1 + team, 128, 0);
-                if (hf == 0) {
-                    m = fmaxf(m, max_s[ti]);
-                    float sc, inv;
-                    pow2_scale(m, NARROW, sc, inv);
-                    co[ti] = beta * inv;
-                    co[C + ti] = beta * g * kinv_s[ti] * inv;
-                    if (ti == C - 1) co[2 * C] = g;
-                    max_s[ti] = sc;
-                }
-                bar_or(1 + team, 128, 0);
-                const float sc = max_s[ti];
+                m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
+                float sc, inv;
+                pow2_scale(m, NARROW, sc, inv);
 #pragma unroll
-                for (int c = 0; c < 4; c += 2) {
-                    uint32_t hi[8], lo[8];
-                    split16(t + 8 * c, sc, hi, lo);
+                for (int c = 0; c < 4; ++c) {                               // chunks of eight columns
+                    const int ch = 4 * (c >> 1) + 2 * hf + (c & 1), at = ti * 128 + ((ch ^ (ti & 7)) << 4);
+                    uint32_t hi[4], lo[4], part[4][3];
 #pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        uint8_t* dst = T_s + ti * 128 + (((4 * hf + c + e) ^ (ti & 7)) << 4);
-                        *reinterpret_cast<uint4*>(dst) = make_uint4(hi[4 * e], hi[4 * e + 1], hi[4 * e + 2], hi[4 * e + 3]);
-                        *reinterpret_cast<uint4*>(dst + TILE) = make_uint4(lo[4 * e], lo[4 * e + 1], lo[4 * e + 2], lo[4 * e + 3]);
+                    for (int e = 0; e < 4; ++e) {
+                        const float a0 = t[8 * c + 2 * e], a1 = t[8 * c + 2 * e + 1];
+                        const float2 c2 = *reinterpret_cast<const float2*>(col_s + 8 * ch + 2 * e);
+                        split_bf16(a0, a1, part[e]);
+                        split2(((a0 * c2.x) * weight) * sc, ((a1 * c2.y) * weight) * sc, hi[e], lo[e]);
                     }
+                    *reinterpret_cast<uint4*>(W_s + at) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+                    *reinterpret_cast<uint4*>(W_s + TILE + at) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+#pragma unroll
+                    for (int p = 0; p < 3; ++p) *reinterpret_cast<uint4*>(T_s + p * TILE + at) = make_uint4(part[0][p], part[1][p], part[2][p], part[3][p]);
                 }
+                if (hf == 0) {
+                    co[ti] = weight;
+                    co[C + ti] = inv;
+                }
+                if (pt == C - 1) co[2 * C] = g + g_rest;
             }
             proxy_fence();
             bar_or(1 + team, 128, 0);
-            if (w4 == 0) {          // Y^T = K^T T'^T: lanes = dk, columns = tokens
+            if (w4 == 0) {          // W^T = K^T T'^T: lanes = dk, columns = tokens
                 tc_fence_after();
-                const uint64_t kd = umma_desc_mn(smem_u32(K_s), TILE), td = umma_desc(smem_u32(T_s));
+                const uint64_t kd = umma_desc_mn(smem_u32(K_s), TILE), td = umma_desc(smem_u32(W_s));
+                constexpr int FIRST = PK > 1 ? 2 : 1;
 #pragma unroll 1
-                for (int t = PK; t >= 0; --t)                               // small terms first: (lo hi,) hi lo, hi hi
+                for (int t = FIRST; t >= 0; --t)                            // small terms first: (lo hi,) hi lo, hi hi
 #pragma unroll
                     for (int ks = 0; ks < C / 16; ++ks)
                         mma_ss(acc_at, kd + (t == 2 ? (KB * TILE) >> 4 : 0) + ((ks * 2048) >> 4), td + (t == 1 ? TILE >> 4 : 0) + ((ks * 32) >> 4),
-                               idesc_f16(C) | A_MN_MAJOR, t != PK || ks);
+                               idesc_f16(C) | A_MN_MAJOR, t != FIRST || ks);
                 mma_commit(bar_prep(team));
+            }
+            // the values ([token][dv]), part `round` of them, as an operand tile over the matrix (which nobody needs any more), in
+            // groups whose loads are in flight together
+            constexpr int CH = D / 8, EACH = C * CH / 128, GROUP = EACH > 4 ? 4 : EACH;
+            uint4 val[GROUP][sizeof(T) / 2];
+            auto load_values = [&](int x0) {
+#pragma unroll
+                for (int x = 0; x < GROUP; ++x) {
+                    const int item = (x0 + x) * 128 + pt, t = t0 + item / CH;
+#pragma unroll
+                    for (int c = 0; c < (int)sizeof(T) / 2; ++c)
+                        val[x][c] = t < a.n_tokens ? __ldg(reinterpret_cast<const uint4*>(vp + t * row_stride + item % CH * 8) + c) : make_uint4(0, 0, 0, 0);
+                }
+            };
+            auto store_values = [&](int x0, int round) {
+#pragma unroll
+                for (int x = 0; x < GROUP; ++x) {
+                    const int item = (x0 + x) * 128 + pt, row = item / CH, ch = item % CH;
+                    uint4 w = val[x][0];
+                    if constexpr (sizeof(T) == 4) {
+                        const uint32_t f[8] = {val[x][0].x, val[x][0].y, val[x][0].z, val[x][0].w, val[x][1].x, val[x][1].y, val[x][1].z, val[x][1].w};
+                        uint32_t part[4][3];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) split_bf16(__uint_as_float(f[2 * e]), __uint_as_float(f[2 * e + 1]), part[e]);
+                        w = round == 0   ? make_uint4(part[0][0], part[1][0], part[2][0], part[3][0])
+                            : round == 1 ? make_uint4(part[0][1], part[1][1], part[2][1], part[3][1])
+                                         : make_uint4(part[0][2], part[1][2], part[2][2], part[3][2]);
+                    }
+                    *reinterpret_cast<uint4*>(V_s + (ch >> 3) * TILE + row * 128 + (((ch & 7) ^ (row & 7)) << 4)) = w;
+                }
+            };
+            load_values(0);
+            if constexpr (VR == 1) {
+#pragma unroll
+                for (int x0 = 0; x0 < EACH; x0 += GROUP) {
+                    if (x0 > 0) load_values(x0);
+                    store_values(x0, 0);
+                }
             }
             wait(bar_prep(team), phase);
             phase ^= 1;
             tc_fence_after();
 #pragma unroll
-            for (int cb = 0; cb < 4; ++cb) {
+            for (int cb = 0; cb < 4; ++cb) {                                // over T', which has been read
                 uint32_t v[16], hi[8], lo[8];
                 tmem_ld16(acc_at + cb * 16 + ((uint32_t)(w4 * 32) << 16), v);
                 tc_wait_ld();
+                float x[16];
 #pragma unroll
-                for (int e = 0; e < 8; ++e) split2(__uint_as_float(v[2 * e]), __uint_as_float(v[2 * e + 1]), hi[e], lo[e]);
+                for (int e = 0; e < 16; ++e) x[e] = __uint_as_float(v[e]);
+                split16(x, 1.f, hi, lo, KEEP_W);
                 if (pt < D) {
 #pragma unroll
                     for (int e = 0; e < 2; ++e) {
-                        uint8_t* dst = Y_s + pt * 128 + (((2 * cb + e) ^ (pt & 7)) << 4);
+                        uint8_t* dst = W_s + pt * 128 + (((2 * cb + e) ^ (pt & 7)) << 4);
                         *reinterpret_cast<uint4*>(dst) = make_uint4(hi[4 * e], hi[4 * e + 1], hi[4 * e + 2], hi[4 * e + 3]);
                         *reinterpret_cast<uint4*>(dst + D * 128) = make_uint4(lo[4 * e], lo[4 * e + 1], lo[4 * e + 2], lo[4 * e + 3]);
                     }
                 }
             }
-            asm volatile("cp.async.wait_all;" ::: "memory");
             proxy_fence();
             tc_fence_before();
-            arrive(bar_full(s));
+            arrive(bar_w(i));
+            // U^T (but for g_C / g) = V^T (T diag(beta))^T: lanes = dv, columns = tokens; bf16 values as they are, fp32 ones in
+            // three rounds of a bf16 part each, the smallest first
+#pragma unroll 1
+            for (int round = VR - 1; round >= 0; --round) {
+                if constexpr (VR > 1) {
+                    if (round < VR - 1) {
+                        if (EACH > GROUP) load_values(0);
+                        wait(bar_prep(team), phase);                        // the tile has been read
+                        phase ^= 1;
+                    }
+#pragma unroll
+                    for (int x0 = 0; x0 < EACH; x0 += GROUP) {
+                        if (x0 > 0) load_values(x0);
+                        store_values(x0, round);
+                    }
+                }
+                proxy_fence();
+                tc_fence_before();
+                bar_or(1 + team, 128, 0);
+                if (w4 == 0) {
+                    tc_fence_after();
+                    const uint64_t vd = umma_desc_mn(smem_u32(V_s), TILE), td = umma_desc(smem_u32(T_s));
+#pragma unroll 1
+                    for (int t = 2 - round; t >= 0; --t)
+#pragma unroll
+                        for (int ks = 0; ks < C / 16; ++ks)
+                            mma_ss(acc_at, vd + ((ks * 2048) >> 4), td + ((t * TILE) >> 4) + ((ks * 32) >> 4), idesc_f16(C) | A_MN_MAJOR | BF16_OPERANDS,
+                                   round != VR - 1 || t != 2 - round || ks);
+                    mma_commit(bar_prep(team));
+                }
+            }
+            wait(bar_prep(team), phase);
+            phase ^= 1;
+            tc_fence_after();
+#pragma unroll
+            for (int cb = 0; cb < 4; ++cb) {                                // over T diag(beta), which has been read
+                uint32_t v[16];
+                tmem_ld16(acc_at + cb * 16 + ((uint32_t)(w4 * 32) << 16), v);
+                tc_wait_ld();
+                if (pt < D) {
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) U_s[(cb * 16 + e) * D + pt] = __uint_as_float(v[e]);
+                }
+            }
+            tc_fence_before();
+            arrive(bar_u(i));
         }
-        asm volatile("cp.async.wait_all;" ::: "memory");
         bar_or(CTA_BARRIER, Z::THREADS, 0);                   // the chains take the rings' memory over
         if (P > 1)
             for (int p = 0; p < P; ++p) cluster_sync();       // (every thread of the cluster meets every one)
@@ -515,7 +665,7 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
     const bool is_m = has_m && (D == 128 ? chain == 1 : r >= D && r < 2 * D);
     const int mrow = D == 128 ? r : r - D;
     const uint32_t taddr = tmem_base + chain * Z::CHAIN_COLS + ((uint32_t)((warp & 3) * 32) << 16);
-    const uint32_t s_at = taddr, d_at = taddr + D;            // S operand / Delta Y ; S K^T / Delta operand
+    const uint32_t s_at = taddr, d_at = taddr + D;            // S operand / Delta K ; S W^T / Delta operand
     const uint32_t s_col = tmem_base + chain * Z::CHAIN_COLS, d_col = s_col + D;      // ... without the warp's lanes
     const bool issuer = (warp & 3) == 0, leader = issuer && lane == 0;
     uint32_t phase = 0;                                       // of the chain's barrier
@@ -532,49 +682,43 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
 #pragma unroll
     for (int d = 0; d < D; ++d) S[d] = is_m && d == mrow ? 1.f : 0.f;
     if ((D < 128 || chain == 0 || has_m) && n > 0) {
-        store_operand(is_m ? 1.f : 0.f);
-        bar_or(team, 128, 0);
+        float largest = is_m ? 1.f : 0.f;                     // of the row
+#pragma unroll 1
         for (int i = 0; i < n; ++i) {
-            const int s = i % Y_STAGES, kvs = i % KV_STAGES;
-            const uint8_t *K_s = smem + kvs * Z::KV_BYTES, *Y_s = y_ring + s * Z::Y_BYTES;
-            const float* co = coef_s + s * (Z::COEF_BYTES / 4);
-            wait(bar_full(s), (i / Y_STAGES) & 1);
-            if (issuer) {                                     // S K^T, small terms first: (hi lo,) lo hi, hi hi
+            store_operand(largest);
+            if (bar_or(team, 128, fail ? 1 : 0)) { fail = true; break; }
+            const int ks_n = i % K_STAGES, ws = i % Z::W_STAGES, us = i % Z::U_STAGES;
+            const uint8_t *K_s = smem + ks_n * Z::K_BYTES, *W_s = w_ring + ws * Z::W_BYTES;
+            const float *U_s = u_ring + us * (Z::U_BYTES / 4), *co = coef_s + us * (Z::COEF_BYTES / 4);
+            wait(bar_w(i), turn(i));
+            if (issuer) {                                     // S W^T, small terms first: hi lo, lo hi, hi hi
                 tc_fence_after();
-                const uint64_t kd = umma_desc(smem_u32(K_s));
+                const uint64_t wd = umma_desc_mn(smem_u32(W_s), D * 128);
 #pragma unroll 1
-                for (int t = PK; t >= 0; --t)
-#pragma unroll 1
-                    for (int kb = 0; kb < KB; ++kb)
+                for (int t = 2; t >= 0; --t)
 #pragma unroll
-                        for (int ks = 0; ks < KS; ++ks)
-                            mma_ts(d_col, s_col + (kb * 4 + ks) * 16 + (t == 1 ? 8 : 0), kd + (t == 2 ? (KB * TILE) >> 4 : 0) + ((kb * TILE + ks * 32) >> 4),
-                                   idesc_f16(C), t != PK || kb || ks);
+                    for (int ks = 0; ks < D / 16; ++ks)
+                        mma_ts(d_col, s_col + ks * 16 + (t == 1 ? 8 : 0), wd + (t == 2 ? (D * 128) >> 4 : 0) + ((ks * 2048) >> 4),
+                               idesc_f16(C) | B_MN_MAJOR, t != 2 || ks);
                 mma_commit(bar_chain(chain));
+                mma_commit(bar_wfree(i));
             }
             wait(bar_chain(chain), phase);
             phase ^= 1;
             tc_fence_after();
-            // Delta (times what undoes Y's row scale), in place; S rows add beta v
+            wait(bar_u(i), turn(i));
+            // Delta (times what undoes the keys' scales) in place; U is the S rows'
             const float neg = -inv_row, g_chunk = co[2 * C];
             float m = 0.f;
-            auto delta = [&](auto with_v) {
+            auto delta = [&](auto with_u) {
 #pragma unroll 1
                 for (int b = 0; b < 4; ++b) {
                     uint32_t v[16];
                     tmem_ld16(d_at + 16 * b, v);
                     float x[16];
-                    if constexpr (decltype(with_v)::value) {
+                    if constexpr (decltype(with_u)::value) {
 #pragma unroll
-                        for (int e = 0; e < 16; ++e) {
-                            if constexpr (Z::V_STAGED) {
-                                const uint8_t* vp = K_s + Z::K_BYTES + ((16 * b + e) * D + r) * 2;
-                                x[e] = __uint_as_float((uint32_t)*reinterpret_cast<const uint16_t*>(vp) << 16);
-                            } else {
-                                const int t = min((c_begin + i) * C + 16 * b + e, a.n_tokens - 1);
-                                x[e] = __ldg(static_cast<const float*>(a.v) + ((long long)t * a.H + h) * D + r);
-                            }
-                        }
+                        for (int e = 0; e < 16; ++e) x[e] = U_s[(16 * b + e) * D + r];
                     }
                     tc_wait_ld();
 #pragma unroll
@@ -582,18 +726,15 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
                         const float4 cc = *reinterpret_cast<const float4*>(co + C + 16 * b + e);
                         const float c4[4] = {cc.x, cc.y, cc.z, cc.w};
                         float b4[4];
-                        if constexpr (decltype(with_v)::value) {
+                        if constexpr (decltype(with_u)::value) {
                             const float4 bb = *reinterpret_cast<const float4*>(co + 16 * b + e);
                             b4[0] = bb.x; b4[1] = bb.y; b4[2] = bb.z; b4[3] = bb.w;
                         }
 #pragma unroll
-                        for (int f = 0; f < 4; f += 2) {
-                            float2 y = __fmul2_rn(make_float2(__uint_as_float(v[e + f]), __uint_as_float(v[e + f + 1])), make_float2(neg, neg));
-                            const float2 c2 = make_float2(c4[f], c4[f + 1]);
-                            if constexpr (decltype(with_v)::value)
-                                y = __ffma2_rn(c2, y, __fmul2_rn(make_float2(b4[f], b4[f + 1]), make_float2(x[e + f], x[e + f + 1])));
-                            else
-                                y = __fmul2_rn(c2, y);
+                        for (int f = 0; f < 4; f += 2) {      // (neg and c are powers of two)
+                            float2 y = __fmul2_rn(__fmul2_rn(make_float2(__uint_as_float(v[e + f]), __uint_as_float(v[e + f + 1])), make_float2(neg, neg)),
+                                                  make_float2(c4[f], c4[f + 1]));
+                            if constexpr (decltype(with_u)::value) y = __ffma2_rn(make_float2(b4[f], b4[f + 1]), make_float2(x[e + f], x[e + f + 1]), y);
                             m = fmaxf(fmaxf(m, fabsf(y.x)), fabsf(y.y));
                             v[e + f] = __float_as_uint(y.x);
                             v[e + f + 1] = __float_as_uint(y.y);
@@ -607,49 +748,69 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
             tc_wait_st();
             float sc, inv_d;
             pow2_scale(m, WIDE, sc, inv_d);
+            // ... and as the next product's A operand: hi and lo in tensor memory; fp32 records: what is left in shared memory (not
+            // for M's chain at dk = 128: S takes M's error times what is left of it after a segment)
+            const bool three = Z::DP == 3 && (D < 128 || chain == 0);
 #pragma unroll 1
             for (int b = 0; b < 4; ++b) {
-                uint32_t v[16];
+                uint32_t v[16], w[16], low[8];
                 tmem_ld16(d_at + 16 * b, v);
                 tc_wait_ld();
                 float x[16];
 #pragma unroll
                 for (int e = 0; e < 16; ++e) x[e] = __uint_as_float(v[e]);
-                split_to_tmem(d_at + 16 * b, x, sc);
+                split16(x, sc, w, w + 8, KEEP_DELTA, Z::DP == 3 ? low : nullptr);
+                tmem_st16(d_at + 16 * b, w);
+                if (three) {
+#pragma unroll
+                    for (int e = 0; e < 2; ++e)
+                        *reinterpret_cast<uint4*>(low_s + r * 128 + (((2 * b + e) ^ (r & 7)) << 4)) = make_uint4(low[4 * e], low[4 * e + 1], low[4 * e + 2], low[4 * e + 3]);
+                }
             }
             tc_wait_st();
+            if (Z::DP == 3) proxy_fence();
             tc_fence_before();
             if (bar_or(team, 128, fail ? 1 : 0)) { fail = true; break; }
-            if (issuer) {                                     // Delta Y: lo hi, hi lo, hi hi, over the S operand (read by now)
+            if (leader) arrive(bar_ufree(i));
+            if (issuer) {                                     // Delta K over the S operand (read by now), small terms first
                 tc_fence_after();
-                const uint64_t yd = umma_desc(smem_u32(Y_s));
-#pragma unroll 1
-                for (int t = 2; t >= 0; --t)
+                const uint64_t kd = umma_desc_mn(smem_u32(K_s), TILE), ld = umma_desc(smem_u32(low_s));
+                bool first = true;
+                auto product = [&](int dp, int kp) {          // part dp of Delta, part kp of the keys
 #pragma unroll
-                    for (int ks = 0; ks < C / 16; ++ks)
-                        mma_ts(s_col, d_col + ks * 16 + (t == 2 ? 8 : 0), yd + (t == 1 ? (D * 128) >> 4 : 0) + ((ks * 32) >> 4), idesc_f16(D), t != 2 || ks);
+                    for (int ks = 0; ks < C / 16; ++ks) {
+                        const uint64_t bd = kd + ((kp * KB * TILE) >> 4) + ((ks * 2048) >> 4);
+                        if (dp == 2) mma_ss(s_col, ld + ((ks * 32) >> 4), bd, idesc_f16(D) | B_MN_MAJOR, !first);
+                        else mma_ts(s_col, d_col + ks * 16 + dp * 8, bd, idesc_f16(D) | B_MN_MAJOR, !first);
+                        first = false;
+                    }
+                };
+                if (three) product(2, 0);
+                if constexpr (PK > 1) {
+                    product(1, 1);
+                    if constexpr (PK > 2) product(0, 2);
+                    product(0, 1);
+                }
+                product(1, 0);
+                product(0, 0);
                 mma_commit(bar_chain(chain));
-                mma_commit(bar_yfree(s));                     // the stages' tiles are read; values and coefficients were before
-                mma_commit(bar_kvfree(kvs));
+                mma_commit(bar_kfree(ks_n));
             }
             wait(bar_chain(chain), phase);
             phase ^= 1;
             tc_fence_after();
-            m = 0.f;
+            largest = 0.f;
 #pragma unroll
             for (int b = 0; b < D / 16; ++b) {
                 uint32_t v[16];
                 tmem_ld16(s_at + 16 * b, v);
                 tc_wait_ld();
 #pragma unroll
-                for (int e = 0; e < 16; e += 2) {
+                for (int e = 0; e < 16; ++e) {
                     S[16 * b + e] = fmaf(g_chunk, S[16 * b + e], __uint_as_float(v[e]) * inv_d);
-                    S[16 * b + e + 1] = fmaf(g_chunk, S[16 * b + e + 1], __uint_as_float(v[e + 1]) * inv_d);
-                    m = fmaxf(fmaxf(m, fabsf(S[16 * b + e])), fabsf(S[16 * b + e + 1]));
+                    largest = fmaxf(largest, fabsf(S[16 * b + e]));
                 }
             }
-            if (i + 1 < n) store_operand(m);
-            if (bar_or(team, 128, fail ? 1 : 0)) { fail = true; break; }
         }
     }
     bar_or(CTA_BARRIER, Z::THREADS, 0);
