@@ -38,10 +38,11 @@
 // (fp32 records: Delta K 5 or 6 products, the lowest part of Delta in shared memory; K K^T three, K^T T'^T three, U six.)
 // What bounds it now: the latency of a chain's step and, as long, the two preparations in flight, about 11 000 cycles per
 // chunk.  16 384 tokens x 32 heads of 128 x 128 bf16: 18.2 ms token by token, 0.44 ms (0.38 ms in the other grouping, whose
-// errors were larger); 1021 tokens x 16 heads of 64 x 64 fp32: 376 -> 39 us (35).
+// errors were larger); 1021 tokens x 16 heads of 64 x 64 fp32: 376 -> 40 us (35).
 //
 // Every wait is bounded: a thread that gives up keeps meeting its team's barriers, whose OR makes the team leave
-// together, and the cluster barriers; ONELA_E_TIMEOUT goes to the status word.
+// together, and the cluster barriers, but hands nothing on; ONELA_E_TIMEOUT goes to the status word.  A team always waits for
+// its own MMAs, so none is in flight when its operands are written again or tensor memory is freed.
 #include <algorithm>
 #include <mutex>
 #include <type_traits>
@@ -209,6 +210,12 @@ __device__ __forceinline__ void rows8(float* acc, const float* rows, const float
     }
 }
 
+#ifdef ONELA_TEST_HOOKS
+// Test-hooks build only (a second library that the product never loads): when set, one thread of the first head's last segment
+// leaves out its arrival for the first chunk's W, so that the chains' wait for it runs out.
+__device__ int g_hook_prefill_drop;
+#endif
+
 template <int D, typename T>
 __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(const PrefillArgs a) {
     using Z = Shape<D, T>;
@@ -267,7 +274,14 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
     bool fail = false;
-    // bounded wait that also gives up as soon as another role has
+    // a team's own MMAs: they complete by themselves, so nobody gives up early and leaves them behind
+    auto wait_mma = [&](uint32_t bar, uint32_t parity) {
+        if (!sm100::mbar_wait(bar, parity)) {
+            fail = true;
+            *abort_flag = 1;
+        }
+    };
+    // what another role has to do: bounded, and given up as soon as a role has
     auto wait = [&](uint32_t bar, uint32_t parity) {
         for (int i = 0; i < sm100::WAIT_LIMIT; ++i) {
             if (sm100::mbar_try_wait(bar, parity)) return;
@@ -390,7 +404,7 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
                     asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
                 }
             }
-            wait(bar_prep(team), phase);
+            wait_mma(bar_prep(team), phase);
             phase ^= 1;
             tc_fence_after();
             // A = beta_i (g_i / g_j) (k_i . k_j), row i by thread i; the gate products run from the right, each as a sum of two
@@ -529,7 +543,7 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
                 if (pt == C - 1) co[2 * C] = g + g_rest;
             }
             proxy_fence();
-            bar_or(1 + team, 128, 0);
+            if (bar_or(1 + team, 128, fail ? 1 : 0)) { fail = true; break; }
             if (w4 == 0) {          // W^T = K^T T'^T: lanes = dk, columns = tokens
                 tc_fence_after();
                 const uint64_t kd = umma_desc_mn(smem_u32(K_s), TILE), td = umma_desc(smem_u32(W_s));
@@ -580,7 +594,7 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
                     store_values(x0, 0);
                 }
             }
-            wait(bar_prep(team), phase);
+            wait_mma(bar_prep(team), phase);
             phase ^= 1;
             tc_fence_after();
 #pragma unroll
@@ -603,7 +617,11 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
             }
             proxy_fence();
             tc_fence_before();
+#ifdef ONELA_TEST_HOOKS
+            if (!(g_hook_prefill_drop && blockIdx.x == gridDim.x - 1 && blockIdx.y == 0 && i == 0 && pt == 0)) arrive(bar_w(i));
+#else
             arrive(bar_w(i));
+#endif
             // U^T (but for g_C / g) = V^T (T diag(beta))^T: lanes = dv, columns = tokens; bf16 values as they are, fp32 ones in
             // three rounds of a bf16 part each, the smallest first
 #pragma unroll 1
@@ -611,7 +629,7 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
                 if constexpr (VR > 1) {
                     if (round < VR - 1) {
                         if (EACH > GROUP) load_values(0);
-                        wait(bar_prep(team), phase);                        // the tile has been read
+                        wait_mma(bar_prep(team), phase);                        // the tile has been read
                         phase ^= 1;
                     }
 #pragma unroll
@@ -635,7 +653,7 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
                     mma_commit(bar_prep(team));
                 }
             }
-            wait(bar_prep(team), phase);
+            wait_mma(bar_prep(team), phase);
             phase ^= 1;
             tc_fence_after();
 #pragma unroll
@@ -651,7 +669,7 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
             tc_fence_before();
             arrive(bar_u(i));
         }
-        bar_or(CTA_BARRIER, Z::THREADS, 0);                   // the chains take the rings' memory over
+        bar_or(CTA_BARRIER, Z::THREADS, fail ? 1 : 0);        // the chains take the rings' memory over
         if (P > 1)
             for (int p = 0; p < P; ++p) cluster_sync();       // (every thread of the cluster meets every one)
     } else {
@@ -703,7 +721,7 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
                 mma_commit(bar_chain(chain));
                 mma_commit(bar_wfree(i));
             }
-            wait(bar_chain(chain), phase);
+            wait_mma(bar_chain(chain), phase);
             phase ^= 1;
             tc_fence_after();
             wait(bar_u(i), turn(i));
@@ -796,7 +814,7 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
                 mma_commit(bar_chain(chain));
                 mma_commit(bar_kfree(ks_n));
             }
-            wait(bar_chain(chain), phase);
+            wait_mma(bar_chain(chain), phase);
             phase ^= 1;
             tc_fence_after();
             largest = 0.f;
@@ -813,7 +831,8 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
             }
         }
     }
-    bar_or(CTA_BARRIER, Z::THREADS, 0);
+    // (a CTA in which somebody gave up has nothing to hand on: it only keeps meeting the cluster)
+    const bool lost = bar_or(CTA_BARRIER, Z::THREADS, fail ? 1 : 0);
 
     // =============================== SEGMENTS IN ORDER ===============================
     // S of the segments so far passes from CTA to CTA as the receiver's A operand (per row dk words in the order of the K
@@ -835,7 +854,7 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
         }
     };
     if (P > 1) {
-        if (has_m && (D < 128 || chain == 1)) {               // M with one scale for all its rows (every warp of the team comes along)
+        if (!lost && has_m && (D < 128 || chain == 1)) {      // M with one scale for all its rows (every warp of the team comes along)
             float m = 0.f, sc, inv;
             if (is_m) {
 #pragma unroll
@@ -864,12 +883,12 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
             }
             proxy_fence();
         }
-        if (rank == 0 && is_s) hand_over();
+        if (!lost && rank == 0 && is_s) hand_over();
         // (one chain holds the S operand; its product lands in the other chain's columns, or beside it)
         const uint32_t o_at = D == 128 ? taddr + Z::CHAIN_COLS : d_at, o_col = D == 128 ? s_col + Z::CHAIN_COLS : d_col;
         for (int p = 1; p < P; ++p) {
             cluster_sync();
-            if (rank != p || chain != 0) continue;
+            if (lost || rank != p || chain != 0) continue;
             const int row = is_s ? r : 0;                     // (rows that are none come along with row 0's data)
             uint32_t peer, peer_inv;
             asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer) : "r"(smem_u32(hand_s + row)), "r"(p - 1));
@@ -902,7 +921,7 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
                                idesc_f16(D) | B_MN_MAJOR, t != 2 || ks);
                 mma_commit(bar_chain(0));
             }
-            wait(bar_chain(0), phase);
+            wait_mma(bar_chain(0), phase);
             phase ^= 1;
             tc_fence_after();
 #pragma unroll
@@ -920,7 +939,7 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
     }
 
     // =============================== RESULT ===============================
-    if (rank == P - 1 && chain == 0) {
+    if (!lost && rank == P - 1 && chain == 0) {
         float m = 0.f;
         if (is_s) {
             float4* dst = reinterpret_cast<float4*>(a.slot + ((long long)h * D + r) * D);
@@ -1052,3 +1071,7 @@ cudaError_t launch_prefill(const void* k, const void* v, const float* alpha, con
 }
 
 }  // namespace onela
+
+#ifdef ONELA_TEST_HOOKS
+extern "C" int onela_testhook_prefill_drop(int on) { return (int)cudaMemcpyToSymbol(onela::g_hook_prefill_drop, &on, sizeof(int)); }
+#endif

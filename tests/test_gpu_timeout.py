@@ -1,4 +1,4 @@
-"""The bounded waits of the tensor-core decode kernels, exercised without a fault: a second build of the library
+"""The bounded waits of the tensor-core kernels, exercised without a fault: a second build of the library
 (same sources, a short wait limit, one test hook) makes ONE fold-warp arrival of CTA 0 go missing, so the wait for
 that group's operand rows runs out.  The kernel must return, the sticky status word must say ONELA_E_TIMEOUT with
 the CTA's index, and the same context must decode correctly afterwards.  Runs in a child process so that the
@@ -112,8 +112,43 @@ def _child_tiled():
     print("timeout reported and recovered")
 
 
+def _child_prefill():
+    """The prefill's wait for a prepared chunk, with one chain per CTA (64 x 64) and with two (128 x 128), on a prompt of one
+    segment: an arrival goes missing, the teams leave together and free their tensor memory; the next prefill of the same
+    context, on a cluster of segments, is right."""
+    import ctypes
+
+    import numpy as np
+
+    sys.path.insert(0, str(ROOT))
+    import oracle
+    import paper_2609_12399_b200 as P
+    from paper_2609_12399_b200 import binding, build, inputs
+
+    binding.LIB_PATH = build.build_testhooks()
+    lib = binding.load_library()
+    lib.onela_testhook_prefill_drop.restype = ctypes.c_int
+    lib.onela_testhook_prefill_drop.argtypes = [ctypes.c_int]
+    for d, dtype in ((128, "bf16"), (128, "fp32"), (64, "fp32")):
+        p = inputs.prompt_tokens(inputs.WORKLOADS[1].scaled(H=2, dk=d, dv=d, dtype=dtype, prompt_len=1000, seed=5), 0, 0)
+        want = oracle.prefill(p["k"], p["v"], p["alpha"], p["beta"])
+        tokens = [p[n].cuda() for n in ("k", "v", "alpha", "beta")]
+        ctx = P.Onela(P.make_config(1, 1, 2, d, d, 8, 1, dtype, "fp32", 16))
+        assert lib.onela_testhook_prefill_drop(1) == 0
+        ctx.onela_prefill_shared_state(0, 0, *(x[:50] for x in tokens))
+        code, _ = ctx.onela_poll_device_status()
+        assert code == binding.E_TIMEOUT, (d, dtype, code)
+        assert lib.onela_testhook_prefill_drop(0) == 0
+        ctx.onela_prefill_shared_state(0, 0, *tokens)
+        got = ctx.onela_export_shared_state(0, 0).cpu().double().numpy()
+        assert ctx.onela_poll_device_status() == (0, 0)
+        err = np.linalg.norm(got - want, axis=(1, 2)) / np.linalg.norm(want, axis=(1, 2))
+        assert err.max() < 2e-6, (d, dtype, err)
+    print("timeout reported and recovered")
+
+
 @pytest.mark.gpu
-@pytest.mark.parametrize("which", ["child", "child_tiled"])
+@pytest.mark.parametrize("which", ["child", "child_tiled", "child_prefill"])
 def test_expired_wait_is_reported_and_the_context_stays_usable(which):
     r = subprocess.run([sys.executable, __file__, which], capture_output=True, text=True, timeout=600)
     assert r.returncode == 0, r.stdout + r.stderr
@@ -124,3 +159,5 @@ if __name__ == "__main__" and sys.argv[1:] == ["child"]:
     _child()
 if __name__ == "__main__" and sys.argv[1:] == ["child_tiled"]:
     _child_tiled()
+if __name__ == "__main__" and sys.argv[1:] == ["child_prefill"]:
+    _child_prefill()
