@@ -173,6 +173,9 @@ def onela_workspace_bytes(cfg: OnelaConfig) -> int:
 class Onela:
     """A context over a torch-owned workspace.  Methods mirror the C entry points one to one."""
 
+    # (on the class: when the interpreter ends, a context may outlive this module's globals)
+    _native_names, _no_native = _NATIVE_CALLS, staticmethod(_no_native_call)
+
     def __init__(self, cfg: OnelaConfig, device="cuda", workspace_ptr: int | None = None):
         self.lib = load_library()
         self.cfg = cfg
@@ -202,8 +205,8 @@ class Onela:
 
     def close(self):
         if getattr(self, "handle", None):
-            for name in _NATIVE_CALLS:
-                setattr(self, "_" + name, _no_native_call)      # (a native caller keeps the raw handle)
+            for name in self._native_names:
+                setattr(self, "_" + name, self._no_native)      # (a native caller keeps the raw handle)
             self.lib.onela_destroy(self.handle)
             self.handle = None
 

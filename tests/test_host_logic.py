@@ -416,3 +416,13 @@ def test_native_calls_built_for_another_torch_are_not_loaded(monkeypatch):
     assert binding.pycall_path() != built and build._stale(binding.pycall_path(), [build.PYCALL_SRC])
     with pytest.raises(RuntimeError, match="is missing"):
         binding._native_caller(binding.load_library(), None, None)
+
+
+def test_a_context_alive_at_exit_is_released_quietly():
+    """A script that ends with a live context: the interpreter clears the binding's globals before it drops the context."""
+    import subprocess
+    import sys
+    code = ("import paper_2609_12399_b200 as P\nfrom paper_2609_12399_b200 import binding\n"
+            "ctx = P.Onela(P.make_config(1, 1, 1, 32, 32, 8, 1, 'fp32', 'fp32', 16, P.FLAG_DRY_RUN), device='cpu')\n")
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, cwd=Path(__file__).parent.parent)
+    assert r.returncode == 0 and r.stderr == "", r.stderr
