@@ -26,8 +26,8 @@
  *  - `stream` is a cudaStream_t passed as void*.  Every call is asynchronous and ordered on that
  *    stream; inputs may be reused as soon as the stream has passed the call.  Only
  *    onela_poll_device_status() synchronises.  Most kernels are launched with programmatic stream serialisation:
- *    they may start while the previous kernel of the stream drains, but read only the library's own shared-state
- *    store before they have waited for that kernel's completion, so stream order holds for every tensor the caller
+ *    they may start while the previous kernels of the stream still run, but read only the library's own shared-state
+ *    store before they have waited for those kernels' completion, so stream order holds for every tensor the caller
  *    passes.  A caller kernel that follows one AND is itself launched with programmatic stream serialisation must
  *    wait for its grid dependency before it reads the outputs, as that launch mode requires of any kernel.
  *  - Tensors are dense, row-major, last index contiguous.  q, k, v use cfg.rec_dtype, outputs

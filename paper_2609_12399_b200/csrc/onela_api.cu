@@ -562,7 +562,6 @@ onela_status launch_decode(onela_ctx* ctx, int32_t req_begin, int32_t req_count,
     a.sidx = ctx->lay.sidx + req_begin * ctx->sidx_req_stride();
     a.ulist = ctx->lay.ulist + req_begin * ctx->sidx_req_stride();
     a.uoff = ctx->lay.uoff + req_begin * ctx->uoff_req_stride();
-    a.urep = ctx->lay.urep + req_begin * ctx->sidx_req_stride();
     a.sg8 = ctx->lay.sg8 + req_begin * ctx->sg8_req_stride();
     a.unode = ctx->lay.unode + (size_t)req_begin * ONELA_UNODE_CAP * 16;
     a.sg8_req_stride = ctx->sg8_req_stride();

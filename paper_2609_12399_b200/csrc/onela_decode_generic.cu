@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(NB* G) decode_generic_kernel(const DecodeArgs 
     const bool active = b < a.W;
     const int bb = active ? b : a.W - 1;  // idle groups shadow a live beam so loads and shuffles stay uniform
 
-    // (the store is written only by the state calls, and a reorder launch always lies between those and a decode)
+    // (read before the wait: see launch_dependent)
     const float* S0h = a.s0 + req * a.s0_req_stride + (long long)h * DV * DK;
     if constexpr (SMALL) {
         for (int i = threadIdx.x; i < DV * DK / 4; i += NB * G) reinterpret_cast<float4*>(S_s)[i] = __ldg(reinterpret_cast<const float4*>(S0h) + i);

@@ -303,8 +303,8 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     };
     // The first segment's S_0 is requested by all warps (one 32-column block each) and put into tensor memory before the
-    // launch's dependencies are waited for: the store is written only by the state calls (a copy or a prefill kernel), and
-    // a reorder launch always separates those from a decode.  (Put there after the first heads had been requested, it stood
+    // launch's dependencies are waited for: see launch_dependent for why the store, and nothing else, may be read
+    // there.  (Put there after the first heads had been requested, it stood
     // between them and the fold: 0.4 us of a launch of 128 x 16 to 512 x 32 units, 1 - 1.5 %; large launches are the same.)
     static_assert(THREADS >= 512, "the first sixteen warps take one 32-column block of the first S_0 each");
     const bool s0_mine = warp < 16;
@@ -359,8 +359,9 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
 
     // Chains that share little - fewer than half of the first request's older levels can be staged, and the beams' parents are
     // more than a quarter as many as there are beams - are gathered through a queue: nothing is staged, and every fold warp
-    // keeps two levels' records on their way by async copies, across quads.  (A decision per CTA, which both roles make alike;
-    // the requests of a batch follow one parent law as a rule.)  A gather into registers waits out L2's latency at every
+    // keeps two levels' records on their way by async copies, across quads.  (A decision per CTA, by the first request of its
+    // range and, of longer chains, by the 32 oldest levels; both roles make it alike.  The requests of a batch follow one parent
+    // law as a rule; where they don't, a request in the other mode costs time, not results.)  A gather into registers waits out L2's latency at every
     // level: 8 x 1024 beams with uniform parents 24 us per level that way, 15 us through the queue (depth 6: 202 -> 165 us).
     // Where the line lies, measured on 4 x 300 beams, uniform parents, depth 4 - 7: staging what can be staged 22.6 us, the
     // queue as soon as one level cannot be staged 21.8 us, but on 2 x 200 beams, Zipf(1.2), 21 us against 18 us with the rule.
@@ -951,7 +952,7 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
                 // neighbouring beams of an output, adds its corr elements, and the pair - packed to bf16 - goes out through
                 // a transposing matrix store, eight outputs of a beam per 16-byte row.  (As 32 x 32-bit rows written
                 // transposed in fp32, read back beside the corr tile and stored by three warps, a group took 1.75 us of
-                // these warps at every depth; 0.8 us now.)
+                // these warps at every depth; 1.1 - 1.2 us now, 0.7 - 0.8 of them up to the barrier below.)
                 float2 w[GN / 8];                             // what undoes the scales of each beam's row
 #pragma unroll
                 for (int nb = 0; nb < GN / 8; ++nb) w[nb] = *reinterpret_cast<const float2*>(inv_s + s * GN + nb * 8 + fc);

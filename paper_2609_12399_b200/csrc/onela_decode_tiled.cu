@@ -167,8 +167,7 @@ __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, 
                        (kb | ks) != 0);
         mma_commit(smem_u32(bar));
     };
-    // The stored states are written by the state calls only, and the index launch that lies between those and any decode
-    // waits for them before it lets this one start: the first operand may be requested before the wait.
+    // (the first operand is requested before the wait: see launch_dependent for why the store may be read there)
     if (tid == 0) load_A(0);        // in flight while the chain is walked
     asm volatile("griddepcontrol.wait;" ::: "memory");
 

@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(THREADS, 1) decode_wy_kernel(const __grid_cons
     bool dead = false;
 
     // The first segment's S_0: requested by the first sixteen warps before the launch's dependencies are waited for
-    // (the store is written only by the state calls, and a reorder launch always separates those from a decode),
+    // (see launch_dependent for why the store may be read there),
     // put into tensor memory as fp16 times the head's power-of-two scale.
     const bool s0_mine = warp < 16;
     float4 s0_first[8];
@@ -463,8 +463,6 @@ __global__ void __launch_bounds__(THREADS, 1) decode_wy_kernel(const __grid_cons
             const int seg_g0 = max(g_begin, pair * groups_per_pair), seg_g1 = min(g_end, (pair + 1) * groups_per_pair);
             const int32_t* uoff = a.uoff + req * a.uoff_req_stride;
             const int32_t* ulist = a.ulist + req * a.ulist_req_stride;
-            const int32_t* urep = a.urep + req * a.ulist_req_stride;
-            const int32_t* sidx = a.sidx + req * a.sidx_req_stride;
             const long long plane_row0 = (long long)h * a.arena_slots;
             const int n = __ldg(uoff + m), nd = __ldg(uoff + m - 1);        // nodes, and nodes older than the parents
             const int n16 = (n + 15) & ~15, nd16 = (nd + 15) & ~15;

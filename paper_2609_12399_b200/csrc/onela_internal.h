@@ -63,7 +63,6 @@ struct DecodeArgs {
     const int32_t* sidx;    // distinct-record index of req_begin (see Layout)
     const int32_t* ulist;
     const int32_t* uoff;
-    const int32_t* urep;
     const uint8_t* sg8;     // byte copies of sidx and the per-record table (see Layout), of req_begin
     const uint8_t* unode;
     long long sg8_req_stride;
@@ -136,10 +135,19 @@ bool decode_tiled_supported(int32_t dk, int32_t dv);
 cudaError_t launch_decode_tiled(const TiledArgs& a, int32_t dk, int32_t dv, int32_t rec_dtype, int32_t out_dtype,
                                 cudaStream_t stream);
 
-// Launch with programmatic stream serialisation: the kernel may start while the previous kernel of the stream drains.
-// Rule for every kernel launched this way: it waits for that kernel (griddepcontrol.wait, every CTA) before it reads or
-// writes anything an earlier launch touches - only the decode kernels read the stored states earlier, see there - and lets
-// its own dependents start (griddepcontrol.launch_dependents) only from every CTA itself.
+// Launch with programmatic stream serialisation: the kernel may start once every CTA of the previous kernel of the stream has
+// let it (griddepcontrol.launch_dependents), and griddepcontrol.wait returns when that kernel has completed.
+//   * Every CTA of a kernel launched this way waits.  So a kernel that has completed has seen its predecessor complete, and
+//     past its own wait a kernel sees everything that earlier launches of the stream have written.
+//   * Before its wait a kernel may count on nothing: the decode kernels let their dependents start before they have waited
+//     themselves, and all others do so behind their wait but before they have written anything.  "Two launches ago" is no
+//     guarantee either.
+//   * The one thing read before the wait is the stored states (with their scales and operand copies), by the decode kernels.
+//     They are written by the state calls alone; the host admits a decode only when a reorder of its request lies between
+//     (finish_state_write restarts the request), and the index kernel of that reorder lets nothing start before its own wait,
+//     so the states were complete when any kernel behind it started.
+// The prefill, the CUDA-core kernels for delta records and grouped heads, and export_chains are ordinary launches: they start
+// when everything before them has completed, and what follows them starts when they have.
 template <class... Params, class... Args>
 cudaError_t launch_dependent(void (*kern)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, const Args&... args) {
     cudaLaunchConfig_t cfg = {};

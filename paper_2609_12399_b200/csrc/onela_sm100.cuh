@@ -1,5 +1,5 @@
-// PTX wrappers and fold primitives shared by the sm_100a decode kernels (dk = dv = 128, bf16 records):
-// mbarriers, bulk async copies, tcgen05 MMA / tensor-memory access, and the per-lane fold step.
+// PTX wrappers shared by the sm_100a kernels (mbarriers, bulk async copies, tcgen05 MMA and tensor-memory access, operand
+// scales) and the per-lane fold step of the decode kernels for dk = dv = 128 with bf16 records.
 #pragma once
 
 #include <cuda_fp16.h>
