@@ -253,13 +253,17 @@ struct Lanes {
         float2 kx[NP2];
 #pragma unroll
         for (int c = 0; c < NCH; ++c) unpack8(rec.k[c], kx + 4 * c);
-        float2 d0 = make_float2(0.f, 0.f), d1 = make_float2(0.f, 0.f);
+        constexpr int NS = NP2 / 4;              // partial sums: chains of four
+        float2 d[NS];
 #pragma unroll
-        for (int e = 0; e < NP2; e += 2) {
-            d0 = __ffma2_rn(kx[e], r[e], d0);
-            d1 = __ffma2_rn(kx[e + 1], r[e + 1], d1);
-        }
-        float dot = (d0.x + d0.y) + (d1.x + d1.y);
+        for (int e = 0; e < NS; ++e) d[e] = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int e = 0; e < NP2; ++e) d[e % NS] = __ffma2_rn(kx[e], r[e], d[e % NS]);
+#pragma unroll
+        for (int n = NS / 2; n > 0; n >>= 1)
+#pragma unroll
+            for (int e = 0; e < n; ++e) d[e] = __fadd2_rn(d[e], d[e + n]);
+        float dot = d[0].x + d[0].y;
 #pragma unroll
         for (int o = LPU / 2; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
         const float bc = REPLAY ? dot : rec.gate.y * dot;
