@@ -272,6 +272,9 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+    // (programmatic dependent launch: set up beside the previous launch; nothing is read before it has completed)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     bool fail = false;
     // a team's own MMAs: they complete by themselves, so nobody gives up early and leaves them behind
@@ -1020,9 +1023,11 @@ cudaError_t launch_dt(const PrefillArgs& args, cudaStream_t stream) {
     cfg.blockDim = dim3(Z::THREADS);
     cfg.dynamicSmemBytes = Z::SMEM;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int* resident = resident_of[dev];
@@ -1048,6 +1053,7 @@ cudaError_t launch_dt(const PrefillArgs& args, cudaStream_t stream) {
     a.rest = cut.rest;
     attr[0].val.clusterDim.x = cut.P;
     cfg.gridDim = dim3(cut.P, a.H);
+    cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, kern, a);
 }
 

@@ -36,6 +36,13 @@ __global__ void __launch_bounds__(256) append_kernel(const char* __restrict__ k,
     if (lane == 0) gate_plane[dst_row] = make_float2(__ldg(alpha + row), __ldg(beta + row));
 }
 
+// Copy of one (request, layer)'s states out of the store, 16 bytes per thread and step.
+__global__ void __launch_bounds__(256) export_state_kernel(const float4* __restrict__ slot, float4* __restrict__ out, int32_t n) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    for (int32_t i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) out[i] = slot[i];
+}
+
 // The operand scale of a head (Layout::s0_scale) from the largest magnitude of its state.
 __device__ __forceinline__ float operand_scale(float peak) {
     const int eb = (int)(__float_as_uint(peak) >> 23) & 255;          // biased exponent of a non-negative number
@@ -165,6 +172,17 @@ cudaError_t launch_store_state(const float* S0_in, float* slot, float* scale_out
 }
 
 cudaError_t launch_export_state(const float* slot, float* S0_out, int32_t H, int32_t dk, int32_t dv, cudaStream_t stream) {
+    // A kernel of our own is a dependent launch, a copy by the runtime is not (a prefill and the export of its states, XXX).
+    // Memory of another device, which a kernel may not reach, is the runtime's.
+    cudaPointerAttributes at;
+    int dev = 0;
+    const bool here = cudaGetDevice(&dev) == cudaSuccess && cudaPointerGetAttributes(&at, S0_out) == cudaSuccess && at.type == cudaMemoryTypeDevice && at.device == dev;
+    const long long n = (long long)H * dk * dv / 4;
+    if (here && n <= 0x7fffffff) {
+        const unsigned blocks = (unsigned)(n / 256 < 1184 ? (n + 255) / 256 : 1184);      // eight per SM at most
+        return launch_dependent(export_state_kernel, dim3(blocks), dim3(256), 0, stream, reinterpret_cast<const float4*>(slot),
+                                reinterpret_cast<float4*>(S0_out), (int32_t)n);
+    }
     return cudaMemcpyAsync(S0_out, slot, (size_t)H * dk * dv * sizeof(float), cudaMemcpyDeviceToDevice, stream);
 }
 
