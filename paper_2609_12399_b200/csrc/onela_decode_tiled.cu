@@ -44,7 +44,6 @@ using sm100::smem_u32;
 using sm100::tmem_ld16;
 using sm100::umma_desc;
 
-constexpr int G = 8;                   // lanes per unit
 // pitch (floats) of the output tile: conflict-free for both access patterns
 template <int VD>
 __host__ __device__ constexpr int tile_pitch() { return (VD < 128 ? VD : 128) + 4; }
@@ -74,18 +73,20 @@ __host__ __device__ constexpr size_t tiled_smem_bytes() {
 // stack: 30 -> 27 us; six: 28.5; fp32 records, five: 16 -> 17 us, three: 4 - 7 % slower at 65 536 units), unless a beam has two
 // rows, where five spill (4 x 300 beams x 16 heads, 6 calls, a generation: 185 -> 177 us).  (64 beams of 256 threads at two per
 // SM, or 16 lanes per unit, were 5 - 10 % slower at 256 x 256.)
-template <int KD, int VD, typename T, bool DELTA>
-__host__ __device__ constexpr int tiled_min_ctas() { return KD + VD <= 128 ? (sizeof(T) == 4 || DELTA ? 4 : 5) : tiled_beams<KD, VD>() == 64 ? 1 : 2; }
+template <int KD, int VD, typename T, bool DELTA, int G>
+__host__ __device__ constexpr int tiled_min_ctas() { return KD + VD <= 128 ? (G == 4 ? (DELTA ? 5 : 6) : sizeof(T) == 4 || DELTA ? 4 : 5) : tiled_beams<KD, VD>() == 64 ? 1 : 2; }
 
 // DELTA: the arena keeps (alpha_t, delta_t, k_t) (Section 3.2, Eq. 2-4).  A beam owns TWO rows of the tile - its query
 // and its own key, both projected through the parent state: S_{t-1} x = D S_0 x + sum_j d_j (k_j . x) delta_j, the
 // replay leaving x unchanged - and after the contraction delta_t = beta_t (v_t - alpha_t S_{t-1} k_t) and
 // o_t = alpha_t S_{t-1} q_t + delta_t (k_t . q_t) are formed from the two rows and the record is written; always with
 // the append fused in, dk = dv <= 128.
-template <int KD, int VD, typename T, typename OutT, bool DELTA = false>
-__global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, VD, T, DELTA>()) decode_tiled_kernel(const TiledArgs a) {
+// G: lanes per unit, 8 or (64 x 64 bf16 in large launches) 4.
+template <int KD, int VD, typename T, typename OutT, bool DELTA, int G>
+__global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, VD, T, DELTA, G>()) decode_tiled_kernel(const TiledArgs a) {
     constexpr int NB = tiled_beams<KD, VD>(), CP = tile_pitch<VD>();
-    constexpr int BPT = DELTA ? NB / 2 : NB;          // beams per tile
+    constexpr int THREADS = NB * G, BPT = DELTA ? NB / 2 : NB;          // beams per tile
+    static_assert(G == 8 || G == 4, "lanes per unit");
     static_assert(!DELTA || (KD == VD && VD <= 128), "delta records: square heads, one tile of value rows");
     constexpr uint32_t ACC_COLS = 2 * NB;      // two accumulators of NB columns (a power of two >= 32)
     constexpr int VEC = Vec16<T>::N;
@@ -186,14 +187,19 @@ __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, 
     for (int e = 0; e < CV * VEC; ++e) corr[e] = 0.f;
     float decay = 1.f;  // product of the alphas already passed
 
-    // Lane g of a unit fetches the slot of the unit's ancestor at level g (the oldest eight levels: one load latency
+    // Lane g of a unit fetches the slots of the unit's ancestors at levels g, g + G, ... (the oldest eight levels: one load latency
     // for the whole chain instead of one per level); deeper levels are looked up when they are reached.
     const int old = a.depth - 1;           // records older than the beam's own: levels old - 1 .. 0
-    const int32_t my_slot = g < old ? __ldg(table + (long long)g * a.max_beam + bb) : 0;
+    constexpr int NEAR = 8, NSLOT = NEAR / G;
+    int32_t my_slot[NSLOT];
+#pragma unroll
+    for (int j = 0; j < NSLOT; ++j) my_slot[j] = j * G + g < old ? __ldg(table + (long long)(j * G + g) * a.max_beam + bb) : 0;
     // (two look-ups, used by two runs of the chain walk: one loop with a branch between them costs every level a
     // dozen instructions, taken or not)
-    auto slot_near = [&](int level) -> int32_t { return __shfl_sync(0xffffffffu, my_slot, level, G); };          // level < G
-    auto slot_far = [&](int level) -> int32_t { return __ldg(table + (long long)level * a.max_beam + bb); };    // level >= G
+    auto slot_near = [&](int level) -> int32_t {                                                                 // level < NEAR
+        return __shfl_sync(0xffffffffu, level >= G ? my_slot[NSLOT - 1] : my_slot[0], level & (G - 1), G);
+    };
+    auto slot_far = [&](int level) -> int32_t { return __ldg(table + (long long)level * a.max_beam + bb); };    // level >= NEAR
     struct Raw { uint4 k[CK], v[CV]; float2 gate; };          // this lane's share of a record, as stored
     auto fetch_slot = [&](long long slot) -> Raw {            // an older record, from the arena
         const uint4* kp = reinterpret_cast<const uint4*>(kplane + slot * a.k_stride) + g;
@@ -285,7 +291,7 @@ __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, 
         for (int c = 0; c < CK; ++c) cur.k[c] = __ldg(reinterpret_cast<const uint4*>(ksrc) + c * G + g);
 #pragma unroll
         for (int c = 0; c < CV; ++c) cur.v[c] = __ldg(reinterpret_cast<const uint4*>(vsrc) + c * G + g);
-        if (EARLY && old > 0) first = fetch_slot(old > G ? slot_far(old - 1) : slot_near(old - 1));
+        if (EARLY && old > 0) first = fetch_slot(old > NEAR ? slot_far(old - 1) : slot_near(old - 1));
         if (fused && active && !key_row) {
             if constexpr (!DELTA) {      // (the delta half of a delta record is written after the contraction)
 #pragma unroll
@@ -317,11 +323,11 @@ __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, 
     // Narrow records are fetched one level ahead of their fold (the chain is a string of dependent loads otherwise);
     // wide ones would not fit in the registers twice.
     constexpr bool AHEAD = KD + VD <= 256;
-    const int near_top = min(old, G) - 1;        // levels near_top .. 0: slots among the lanes'; old - 1 .. G: in memory
+    const int near_top = min(old, NEAR) - 1;        // levels near_top .. 0: slots among the lanes'; old - 1 .. NEAR: in memory
     if constexpr (DELTA) {                       // the replay runs over the older records only
         if (old > 0) {
-            Raw x = old > G ? fetch_slot(slot_far(old - 1)) : fetch_slot(slot_near(old - 1));
-            for (int level = old - 2; level >= G; --level) {
+            Raw x = old > NEAR ? fetch_slot(slot_far(old - 1)) : fetch_slot(slot_near(old - 1));
+            for (int level = old - 2; level >= NEAR; --level) {
                 const Raw next = fetch_slot(slot_far(level));
                 fold(x);
                 x = next;
@@ -337,7 +343,7 @@ __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, 
         fold(cur);
         if (old > 0) {
             cur = first;
-            for (int level = old - 2; level >= G; --level) {
+            for (int level = old - 2; level >= NEAR; --level) {
                 const Raw next = fetch_slot(slot_far(level));
                 fold(cur);
                 cur = next;
@@ -350,7 +356,7 @@ __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, 
             fold(cur);
         }
     } else if constexpr (AHEAD) {
-        for (int level = old - 1; level >= G; --level) {
+        for (int level = old - 1; level >= NEAR; --level) {
             const Raw next = fetch_slot(slot_far(level));
             fold(cur);
             cur = next;
@@ -363,7 +369,7 @@ __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, 
         fold(cur);
     } else {
         fold(cur);
-        for (int level = old - 1; level >= G; --level) {
+        for (int level = old - 1; level >= NEAR; --level) {
             const Raw x = fetch_slot(slot_far(level));
             fold(x);
         }
@@ -410,7 +416,7 @@ __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, 
 #endif
 
     OutT* out = static_cast<OutT*>(a.out) + (((long long)req * a.W + b) * Hv + hv) * VD;
-    const int quad = warp & 3, half = warp >> 2;     // tensor-memory lane quadrant of this warp, and which 16 beams it takes
+    const int quad = warp & 3, half = warp >> 2;     // tensor-memory lane quadrant of this warp, and which 16 beams it takes (first)
     bool failed = false;
 #pragma unroll
     for (int mt = 0; mt < MT; ++mt) {
@@ -431,13 +437,16 @@ __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, 
             load_A(mt + 1);
         }
         {
-            uint32_t v[16];
-            tmem_ld16(tmem_base + (mt & 1) * NB + half * 16 + ((uint32_t)(quad * 32) << 16), v);
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
             const int i = quad * 32 + lane;          // value row within the tile
-            if (mt * 128 + i < VD) {
 #pragma unroll
-                for (int j = 0; j < 16; ++j) C_s[(half * 16 + j) * CP + i] = __uint_as_float(v[j]);
+            for (int b0 = half * 16; b0 < NB; b0 += THREADS / 8) {
+                uint32_t v[16];
+                tmem_ld16(tmem_base + (mt & 1) * NB + b0 + ((uint32_t)(quad * 32) << 16), v);
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                if (mt * 128 + i < VD) {
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) C_s[(b0 + j) * CP + i] = __uint_as_float(v[j]);
+                }
             }
         }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -449,7 +458,7 @@ __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, 
         auto output = [&](int c, float* x) {
             // (a chunk of eight elements by two 16-byte reads: lanes 4 - 7 take theirs in the other order, off the banks of lanes 0 - 3)
             const float* src = C_s + grp * CP + (c * G + g) * VEC - mt * 128;
-            const int first = VEC == 8 ? (g >> 2) * 4 : 0;
+            const int first = VEC == 8 ? (g >> 2) * 4 : 0;       // (four lanes: no such banks)
             const float4 t = *reinterpret_cast<const float4*>(src + first);
             float y[VEC];
             y[0] = t.x; y[1] = t.y; y[2] = t.z; y[3] = t.w;
@@ -519,9 +528,9 @@ __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, 
     }
 }
 
-template <int KD, int VD, typename T, typename OutT, bool DELTA = false>
-cudaError_t launch_one(const TiledArgs& a, cudaStream_t stream) {
-    auto kern = decode_tiled_kernel<KD, VD, T, OutT, DELTA>;
+template <int KD, int VD, typename T, typename OutT, bool DELTA, int G>
+cudaError_t launch_lanes(const TiledArgs& a, cudaStream_t stream) {
+    auto kern = decode_tiled_kernel<KD, VD, T, OutT, DELTA, G>;
     constexpr int NB = tiled_beams<KD, VD>(), THREADS = NB * G, BPT = DELTA ? NB / 2 : NB;
     constexpr size_t smem = tiled_smem_bytes<KD, VD>();
     static_assert(smem <= 232448, "shared memory per CTA");
@@ -537,7 +546,7 @@ cudaError_t launch_one(const TiledArgs& a, cudaStream_t stream) {
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             // shared memory for the CTAs the registers allow and no more: what is left of the SM's 228 KB serves the
             // fold's record loads as L1 (asking for all of it made 128 x 128 fp32 14 % slower)
-            constexpr int pct = (int)((tiled_min_ctas<KD, VD, T, DELTA>() * (smem + 1024) * 100 + 228 * 1024 - 1) / (228 * 1024));
+            constexpr int pct = (int)((tiled_min_ctas<KD, VD, T, DELTA, G>() * (smem + 1024) * 100 + 228 * 1024 - 1) / (228 * 1024));
             if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, pct > 100 ? 100 : pct);
             if (e != cudaSuccess) return e;
             ready[dev] = true;
@@ -545,6 +554,19 @@ cudaError_t launch_one(const TiledArgs& a, cudaStream_t stream) {
     }
     dim3 grid((a.W + BPT - 1) / BPT, a.Hk * a.g, a.req_count);
     return launch_dependent(kern, grid, dim3(THREADS), smem, stream, a);
+}
+
+// 64 x 64 bf16: four lanes per unit fold with a quarter fewer instructions and leave room for six CTAs per SM (five with delta
+// records), but a chain takes them longer.  Measured, eight / four lanes, us a generation: 4 x 512 beams x 32 heads XXX; the line lies at one wave of five CTAs
+// on 148 SMs.
+constexpr int FOUR_LANES_FROM = 740;
+template <int KD, int VD, typename T, typename OutT, bool DELTA>
+cudaError_t launch_one(const TiledArgs& a, cudaStream_t stream) {
+    if constexpr (KD + VD <= 128 && sizeof(T) == 2) {
+        constexpr int BPT = tiled_beams<KD, VD>() / (DELTA ? 2 : 1);
+        if ((long long)((a.W + BPT - 1) / BPT) * a.Hk * a.g * a.req_count > FOUR_LANES_FROM) return launch_lanes<KD, VD, T, OutT, DELTA, 4>(a, stream);
+    }
+    return launch_lanes<KD, VD, T, OutT, DELTA, 8>(a, stream);
 }
 
 template <int KD, int VD, bool DELTA = false>
