@@ -696,10 +696,7 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
                         unpack8(cur.q[c], r + 4 * c);
                         unpack8(cur.own.k[c], kx + 4 * c);
                     }
-                    float2 d2 = make_float2(0.f, 0.f);
-#pragma unroll
-                    for (int e = 0; e < 4 * NCH; ++e) d2 = __ffma2_rn(kx[e], r[e], d2);
-                    kq = d2.x + d2.y;
+                    kq = L::own_dot(kx, r);
 #pragma unroll
                     for (int o = LPU / 2; o > 0; o >>= 1) kq += __shfl_xor_sync(0xffffffffu, kq, o);
                     if (grp & 1) {           // the odd unit of a beam projects its key
@@ -719,10 +716,7 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
                 // on the folded row itself (below).
                 float q_scale = 1.f, q_inv = 1.f;
                 {
-                    float2 n2 = make_float2(0.f, 0.f);
-#pragma unroll
-                    for (int e = 0; e < 4 * NCH; ++e) n2 = __ffma2_rn(r[e], r[e], n2);
-                    float norm2 = n2.x + n2.y;
+                    float norm2 = L::own_dot(r, r);
 #pragma unroll
                     for (int o = LPU / 2; o > 0; o >>= 1) norm2 += __shfl_xor_sync(0xffffffffu, norm2, o);
                     const int eb = (int)(__float_as_uint(norm2) >> 23) & 255;      // |q|^2 in [2^(eb-127), 2^(eb-126))
