@@ -44,18 +44,15 @@ namespace {
 using namespace sm100;
 
 #ifndef ONELA_FOLD_WARPS
-#define ONELA_FOLD_WARPS 8
+#define ONELA_FOLD_WARPS 12
 #endif
 constexpr int FOLD_WARPS = ONELA_FOLD_WARPS;
-constexpr int LPU = 4;                              // lanes per (beam, head) unit
-constexpr int UPW = 32 / LPU;                       // units a fold warp folds at a time (a "quad" below)
+constexpr int LPU = 8;                              // lanes per (beam, head) unit
+constexpr int UPW = 32 / LPU;                       // units a fold warp folds at a time (a "quad" when LPU = 8)
 constexpr int NCH = 16 / LPU;                       // 16-byte chunks per lane per 256-byte vector
-constexpr int THREADS = (FOLD_WARPS + 8) * 32;      // + 4 epilogue warps + the warp that issues the MMAs and three that complete its warpgroup
-// Registers: 16 warps start with 128 each; the fold warps take what the issuing warp's group leaves.
-constexpr int FOLD_REGS = 160, EPI_REGS = 136, MMA_REGS = 56;
-static_assert(FOLD_WARPS * FOLD_REGS + 4 * EPI_REGS + 4 * MMA_REGS <= 16 * 128, "a split beyond the launch's registers waits for ever");
+constexpr int THREADS = (FOLD_WARPS + 5) * 32;      // + 4 epilogue warps + the warp that issues the MMAs
 constexpr int MMA_WARP = FOLD_WARPS + 4;
-constexpr int GN = FOLD_WARPS * UPW;                // beams per group = MMA N (64)
+constexpr int GN = FOLD_WARPS * UPW;                // beams per group = MMA N (48)
 constexpr int R_KB_STRIDE = GN * 128;               // bytes between the two K blocks (64 fp16 each) of the operand
 constexpr int OUT_PITCH = 256 + 16;                 // bytes between the rows of a group's bf16 outputs (bank-conflict-free)
 constexpr int R_BYTES = GN * OUT_PITCH;             // a slot's first tile: the group's operand rows, later its outputs as bf16
@@ -89,15 +86,15 @@ constexpr int SMEM_BYTES = SLOTS * SLOT_BYTES + STAGE_BYTES + GATE_BYTES + HEADS
 constexpr int DELTA_BEAMS = GN / 2;
 constexpr int DELTA_V_PITCH = DV * 2 + 16;       // (bank-conflict-free)
 constexpr int DELTA_SLOT_BYTES = DELTA_BEAMS * DELTA_V_PITCH + DELTA_BEAMS * 16;
-constexpr int SMEM_BYTES_DELTA = SMEM_BYTES - HEADS_TOTAL / 2 + SLOTS * DELTA_SLOT_BYTES;      // (the two units of a beam share its heads)
+constexpr int SMEM_BYTES_DELTA = SMEM_BYTES + SLOTS * DELTA_SLOT_BYTES;
 static_assert(SMEM_BYTES_DELTA <= 232448, "shared memory per CTA (delta records)");
 constexpr uint32_t S0_COL = 128;                 // accumulators of the ring slots in [0, SLOTS * GN); S_0 buffers (64 columns) at 128 and 256
 constexpr int R_TARGET = 8;                      // a scaled operand row's largest element lies in [2^8, 2^9) x (decay in [1, 2)): far inside fp16's range
 constexpr uint32_t TMEM_COLS = 512;
-static_assert(SLOTS * GN <= 128 && GN == 64, "accumulator columns");
+static_assert(SLOTS * GN <= 128 && GN == 48, "accumulator columns");
 // Where chains share too little to be staged (see gather_queued) the staging area holds two gathered records per unit instead.
-constexpr int QUEUE_SLOT = UPW * REC_BYTES;          // a quad's records of one level (their gates lie where the staged ones' do)
-static_assert(FOLD_WARPS * 2 * QUEUE_SLOT <= STAGE_BYTES && FOLD_WARPS * 2 * UPW * 8 <= GATE_BYTES, "gather queues");
+constexpr int QUEUE_SLOT = UPW * REC_BYTES + 64;     // a quad's records of one level, then their gates
+static_assert(FOLD_WARPS * 2 * QUEUE_SLOT <= STAGE_BYTES && LPU >= 8, "gather queues");
 static_assert(2 * STAGE_BUF <= 128, "one staged record per epilogue lane");
 static_assert(SMEM_BYTES <= 232448, "shared memory per CTA");
 static_assert(GN % 16 == 0 && GN >= 16 && GN <= 256, "MMA N");
@@ -143,7 +140,7 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 
 // Position of 16-byte chunk q (4 floats) of a corr-tile row: chunks swap in pairs in every other 128-byte stretch,
 // which keeps the fold warps' 32-byte-strided writes and the epilogue's 32-byte-strided reads off shared banks.
-__device__ __forceinline__ int corr_chunk(int q, int row) { return q ^ (((q >> 3) ^ row) & 1); }
+__device__ __forceinline__ int corr_chunk(int q) { return q ^ ((q >> 3) & 1); }
 
 struct Head {           // what a unit's fold needs first
     uint4 q[NCH];
@@ -175,15 +172,14 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
     uint8_t* stage = ring + SLOTS * SLOT_BYTES;
     float2* gates_s = reinterpret_cast<float2*>(stage + STAGE_BYTES);
     uint8_t* heads = stage + STAGE_BYTES + GATE_BYTES;
-    constexpr int HEADS = DELTA ? HEADS_TOTAL / 2 : HEADS_TOTAL;
-    uint64_t* bars = reinterpret_cast<uint64_t*>(heads + HEADS);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(heads + HEADS_TOTAL);
     // bars: per S_0 / staging buffer b: S_0 in tensor memory, records staged, staging buffer read out;
     //       per ring slot s: full, MMA done, free
     const uint32_t bar_s0_first = smem_u32(bars + 6 + 3 * SLOTS);   // the first segment's S_0, put there by all warps
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 7 + 3 * SLOTS);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-    float* inv_s = reinterpret_cast<float*>(heads + HEADS + 256);      // [SLOTS][GN]
-    uint8_t* delta_s = heads + HEADS + 256 + INV_BYTES;                // DELTA: [SLOTS][value rows | scalars]
+    float* inv_s = reinterpret_cast<float*>(heads + HEADS_TOTAL + 256);      // [SLOTS][GN]
+    uint8_t* delta_s = heads + HEADS_TOTAL + 256 + INV_BYTES;                // DELTA: [SLOTS][value rows | scalars]
 #ifdef ONELA_WS_TL
     unsigned long long* tl_s = reinterpret_cast<unsigned long long*>(delta_s + (DELTA ? SLOTS * DELTA_SLOT_BYTES : 0));
     const int tl_role = (int)blockIdx.x != g_ws_tl_cta ? -1 : warp == 0 ? 0 : warp == MMA_WARP ? 1 : warp == FOLD_WARPS ? 2 : -1;
@@ -209,7 +205,7 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
             mbar_init(bar_done(s), 1);                // tcgen05.commit
             mbar_init(bar_free(s), 4);                // the four epilogue warps
         }
-        mbar_init(bar_s0_first, FOLD_WARPS);          // the fold warps, which bring the first S_0 in
+        mbar_init(bar_s0_first, 16);                  // the sixteen warps that bring the first S_0 in
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -256,12 +252,6 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
                        : kv + ((long long)h * a.arena_slots + slot) * REC_BYTES + DK * 2;
     };
     const int grp = lane / LPU, g = lane % LPU;
-    // A lane owns 16-byte chunks (its elements [8 x, 8 x + 8)) of every 256-byte vector: LPU consecutive lanes take 64
-    // consecutive bytes, and every other unit of a warp takes the 64-byte halves of a 128-byte stretch in the opposite order, so
-    // that two units reading different rows of shared memory never meet on a bank.  Byte offset of the lane's c-th chunk:
-    const int chunk_even = g * 16 + (grp & 1) * 64, chunk_odd = chunk_even ^ 64;
-    auto chunk = [&](int c) { return ((c & 1) ? chunk_odd : chunk_even) + (c >> 1) * 128; };
-    static_assert(LPU == 4 && NCH == 4, "chunk order");
     bool dead = false;                    // this warp gave up (timeout or abort raised elsewhere)
 
     // S_0 of a (request, head) goes to tensor memory as fp16 (TF32's mantissa; K = 16 per MMA instead of 8), times
@@ -316,29 +306,24 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
     // launch's dependencies are waited for: see launch_dependent for why the store, and nothing else, may be read
     // there.  (Put there after the first heads had been requested, it stood
     // between them and the fold: 0.4 us of a launch of 128 x 16 to 512 x 32 units, 1 - 1.5 %; large launches are the same.)
-    static_assert(FOLD_WARPS == 8, "a fold warp takes two 32-column blocks of the first S_0");
-    const bool s0_mine = warp < FOLD_WARPS;
-    float4 s0_first[2][8];
+    static_assert(THREADS >= 512, "the first sixteen warps take one 32-column block of the first S_0 each");
+    const bool s0_mine = warp < 16;
+    float4 s0_first[8];
     float s0_first_scale = 1.f;
     if (n_segs > 0 && s0_mine) {
         const int req = req_begin, h = h_begin;
         s0_first_scale = __ldg(a.s0_scale + req * a.s0_scale_req_stride + value_head(h));
-#pragma unroll
-        for (int j = 0; j < 2; ++j)
-            request_s0(a.s0 + req * a.s0_req_stride + (long long)h * (DV * DK) + s0_fragment(warp & 3) + ((warp >> 2) * 2 + j) * 32, s0_first[j]);
+        request_s0(a.s0 + req * a.s0_req_stride + (long long)h * (DV * DK) + s0_fragment(warp & 3) + (warp >> 2) * 32, s0_first);
         if (n_segs > 1) {
             int nreq, nh;
             pair_of(1, nreq, nh);
-            const float* nrow = a.s0 + nreq * a.s0_req_stride + (long long)nh * (DV * DK) + (long long)((warp & 3) * 32 + lane) * DK + (warp >> 2) * 64;
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(nrow));
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(nrow + 32));
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(a.s0 + nreq * a.s0_req_stride + (long long)nh * (DV * DK) +
+                                                          (long long)((warp & 3) * 32 + lane) * DK + (warp >> 2) * 32));
         }
     }
     auto put_first_s0 = [&]() {
         if (n_segs == 0 || !s0_mine) return;
-#pragma unroll
-        for (int j = 0; j < 2; ++j)
-            store_s0(tmem_base + S0_COL + ((warp >> 2) * 2 + j) * 16 + ((uint32_t)((warp & 3) * 32) << 16), s0_first[j], s0_first_scale);
+        store_s0(tmem_base + S0_COL + (warp >> 2) * 16 + ((uint32_t)((warp & 3) * 32) << 16), s0_first, s0_first_scale);
         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncwarp();
@@ -391,13 +376,10 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
     };
 
     if (warp < FOLD_WARPS) {
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(FOLD_REGS));
         // =============================== FOLD ===============================
         // Quad k of this warp belongs to group g_begin + k: rows UPW * warp .. + UPW - 1 of the group.
         const int n_quads = g_end - g_begin;
-        constexpr int HEAD_ROWS = DELTA ? UPW / 2 : UPW;        // (DELTA: the two units of a beam share its head)
-        uint8_t* my_heads = heads + warp * (HEAD_ROWS * (HEAD_BYTES / UPW));
-        const int hrow = DELTA ? grp >> 1 : grp;
+        uint8_t* my_heads = heads + warp * HEAD_BYTES;
         // segment, request, head, group within the (request, head) pair; GROUPED: the head's key head and its place among that
         // key head's heads, its value head and its place among that one's tiles - carried along, not divided out for every quad
         // (the divisions were a sixth of the grouped launches' time: 128 x 256 on 16 value heads 24.2 -> 20.8 us)
@@ -440,10 +422,9 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
         // registers.  The lines of the FIRST quad are requested into L2 before the launch's dependencies are waited
         // for (requesting every later quad's lines a quad ahead of its copies as well measured 2 % slower).
         auto request_heads = [&](const Unit& n) {        // the 128-byte lines of a quad's heads, into L2
-#pragma unroll 1
-            for (int x = lane; x < HEAD_ROWS * 6; x += 32) {
-                const int un = x / 6, item = x % 6;
-                const int b2 = min(n.gip * BPG + HEAD_ROWS * warp + un, a.W - 1);
+            if (lane < UPW * 6) {
+                const int un = lane / 6, item = lane % 6;
+                const int b2 = min(n.gip * BPG + (DELTA ? (UPW * warp + un) >> 1 : UPW * warp + un), a.W - 1);
                 const long long krow2 = krow_of(n, b2), vrow2 = vrow_in(n.req, b2, n.h);
                 const long long slot2 = a.bases.base[n.req] + b2;
                 const char* p2 = item < 2 ? reinterpret_cast<const char*>(qbase) + krow2 * (DK * 2)
@@ -454,36 +435,30 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
             }
         };
         auto issue_head = [&](const Unit& u) {
-            const uint32_t dst = smem_u32(my_heads) + hrow * REC_BYTES, qdst = smem_u32(my_heads) + HEAD_ROWS * REC_BYTES + hrow * (DK * 2);
+            const uint32_t dst = smem_u32(my_heads);
             const int bb = live_beam(u);
             const long long krow = krow_of(u, bb);
-            const char* qr = reinterpret_cast<const char*>(qbase + krow * DK);
-            const char *kr, *vr;
+            const char* qr = reinterpret_cast<const char*>(qbase + krow * DK) + g * 16;
             if (fused) {   // the call's records come straight from the caller's k and v tensors
-                kr = static_cast<const char*>(a.k_in) + krow * (DK * 2);
-                vr = static_cast<const char*>(a.v_in) + vrow_in(u.req, bb, u.h) * (DV * 2);
-            } else {
-                const long long slot = a.bases.base[u.req] + bb;
-                kr = k_of(u, slot);
-                vr = v_of(u, slot);
-            }
-            if constexpr (DELTA) {     // a beam's even unit copies the key, its odd one the value, each half of the query
-                const char* from = (grp & 1) ? vr : kr;
-                const uint32_t to = dst + (grp & 1) * (DK * 2);
-#pragma unroll
-                for (int c = 0; c < NCH; ++c) cp_async16(to + chunk(c), from + chunk(c));
-                const int half = (grp & 1) * 128;
-#pragma unroll
-                for (int c = 0; c < NCH / 2; ++c) cp_async16(qdst + half + chunk(c), qr + half + chunk(c));
-            } else {
+                const char* kr = static_cast<const char*>(a.k_in) + krow * (DK * 2) + g * 16;
+                const char* vr = static_cast<const char*>(a.v_in) + vrow_in(u.req, bb, u.h) * (DV * 2) + g * 16;
 #pragma unroll
                 for (int c = 0; c < NCH; ++c) {
-                    cp_async16(dst + chunk(c), kr + chunk(c));
-                    cp_async16(dst + DK * 2 + chunk(c), vr + chunk(c));
+                    cp_async16(dst + grp * REC_BYTES + (c * LPU + g) * 16, kr + c * LPU * 16);
+                    cp_async16(dst + grp * REC_BYTES + (16 + c * LPU + g) * 16, vr + c * LPU * 16);
                 }
+            } else {
+                const long long slot = a.bases.base[u.req] + bb;
+                const char* kr = k_of(u, slot) + g * 16;
+                const char* vr = v_of(u, slot) + g * 16;
 #pragma unroll
-                for (int c = 0; c < NCH; ++c) cp_async16(qdst + chunk(c), qr + chunk(c));
+                for (int c = 0; c < NCH; ++c) {
+                    cp_async16(dst + grp * REC_BYTES + (c * LPU + g) * 16, kr + c * LPU * 16);
+                    cp_async16(dst + grp * REC_BYTES + (16 + c * LPU + g) * 16, vr + c * LPU * 16);
+                }
             }
+#pragma unroll
+            for (int c = 0; c < NCH; ++c) cp_async16(dst + UPW * REC_BYTES + grp * (DK * 2) + (c * LPU + g) * 16, qr + c * LPU * 16);
             asm volatile("cp.async.commit_group;" ::: "memory");
         };
         auto load_gate = [&](const Unit& u) {
@@ -502,10 +477,6 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
         constexpr int NIDX = LPU >= 8 ? 1 : 8 / LPU;     // the unit's lanes hold the indices of its first 8 levels
         static_assert(NIDX * LPU >= 8, "staging_of stages up to eight levels: their indices must be among the lanes'");
         struct Idx { int32_t v[NIDX]; };
-        auto near_idx = [&](const Idx& x, int level) -> int32_t {          // level < NIDX * LPU
-            static_assert(NIDX <= 2, "the index of a level");
-            return __shfl_sync(0xffffffffu, NIDX > 1 && level >= LPU ? x.v[NIDX - 1] : x.v[0], level & (LPU - 1), LPU);
-        };
         auto load_idx = [&](const Unit& u) -> Idx {
             const int sl = staged_levels_of(u.req);
             const int bb = live_beam(u);
@@ -534,24 +505,21 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
         // The first quad's indices, asked for in both places where they may stand, beside the levels' ends that tell which
         // of the two counts: one latency instead of two.  (With the same for the first staging list and no wait for the
         // segment's scale: 8 layers x 128 beams x 16 heads, depth 4, 209 -> 201 us a generation; 4 x 512 x 32, 1.5 %.)
-        int32_t in_table[NIDX] = {}, in_list[NIDX] = {};
+        int32_t in_table = 0, in_list = 0;
         int ends = 0x7fffffff;
         if (n_quads > 0) {
             ends = ends_of(req_begin);
-#pragma unroll
-            for (int j = 0; j < NIDX; ++j)
-                if (j * LPU + g < old) {
-                    const long long at = (long long)(j * LPU + g) * a.max_beam + live_beam(u0);
-                    in_table[j] = __ldg(a.table + u0.req * a.table_req_stride + at);
-                    in_list[j] = __ldg(a.sidx + u0.req * a.sidx_req_stride + at);
-                }
+            if (g < old) {
+                const long long at = (long long)g * a.max_beam + live_beam(u0);
+                in_table = __ldg(a.table + u0.req * a.table_req_stride + at);
+                in_list = __ldg(a.sidx + u0.req * a.sidx_req_stride + at);
+            }
         }
         TL(2, 0);   // dependencies waited for, first heads requested
         if (n_quads > 0) {
             queued = gather_queued(ends, info_levels, info_count);
             info_req = req_begin;
-#pragma unroll
-            for (int j = 0; j < NIDX; ++j) idx_next.v[j] = j * LPU + g < info_levels ? in_list[j] : in_table[j];
+            idx_next.v[0] = g < info_levels ? in_list : in_table;
         }
         TL(3, 0);   // first indices there
         int cur_seg = -1, buf = 0, staged_levels = 0;
@@ -564,21 +532,20 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
             constexpr bool QUEUE = decltype(queue_tag)::value;
             const bool two = old >= 2;               // gathers in flight: two, or the one older level there is
             uint8_t* my_queue = stage + warp * (2 * QUEUE_SLOT);
-            float2* my_queue_gates = gates_s + warp * (2 * UPW);
             const uint32_t queue_at = smem_u32(my_queue);
             int q_in = 0, q_out = 0;                 // place in the queue of the next request / the next record
             auto queue_record = [&](const Unit& n, const Idx& ix, int item) {      // the item-th older record, newest first, of quad n's units
                 const int level = old - 1 - item;
-                const int32_t near = near_idx(ix, level);
-                const int32_t slot = level < NIDX * LPU ? near : __ldg(a.table + n.req * a.table_req_stride + (long long)level * a.max_beam + live_beam(n));
-                const char *kp = k_of(n, slot), *vp = v_of(n, slot);
-                const uint32_t dst = queue_at + q_in * QUEUE_SLOT + grp * REC_BYTES;
+                const int32_t near = __shfl_sync(0xffffffffu, ix.v[0], level & (LPU - 1), LPU);
+                const int32_t slot = level < LPU ? near : __ldg(a.table + n.req * a.table_req_stride + (long long)level * a.max_beam + live_beam(n));
+                const char *kp = k_of(n, slot) + g * 16, *vp = v_of(n, slot) + g * 16;
+                const uint32_t dst = queue_at + q_in * QUEUE_SLOT + grp * REC_BYTES + g * 16;
 #pragma unroll
                 for (int c = 0; c < NCH; ++c) {
-                    cp_async16(dst + chunk(c), kp + chunk(c));
-                    cp_async16(dst + DK * 2 + chunk(c), vp + chunk(c));
+                    cp_async16(dst + c * LPU * 16, kp + c * LPU * 16);
+                    cp_async16(dst + DK * 2 + c * LPU * 16, vp + c * LPU * 16);
                 }
-                if (g == 0) cp_async8(smem_u32(my_queue_gates + q_in * UPW + grp), a.gates + (long long)value_head_of(n) * a.arena_slots + slot);
+                if (g == 0) cp_async8(queue_at + q_in * QUEUE_SLOT + UPW * REC_BYTES + grp * 8, a.gates + (long long)value_head_of(n) * a.arena_slots + slot);
                 q_in ^= two ? 1 : 0;
             };
             auto commit = [&]() { asm volatile("cp.async.commit_group;" ::: "memory"); };
@@ -615,16 +582,14 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
                     if (QUEUE) wait_but(std::integral_constant<int, 1>{});      // (younger: the first gathers of this quad)
                     else asm volatile("cp.async.wait_group 0;" ::: "memory");
                     TL(11, k);  // fold: heads landed
-                    if (DELTA) __syncwarp();                 // (each unit of a beam has copied a part)
-                    const uint8_t* rec = my_heads + hrow * REC_BYTES;
-                    const uint8_t* qv = my_heads + HEAD_ROWS * REC_BYTES + hrow * (DK * 2);
+                    const uint4* rec = reinterpret_cast<const uint4*>(my_heads + grp * REC_BYTES) + g;
+                    const uint4* qv = reinterpret_cast<const uint4*>(my_heads + UPW * REC_BYTES + grp * (DK * 2)) + g;
 #pragma unroll
                     for (int c = 0; c < NCH; ++c) {
-                        cur.own.k[c] = *reinterpret_cast<const uint4*>(rec + chunk(c));
-                        cur.own.v[c] = *reinterpret_cast<const uint4*>(rec + DK * 2 + chunk(c));
-                        cur.q[c] = *reinterpret_cast<const uint4*>(qv + chunk(c));
+                        cur.own.k[c] = rec[c * LPU];
+                        cur.own.v[c] = rec[16 + c * LPU];
+                        cur.q[c] = qv[c * LPU];
                     }
-                    if (DELTA) __syncwarp();
                     cur.own.gate = gate0;
                     // the next quad's copies go out before this quad's stores (each lane overwrites only the chunks it
                     // has just read)
@@ -633,28 +598,28 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
                     if (DELTA) {
                         // the key half of the record and the gates; delta_t follows from the epilogue
                         if ((grp & 1) == 0 && beam_of(u0) < a.W) {
-                            char* dst = a.kv_out + (own_row0 + bb) * REC_BYTES;
+                            uint4* dst = reinterpret_cast<uint4*>(a.kv_out + (own_row0 + bb) * REC_BYTES) + g;
 #pragma unroll
-                            for (int c = 0; c < NCH; ++c) *reinterpret_cast<uint4*>(dst + chunk(c)) = cur.own.k[c];
+                            for (int c = 0; c < NCH; ++c) dst[c * LPU] = cur.own.k[c];
                             if (g == 0) a.gates_out[own_row0 + bb] = gate0;
                         }
                     } else if (fused && beam_of(u0) < a.W) {   // the append: this beam's record goes to its arena slot, bit for bit
                         if constexpr (GROUPED) {
                             const long long slot = a.bases.base[u0.req] + bb;
-                            char* vdst = a.vv_out + (v_of(u0, slot) - a.vv);
+                            uint4* vdst = reinterpret_cast<uint4*>(a.vv_out + (v_of(u0, slot) - a.vv)) + g;
 #pragma unroll
-                            for (int c = 0; c < NCH; ++c) *reinterpret_cast<uint4*>(vdst + chunk(c)) = cur.own.v[c];
+                            for (int c = 0; c < NCH; ++c) vdst[c * LPU] = cur.own.v[c];
                             if (u0.ki == 0) {     // the key is stored once per key head: by its first value head
-                                char* kdst = a.kv_out + (k_of(u0, slot) - kv);
+                                uint4* kdst = reinterpret_cast<uint4*>(a.kv_out + (k_of(u0, slot) - kv)) + g;
 #pragma unroll
-                                for (int c = 0; c < NCH; ++c) *reinterpret_cast<uint4*>(kdst + chunk(c)) = cur.own.k[c];
+                                for (int c = 0; c < NCH; ++c) kdst[c * LPU] = cur.own.k[c];
                             }
                         } else {
-                            char* dst = a.kv_out + (own_row0 + bb) * REC_BYTES;
+                            uint4* dst = reinterpret_cast<uint4*>(a.kv_out + (own_row0 + bb) * REC_BYTES) + g;
 #pragma unroll
                             for (int c = 0; c < NCH; ++c) {
-                                *reinterpret_cast<uint4*>(dst + chunk(c)) = cur.own.k[c];
-                                *reinterpret_cast<uint4*>(dst + DK * 2 + chunk(c)) = cur.own.v[c];
+                                dst[c * LPU] = cur.own.k[c];
+                                dst[16 + c * LPU] = cur.own.v[c];
                             }
                         }
                         if (g == 0 && (!GROUPED || u0.vi == 0)) a.gates_out[own_row0 + bb] = gate0;
@@ -668,23 +633,27 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
                 const Idx my_idx = idx_next;
                 if (k + 1 < n_quads) idx_next = load_idx(u1);
                 auto idx_of = [&](int level) -> int32_t {
-                    const int32_t t = near_idx(my_idx, level);
+                    int32_t t = 0;
+#pragma unroll
+                    for (int j = 0; j < NIDX; ++j) {
+                        const int32_t x = __shfl_sync(0xffffffffu, my_idx.v[j], level & (LPU - 1), LPU);
+                        if (j == level / LPU) t = x;
+                    }
                     return level < NIDX * LPU ? t
                                               : __ldg((level < staged_levels ? sidx_r : table_r) + (long long)level * a.max_beam + bb);
                 };
                 // The same for a staged level: always among the lanes' (staging_of stages no level beyond them), so no
                 // branch to the look-up in memory stands in the staged fold - merely being there, never taken, it cost
                 // every level a dozen instructions (2.77 -> 2.5 us per level on the beam-512 stack).
-                auto staged_idx_of = [&](int level) -> int32_t { return near_idx(my_idx, level); };
-                auto record_at = [&](const uint8_t* p, const float2* gate) {         // a record in shared memory
-                    RecT rec;
+                auto staged_idx_of = [&](int level) -> int32_t {
+                    if constexpr (NIDX == 1) return __shfl_sync(0xffffffffu, my_idx.v[0], level, LPU);   // level < LPU
+                    int32_t t = 0;
 #pragma unroll
-                    for (int c = 0; c < NCH; ++c) {
-                        rec.k[c] = *reinterpret_cast<const uint4*>(p + chunk(c));
-                        rec.v[c] = *reinterpret_cast<const uint4*>(p + DK * 2 + chunk(c));
+                    for (int j = 0; j < NIDX; ++j) {
+                        const int32_t x = __shfl_sync(0xffffffffu, my_idx.v[j], level & (LPU - 1), LPU);
+                        if (j == level / LPU) t = x;
                     }
-                    rec.gate = *gate;
-                    return rec;
+                    return t;
                 };
 
                 float2 r[4 * NCH], corr[4 * NCH];
@@ -696,7 +665,10 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
                         unpack8(cur.q[c], r + 4 * c);
                         unpack8(cur.own.k[c], kx + 4 * c);
                     }
-                    kq = L::own_dot(kx, r);
+                    float2 d2 = make_float2(0.f, 0.f);
+#pragma unroll
+                    for (int e = 0; e < 4 * NCH; ++e) d2 = __ffma2_rn(kx[e], r[e], d2);
+                    kq = d2.x + d2.y;
 #pragma unroll
                     for (int o = LPU / 2; o > 0; o >>= 1) kq += __shfl_xor_sync(0xffffffffu, kq, o);
                     if (grp & 1) {           // the odd unit of a beam projects its key
@@ -716,7 +688,10 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
                 // on the folded row itself (below).
                 float q_scale = 1.f, q_inv = 1.f;
                 {
-                    float norm2 = L::own_dot(r, r);
+                    float2 n2 = make_float2(0.f, 0.f);
+#pragma unroll
+                    for (int e = 0; e < 4 * NCH; ++e) n2 = __ffma2_rn(r[e], r[e], n2);
+                    float norm2 = n2.x + n2.y;
 #pragma unroll
                     for (int o = LPU / 2; o > 0; o >>= 1) norm2 += __shfl_xor_sync(0xffffffffu, norm2, o);
                     const int eb = (int)(__float_as_uint(norm2) >> 23) & 255;      // |q|^2 in [2^(eb-127), 2^(eb-126))
@@ -728,15 +703,20 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
                 }
                 auto gather = [&](int level) {
                                   const long long slot = idx_of(level);
-                                  RecT rec;
-                                  const char *kp = k_of(u0, slot), *vp = v_of(u0, slot);
+                                  if constexpr (GROUPED) {
+                                      RecT rec;
+                                      const uint4* kp = reinterpret_cast<const uint4*>(k_of(u0, slot)) + g;
+                                      const uint4* vp = reinterpret_cast<const uint4*>(v_of(u0, slot)) + g;
 #pragma unroll
-                                  for (int c = 0; c < NCH; ++c) {
-                                      rec.k[c] = __ldg(reinterpret_cast<const uint4*>(kp + chunk(c)));
-                                      rec.v[c] = __ldg(reinterpret_cast<const uint4*>(vp + chunk(c)));
+                                      for (int c = 0; c < NCH; ++c) {
+                                          rec.k[c] = __ldg(kp + c * LPU);
+                                          rec.v[c] = __ldg(vp + c * LPU);
+                                      }
+                                      rec.gate = __ldg(a.gates + plane_row0 + slot);
+                                      return rec;
+                                  } else {
+                                      return L::load_global(kv, a.gates, plane_row0 + slot, g);
                                   }
-                                  rec.gate = __ldg(a.gates + plane_row0 + slot);
-                                  return rec;
                               };
                 if constexpr (QUEUE) {
                     if (!DELTA) L::template fold_step<false>(cur.own, r, corr, decay);
@@ -746,7 +726,15 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
                         if (item < (two ? 2 : 1)) wait_but(std::integral_constant<int, 1>{});
                         else wait_but(std::integral_constant<int, 0>{});
                         __syncwarp();                        // (the gates were copied by the unit's first lane)
-                        const RecT rec = record_at(my_queue + q_out * QUEUE_SLOT + grp * REC_BYTES, my_queue_gates + q_out * UPW + grp);
+                        const uint8_t* slot_s = my_queue + q_out * QUEUE_SLOT;
+                        const uint4* p = reinterpret_cast<const uint4*>(slot_s + grp * REC_BYTES) + g;
+                        RecT rec;
+#pragma unroll
+                        for (int c = 0; c < NCH; ++c) {
+                            rec.k[c] = p[c * LPU];
+                            rec.v[c] = p[16 + c * LPU];
+                        }
+                        rec.gate = *reinterpret_cast<const float2*>(slot_s + UPW * REC_BYTES + grp * 8);
                         q_out ^= two ? 1 : 0;
                         __syncwarp();                        // the place is read out: the record after the next (the next) takes it
                         const int next = item + (two ? 2 : 1);
@@ -772,12 +760,9 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
                 if (staged_levels > 0) {
                     const uint8_t* st = stage + buf * (STAGE_BUF * REC_BYTES);
                     const float2* gs = gates_s + buf * STAGE_BUF;
-                    auto staged = [&](int level) {
-                        const int32_t at = staged_idx_of(level);
-                        return record_at(st + at * REC_BYTES, gs + at);
-                    };
-                    const RecT newest = staged(staged_levels - 1);
-                    L::template fold_chain_simple<DELTA>(newest, staged_levels - 2, 0, staged, r, corr, decay);
+                    const RecT newest = L::load_shared(st, gs, staged_idx_of(staged_levels - 1), g);
+                    L::template fold_chain_simple<DELTA>(newest, staged_levels - 2, 0,
+                                  [&](int level) { return L::load_shared(st, gs, staged_idx_of(level), g); }, r, corr, decay);
                 }
                 if (seg_last) {                    // this warp's last read of the segment's staging buffer
                     __syncwarp();
@@ -791,9 +776,10 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
                 uint8_t* R_s = ring + s * SLOT_BYTES;
                 float* C_s = reinterpret_cast<float*>(R_s + R_BYTES);
                 {
-                    // Bank conflicts: the units of a warp's even and odd rows write opposite halves of a 128-byte stretch at a time
-                    // (see chunk); the corr tile (a layout of our own) swaps each pair of 16-byte chunks in every other 128-byte
-                    // stretch of a row, starting with the first in odd rows (corr_chunk; the epilogue reads it the same way).
+                    // Bank conflicts: the lanes g and g + 4 of a unit own the same chunk positions of two operand rows
+                    // 48 * 128 bytes apart, so the upper four lanes write their two chunks in the opposite order;
+                    // the corr tile (a layout of our own) swaps each pair of 16-byte chunks in every other 128-byte
+                    // stretch of a row instead (corr_chunk; the epilogue reads it the same way).
                     const int sw = u & 7;
                     // The folded query decay * r~ goes out as fp16 times two powers of two: the one that brings the decay into
                     // [1, 2) and the row's own (the guess taken from |q| when the quad started: |r~| < 2^R_TARGET / q_scale).
@@ -824,20 +810,20 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
                     const float2 dc = make_float2(dcs, dcs);
 #pragma unroll
                     for (int c = 0; c < NCH; ++c) {
-                        const int ci = chunk(c) >> 4;               // elements [8 ci, 8 ci + 8)
+                        const int ci = c * LPU + g;                 // elements [8 ci, 8 ci + 8)
                         float2 x[4];
 #pragma unroll
                         for (int e = 0; e < 4; ++e) x[e] = __fmul2_rn(r[4 * c + e], dc);
                         // fp16 operand rows: K blocks of 64 elements (128 bytes, 128-byte swizzle), one 16-byte chunk
                         // per lane and c; a warp's four rows are 512 consecutive bytes: no bank conflicts
-                        uint8_t* row = R_s + (c >> 1) * R_KB_STRIDE + u * 128;
+                        uint8_t* row = R_s + (ci >> 3) * R_KB_STRIDE + u * 128;
                         *reinterpret_cast<uint4*>(row + (((ci & 7) ^ sw) << 4)) =
                             make_uint4(pack_f16x2(x[0].x, x[0].y), pack_f16x2(x[1].x, x[1].y), pack_f16x2(x[2].x, x[2].y),
                                        pack_f16x2(x[3].x, x[3].y));
                         float* crow = C_s + u * C_PITCH;
-                        *reinterpret_cast<float4*>(crow + (2 * ci + (c & 1)) * 4) =
+                        *reinterpret_cast<float4*>(crow + corr_chunk(2 * ci) * 4) =
                             make_float4(corr[4 * c].x, corr[4 * c].y, corr[4 * c + 1].x, corr[4 * c + 1].y);
-                        *reinterpret_cast<float4*>(crow + (2 * ci + 1 - (c & 1)) * 4) =
+                        *reinterpret_cast<float4*>(crow + corr_chunk(2 * ci + 1) * 4) =
                             make_float4(corr[4 * c + 2].x, corr[4 * c + 2].y, corr[4 * c + 3].x, corr[4 * c + 3].y);
                     }
                 }
@@ -845,7 +831,7 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
                     uint8_t* ds = delta_s + s * DELTA_SLOT_BYTES;
                     const int bq = u >> 1;
 #pragma unroll
-                    for (int c = 0; c < NCH; ++c) *reinterpret_cast<uint4*>(ds + bq * DELTA_V_PITCH + chunk(c)) = cur.own.v[c];
+                    for (int c = 0; c < NCH; ++c) *reinterpret_cast<uint4*>(ds + bq * DELTA_V_PITCH + (c * LPU + g) * 16) = cur.own.v[c];
                     if (g == 0) *reinterpret_cast<float4*>(ds + DELTA_BEAMS * DELTA_V_PITCH + bq * 16) = make_float4(cur.own.gate.x, cur.own.gate.y, kq, 0.f);
                 }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy writes -> visible to the MMA
@@ -859,9 +845,7 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
         };
         if (queued) fold_quads(std::true_type{});
         else fold_quads(std::false_type{});
-    } else if (warp >= MMA_WARP) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(MMA_REGS));
-        if (warp == MMA_WARP) {
+    } else if (warp == MMA_WARP) {
         // =============================== MMA ISSUE ===============================
         // A group's 8 MMAs go out as soon as its rows are written and its segment's S_0 is in place (complete rows imply that
         // the epilogue has read the accumulators of two groups ago: a slot's rows are written after it was handed back).
@@ -890,10 +874,9 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
             if (seg_first) { gip = 0; ++seg; }
         }
         if (dead && lane == 0) *abort_flag = 1;
-        }
     } else {
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(EPI_REGS));
         // =============================== EPILOGUE (+ preparation of the next segments) ===============================
+        put_first_s0();
         dependency_wait();
         const int quad = warp & 3;                    // tensor-memory lane quadrant of this warp
         // the first request's levels and its list, asked for together (beyond the list's end: not used)
@@ -979,17 +962,16 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
                     uint32_t v[GN / 2];
                     const uint32_t taddr = tmem_base + s * GN + ((uint32_t)(quad * 32 + half * 16) << 16);
                     tmem_ld_16x32(taddr, v);
-                    tmem_ld_16x32(taddr + 32, v + 16);
+                    tmem_ld_16x16(taddr + 32, v + 16);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
                     const int dv0 = quad * 32 + half * 16 + fr;
-                    // where the corr tile keeps outputs dv0 and dv0 + 8 of an even row, and of the odd one behind it
-                    const int p0 = corr_chunk(dv0 >> 2, 0) * 4 + (dv0 & 3), p1 = corr_chunk((dv0 + 8) >> 2, 0) * 4 + (dv0 & 3);
-                    const int n0 = C_PITCH + (p0 ^ 4), n1 = C_PITCH + (p1 ^ 4);
+                    // where the corr tile keeps outputs dv0 and dv0 + 8 of a row
+                    const int p0 = corr_chunk(dv0 >> 2) * 4 + (dv0 & 3), p1 = corr_chunk((dv0 + 8) >> 2) * 4 + (dv0 & 3);
 #pragma unroll
                     for (int nb = 0; nb < GN / 8; ++nb) {
                         float* c = C_s + (nb * 8 + fc) * C_PITCH;
-                        float o[4] = {fmaf(__uint_as_float(v[4 * nb]), w[nb].x, c[p0]), fmaf(__uint_as_float(v[4 * nb + 1]), w[nb].y, c[n0]),
-                                      fmaf(__uint_as_float(v[4 * nb + 2]), w[nb].x, c[p1]), fmaf(__uint_as_float(v[4 * nb + 3]), w[nb].y, c[n1])};
+                        float o[4] = {fmaf(__uint_as_float(v[4 * nb]), w[nb].x, c[p0]), fmaf(__uint_as_float(v[4 * nb + 1]), w[nb].y, c[C_PITCH + p0]),
+                                      fmaf(__uint_as_float(v[4 * nb + 2]), w[nb].x, c[p1]), fmaf(__uint_as_float(v[4 * nb + 3]), w[nb].y, c[C_PITCH + p1])};
                         if constexpr (DELTA) {
                             // Eq. 2 and 4 on the two projections of a beam (its rows of the group are neighbours):
                             //   delta_t = beta_t (v_t - alpha_t S_{t-1} k_t) ,  o_t = alpha_t S_{t-1} q_t + delta_t (k_t . q_t)
@@ -1008,9 +990,9 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
                             packed[2 * half + 1][nb] = pack_bf16x2(o[2], o[3]);
                         } else {                              // fp32 outputs: in place of the corr elements
                             c[p0] = o[0];
-                            c[n0] = o[1];
+                            c[C_PITCH + p0] = o[1];
                             c[p1] = o[2];
-                            c[n1] = o[3];
+                            c[C_PITCH + p1] = o[3];
                         }
                     }
                 }
@@ -1044,7 +1026,7 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
                                               : reinterpret_cast<char*>(out0 + (long long)(j >> 1) * a.H * DV);
                         *reinterpret_cast<uint4*>(dst + ch * 16) = x;
                     } else {
-                        const float4 x = *reinterpret_cast<const float4*>(C_s + j * C_PITCH + corr_chunk(ch, j) * 4);
+                        const float4 x = *reinterpret_cast<const float4*>(C_s + j * C_PITCH + corr_chunk(ch) * 4);
                         if (DELTA && (j & 1))
                             *reinterpret_cast<uint2*>(rec0 + (long long)(j >> 1) * REC_BYTES + ch * 8) = make_uint2(pack_bf16x2(x.x, x.y), pack_bf16x2(x.z, x.w));
                         else
@@ -1123,7 +1105,7 @@ struct PartitionCost {
     int group, seg, more;        // more: the third segment and on
     bool operator==(const PartitionCost& o) const { return group == o.group && seg == o.seg && more == o.more; }
 };
-PartitionCost partition_cost(int depth) { return {10 + (depth > 1 ? depth - 1 : 0), 6, depth <= 3 ? 12 : 6}; }
+PartitionCost partition_cost(int depth) { return {8 + (depth > 1 ? depth - 1 : 0), 6, depth <= 3 ? 12 : 6}; }
 template <class Begin>
 int greedy_fill(int total_groups, int gpp, int limit, int max_ctas, PartitionCost c, Begin* begin) {
     int n = 0, gi = 0;

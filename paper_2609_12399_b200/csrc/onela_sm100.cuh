@@ -244,22 +244,6 @@ struct Lanes {
         r.gate = gates_s[idx];
         return r;
     }
-    // This lane's part of a dot product: a sum per chunk, added up so that neighbouring chunks may change places (a kernel may
-    // hold them in either order) without a change of the result.
-    static __device__ __forceinline__ float own_dot(const float2* x, const float2* y) {
-        float2 d[NCH];
-#pragma unroll
-        for (int c = 0; c < NCH; ++c) {
-            d[c] = make_float2(0.f, 0.f);
-#pragma unroll
-            for (int e = 4 * c; e < 4 * c + 4; ++e) d[c] = __ffma2_rn(x[e], y[e], d[c]);
-        }
-#pragma unroll
-        for (int n = NCH / 2; n > 0; n >>= 1)
-#pragma unroll
-            for (int c = 0; c < n; ++c) d[c] = __fadd2_rn(d[c], d[c + n]);
-        return d[0].x + d[0].y;
-    }
     // One fold step on this lane's elements (packed fp32x2 FMAs), with the LPU-lane dot reduction:
     //   c~ = k . r~ ;  corr += (decay beta c~) v ;  r~ -= (beta c~) k ;  decay *= alpha
     // REPLAY (records (alpha, delta, k), Eq. 3): the vector is not changed, the record's second half is the stored
@@ -269,7 +253,13 @@ struct Lanes {
         float2 kx[NP2];
 #pragma unroll
         for (int c = 0; c < NCH; ++c) unpack8(rec.k[c], kx + 4 * c);
-        float dot = own_dot(kx, r);
+        float2 d0 = make_float2(0.f, 0.f), d1 = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int e = 0; e < NP2; e += 2) {
+            d0 = __ffma2_rn(kx[e], r[e], d0);
+            d1 = __ffma2_rn(kx[e + 1], r[e + 1], d1);
+        }
+        float dot = (d0.x + d0.y) + (d1.x + d1.y);
 #pragma unroll
         for (int o = LPU / 2; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
         const float bc = REPLAY ? dot : rec.gate.y * dot;
