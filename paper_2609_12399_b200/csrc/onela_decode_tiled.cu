@@ -556,9 +556,13 @@ cudaError_t launch_lanes(const TiledArgs& a, cudaStream_t stream) {
     return launch_dependent(kern, grid, dim3(THREADS), smem, stream, a);
 }
 
-// 64 x 64 bf16: four lanes per unit fold with a quarter fewer instructions and leave room for six CTAs per SM (five with delta
-// records), but a chain takes them longer.  Measured, eight / four lanes, us a generation: 4 x 512 beams x 32 heads XXX; the line lies at one wave of five CTAs
-// on 148 SMs.
+// 64 x 64 bf16: four lanes per unit take a quarter fewer instructions per fold and leave room for six CTAs of 128 threads per SM
+// (five with delta records), 192 units in flight instead of 160; but a warp's chain is longer.  Eight / four lanes, us a
+// generation: 4 x 512 beams x 32 heads, 8 calls 384 / 375; 8 x 777, 4 calls 458 / 420; 2 x 400, 4 calls (832 tiles: two waves
+// of five CTAs, one of six) 90.6 / 74.4; 3 x 333 grouped heads 124.6 / 121.1; delta records 4 x 512 506 / 493, 4 x 300 182 /
+// 175.  Below one wave of five the longer chain shows: 2 x 300 beams x 16 heads (320 tiles) 74.3 / 75.5, 1 x 100 beams x 32
+// heads 33.3 / 33.5.  So the line lies at one wave of five CTAs on 148 SMs.  (Seven or eight CTAs spill; 64 beams per CTA 377
+// on the first, 13 % slower on the last; fp32 records 5 % slower and more.)
 constexpr int FOUR_LANES_FROM = 740;
 template <int KD, int VD, typename T, typename OutT, bool DELTA>
 cudaError_t launch_one(const TiledArgs& a, cudaStream_t stream) {

@@ -146,8 +146,8 @@ cudaError_t launch_decode_tiled(const TiledArgs& a, int32_t dk, int32_t dv, int3
 //     They are written by the state calls alone; the host admits a decode only when a reorder of its request lies between
 //     (finish_state_write restarts the request), and the index kernel of that reorder lets nothing start before its own wait,
 //     so the states were complete when any kernel behind it started.
-// The prefill, the CUDA-core kernels for delta records and grouped heads, and export_chains are ordinary launches: they start
-// when everything before them has completed, and what follows them starts when they have.
+// The CUDA-core kernels for delta records and grouped heads, and export_chains are ordinary launches: they start when
+// everything before them has completed, and what follows them starts when they have.
 template <class... Params, class... Args>
 cudaError_t launch_dependent(void (*kern)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, const Args&... args) {
     cudaLaunchConfig_t cfg = {};

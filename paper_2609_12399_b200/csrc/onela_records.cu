@@ -36,7 +36,8 @@ __global__ void __launch_bounds__(256) append_kernel(const char* __restrict__ k,
     if (lane == 0) gate_plane[dst_row] = make_float2(__ldg(alpha + row), __ldg(beta + row));
 }
 
-// Copy of one (request, layer)'s states out of the store, 16 bytes per thread and step.
+// Copy of one (request, layer)'s states out of the store, 16 bytes per thread and step (a prefill has just left them in L2: the
+// launch is what it costs).
 __global__ void __launch_bounds__(256) export_state_kernel(const float4* __restrict__ slot, float4* __restrict__ out, int32_t n) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -172,8 +173,10 @@ cudaError_t launch_store_state(const float* S0_in, float* slot, float* scale_out
 }
 
 cudaError_t launch_export_state(const float* slot, float* S0_out, int32_t H, int32_t dk, int32_t dv, cudaStream_t stream) {
-    // A kernel of our own is a dependent launch, a copy by the runtime is not (a prefill and the export of its states, XXX).
-    // Memory of another device, which a kernel may not reach, is the runtime's.
+    // A kernel of our own is a dependent launch, a copy by the runtime is not.  (Together with the prefill's own dependent
+    // launch, us a pass of prefill + export: 3 x 100 tokens x 32 heads of 64 x 64 bf16 62 -> 45, 2 x 1021 tokens x 16 heads
+    // fp32 82 -> 74.5, 3 x 900 tokens x 16 heads of 128 x 128 160 -> 147, 16 384 tokens 450 -> 445.)  Memory of another device,
+    // which a kernel may not reach, is the runtime's.
     cudaPointerAttributes at;
     int dev = 0;
     const bool here = cudaGetDevice(&dev) == cudaSuccess && cudaPointerGetAttributes(&at, S0_out) == cudaSuccess && at.type == cudaMemoryTypeDevice && at.device == dev;
