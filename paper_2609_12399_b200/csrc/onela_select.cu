@@ -300,7 +300,9 @@ __device__ __forceinline__ void emit(unsigned long long x, int rank, const Score
     const uint32_t idx = 0xffffffffu - (uint32_t)(x & 0xffffffffull), par = src.parent(idx);
     parents[rank] = (int)par;
     codes[rank] = (int)(idx - par * (uint32_t)src.C);
-    scores[rank] = __ldg(src.bs + par) + __ldg(src.lp + idx);
+    // the score is in the composite, but for NaNs' payloads and the sign of zero (0 and 0x80000000 there)
+    const uint32_t u = (uint32_t)(x >> 32);
+    scores[rank] = (u & 0x7fffffffu) == 0u ? __ldg(src.bs + par) + __ldg(src.lp + idx) : __uint_as_float((u & 0x80000000u) ? u ^ 0x80000000u : ~u);
 }
 
 // Orders list[0 .. n) best first (n <= 1024 E; `spare`: as much room again) and writes the k best out.  The scores at hand are
@@ -437,22 +439,34 @@ struct Best {
 // consecutive candidates of a stripe, turned by SEL_ROTATE from stripe to stripe.
 __device__ __forceinline__ uint32_t place_of(int j, uint32_t me, uint32_t span) { return (uint32_t)j * span + ((me + (uint32_t)j * SEL_ROTATE) & (span - 1)); }
 
-// Requests of more candidates than a cluster's registers hold: the largest of every share of SEL_HELD, one CTA per 16 384
-// candidates, to scratch[request][share].
-__global__ void __launch_bounds__(SEL_THREADS) select_shares_kernel(const float* __restrict__ beam_scores, const float* __restrict__ cand_logp, int W_prev, int C,
-                                                                    uint32_t magic, int shift, unsigned long long* __restrict__ scratch) {
+// The largest of every share of SEL_HELD candidates, to scratch[request][share].  Share t of 16 384 candidates has its members at
+// place_of(m, t, 1024); a CTA finds 64 shares' largest, four members per thread, so that the loads spread over all SMs.
+constexpr int SHARE_THREADS = 256, SHARES_PER_CTA = 64;
+__global__ void __launch_bounds__(SHARE_THREADS) select_shares_kernel(const float* __restrict__ beam_scores, const float* __restrict__ cand_logp, int W_prev, int C,
+                                                                      uint32_t magic, int shift, unsigned long long* __restrict__ scratch) {
+    constexpr int MEMBERS = SEL_HELD * SHARES_PER_CTA / SHARE_THREADS;
+    static_assert(SEL_THREADS % SHARES_PER_CTA == 0 && SHARES_PER_CTA % 32 == 0 && MEMBERS * SHARE_THREADS == SEL_HELD * SHARES_PER_CTA, "shares of a CTA");
+    __shared__ unsigned long long part[SHARE_THREADS];
     const int tid = threadIdx.x, req = blockIdx.y;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const uint32_t N = (uint32_t)W_prev * (uint32_t)C, first = blockIdx.x * (SEL_HELD * SEL_THREADS);
+    const uint32_t N = (uint32_t)W_prev * (uint32_t)C, share = blockIdx.x * SHARES_PER_CTA + (tid & (SHARES_PER_CTA - 1));
+    const uint32_t first = share / SEL_THREADS * (SEL_HELD * SEL_THREADS);
     const ScoreSource src{beam_scores + (long long)req * W_prev, cand_logp + (long long)req * N, magic, shift, C};
     Best best;
-#pragma unroll 8
-    for (int j = 0; j < SEL_HELD; ++j) {
-        const uint32_t i = first + place_of(j, tid, SEL_THREADS);
+#pragma unroll
+    for (int j = 0; j < MEMBERS; ++j) {
+        const uint32_t i = first + place_of(tid / SHARES_PER_CTA * MEMBERS + j, share & (SEL_THREADS - 1), SEL_THREADS);
         if (i < N) best.take(src.score(i), i);
     }
-    scratch[(long long)req * (ONELA_SELECT_PARTS * SEL_CAP) + blockIdx.x * SEL_THREADS + tid] = best.composite(src);
+    part[tid] = best.composite(src);
+    __syncthreads();
+    if (tid < SHARES_PER_CTA) {
+        unsigned long long x = part[tid];
+#pragma unroll
+        for (int j = SHARES_PER_CTA; j < SHARE_THREADS; j += SHARES_PER_CTA) x = max(x, part[j + tid]);
+        scratch[(long long)req * (ONELA_SELECT_PARTS * SEL_CAP) + share] = x;
+    }
 }
 
 // grid (CTAs of a cluster, requests).  SHARES: the candidates' largest per share of SEL_HELD come from scratch
@@ -601,7 +615,12 @@ __global__ void __launch_bounds__(SEL_THREADS) select_kernel(const float* __rest
 
 }  // namespace
 
-int select_launches(long long candidates) { return candidates > (long long)SEL_CTAS * SEL_HELD * SEL_THREADS ? 2 : 1; }
+// From how many candidates on the shares' largest come from a launch of their own (XXX).
+#ifndef X_SF
+#define X_SF 32768
+#endif
+constexpr long long SEL_SHARES_FROM = X_SF;
+int select_launches(long long candidates) { return candidates > SEL_SHARES_FROM ? 2 : 1; }
 
 cudaError_t launch_select(const float* beam_scores, const float* cand_logp, int32_t req_count, int32_t W_prev, int32_t C,
                           int32_t W_new, unsigned long long* scratch, int32_t* parents, int32_t* codes, float* scores,
@@ -611,8 +630,9 @@ cudaError_t launch_select(const float* beam_scores, const float* cand_logp, int3
     // CTAs per request: one while the candidates are at most four per thread (the exchange between CTAs costs more than the
     // loads it shares out), then as many as keep them in registers, up to a portable cluster; beyond that the candidates are
     // cut into shares first, on as many SMs as there are (one cluster alone read a million candidates at 31 us)
-    const int ctas = N <= 4 * SEL_THREADS ? 1 : N <= 2 * SEL_HELD * SEL_THREADS ? 2 : N <= 4 * SEL_HELD * SEL_THREADS ? 4 : SEL_CTAS;
+    const int blocks = (int)((N + SEL_HELD * SEL_THREADS - 1) / (SEL_HELD * SEL_THREADS));      // of shares
     const bool shares = scratch && select_launches(N) > 1;
+    const int ctas = shares ? (blocks <= 2 ? 2 : blocks <= 4 ? 4 : SEL_CTAS) : N <= 4 * SEL_THREADS ? 1 : N <= 2 * SEL_HELD * SEL_THREADS ? 2 : N <= 4 * SEL_HELD * SEL_THREADS ? 4 : SEL_CTAS;
     // the threads' largest, later list and sort buffer: 64 KB; the shares that reach the bound: 16 KB
     constexpr int SMEM = SEL_CTAS * SEL_THREADS * (int)sizeof(unsigned long long) + SEL_SHARES / SEL_CTAS * (int)sizeof(uint16_t);
     static_assert(2 * SEL_LIST == SEL_CTAS * SEL_THREADS, "list and sort buffer");
@@ -636,8 +656,7 @@ cudaError_t launch_select(const float* beam_scores, const float* cand_logp, int3
     int shift;
     divide_by(C, magic, shift);
     if (shares) {
-        const unsigned parts = (unsigned)((N + SEL_HELD * SEL_THREADS - 1) / (SEL_HELD * SEL_THREADS));
-        const cudaError_t e = launch_dependent(select_shares_kernel, dim3(parts, req_count), dim3(SEL_THREADS), 0, stream, beam_scores, cand_logp, W_prev,
+        const cudaError_t e = launch_dependent(select_shares_kernel, dim3(blocks * (SEL_THREADS / SHARES_PER_CTA), req_count), dim3(SHARE_THREADS), 0, stream, beam_scores, cand_logp, W_prev,
                                                C, magic, shift, scratch);
         if (e != cudaSuccess) return e;
     }
