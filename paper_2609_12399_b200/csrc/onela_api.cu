@@ -418,7 +418,7 @@ onela_status onela_select_beams(onela_ctx* ctx, int32_t req_begin, int32_t req_c
                       ctx->lay.select_scratch + (size_t)req_begin * ONELA_SELECT_PARTS * ONELA_SELECT_CAP, parents_out_dev,
                       codes_out_dev, scores_out_dev, s) != cudaSuccess)
         return ONELA_E_CUDA;
-    ctx->launches += select_launches(W_prev * C);
+    ctx->launches += select_launches(W_prev * C, W_new);
     return ONELA_OK;
 }
 

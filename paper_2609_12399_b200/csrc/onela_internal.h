@@ -184,7 +184,7 @@ cudaError_t launch_export_chains(const int32_t* table_cur, int32_t W, int32_t de
 cudaError_t launch_select(const float* beam_scores, const float* cand_logp, int32_t req_count, int32_t W_prev, int32_t C,
                           int32_t W_new, unsigned long long* scratch, int32_t* parents, int32_t* codes, float* scores,
                           cudaStream_t stream);
-int select_launches(long long candidates);      // kernels a call with a scratch launches
+int select_launches(long long candidates, int32_t W_new);      // kernels a call with a scratch launches
 
 // record / state kernels
 cudaError_t launch_append(const void* k, const void* v, const float* alpha, const float* beta, char* kv_plane,

@@ -422,6 +422,13 @@ __device__ void sort_and_emit(unsigned long long* list, unsigned long long* spar
         if (e * SEL_THREADS + tid < k) emit(x[e], e * SEL_THREADS + tid, src, parents, codes, scores);
 }
 
+// ... of a list of at most SEL_LIST in `room`, the sort buffer behind it.
+__device__ __forceinline__ void order_and_emit(unsigned long long* room, int n, int k, SelectShared& sh, const ScoreSource& src, int32_t* parents, int32_t* codes, float* scores) {
+    if (n <= SEL_THREADS) sort_and_emit<1>(room, room + SEL_LIST, n, k, sh, src, parents, codes, scores);
+    else if (n <= 2 * SEL_THREADS) sort_and_emit<2>(room, room + SEL_LIST, n, k, sh, src, parents, codes, scores);
+    else sort_and_emit<SEL_LIST / SEL_THREADS>(room, room + SEL_LIST, n, k, sh, src, parents, codes, scores);
+}
+
 // Running maximum of a thread's candidates in increasing index order: the larger score, the earlier one of equals, NaN below
 // every number (the order of the composites, on floats: a third of the instructions).
 struct Best {
@@ -439,40 +446,102 @@ struct Best {
 // consecutive candidates of a stripe, turned by SEL_ROTATE from stripe to stripe.
 __device__ __forceinline__ uint32_t place_of(int j, uint32_t me, uint32_t span) { return (uint32_t)j * span + ((me + (uint32_t)j * SEL_ROTATE) & (span - 1)); }
 
-// The largest of every share of SEL_HELD candidates, to scratch[request][share].  Share t of 16 384 candidates has its members at
-// place_of(m, t, 1024); a CTA finds 64 shares' largest, four members per thread, so that the loads spread over all SMs.
-constexpr int SHARE_THREADS = 256, SHARES_PER_CTA = 64;
+// The largest of every share of 16 V consecutive candidates, to scratch[request][share]: V candidates per thread and step, the
+// largest of sixteen threads' by shuffles; a CTA takes 1024 candidates, so that the loads spread over all SMs.
+constexpr int SHARE_THREADS = 256;
+template <int V>
 __global__ void __launch_bounds__(SHARE_THREADS) select_shares_kernel(const float* __restrict__ beam_scores, const float* __restrict__ cand_logp, int W_prev, int C,
                                                                       uint32_t magic, int shift, unsigned long long* __restrict__ scratch) {
-    constexpr int MEMBERS = SEL_HELD * SHARES_PER_CTA / SHARE_THREADS;
-    static_assert(SEL_THREADS % SHARES_PER_CTA == 0 && SHARES_PER_CTA % 32 == 0 && MEMBERS * SHARE_THREADS == SEL_HELD * SHARES_PER_CTA, "shares of a CTA");
-    __shared__ unsigned long long part[SHARE_THREADS];
     const int tid = threadIdx.x, req = blockIdx.y;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const uint32_t N = (uint32_t)W_prev * (uint32_t)C, share = blockIdx.x * SHARES_PER_CTA + (tid & (SHARES_PER_CTA - 1));
-    const uint32_t first = share / SEL_THREADS * (SEL_HELD * SEL_THREADS);
+    const uint32_t N = (uint32_t)W_prev * (uint32_t)C;
     const ScoreSource src{beam_scores + (long long)req * W_prev, cand_logp + (long long)req * N, magic, shift, C};
-    Best best;
+    scratch += (long long)req * (ONELA_SELECT_PARTS * SEL_CAP);
+    unsigned long long best[4 / V];
 #pragma unroll
-    for (int j = 0; j < MEMBERS; ++j) {
-        const uint32_t i = first + place_of(tid / SHARES_PER_CTA * MEMBERS + j, share & (SEL_THREADS - 1), SEL_THREADS);
-        if (i < N) best.take(src.score(i), i);
+    for (int j = 0; j < 4 / V; ++j) {
+        best[j] = 0ull;
+#pragma unroll
+        for (int e = 0; e < V; ++e) {
+            const uint32_t i = blockIdx.x * 1024u + (j * SHARE_THREADS + tid) * V + e;
+            if (i < N) best[j] = max(best[j], src(i));
+        }
     }
-    part[tid] = best.composite(src);
-    __syncthreads();
-    if (tid < SHARES_PER_CTA) {
-        unsigned long long x = part[tid];
 #pragma unroll
-        for (int j = SHARES_PER_CTA; j < SHARE_THREADS; j += SHARES_PER_CTA) x = max(x, part[j + tid]);
-        scratch[(long long)req * (ONELA_SELECT_PARTS * SEL_CAP) + share] = x;
+    for (int j = 0; j < 4 / V; ++j) {
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) best[j] = max(best[j], __shfl_xor_sync(0xffffffffu, best[j], o));
+        const uint32_t share = blockIdx.x * (64u / V) + (j * SHARE_THREADS + tid) / 16;
+        if ((tid & 15) == 0 && share * (16u * V) < N) scratch[share] = best[j];
     }
 }
 
-// grid (CTAs of a cluster, requests).  SHARES: the candidates' largest per share of SEL_HELD come from scratch
-// (select_shares_kernel), and only the shares that reach the bound are looked into.  `scratch` ([request][ONELA_SELECT_PARTS *
-// SEL_CAP], or null): also where the candidates that reach the bound go when they do not fit in shared memory (behind the shares).
-template <bool SHARES>
+// The k best of a request from its shares' largest (at most 16 384), one CTA: a bound that at least k of the shares reach, the
+// candidates of those shares that reach it, their order.  (A cluster that shared this work out spent 4 us of 14 in its barriers.)
+__global__ void __launch_bounds__(SEL_THREADS) select_of_shares_kernel(const float* __restrict__ beam_scores, const float* __restrict__ cand_logp, int W_prev, int C,
+                                                                       uint32_t magic, int shift, int k, int log2_share, unsigned long long* __restrict__ scratch,
+                                                                       int32_t* __restrict__ parents, int32_t* __restrict__ codes, float* __restrict__ scores) {
+    extern __shared__ unsigned long long room[];             // [2][SEL_LIST]: list and sort buffer; the shares that reach the bound
+    __shared__ SelectShared sh;
+    __shared__ unsigned n_list, n_hits;
+    const int tid = threadIdx.x, req = blockIdx.x;
+    if (tid == 0) n_list = n_hits = 0u;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const uint32_t N = (uint32_t)W_prev * (uint32_t)C, shares = (N + (1u << log2_share) - 1) >> log2_share;
+    const ScoreSource src{beam_scores + (long long)req * W_prev, cand_logp + (long long)req * N, magic, shift, C};
+    parents += (long long)req * k;
+    codes += (long long)req * k;
+    scores += (long long)req * k;
+    scratch += (long long)req * (ONELA_SELECT_PARTS * SEL_CAP);
+    unsigned long long held[SEL_HELD];
+#pragma unroll
+    for (int j = 0; j < SEL_HELD; ++j) {
+        const uint32_t i = (uint32_t)j * SEL_THREADS + tid;
+        held[j] = i < shares ? __ldcg(scratch + i) : 0ull;
+    }
+    const unsigned long long bound = bound_of(held, k, sh);
+    uint16_t* hits = reinterpret_cast<uint16_t*>(room + 2 * SEL_LIST);
+#pragma unroll
+    for (int j = 0; j < SEL_HELD; ++j)
+        if (held[j] >= bound) hits[atomicAdd(&n_hits, 1u)] = (uint16_t)(j * SEL_THREADS + tid);
+    __syncthreads();
+    auto each = [&](auto&& put) {
+        const uint32_t todo = n_hits << log2_share;
+#pragma unroll 4
+        for (uint32_t x = tid; x < todo; x += SEL_THREADS) {
+            const uint32_t i = ((uint32_t)hits[x >> log2_share] << log2_share) + (x & ((1u << log2_share) - 1u));
+            if (i < N) {
+                const unsigned long long c = src(i);
+                if (c >= bound) put(c);
+            }
+        }
+    };
+    each([&](unsigned long long c) {
+        const unsigned at = atomicAdd(&n_list, 1u);
+        if (at < SEL_LIST) room[at] = c;
+    });
+    __syncthreads();
+    const unsigned n = n_list;
+    if (n <= SEL_LIST) {
+        order_and_emit(room, (int)n, k, sh, src, parents, codes, scores);
+        return;
+    }
+    // too many for shared memory (candidates that gather in few shares): the list again, to global memory
+    __syncthreads();
+    if (tid == 0) n_list = 0u;
+    __syncthreads();
+    unsigned long long* list = scratch + SEL_SHARES;
+    each([&](unsigned long long c) { list[atomicAdd(&n_list, 1u)] = c; });
+    __threadfence_block();
+    __syncthreads();
+    select_topk<SEL_HELD>([&](uint32_t i) { return __ldcg(list + i); }, n, k, sh);
+    sort_and_emit<1>(sh.sel, room, k, k, sh, src, parents, codes, scores);
+}
+
+// grid (CTAs of a cluster, requests).  `scratch` ([request][ONELA_SELECT_PARTS * SEL_CAP], or null): where the candidates that
+// reach the bound go when they do not fit in shared memory.
 __global__ void __launch_bounds__(SEL_THREADS) select_kernel(const float* __restrict__ beam_scores, const float* __restrict__ cand_logp, int W_prev, int C,
                                                              uint32_t magic, int shift, int k, unsigned long long* __restrict__ scratch,
                                                              int32_t* __restrict__ parents, int32_t* __restrict__ codes, float* __restrict__ scores) {
@@ -492,25 +561,15 @@ __global__ void __launch_bounds__(SEL_THREADS) select_kernel(const float* __rest
     scores += (long long)req * k;
     if (scratch) scratch += (long long)req * (ONELA_SELECT_PARTS * SEL_CAP);
     const uint32_t span = (uint32_t)ctas * SEL_THREADS, me = (uint32_t)rank * SEL_THREADS + tid;
-    const uint32_t items = SHARES ? (N + SEL_HELD * SEL_THREADS - 1) / (SEL_HELD * SEL_THREADS) * SEL_THREADS : N;     // candidates, or shares
-    const int stripes = (int)((items + span - 1) / span);
-    // 1. this thread's candidates (shares)
-    unsigned long long best = 0ull;
-    if constexpr (SHARES) {
+    const int stripes = (int)((N + span - 1) / span);
+    // 1. this thread's candidates
+    Best top;
 #pragma unroll 8
-        for (int j = 0; j < stripes; ++j) {
-            const uint32_t i = place_of(j, me, span);
-            if (i < items) best = max(best, __ldcg(scratch + i));
-        }
-    } else {
-        Best top;
-#pragma unroll 8
-        for (int j = 0; j < stripes; ++j) {
-            const uint32_t i = place_of(j, me, span);
-            if (i < N) top.take(src.score(i), i);
-        }
-        best = top.composite(src);
+    for (int j = 0; j < stripes; ++j) {
+        const uint32_t i = place_of(j, me, span);
+        if (i < N) top.take(src.score(i), i);
     }
+    const unsigned long long best = top.composite(src);
     // 2. the bound
     unsigned long long bound = 1ull;                         // (a composite is never 0: the index word of a candidate is not)
     if (ctas > 1) {
@@ -535,30 +594,17 @@ __global__ void __launch_bounds__(SEL_THREADS) select_kernel(const float* __rest
     }
     // 3. the candidates that reach it: the shares whose largest does are listed, then all threads look into their members;
     // what they find goes to a list of this CTA's, which is then appended to the first CTA's
-    uint16_t* hits = reinterpret_cast<uint16_t*>(room + 2 * SEL_LIST);      // thread (+ 1024 x stripe: share), of this CTA
-    if constexpr (SHARES) {
-        if (best >= bound)
-            for (int j = 0; j < stripes; ++j) {
-                const uint32_t i = place_of(j, me, span);
-                if (i < items && __ldcg(scratch + i) >= bound) hits[atomicAdd(&n_hits, 1u)] = (uint16_t)(j * SEL_THREADS + tid);
-            }
-    } else if (best >= bound) {
-        hits[atomicAdd(&n_hits, 1u)] = (uint16_t)tid;
-    }
+    uint16_t* hits = reinterpret_cast<uint16_t*>(room + 2 * SEL_LIST);      // threads of this CTA
+    if (best >= bound) hits[atomicAdd(&n_hits, 1u)] = (uint16_t)tid;
     __syncthreads();
-    const int members = SHARES ? SEL_HELD : stripes;
+    const int members = stripes;
     auto each = [&](auto&& put) {
         const int todo = (int)n_hits * members;
 #pragma unroll 2
         for (int x = tid; x < todo; x += SEL_THREADS) {
             const int q = x / members, m = x - q * members;
             uint32_t i = hits[q];
-            if constexpr (SHARES) {                          // share i of stripe j: member m among the 16 384 candidates of its CTA
-                i = place_of((int)(i / SEL_THREADS), (uint32_t)rank * SEL_THREADS + (i & (SEL_THREADS - 1)), span);
-                i = i / SEL_THREADS * (SEL_HELD * SEL_THREADS) + place_of(m, i & (SEL_THREADS - 1), SEL_THREADS);
-            } else {
-                i = place_of(m, (uint32_t)rank * SEL_THREADS + i, span);
-            }
+            i = place_of(m, (uint32_t)rank * SEL_THREADS + i, span);
             if (i < N) {
                 const unsigned long long c = src(i);
                 if (c >= bound) put(c);
@@ -596,12 +642,8 @@ __global__ void __launch_bounds__(SEL_THREADS) select_kernel(const float* __rest
     }
     asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
     if (rank != 0) return;
-    if (n <= SEL_THREADS) {
-        sort_and_emit<1>(room, room + SEL_LIST, (int)n, k, sh, src, parents, codes, scores);
-    } else if (n <= 2 * SEL_THREADS) {
-        sort_and_emit<2>(room, room + SEL_LIST, (int)n, k, sh, src, parents, codes, scores);
-    } else if (n <= SEL_LIST) {
-        sort_and_emit<SEL_LIST / SEL_THREADS>(room, room + SEL_LIST, (int)n, k, sh, src, parents, codes, scores);
+    if (n <= SEL_LIST) {
+        order_and_emit(room, (int)n, k, sh, src, parents, codes, scores);
     } else {                                                 // exhaustively, over the list or over all candidates
         if (scratch) {
             const unsigned long long* list = scratch + SEL_SHARES;
@@ -615,12 +657,13 @@ __global__ void __launch_bounds__(SEL_THREADS) select_kernel(const float* __rest
 
 }  // namespace
 
-// From how many candidates on the shares' largest come from a launch of their own (XXX).
+// Whether the shares' largest come from a launch of their own (XXX).  The shares have to be a few times as many as the survivors
+// for their bound to leave little more than those.
 #ifndef X_SF
-#define X_SF 32768
+#define X_SF 16384
 #endif
-constexpr long long SEL_SHARES_FROM = X_SF;
-int select_launches(long long candidates) { return candidates > SEL_SHARES_FROM ? 2 : 1; }
+bool from_shares(long long candidates, int k) { return candidates > X_SF && candidates >= 16ll * 3 * k; }
+int select_launches(long long candidates, int32_t W_new) { return from_shares(candidates, W_new) ? 2 : 1; }
 
 cudaError_t launch_select(const float* beam_scores, const float* cand_logp, int32_t req_count, int32_t W_prev, int32_t C,
                           int32_t W_new, unsigned long long* scratch, int32_t* parents, int32_t* codes, float* scores,
@@ -628,13 +671,12 @@ cudaError_t launch_select(const float* beam_scores, const float* cand_logp, int3
     const long long N = (long long)W_prev * C;
     if (N > (long long)ONELA_SELECT_PARTS * 4096) return cudaErrorInvalidValue;
     // CTAs per request: one while the candidates are at most four per thread (the exchange between CTAs costs more than the
-    // loads it shares out), then as many as keep them in registers, up to a portable cluster; beyond that the candidates are
-    // cut into shares first, on as many SMs as there are (one cluster alone read a million candidates at 31 us)
-    const int blocks = (int)((N + SEL_HELD * SEL_THREADS - 1) / (SEL_HELD * SEL_THREADS));      // of shares
-    const bool shares = scratch && select_launches(N) > 1;
-    const int ctas = shares ? (blocks <= 2 ? 2 : blocks <= 4 ? 4 : SEL_CTAS) : N <= 4 * SEL_THREADS ? 1 : N <= 2 * SEL_HELD * SEL_THREADS ? 2 : N <= 4 * SEL_HELD * SEL_THREADS ? 4 : SEL_CTAS;
+    // loads it shares out), then as many as keep them in registers, up to a portable cluster
+    const int ctas = N <= 4 * SEL_THREADS ? 1 : N <= 2 * SEL_HELD * SEL_THREADS ? 2 : N <= 4 * SEL_HELD * SEL_THREADS ? 4 : SEL_CTAS;
+    const bool shares = scratch && from_shares(N, W_new);
     // the threads' largest, later list and sort buffer: 64 KB; the shares that reach the bound: 16 KB
-    constexpr int SMEM = SEL_CTAS * SEL_THREADS * (int)sizeof(unsigned long long) + SEL_SHARES / SEL_CTAS * (int)sizeof(uint16_t);
+    constexpr int SMEM = SEL_CTAS * SEL_THREADS * (int)sizeof(unsigned long long) + 2 * SEL_THREADS * (int)sizeof(uint16_t);
+    static_assert(SEL_CAP + SEL_CAP / 8 <= 2 * SEL_THREADS && SEL_CAP / 8 >= 32, "shares (threads) that the bound may leave");
     static_assert(2 * SEL_LIST == SEL_CTAS * SEL_THREADS, "list and sort buffer");
     static_assert(SEL_SHARES + (SEL_CAP + SEL_CAP / 8) * (ONELA_SELECT_PARTS * 4096 / (SEL_CTAS * SEL_THREADS)) <= ONELA_SELECT_PARTS * SEL_CAP, "scratch");
     // one-time set-up per device (function attributes belong to a device's context)
@@ -646,8 +688,8 @@ cudaError_t launch_select(const float* beam_scores, const float* cand_logp, int3
     {
         std::lock_guard<std::mutex> lock(setup_mutex);
         if (!ready[dev]) {
-            cudaError_t e = cudaFuncSetAttribute(select_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
-            if (e == cudaSuccess) e = cudaFuncSetAttribute(select_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+            cudaError_t e = cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(select_of_shares_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
             if (e != cudaSuccess) return e;
             ready[dev] = true;
         }
@@ -656,9 +698,14 @@ cudaError_t launch_select(const float* beam_scores, const float* cand_logp, int3
     int shift;
     divide_by(C, magic, shift);
     if (shares) {
-        const cudaError_t e = launch_dependent(select_shares_kernel, dim3(blocks * (SEL_THREADS / SHARES_PER_CTA), req_count), dim3(SHARE_THREADS), 0, stream, beam_scores, cand_logp, W_prev,
-                                               C, magic, shift, scratch);
+        // shares of 16 candidates, or of 64 where those would be more than a CTA's threads hold
+        const bool wide = N > 16ll * SEL_HELD * SEL_THREADS;
+        static_assert(64ll * SEL_HELD * SEL_THREADS >= (long long)ONELA_SELECT_PARTS * 4096, "the shares of the largest request");
+        const cudaError_t e = launch_dependent(wide ? select_shares_kernel<4> : select_shares_kernel<1>, dim3((unsigned)((N + 1023) / 1024), req_count),
+                                               dim3(SHARE_THREADS), 0, stream, beam_scores, cand_logp, W_prev, C, magic, shift, scratch);
         if (e != cudaSuccess) return e;
+        return launch_dependent(select_of_shares_kernel, dim3(req_count), dim3(SEL_THREADS), SMEM, stream, beam_scores, cand_logp, W_prev, C, magic, shift,
+                                W_new, wide ? 6 : 4, scratch, parents, codes, scores);
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(ctas, req_count);
@@ -673,8 +720,7 @@ cudaError_t launch_select(const float* beam_scores, const float* cand_logp, int3
     attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    auto kern = shares ? select_kernel<true> : select_kernel<false>;
-    return cudaLaunchKernelEx(&cfg, kern, beam_scores, cand_logp, W_prev, C, magic, shift, W_new, scratch, parents, codes, scores);
+    return cudaLaunchKernelEx(&cfg, select_kernel, beam_scores, cand_logp, W_prev, C, magic, shift, W_new, scratch, parents, codes, scores);
 }
 
 }  // namespace onela
