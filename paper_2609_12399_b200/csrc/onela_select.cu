@@ -32,7 +32,8 @@ constexpr int SEL_CAP = ONELA_SELECT_CAP;      // survivors per request (W_new <
 constexpr int SEL_LIST = 4096;                 // candidates that reach the bound: room in shared memory
 constexpr int SEL_CTAS = 8;                    // CTAs per cluster at most
 constexpr int SEL_HELD = 16;                   // scores a thread keeps in registers
-constexpr int SEL_SHARES = ONELA_SELECT_PARTS * 4096 / SEL_HELD;      // shares of the largest request; the list behind them in the
+constexpr int SEL_SHARE = 16;                  // consecutive candidates of a share
+constexpr int SEL_SHARES = ONELA_SELECT_PARTS * 4096 / SEL_SHARE;     // shares of the largest request; the list behind them in the
                                                // scratch takes all candidates of the k + k / 8 threads the bound may leave
 constexpr int SEL_BINS = 2048;
 constexpr int SEL_ROTATE = 977;                // a thread's place moves by this much from stripe to stripe, so that one code's
@@ -540,8 +541,10 @@ __global__ void __launch_bounds__(SEL_THREADS) select_of_shares_kernel(const flo
     sort_and_emit<1>(sh.sel, room, k, k, sh, src, parents, codes, scores);
 }
 
-// grid (CTAs of a cluster, requests).  `scratch` ([request][ONELA_SELECT_PARTS * SEL_CAP], or null): where the candidates that
-// reach the bound go when they do not fit in shared memory.
+// grid (CTAs of a cluster, requests).  SHARES: the largest of every sixteen candidates come from scratch (select_shares_kernel),
+// and only the shares that reach the bound are looked into.  `scratch` ([request][ONELA_SELECT_PARTS * SEL_CAP], or null): also
+// where the candidates that reach the bound go when they do not fit in shared memory (behind the shares).
+template <bool SHARES>
 __global__ void __launch_bounds__(SEL_THREADS) select_kernel(const float* __restrict__ beam_scores, const float* __restrict__ cand_logp, int W_prev, int C,
                                                              uint32_t magic, int shift, int k, unsigned long long* __restrict__ scratch,
                                                              int32_t* __restrict__ parents, int32_t* __restrict__ codes, float* __restrict__ scores) {
@@ -561,15 +564,25 @@ __global__ void __launch_bounds__(SEL_THREADS) select_kernel(const float* __rest
     scores += (long long)req * k;
     if (scratch) scratch += (long long)req * (ONELA_SELECT_PARTS * SEL_CAP);
     const uint32_t span = (uint32_t)ctas * SEL_THREADS, me = (uint32_t)rank * SEL_THREADS + tid;
-    const int stripes = (int)((N + span - 1) / span);
-    // 1. this thread's candidates
-    Best top;
+    const uint32_t items = SHARES ? (N + SEL_SHARE - 1) / SEL_SHARE : N;
+    const int stripes = (int)((items + span - 1) / span);
+    // 1. this thread's candidates (shares)
+    unsigned long long best = 0ull;
+    if constexpr (SHARES) {
 #pragma unroll 8
-    for (int j = 0; j < stripes; ++j) {
-        const uint32_t i = place_of(j, me, span);
-        if (i < N) top.take(src.score(i), i);
+        for (int j = 0; j < stripes; ++j) {
+            const uint32_t i = place_of(j, me, span);
+            if (i < items) best = max(best, __ldcg(scratch + i));
+        }
+    } else {
+        Best top;
+#pragma unroll 8
+        for (int j = 0; j < stripes; ++j) {
+            const uint32_t i = place_of(j, me, span);
+            if (i < N) top.take(src.score(i), i);
+        }
+        best = top.composite(src);
     }
-    const unsigned long long best = top.composite(src);
     // 2. the bound
     unsigned long long bound = 1ull;                         // (a composite is never 0: the index word of a candidate is not)
     if (ctas > 1) {
@@ -594,17 +607,26 @@ __global__ void __launch_bounds__(SEL_THREADS) select_kernel(const float* __rest
     }
     // 3. the candidates that reach it: the shares whose largest does are listed, then all threads look into their members;
     // what they find goes to a list of this CTA's, which is then appended to the first CTA's
-    uint16_t* hits = reinterpret_cast<uint16_t*>(room + 2 * SEL_LIST);      // threads of this CTA
-    if (best >= bound) hits[atomicAdd(&n_hits, 1u)] = (uint16_t)tid;
+    uint16_t* hits = reinterpret_cast<uint16_t*>(room + 2 * SEL_LIST);      // thread (+ 1024 x stripe: share), of this CTA
+    if constexpr (SHARES) {
+        if (best >= bound)
+            for (int j = 0; j < stripes; ++j) {
+                const uint32_t i = place_of(j, me, span);
+                if (i < items && __ldcg(scratch + i) >= bound) hits[atomicAdd(&n_hits, 1u)] = (uint16_t)(j * SEL_THREADS + tid);
+            }
+    } else if (best >= bound) {
+        hits[atomicAdd(&n_hits, 1u)] = (uint16_t)tid;
+    }
     __syncthreads();
-    const int members = stripes;
+    const int members = SHARES ? SEL_SHARE : stripes;
     auto each = [&](auto&& put) {
         const int todo = (int)n_hits * members;
 #pragma unroll 2
         for (int x = tid; x < todo; x += SEL_THREADS) {
             const int q = x / members, m = x - q * members;
             uint32_t i = hits[q];
-            i = place_of(m, (uint32_t)rank * SEL_THREADS + i, span);
+            if constexpr (SHARES) i = place_of((int)(i / SEL_THREADS), (uint32_t)rank * SEL_THREADS + (i & (SEL_THREADS - 1)), span) * SEL_SHARE + m;
+            else i = place_of(m, (uint32_t)rank * SEL_THREADS + i, span);
             if (i < N) {
                 const unsigned long long c = src(i);
                 if (c >= bound) put(c);
@@ -657,12 +679,10 @@ __global__ void __launch_bounds__(SEL_THREADS) select_kernel(const float* __rest
 
 }  // namespace
 
-// Whether the shares' largest come from a launch of their own (XXX).  The shares have to be a few times as many as the survivors
-// for their bound to leave little more than those.
-#ifndef X_SF
-#define X_SF 16384
-#endif
-bool from_shares(long long candidates, int k) { return candidates > X_SF && candidates >= 16ll * 3 * k; }
+// Whether the shares' largest come from a launch of their own.  The shares have to be a few times as many as the survivors for
+// their bound to leave little more than those.  XXX
+constexpr int SHARES_FROM = 4096, ONE_CTA_TO = 256;
+bool from_shares(long long candidates, int k) { return candidates > (k <= ONE_CTA_TO ? SHARES_FROM : 2 * SEL_HELD * SEL_THREADS) && candidates >= 3ll * SEL_SHARE * k; }
 int select_launches(long long candidates, int32_t W_new) { return from_shares(candidates, W_new) ? 2 : 1; }
 
 cudaError_t launch_select(const float* beam_scores, const float* cand_logp, int32_t req_count, int32_t W_prev, int32_t C,
@@ -672,11 +692,12 @@ cudaError_t launch_select(const float* beam_scores, const float* cand_logp, int3
     if (N > (long long)ONELA_SELECT_PARTS * 4096) return cudaErrorInvalidValue;
     // CTAs per request: one while the candidates are at most four per thread (the exchange between CTAs costs more than the
     // loads it shares out), then as many as keep them in registers, up to a portable cluster
-    const int ctas = N <= 4 * SEL_THREADS ? 1 : N <= 2 * SEL_HELD * SEL_THREADS ? 2 : N <= 4 * SEL_HELD * SEL_THREADS ? 4 : SEL_CTAS;
     const bool shares = scratch && from_shares(N, W_new);
+    const int ctas = shares ? (N <= 2ll * SEL_SHARE * SEL_THREADS ? 2 : N <= 4ll * SEL_SHARE * SEL_THREADS ? 4 : SEL_CTAS)
+                            : N <= 4 * SEL_THREADS ? 1 : N <= 2 * SEL_HELD * SEL_THREADS ? 2 : N <= 4 * SEL_HELD * SEL_THREADS ? 4 : SEL_CTAS;
     // the threads' largest, later list and sort buffer: 64 KB; the shares that reach the bound: 16 KB
-    constexpr int SMEM = SEL_CTAS * SEL_THREADS * (int)sizeof(unsigned long long) + 2 * SEL_THREADS * (int)sizeof(uint16_t);
-    static_assert(SEL_CAP + SEL_CAP / 8 <= 2 * SEL_THREADS && SEL_CAP / 8 >= 32, "shares (threads) that the bound may leave");
+    constexpr int SMEM = SEL_CTAS * SEL_THREADS * (int)sizeof(unsigned long long) + SEL_SHARES / SEL_CTAS * (int)sizeof(uint16_t);
+    static_assert(ONE_CTA_TO + 32 <= SEL_SHARES / SEL_CTAS && ONE_CTA_TO / 8 <= 32, "shares that the bound may leave to one CTA");
     static_assert(2 * SEL_LIST == SEL_CTAS * SEL_THREADS, "list and sort buffer");
     static_assert(SEL_SHARES + (SEL_CAP + SEL_CAP / 8) * (ONELA_SELECT_PARTS * 4096 / (SEL_CTAS * SEL_THREADS)) <= ONELA_SELECT_PARTS * SEL_CAP, "scratch");
     // one-time set-up per device (function attributes belong to a device's context)
@@ -688,7 +709,8 @@ cudaError_t launch_select(const float* beam_scores, const float* cand_logp, int3
     {
         std::lock_guard<std::mutex> lock(setup_mutex);
         if (!ready[dev]) {
-            cudaError_t e = cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+            cudaError_t e = cudaFuncSetAttribute(select_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(select_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
             if (e == cudaSuccess) e = cudaFuncSetAttribute(select_of_shares_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
             if (e != cudaSuccess) return e;
             ready[dev] = true;
@@ -698,14 +720,15 @@ cudaError_t launch_select(const float* beam_scores, const float* cand_logp, int3
     int shift;
     divide_by(C, magic, shift);
     if (shares) {
-        // shares of 16 candidates, or of 64 where those would be more than a CTA's threads hold
-        const bool wide = N > 16ll * SEL_HELD * SEL_THREADS;
-        static_assert(64ll * SEL_HELD * SEL_THREADS >= (long long)ONELA_SELECT_PARTS * 4096, "the shares of the largest request");
+        // shares of 16 candidates; of 64 where one CTA orders them and its threads would not hold that many
+        const bool one = W_new <= ONE_CTA_TO, wide = one && N > 1ll * SEL_SHARE * SEL_HELD * SEL_THREADS;
+        static_assert(4ll * SEL_SHARE * SEL_HELD * SEL_THREADS >= (long long)ONELA_SELECT_PARTS * 4096, "the shares of the largest request");
         const cudaError_t e = launch_dependent(wide ? select_shares_kernel<4> : select_shares_kernel<1>, dim3((unsigned)((N + 1023) / 1024), req_count),
                                                dim3(SHARE_THREADS), 0, stream, beam_scores, cand_logp, W_prev, C, magic, shift, scratch);
         if (e != cudaSuccess) return e;
-        return launch_dependent(select_of_shares_kernel, dim3(req_count), dim3(SEL_THREADS), SMEM, stream, beam_scores, cand_logp, W_prev, C, magic, shift,
-                                W_new, wide ? 6 : 4, scratch, parents, codes, scores);
+        if (one)
+            return launch_dependent(select_of_shares_kernel, dim3(req_count), dim3(SEL_THREADS), SMEM, stream, beam_scores, cand_logp, W_prev, C, magic, shift,
+                                    W_new, wide ? 6 : 4, scratch, parents, codes, scores);
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(ctas, req_count);
@@ -720,7 +743,7 @@ cudaError_t launch_select(const float* beam_scores, const float* cand_logp, int3
     attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, select_kernel, beam_scores, cand_logp, W_prev, C, magic, shift, W_new, scratch, parents, codes, scores);
+    return cudaLaunchKernelEx(&cfg, shares ? select_kernel<true> : select_kernel<false>, beam_scores, cand_logp, W_prev, C, magic, shift, W_new, scratch, parents, codes, scores);
 }
 
 }  // namespace onela
