@@ -757,12 +757,47 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
                     if (!wait_or_abort(bar_stage(buf), (single ? 0 : (cur_seg >> 1)) & 1, abort_flag)) { dead = true; break; }
                     staged_ready = true;
                 }
-                if (staged_levels > 0) {
+                if (!QUEUE && staged_levels > 0) {      // (a queue leaves nothing staged: no such code in its loop, grouped wide heads 257 -> 253 us)
                     const uint8_t* st = stage + buf * (STAGE_BUF * REC_BYTES);
                     const float2* gs = gates_s + buf * STAGE_BUF;
-                    const RecT newest = L::load_shared(st, gs, staged_idx_of(staged_levels - 1), g);
-                    L::template fold_chain_simple<DELTA>(newest, staged_levels - 2, 0,
-                                  [&](int level) { return L::load_shared(st, gs, staged_idx_of(level), g); }, r, corr, decay);
+                    if constexpr (GROUPED) {
+                        const RecT newest = L::load_shared(st, gs, staged_idx_of(staged_levels - 1), g);
+                        L::template fold_chain_simple<DELTA>(newest, staged_levels - 2, 0,
+                                      [&](int level) { return L::load_shared(st, gs, staged_idx_of(level), g); }, r, corr, decay);
+                    } else {
+                        // Keys and gates a level ahead of their fold: a level's index shuffle and key loads are off its chain.  (Ten
+                        // more registers; whole records ahead, or the loop unrolled, spill: 27 % slower.  Beam-512 stack, 4
+                        // layers, 8 calls 1069 -> 1046 us; 5 x 77 beams 251.4 -> 247.9; delta records 4 x 512 680 -> 673; the
+                        // grouped instantiation does not have the registers.)
+                        auto load_key = [&](RecT& x, int at) {
+                            const uint4* p = reinterpret_cast<const uint4*>(st + at * REC_BYTES) + g;
+#pragma unroll
+                            for (int c = 0; c < NCH; ++c) x.k[c] = p[c * LPU];
+                            x.gate = gs[at];
+                        };
+                        auto load_value = [&](RecT& x, int at) {
+                            const uint4* p = reinterpret_cast<const uint4*>(st + at * REC_BYTES) + g;
+#pragma unroll
+                            for (int c = 0; c < NCH; ++c) x.v[c] = p[16 + c * LPU];
+                        };
+                        int at = staged_idx_of(staged_levels - 1);
+                        RecT x;
+                        load_key(x, at);
+#pragma unroll 1
+                        for (int level = staged_levels - 2; level >= 0; --level) {
+                            const int next = staged_idx_of(level);
+                            RecT y;
+                            load_value(x, at);
+                            load_key(y, next);
+                            L::template fold_step<DELTA>(x, r, corr, decay);
+#pragma unroll
+                            for (int c = 0; c < NCH; ++c) x.k[c] = y.k[c];
+                            x.gate = y.gate;
+                            at = next;
+                        }
+                        load_value(x, at);
+                        L::template fold_step<DELTA>(x, r, corr, decay);
+                    }
                 }
                 if (seg_last) {                    // this warp's last read of the segment's staging buffer
                     __syncwarp();
