@@ -447,9 +447,38 @@ struct Best {
 // consecutive candidates of a stripe, turned by SEL_ROTATE from stripe to stripe.
 __device__ __forceinline__ uint32_t place_of(int j, uint32_t me, uint32_t span) { return (uint32_t)j * span + ((me + (uint32_t)j * SEL_ROTATE) & (span - 1)); }
 
+// The largest of every share of SEL_HELD candidates, to scratch[request][share].  Share t of 16 384 candidates has its members at
+// place_of(m, t, 1024); a CTA finds 64 shares' largest, four members per thread, so that the loads spread over all SMs.
+constexpr int SHARE_THREADS = 256, SHARES_PER_CTA = 64;
+__global__ void __launch_bounds__(SHARE_THREADS) spread_shares_kernel(const float* __restrict__ beam_scores, const float* __restrict__ cand_logp, int W_prev, int C,
+                                                                      uint32_t magic, int shift, unsigned long long* __restrict__ scratch) {
+    constexpr int MEMBERS = SEL_HELD * SHARES_PER_CTA / SHARE_THREADS;
+    static_assert(SEL_THREADS % SHARES_PER_CTA == 0 && SHARES_PER_CTA % 32 == 0 && MEMBERS * SHARE_THREADS == SEL_HELD * SHARES_PER_CTA, "shares of a CTA");
+    __shared__ unsigned long long part[SHARE_THREADS];
+    const int tid = threadIdx.x, req = blockIdx.y;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const uint32_t N = (uint32_t)W_prev * (uint32_t)C, share = blockIdx.x * SHARES_PER_CTA + (tid & (SHARES_PER_CTA - 1));
+    const uint32_t first = share / SEL_THREADS * (SEL_HELD * SEL_THREADS);
+    const ScoreSource src{beam_scores + (long long)req * W_prev, cand_logp + (long long)req * N, magic, shift, C};
+    Best best;
+#pragma unroll
+    for (int j = 0; j < MEMBERS; ++j) {
+        const uint32_t i = first + place_of(tid / SHARES_PER_CTA * MEMBERS + j, share & (SEL_THREADS - 1), SEL_THREADS);
+        if (i < N) best.take(src.score(i), i);
+    }
+    part[tid] = best.composite(src);
+    __syncthreads();
+    if (tid < SHARES_PER_CTA) {
+        unsigned long long x = part[tid];
+#pragma unroll
+        for (int j = SHARES_PER_CTA; j < SHARE_THREADS; j += SHARES_PER_CTA) x = max(x, part[j + tid]);
+        scratch[(long long)req * (ONELA_SELECT_PARTS * SEL_CAP) + share] = x;
+    }
+}
+
 // The largest of every share of 16 V consecutive candidates, to scratch[request][share]: V candidates per thread and step, the
 // largest of sixteen threads' by shuffles; a CTA takes 1024 candidates, so that the loads spread over all SMs.
-constexpr int SHARE_THREADS = 256;
 template <int V>
 __global__ void __launch_bounds__(SHARE_THREADS) select_shares_kernel(const float* __restrict__ beam_scores, const float* __restrict__ cand_logp, int W_prev, int C,
                                                                       uint32_t magic, int shift, unsigned long long* __restrict__ scratch) {
@@ -541,7 +570,7 @@ __global__ void __launch_bounds__(SEL_THREADS) select_of_shares_kernel(const flo
     sort_and_emit<1>(sh.sel, room, k, k, sh, src, parents, codes, scores);
 }
 
-// grid (CTAs of a cluster, requests).  SHARES: the largest of every sixteen candidates come from scratch (select_shares_kernel),
+// grid (CTAs of a cluster, requests).  SHARES: the shares' largest come from scratch (spread_shares_kernel),
 // and only the shares that reach the bound are looked into.  `scratch` ([request][ONELA_SELECT_PARTS * SEL_CAP], or null): also
 // where the candidates that reach the bound go when they do not fit in shared memory (behind the shares).
 template <bool SHARES>
@@ -564,7 +593,7 @@ __global__ void __launch_bounds__(SEL_THREADS) select_kernel(const float* __rest
     scores += (long long)req * k;
     if (scratch) scratch += (long long)req * (ONELA_SELECT_PARTS * SEL_CAP);
     const uint32_t span = (uint32_t)ctas * SEL_THREADS, me = (uint32_t)rank * SEL_THREADS + tid;
-    const uint32_t items = SHARES ? (N + SEL_SHARE - 1) / SEL_SHARE : N;
+    const uint32_t items = SHARES ? (N + SEL_HELD * SEL_THREADS - 1) / (SEL_HELD * SEL_THREADS) * SEL_THREADS : N;     // candidates, or shares
     const int stripes = (int)((items + span - 1) / span);
     // 1. this thread's candidates (shares)
     unsigned long long best = 0ull;
@@ -618,15 +647,19 @@ __global__ void __launch_bounds__(SEL_THREADS) select_kernel(const float* __rest
         hits[atomicAdd(&n_hits, 1u)] = (uint16_t)tid;
     }
     __syncthreads();
-    const int members = SHARES ? SEL_SHARE : stripes;
+    const int members = SHARES ? SEL_HELD : stripes;
     auto each = [&](auto&& put) {
         const int todo = (int)n_hits * members;
 #pragma unroll 2
         for (int x = tid; x < todo; x += SEL_THREADS) {
             const int q = x / members, m = x - q * members;
             uint32_t i = hits[q];
-            if constexpr (SHARES) i = place_of((int)(i / SEL_THREADS), (uint32_t)rank * SEL_THREADS + (i & (SEL_THREADS - 1)), span) * SEL_SHARE + m;
-            else i = place_of(m, (uint32_t)rank * SEL_THREADS + i, span);
+            if constexpr (SHARES) {                          // share i of stripe j: member m among the 16 384 candidates it lies in
+                i = place_of((int)(i / SEL_THREADS), (uint32_t)rank * SEL_THREADS + (i & (SEL_THREADS - 1)), span);
+                i = i / SEL_THREADS * (SEL_HELD * SEL_THREADS) + place_of(m, i & (SEL_THREADS - 1), SEL_THREADS);
+            } else {
+                i = place_of(m, (uint32_t)rank * SEL_THREADS + i, span);
+            }
             if (i < N) {
                 const unsigned long long c = src(i);
                 if (c >= bound) put(c);
@@ -693,7 +726,8 @@ cudaError_t launch_select(const float* beam_scores, const float* cand_logp, int3
     // CTAs per request: one while the candidates are at most four per thread (the exchange between CTAs costs more than the
     // loads it shares out), then as many as keep them in registers, up to a portable cluster
     const bool shares = scratch && from_shares(N, W_new);
-    const int ctas = shares ? (N <= 2ll * SEL_SHARE * SEL_THREADS ? 2 : N <= 4ll * SEL_SHARE * SEL_THREADS ? 4 : SEL_CTAS)
+    const long long blocks = (N + SEL_HELD * SEL_THREADS - 1) / (SEL_HELD * SEL_THREADS);       // of 1024 shares
+    const int ctas = shares ? (blocks <= 2 ? 2 : blocks <= 4 ? 4 : SEL_CTAS)
                             : N <= 4 * SEL_THREADS ? 1 : N <= 2 * SEL_HELD * SEL_THREADS ? 2 : N <= 4 * SEL_HELD * SEL_THREADS ? 4 : SEL_CTAS;
     // the threads' largest, later list and sort buffer: 64 KB; the shares that reach the bound: 16 KB
     constexpr int SMEM = SEL_CTAS * SEL_THREADS * (int)sizeof(unsigned long long) + SEL_SHARES / SEL_CTAS * (int)sizeof(uint16_t);
@@ -720,15 +754,19 @@ cudaError_t launch_select(const float* beam_scores, const float* cand_logp, int3
     int shift;
     divide_by(C, magic, shift);
     if (shares) {
-        // shares of 16 candidates; of 64 where one CTA orders them and its threads would not hold that many
-        const bool one = W_new <= ONE_CTA_TO, wide = one && N > 1ll * SEL_SHARE * SEL_HELD * SEL_THREADS;
-        static_assert(4ll * SEL_SHARE * SEL_HELD * SEL_THREADS >= (long long)ONELA_SELECT_PARTS * 4096, "the shares of the largest request");
-        const cudaError_t e = launch_dependent(wide ? select_shares_kernel<4> : select_shares_kernel<1>, dim3((unsigned)((N + 1023) / 1024), req_count),
-                                               dim3(SHARE_THREADS), 0, stream, beam_scores, cand_logp, W_prev, C, magic, shift, scratch);
-        if (e != cudaSuccess) return e;
-        if (one)
+        cudaError_t e;
+        if (W_new <= ONE_CTA_TO) {       // shares of 16 candidates; of 64 where the CTA's threads would not hold that many
+            const bool wide = N > 1ll * SEL_SHARE * SEL_HELD * SEL_THREADS;
+            static_assert(4ll * SEL_SHARE * SEL_HELD * SEL_THREADS >= (long long)ONELA_SELECT_PARTS * 4096, "the shares of the largest request");
+            e = launch_dependent(wide ? select_shares_kernel<4> : select_shares_kernel<1>, dim3((unsigned)((N + 1023) / 1024), req_count), dim3(SHARE_THREADS), 0,
+                                 stream, beam_scores, cand_logp, W_prev, C, magic, shift, scratch);
+            if (e != cudaSuccess) return e;
             return launch_dependent(select_of_shares_kernel, dim3(req_count), dim3(SEL_THREADS), SMEM, stream, beam_scores, cand_logp, W_prev, C, magic, shift,
                                     W_new, wide ? 6 : 4, scratch, parents, codes, scores);
+        }
+        e = launch_dependent(spread_shares_kernel, dim3((unsigned)(blocks * (SEL_THREADS / SHARES_PER_CTA)), req_count), dim3(SHARE_THREADS), 0, stream, beam_scores,
+                             cand_logp, W_prev, C, magic, shift, scratch);
+        if (e != cudaSuccess) return e;
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(ctas, req_count);
