@@ -727,7 +727,7 @@ cudaError_t launch_select(const float* beam_scores, const float* cand_logp, int3
     // loads it shares out), then as many as keep them in registers, up to a portable cluster
     const bool shares = scratch && from_shares(N, W_new);
     const long long blocks = (N + SEL_HELD * SEL_THREADS - 1) / (SEL_HELD * SEL_THREADS);       // of 1024 shares
-    const int ctas = shares ? (blocks <= 2 ? 2 : blocks <= 4 ? 4 : SEL_CTAS)
+    const int ctas = shares ? (blocks <= 4 ? 4 : SEL_CTAS)
                             : N <= 4 * SEL_THREADS ? 1 : N <= 2 * SEL_HELD * SEL_THREADS ? 2 : N <= 4 * SEL_HELD * SEL_THREADS ? 4 : SEL_CTAS;
     // the threads' largest, later list and sort buffer: 64 KB; the shares that reach the bound: 16 KB
     constexpr int SMEM = SEL_CTAS * SEL_THREADS * (int)sizeof(unsigned long long) + SEL_SHARES / SEL_CTAS * (int)sizeof(uint16_t);
