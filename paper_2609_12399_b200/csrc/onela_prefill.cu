@@ -839,7 +839,10 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
 
     // =============================== SEGMENTS IN ORDER ===============================
     // S of the segments so far passes from CTA to CTA as the receiver's A operand (per row dk words in the order of the K
-    // steps, and what undoes the row's scale), written to the sender's shared memory and read over the cluster
+    // steps, and what undoes the row's scale), written to the receiver's shared memory over the cluster: what it then waits for
+    // is the barrier and local reads.  (Read over the cluster by the receiver, a hop had their latency four to eight times over:
+    // 2000 tokens x 8 heads of 128 x 128 bf16 69.1 -> 65.7 us, 400 tokens 38.7 -> 37.5, 3000 tokens x 8 heads of 64 x 64
+    // 49.0 -> 47.4.)
     uint4* hand_s = reinterpret_cast<uint4*>(smem);           // [dk / 4][128 rows]
     uint8_t* M_s = smem + D * 128 * 4;                        // M_p as an MN-major B operand: [hi, lo][blocks of 64][dk rows][128 bytes]
     auto hand_over = [&]() {
@@ -847,13 +850,19 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
 #pragma unroll
         for (int d = 0; d < D; d += 2) m = fmaxf(fmaxf(m, fabsf(S[d])), fabsf(S[d + 1]));
         pow2_scale(m, WIDE, sc, inv);
-        hinv_s[r] = inv;
+        uint32_t peer, peer_inv;
+        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer) : "r"(smem_u32(hand_s + r)), "r"(rank + 1));
+        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer_inv) : "r"(smem_u32(hinv_s + r)), "r"(rank + 1));
+        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(peer_inv), "f"(inv) : "memory");
 #pragma unroll
         for (int b = 0; b < D / 16; ++b) {
             uint32_t w[16];
             split16(S + 16 * b, sc, w, w + 8);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) hand_s[(4 * b + q) * 128 + r] = make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+            for (int q = 0; q < 4; ++q)
+                asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(peer + (4 * b + q) * (128 * 16)), "r"(w[4 * q]), "r"(w[4 * q + 1]),
+                             "r"(w[4 * q + 2]), "r"(w[4 * q + 3])
+                             : "memory");
         }
     };
     if (P > 1) {
@@ -886,6 +895,7 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
             }
             proxy_fence();
         }
+        cluster_sync();                                       // every CTA is through its chunks: its rings may be written
         if (!lost && rank == 0 && is_s) hand_over();
         // (one chain holds the S operand; its product lands in the other chain's columns, or beside it)
         const uint32_t o_at = D == 128 ? taddr + Z::CHAIN_COLS : d_at, o_col = D == 128 ? s_col + Z::CHAIN_COLS : d_col;
@@ -893,20 +903,15 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
             cluster_sync();
             if (lost || rank != p || chain != 0) continue;
             const int row = is_s ? r : 0;                     // (rows that are none come along with row 0's data)
-            uint32_t peer, peer_inv;
-            asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer) : "r"(smem_u32(hand_s + row)), "r"(p - 1));
-            asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer_inv) : "r"(smem_u32(hinv_s + row)), "r"(p - 1));
-            float inv;
-            asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(inv) : "r"(peer_inv) : "memory");
+            float inv = hinv_s[row];
 #pragma unroll 2
             for (int b = 0; b < D / 16; ++b) {
                 uint32_t w[16];
 #pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    asm volatile("ld.shared::cluster.v4.b32 {%0, %1, %2, %3}, [%4];"
-                                 : "=r"(w[4 * q]), "=r"(w[4 * q + 1]), "=r"(w[4 * q + 2]), "=r"(w[4 * q + 3])
-                                 : "r"(peer + (4 * b + q) * (128 * 16))
-                                 : "memory");
+                for (int q = 0; q < 4; ++q) {
+                    const uint4 x = hand_s[(4 * b + q) * 128 + row];
+                    w[4 * q] = x.x; w[4 * q + 1] = x.y; w[4 * q + 2] = x.z; w[4 * q + 3] = x.w;
+                }
                 tmem_st16(s_at + 16 * b, w);
             }
             tc_wait_st();
@@ -938,7 +943,6 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
             tc_fence_before();
             if (p + 1 < P && is_s) hand_over();
         }
-        cluster_sync();                                       // nobody leaves while its shared memory may be read
     }
 
     // =============================== RESULT ===============================
@@ -982,12 +986,14 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
 
 // How a prompt of `chunks` chunks is cut: P segments (a cluster of P CTAs per head), the first of `first` chunks, the
 // others of `rest`.  Cost model, in chunk steps of a segment that carries M: a chunk of the first segment counts FIRST, one
-// fold at the end FOLD, and `resident[P]` clusters of P run at a time.
+// fold at the end FOLD, and `resident[P]` clusters of P run at a time.  FOLD, measured around the cuts it decides: 64 x 64 fp32,
+// 700 tokens 32.7 us at 0.8, 29.8 at 0.4, 2 x 1021 tokens 73.5 / 72.7; 32 x 32, 200 tokens 17.1 / 14.6; 128 x 128 bf16, 250 tokens
+// 29.8 / 31.4, 800 tokens 45.4 / 49.0.
 struct Cut {
     int P, first, rest;
 };
 Cut cut_prompt(int chunks, int H, bool two_chains, const int* resident) {
-    const double first_cost = two_chains ? 0.95 : 1.0, fold = 0.8;
+    const double first_cost = two_chains ? 0.95 : 1.0, fold = two_chains ? 0.8 : 0.4;
     Cut best{1, chunks, 0};
     double best_cost = 1e30;
     for (int P = 1; P <= MAX_SEGMENTS && P <= chunks; ++P) {
