@@ -7,18 +7,18 @@
 // order-preserving bits; NaN lowest, -0 = +0) in the high word, 0xffffffff - flat index in the low word, so
 // composites are distinct and "larger" means "better, ties to the smaller flat index".
 //
-// A cluster of up to eight CTAs of 1024 threads per request (`select_kernel`):
-//   1. every thread takes a strided share of the candidates and keeps its largest;
-//   2. the cluster's first CTA finds a bound that at least k of the threads' largest reach - so at least k candidates
-//      reach it, and with shares spread over all parents and codes hardly more do (1094 expected for k = 1024 of a million);
-//   3. the shares whose largest reaches the bound are looked into, what reaches it is gathered in the first CTA's shared
-//      memory (distributed shared memory, one remote atomic per CTA), ordered through a histogram of the scores and written
-//      out best first.
-// Requests beyond 131 072 candidates have the shares' largest found by a launch of its own over all SMs.
-// What bounds it: latency - the candidates are read once (512 KB for 512 x 256), then four cluster barriers and a dozen of a
-// CTA's; the code runs once per launch, so loops stay rolled.  (As two launches - every 4096 candidates by an eight-pass radix
-// select of their own, one CTA to merge the parts' lists - the 512 x 256 -> 512 selection took 36 - 43 us; 14 us now, and
-// 23 us for 4 requests of 1024 x 1000 -> 1024.)
+// The candidates are cut into shares, the shares' largest give a bound that at least k of them reach - so at least k candidates
+// reach it, and hardly more do (1094 expected for k = 1024 of a million) - and only the shares that reach it are looked into:
+//   * up to 32 768 candidates, or without scratch, a share is a thread's, in a cluster of up to eight CTAs of 1024 threads per
+//     request (`select_kernel`): the first CTA finds the bound, what reaches it is gathered in its shared memory (distributed
+//     shared memory, one remote atomic per CTA), ordered through a histogram of the scores and written out best first;
+//   * beyond, shares of sixteen are spread over all SMs by a launch of their own (`spread_shares_kernel`), and the cluster goes on
+//     from their largest (`select_kernel<true>`).  A cluster alone waited 7.7 us for 512 x 256 candidates out of HBM;
+//   * where few survive (k <= 256), one CTA does the rest without a cluster's barriers, from shares of neighbours, whose members
+//     one CTA can fetch in full lines (`select_shares_kernel`, `select_of_shares_kernel`).
+// What bounds it: latency - the shares (2 us), then for a cluster four barriers (4 us of 12) and a dozen of a CTA's; the code runs
+// once per launch, so loops stay rolled.  (As two launches - every 4096 candidates by an eight-pass radix select of their own, one
+// CTA to merge the parts' lists - the 512 x 256 -> 512 selection took 36 - 43 us, one cluster 14 warm and 18 out of HBM.)
 #include <mutex>
 
 #include "onela_internal.h"
@@ -713,7 +713,11 @@ __global__ void __launch_bounds__(SEL_THREADS) select_kernel(const float* __rest
 }  // namespace
 
 // Whether the shares' largest come from a launch of their own.  The shares have to be a few times as many as the survivors for
-// their bound to leave little more than those.  XXX
+// their bound to leave little more than those (three times: 1.2 k candidates expected).  Where the lines lie, measured as whole
+// generations (select, index, decode; us, one cluster reading all candidates / from shares): one CTA for the rest - 100 x 128 ->
+// 100 66.8 / 64.0, 8 x 60 x 256 -> 60 101 / 95, 128 x 1000 -> 128 115 / 101, 4 x 200 x 512 -> 200 98.5 / 94.2; a cluster for the
+// rest - 2 x 512 x 128 -> 512 127.5 / 121.4, 8 x 512 x 512 -> 512 215 / 193, 3 x 333 x 512 -> 333 281 / 250.  One CTA at 512 survivors
+// of 8 x 512 x 512 198, at 1000 of 4 x 1000 x 1000 194 against the cluster's 152: it then fetches 16 000 candidates by itself.
 constexpr int SHARES_FROM = 4096, ONE_CTA_TO = 256;
 bool from_shares(long long candidates, int k) { return candidates > (k <= ONE_CTA_TO ? SHARES_FROM : 2 * SEL_HELD * SEL_THREADS) && candidates >= 3ll * SEL_SHARE * k; }
 int select_launches(long long candidates, int32_t W_new) { return from_shares(candidates, W_new) ? 2 : 1; }
