@@ -189,7 +189,8 @@ onela_status onela_release_request(onela_ctx* ctx, int32_t request);
  * the form reorder_beams takes), codes_out_dev [req_count][W_new] int32, scores_out_dev [req_count][W_new] fp32.
  * Equal scores go to the smaller flat index p * C + c; NaN ranks below every number; -0 equals +0.  Reads and
  * writes only the caller's buffers and changes no state of the context, so selection, reorder and the layers'
- * decode launches of a step can be captured in one CUDA graph.  1 <= W_new <= min(1024, W_prev * C), else
+ * decode launches of a step can be captured in one CUDA graph.  (Larger selections use scratch of the workspace, one
+ * per request: two selections of ONE request have to be ordered like its other calls.)  1 <= W_new <= min(1024, W_prev * C), else
  * ONELA_E_CAPACITY. */
 onela_status onela_select_beams(onela_ctx* ctx, int32_t req_begin, int32_t req_count, const float* beam_scores_dev,
                                 const float* cand_logp_dev, int32_t C, int32_t W_new, int32_t* parents_out_dev,
