@@ -190,14 +190,15 @@ __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, 
     // Lane g of a unit fetches the slots of the unit's ancestors at levels g, g + G, ... (the oldest eight levels: one load latency
     // for the whole chain instead of one per level); deeper levels are looked up when they are reached.
     const int old = a.depth - 1;           // records older than the beam's own: levels old - 1 .. 0
-    constexpr int NEAR = 8, NSLOT = NEAR / G;
-    int32_t my_slot[NSLOT];
-#pragma unroll
-    for (int j = 0; j < NSLOT; ++j) my_slot[j] = j * G + g < old ? __ldg(table + (long long)(j * G + g) * a.max_beam + bb) : 0;
+    constexpr int NEAR = 8;
+    const int32_t my_slot = g < old ? __ldg(table + (long long)g * a.max_beam + bb) : 0;
+    int32_t my_slot2 = 0;
+    if constexpr (G < NEAR) my_slot2 = G + g < old ? __ldg(table + (long long)(G + g) * a.max_beam + bb) : 0;
     // (two look-ups, used by two runs of the chain walk: one loop with a branch between them costs every level a
     // dozen instructions, taken or not)
     auto slot_near = [&](int level) -> int32_t {                                                                 // level < NEAR
-        return __shfl_sync(0xffffffffu, level >= G ? my_slot[NSLOT - 1] : my_slot[0], level & (G - 1), G);
+        if constexpr (G == NEAR) return __shfl_sync(0xffffffffu, my_slot, level, G);
+        else return __shfl_sync(0xffffffffu, level >= G ? my_slot2 : my_slot, level & (G - 1), G);
     };
     auto slot_far = [&](int level) -> int32_t { return __ldg(table + (long long)level * a.max_beam + bb); };    // level >= NEAR
     struct Raw { uint4 k[CK], v[CV]; float2 gate; };          // this lane's share of a record, as stored
@@ -439,7 +440,8 @@ __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, 
         {
             const int i = quad * 32 + lane;          // value row within the tile
 #pragma unroll
-            for (int b0 = half * 16; b0 < NB; b0 += THREADS / 8) {
+            for (int pass = 0; pass < NB * 8 / THREADS; ++pass) {
+                const int b0 = half * 16 + pass * (THREADS / 8);
                 uint32_t v[16];
                 tmem_ld16(tmem_base + (mt & 1) * NB + b0 + ((uint32_t)(quad * 32) << 16), v);
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
