@@ -3,7 +3,8 @@
 // Section 4.1).  The chain walk is the CUDA-core one (see onela_decode_generic.cu); what moves to the tensor cores is
 // the contraction with S_0, which dominates these shapes (dv x dk multiply-adds per unit against 3 dk per record).
 //
-// One CTA = (request, value head, tile of 32 beams - 64 at key width 256), 8 lanes per (beam, head) unit.
+// One CTA = (request, value head, tile of 32 beams - 64 from 128 x 128 up), 8 lanes per (beam, head) unit (4 in large launches of
+// 64 x 64 bf16: see launch_one).
 //   1. Every unit folds its query through its records, newest first:  c = k.r ; corr += beta c v ; r -= beta c k,
 //      the decay a running scalar.  corr stays in registers.  With the append fused in, the newest record comes from
 //      the caller's tensors and the unit also writes it to its arena slot.
@@ -16,8 +17,9 @@
 // What bounds it: the phases of a CTA in sequence (inputs from HBM, dependent gathers, MMAs, accumulators through shared
 // memory), overlapped only by the other CTAs of the SM - one at the widest shapes.  us per launch on the beam-512 stack
 // before / after corr was left in registers, the MMAs issued by an elected lane of a converged warp and the loads moved ahead
-// of the first barrier: 64 x 64 bf16 29.8 / 24.0 (depth 1 - 8), 256 x 256 bf16 79.9 / 70.9, 256 x 512 bf16 (600 beams x 16
-// heads) 36.6 / 32.0, 128 x 256 fp32 23.5 / 21.5.  Requests of the next wave's inputs into L2 made it 3 % slower; a persistent
+// of the first barrier: 64 x 64 bf16 29.8 / 24.0 (depth 1 - 8; 23.4 since with four lanes), 256 x 256 bf16 79.9 / 70.9 (68 since with requests a level ahead), 256 x 512 bf16 (600 beams x 16
+// heads) 36.6 / 32.0, 128 x 256 fp32 23.5 / 21.5.  Requests of the next wave's inputs into L2 made it 3 % slower, of all older
+// records ahead of the fold at 64 x 64 8 - 13 % (other CTAs hide them, the instructions are paid); a persistent
 // loop over the tiles of beams spills (the invariants of every pointer stay live): 64 x 64 40 us.
 // The only wait is for the MMAs' completion; it is bounded, and all threads agree on its outcome before going on
 // (ONELA_E_TIMEOUT in the status word otherwise).

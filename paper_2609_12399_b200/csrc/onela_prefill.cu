@@ -37,8 +37,9 @@
 //   per chunk:            K K^T (dk / 16 MMAs), K^T T'^T (2 x 4), V^T (T diag(beta))^T (3 x 4), A = the tile read MN-major
 // (fp32 records: Delta K 5 or 6 products, the lowest part of Delta in shared memory; K K^T three, K^T T'^T three, U six.)
 // What bounds it now: the latency of a chain's step and, as long, the two preparations in flight, about 11 000 cycles per
-// chunk.  16 384 tokens x 32 heads of 128 x 128 bf16: 18.2 ms token by token, 0.44 ms (0.38 ms in the other grouping, whose
-// errors were larger); 1021 tokens x 16 heads of 64 x 64 fp32: 376 -> 40 us (35).
+// chunk.  16 384 tokens x 32 heads of 128 x 128 bf16: 18.2 ms token by token, 0.435 ms (0.38 ms in the other grouping, whose
+// errors were larger); 1021 tokens x 16 heads of 64 x 64 fp32: 376 -> 35 us.  M's chain retired once M has decayed to zero: 0.44 ->
+// 0.50 ms, by spills.  The loops of gates or of Delta unrolled at dk <= 64: within 1 % either way, up to 6 % slower together.
 //
 // Every wait is bounded: a thread that gives up keeps meeting its team's barriers, whose OR makes the team leave
 // together, and the cluster barriers, but hands nothing on; ONELA_E_TIMEOUT goes to the status word.  A team always waits for
