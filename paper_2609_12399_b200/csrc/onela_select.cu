@@ -9,7 +9,7 @@
 //
 // The candidates are cut into shares, the shares' largest give a bound that at least k of them reach - so at least k candidates
 // reach it, and hardly more do (1094 expected for k = 1024 of a million) - and only the shares that reach it are looked into:
-//   * up to 32 768 candidates, or without scratch, a share is a thread's, in a cluster of up to eight CTAs of 1024 threads per
+//   * up to 16 384 candidates (32 768 where many survive), or without scratch, a share is a thread's, in a cluster of up to eight CTAs of 1024 threads per
 //     request (`select_kernel`): the first CTA finds the bound, what reaches it is gathered in its shared memory (distributed
 //     shared memory, one remote atomic per CTA), ordered through a histogram of the scores and written out best first;
 //   * beyond, shares of sixteen are spread over all SMs by a launch of their own (`spread_shares_kernel`), and the cluster goes on
@@ -714,11 +714,12 @@ __global__ void __launch_bounds__(SEL_THREADS) select_kernel(const float* __rest
 
 // Whether the shares' largest come from a launch of their own.  The shares have to be a few times as many as the survivors for
 // their bound to leave little more than those (three times: 1.2 k candidates expected).  Where the lines lie, measured as whole
-// generations (select, index, decode; us, one cluster reading all candidates / from shares): one CTA for the rest - 100 x 128 ->
-// 100 66.8 / 64.0, 8 x 60 x 256 -> 60 101 / 95, 128 x 1000 -> 128 115 / 101, 4 x 200 x 512 -> 200 98.5 / 94.2; a cluster for the
-// rest - 2 x 512 x 128 -> 512 127.5 / 121.4, 8 x 512 x 512 -> 512 215 / 193, 3 x 333 x 512 -> 333 281 / 250.  One CTA at 512 survivors
-// of 8 x 512 x 512 198, at 1000 of 4 x 1000 x 1000 194 against the cluster's 152: it then fetches 16 000 candidates by itself.
-constexpr int SHARES_FROM = 4096, ONE_CTA_TO = 256;
+// generations (select, index, decode; us, one cluster reading all candidates / from shares): one CTA for the rest - 128 x 1000 ->
+// 128 115 / 101, 4 x 200 x 512 -> 200 98.5 / 94.2; a cluster for the rest - 2 x 512 x 128 -> 512 127.5 / 121.4, 8 x 512 x 512 -> 512
+// 215 / 193, 3 x 333 x 512 -> 333 281 / 250.  One CTA at 512 survivors of 8 x 512 x 512 198, at 1000 of 4 x 1000 x 1000 194 against the
+// cluster's 152: it then fetches 16 000 candidates by itself.  Below 16 384 candidates the second launch is not worth its host time:
+// 100 x 128 -> 100 66.8 / 64.0 as a graph, but 7 x 10 x 1000 -> 10, issued eagerly, 95.1 / 95.8.
+constexpr int SHARES_FROM = 16384, ONE_CTA_TO = 256;
 bool from_shares(long long candidates, int k) { return candidates > (k <= ONE_CTA_TO ? SHARES_FROM : 2 * SEL_HELD * SEL_THREADS) && candidates >= 3ll * SEL_SHARE * k; }
 int select_launches(long long candidates, int32_t W_new) { return from_shares(candidates, W_new) ? 2 : 1; }
 
