@@ -996,14 +996,16 @@ __global__ void __launch_bounds__(Shape<D, T>::THREADS, 1) prefill_chunk_kernel(
 
 // How a prompt of `chunks` chunks is cut: P segments (a cluster of P CTAs per head), the first of `first` chunks, the
 // others of `rest`.  Cost model, in chunk steps of a segment that carries M: a chunk of the first segment counts FIRST, one
-// fold at the end FOLD, and `resident[P]` clusters of P run at a time.  FOLD, measured around the cuts it decides: 64 x 64 fp32,
-// 700 tokens 32.7 us at 0.8, 29.8 at 0.4, 2 x 1021 tokens 73.5 / 72.7; 32 x 32, 200 tokens 17.1 / 14.6; 128 x 128 bf16, 250 tokens
-// 29.8 / 31.4, 800 tokens 45.4 / 49.0.
+// fold at the end FOLD, and `resident[P]` clusters of P run at a time.  FOLD, measured around the cuts it decides: 128 x 128 bf16,
+// 250 tokens 29.8 us at 0.8, 31.4 at 0.4, 800 tokens 45.4 / 49.0; 64 x 64 fp32, 700 tokens 32.7 / 29.8, 2 x 1021 tokens 73.5 / 72.7;
+// 32 x 32, 200 tokens 17.1 / 14.6.  One chain is cut no finer for that: every fold takes the whole state through two fp16 parts.
+// Relative error against 64 bits at 0.8 / at 0.4, 64 x 64 without decay: 200 tokens 1.6e-7 / 2.4e-7, 300 1.6e-7 / 2.3e-7, 969
+// 1.6e-7 / 1.9e-7; gates in [0.9, 1], 200 tokens 0.8e-7 / 1.1e-7.
 struct Cut {
     int P, first, rest;
 };
 Cut cut_prompt(int chunks, int H, bool two_chains, const int* resident) {
-    const double first_cost = two_chains ? 0.95 : 1.0, fold = two_chains ? 0.8 : 0.4;
+    const double first_cost = two_chains ? 0.95 : 1.0, fold = 0.8;
     Cut best{1, chunks, 0};
     double best_cost = 1e30;
     for (int P = 1; P <= MAX_SEGMENTS && P <= chunks; ++P) {
