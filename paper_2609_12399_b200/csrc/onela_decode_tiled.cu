@@ -83,7 +83,9 @@ __host__ __device__ constexpr int tiled_min_ctas() { return KD + VD <= 128 ? (G 
 // replay leaving x unchanged - and after the contraction delta_t = beta_t (v_t - alpha_t S_{t-1} k_t) and
 // o_t = alpha_t S_{t-1} q_t + delta_t (k_t . q_t) are formed from the two rows and the record is written; always with
 // the append fused in, dk = dv <= 128.
-// G: lanes per unit, 8 or (64 x 64 bf16 in large launches) 4.
+// G: lanes per unit, 8 or (64 x 64 bf16 in large launches) 4.  Four lanes add up what eight do, in eight lanes' order: lane g holds
+// the chunks of lanes g and g + 4, sums each by itself and adds the two, which is what the first exchange among eight lanes does.  So
+// a request's results do not depend on how many others share its launch.
 template <int KD, int VD, typename T, typename OutT, bool DELTA, int G>
 __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, VD, T, DELTA, G>()) decode_tiled_kernel(const TiledArgs a) {
     constexpr int NB = tiled_beams<KD, VD>(), CP = tile_pitch<VD>();
@@ -246,14 +248,16 @@ __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, 
             float2 d0 = make_float2(0.f, 0.f), d1 = d0;
 #pragma unroll
             for (int c = 0; c < CK; ++c) {
+                if (G == 4) d0 = d1 = make_float2(0.f, 0.f);       // chunk by chunk: see the kernel's head
                 Vec16<T>::unpack(x.k[c], kx + c * VEC);
 #pragma unroll
                 for (int e = c * VEC; e < (c + 1) * VEC; e += 4) {
                     d0 = __ffma2_rn(make_float2(kx[e], kx[e + 1]), make_float2(r[e], r[e + 1]), d0);
                     d1 = __ffma2_rn(make_float2(kx[e + 2], kx[e + 3]), make_float2(r[e + 2], r[e + 3]), d1);
                 }
+                if (G == 4) dot = c == 0 ? (d0.x + d0.y) + (d1.x + d1.y) : dot + ((d0.x + d0.y) + (d1.x + d1.y));
             }
-            dot = (d0.x + d0.y) + (d1.x + d1.y);
+            if (G != 4) dot = (d0.x + d0.y) + (d1.x + d1.y);
         } else {
 #pragma unroll
             for (int c = 0; c < CK; ++c) {
@@ -325,8 +329,10 @@ __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, 
 #pragma unroll
         for (int c = 0; c < CK; ++c) {
             Vec16<T>::unpack(cur.k[c], kx + c * VEC);
+            float part = G == 4 ? 0.f : kq;
 #pragma unroll
-            for (int e = 0; e < VEC; ++e) kq = fmaf(kx[c * VEC + e], r[c * VEC + e], kq);
+            for (int e = 0; e < VEC; ++e) part = fmaf(kx[c * VEC + e], r[c * VEC + e], part);
+            kq = G == 4 && c > 0 ? kq + part : part;
         }
 #pragma unroll
         for (int off = G / 2; off > 0; off >>= 1) kq += __shfl_xor_sync(0xffffffffu, kq, off);

@@ -39,3 +39,12 @@ def test_raw_records(R, H, W, D, out_dtype, fused):
 @pytest.mark.parametrize("R,H,W,D,out_dtype", [(12, 31, 17, 4, "bf16"), (12, 31, 32, 10, "fp32")])      # tiles of 16 beams: 744
 def test_delta_records(R, H, W, D, out_dtype):
     _check(CFG1.scaled(R=R, H=H, dk=64, dv=64, W=W, D=D, prompt_len=8, seed=R + W), out_dtype, P.FLAG_GTR_DELTA)
+
+
+@pytest.mark.parametrize("W,D,out_dtype,flags", [(33, 10, "fp32", 0), (33, 3, "bf16", 0), (17, 10, "fp32", P.FLAG_GTR_DELTA)])
+def test_results_do_not_depend_on_the_other_requests_of_a_call(W, D, out_dtype, flags):
+    """Twelve requests in one call (744 tiles: four lanes) and the same requests one by one (62 tiles: eight), bit for bit."""
+    case = make_case(CFG1.scaled(R=12, H=31, dk=64, dv=64, W=W, D=D, prompt_len=8, parents="zipf", zipf_s=1.3, seed=W + D))
+    outs, _, _ = run_library(case, out_dtype=out_dtype, flags=flags, fused=True)
+    alone, _, _ = run_library(case, out_dtype=out_dtype, flags=flags, fused=True, batched=False)
+    assert all(np.array_equal(outs[key].numpy(), alone[key].numpy()) for key in outs)
