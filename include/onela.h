@@ -187,11 +187,11 @@ onela_status onela_release_request(onela_ctx* ctx, int32_t request);
  * W_prev beams of the request's current decode call (W_prev = 1, the root, before the first call) and c over the C
  * codes.  The W_new best are written best first: parents_out_dev [req_count][W_new] int32 (the parent map pi_t in
  * the form reorder_beams takes), codes_out_dev [req_count][W_new] int32, scores_out_dev [req_count][W_new] fp32.
- * Equal scores go to the smaller flat index p * C + c; NaN ranks below every number; -0 equals +0.  Reads and
- * writes only the caller's buffers and changes no state of the context, so selection, reorder and the layers'
- * decode launches of a step can be captured in one CUDA graph.  (Larger selections use scratch of the workspace, one
- * per request: two selections of ONE request have to be ordered like its other calls.)  1 <= W_new <= min(1024, W_prev * C), else
- * ONELA_E_CAPACITY. */
+ * Equal scores go to the smaller flat index p * C + c; NaN ranks below every number; -0 equals +0.  Changes
+ * no state of the context, so selection, reorder and the layers' decode launches of a step can be captured in one CUDA
+ * graph, and selections of one request with output buffers of their own may run on several streams at once.  (Beyond
+ * 4096 candidates a selection may use scratch of the request's workspace; one that finds it in use goes without it,
+ * which takes it some hundred microseconds.)  1 <= W_new <= min(1024, W_prev * C), else ONELA_E_CAPACITY. */
 onela_status onela_select_beams(onela_ctx* ctx, int32_t req_begin, int32_t req_count, const float* beam_scores_dev,
                                 const float* cand_logp_dev, int32_t C, int32_t W_new, int32_t* parents_out_dev,
                                 int32_t* codes_out_dev, float* scores_out_dev, void* stream);

@@ -44,6 +44,9 @@ bool uses_tiled_kernel(const onela_config& c) {
     return decode_tiled_supported(c.dk, c.dv) && (!(c.flags & ONELA_FLAG_GTR_DELTA) || c.dk == c.dv);   // delta records: square heads
 }
 
+// The status words and the selections' claims: what has to be zero before the first launch.
+size_t status_bytes(const onela_config& c) { return 4 * sizeof(int32_t) + (size_t)c.num_requests * sizeof(unsigned long long); }
+
 // Carve the workspace.  `base` may be null (size query only).
 Layout carve(const onela_config& c, char* base) {
     const size_t es = c.rec_dtype == ONELA_DTYPE_BF16 ? 2 : 4;
@@ -55,7 +58,8 @@ Layout carve(const onela_config& c, char* base) {
         off += align_up(bytes);
         return p;
     };
-    l.status = reinterpret_cast<int32_t*>(take(4 * sizeof(int32_t)));
+    l.status = reinterpret_cast<int32_t*>(take(status_bytes(c)));
+    l.select_claims = reinterpret_cast<unsigned long long*>(l.status + 4);
     l.tables = reinterpret_cast<int32_t*>(take((size_t)c.num_requests * 2 * c.max_steps * c.max_beam * sizeof(int32_t)));
     l.sidx = reinterpret_cast<int32_t*>(take((size_t)c.num_requests * c.max_steps * c.max_beam * sizeof(int32_t)));
     l.ulist = reinterpret_cast<int32_t*>(take((size_t)c.num_requests * c.max_steps * c.max_beam * sizeof(int32_t)));
@@ -120,7 +124,7 @@ struct onela_ctx {
 
     onela_status prepare(cudaStream_t s) {
         if (dry() || status_cleared) return ONELA_OK;
-        if (cudaMemsetAsync(lay.status, 0, 4 * sizeof(int32_t), s) != cudaSuccess) return ONELA_E_CUDA;
+        if (cudaMemsetAsync(lay.status, 0, status_bytes(cfg), s) != cudaSuccess) return ONELA_E_CUDA;
         status_cleared = true;
         return ONELA_OK;
     }
@@ -415,8 +419,8 @@ onela_status onela_select_beams(onela_ctx* ctx, int32_t req_begin, int32_t req_c
     if ((st = ctx->prepare(s)) != ONELA_OK) return st;
     if (ctx->dry()) return ONELA_OK;
     if (launch_select(beam_scores_dev, cand_logp_dev, req_count, (int32_t)W_prev, C, W_new,
-                      ctx->lay.select_scratch + (size_t)req_begin * ONELA_SELECT_PARTS * ONELA_SELECT_CAP, parents_out_dev,
-                      codes_out_dev, scores_out_dev, s) != cudaSuccess)
+                      ctx->lay.select_scratch + (size_t)req_begin * ONELA_SELECT_PARTS * ONELA_SELECT_CAP,
+                      ctx->lay.select_claims + req_begin, parents_out_dev, codes_out_dev, scores_out_dev, s) != cudaSuccess)
         return ONELA_E_CUDA;
     ctx->launches += select_launches(W_prev * C, W_new);
     return ONELA_OK;

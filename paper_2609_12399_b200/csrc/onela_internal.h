@@ -12,6 +12,7 @@ namespace onela {
 // Device addresses of the sub-buffers carved out of the caller's workspace.
 struct Layout {
     int32_t* status;   // [4]: code, detail, spare, spare
+    unsigned long long* select_claims;   // [request], behind the status, zero from the start: whose select_scratch is (see onela_select.cu)
     int32_t* tables;   // [request][2][max_steps][max_beam] global slot ids (double-buffered per request)
     int32_t* sidx;     // [request][max_steps][max_beam] per (level, beam): index into the request's distinct-record list
     int32_t* ulist;    // [request][max_steps*max_beam] distinct record slots of the live chains, oldest level first
@@ -25,7 +26,8 @@ struct Layout {
     char* kv;          // [layer][head][arena_slots][dk + dv] in rec_dtype: one row = k | v of one record
                        // (grouped value heads: keys only, [layer][key head][arena_slots][dk])
     char* vv;          // grouped value heads only: values [layer][value head][arena_slots][dv]
-    unsigned long long* select_scratch;   // [request][ONELA_SELECT_PARTS * ONELA_SELECT_CAP]: beam selection, candidates beyond its shared memory
+    unsigned long long* select_scratch;   // [request][ONELA_SELECT_PARTS * ONELA_SELECT_CAP]: beam selection, the largest of shares of
+                                          // the candidates; behind them candidates beyond its shared memory
     float* s0_scale;   // [request][layer][head]: the power of two that brings the head's largest |S_0| element into
                        // [2^11, 2^12) (1 for an all-zero or non-finite state); written with the state, read by the
                        // tensor-core kernel, whose fp16 operand it keeps in range
@@ -178,12 +180,13 @@ cudaError_t launch_export_chains(const int32_t* table_cur, int32_t W, int32_t de
 
 // global beam selection: the W_new best (parent, code) pairs per request, best first (see onela_select.cu).
 // At most ONELA_SELECT_PARTS * 4096 candidates per request.  `scratch` ([request][ONELA_SELECT_PARTS * ONELA_SELECT_CAP] 64-bit
-// words, or null) takes the candidates that the selection bound leaves where shared memory cannot hold them.
+// words, or null) takes the largest of shares of the candidates and, behind them, the candidates that the selection bound leaves where
+// shared memory cannot hold them; `claims` ([request], see Layout): whose it is.
 #define ONELA_SELECT_CAP 1024
 #define ONELA_SELECT_PARTS 256
 cudaError_t launch_select(const float* beam_scores, const float* cand_logp, int32_t req_count, int32_t W_prev, int32_t C,
-                          int32_t W_new, unsigned long long* scratch, int32_t* parents, int32_t* codes, float* scores,
-                          cudaStream_t stream);
+                          int32_t W_new, unsigned long long* scratch, unsigned long long* claims, int32_t* parents, int32_t* codes,
+                          float* scores, cudaStream_t stream);
 int select_launches(long long candidates, int32_t W_new);      // kernels a call with a scratch launches
 
 // record / state kernels

@@ -447,17 +447,47 @@ struct Best {
 // consecutive candidates of a stripe, turned by SEL_ROTATE from stripe to stripe.
 __device__ __forceinline__ uint32_t place_of(int j, uint32_t me, uint32_t span) { return (uint32_t)j * span + ((me + (uint32_t)j * SEL_ROTATE) & (span - 1)); }
 
+// A request's scratch is one selection's at a time, and selections of one request may be in flight on several streams: who uses it
+// has claimed it.  The claim (a word per request, zero when the context starts): the address the claimant's parents go to, which is
+// its alone while it is in flight, and how many CTAs of its launch of shares found the claim theirs, so that one word says all.
+// Nobody waits for a claim: a launch of shares that does not get it for all of its CTAs leaves the next launch to select
+// exhaustively from the candidates themselves, by one CTA - slow, but two selections of one request at a time are rare.  (Cost, us a
+// selection: 0.3 for the claim, 0.3 for the code beside the path; marks in the shares' entries in place of a claim, read and written
+// with them as 128 bits, 0.7 for the cluster and 1.8 for one CTA.)
+struct Claim {
+    static constexpr int COUNT_BITS = 11;                    // of at most ONELA_SELECT_PARTS * 4 CTAs
+    static_assert(ONELA_SELECT_PARTS * 4 < 1 << COUNT_BITS, "CTAs of a launch of shares");
+    unsigned long long *word, token;
+    __device__ __forceinline__ Claim(unsigned long long* claims, int req, const int32_t* parents_of_request)
+        : word(claims + req), token(reinterpret_cast<unsigned long long>(parents_of_request) >> 2 << COUNT_BITS) {}
+    // one thread of a CTA: ask, and later (the answer takes as long as a load) settle
+    __device__ __forceinline__ unsigned long long ask() const { return atomicCAS(word, 0ull, token + 1); }
+    __device__ __forceinline__ bool settle(unsigned long long answer) const {
+        if (answer == 0ull) return true;
+        if ((answer ^ token) >> COUNT_BITS) return false;
+        atomicAdd(word, 1ull);
+        return true;
+    }
+    __device__ __forceinline__ unsigned long long state() const { return __ldcg(word); }
+    __device__ __forceinline__ bool mine(unsigned long long state) const { return ((state ^ token) >> COUNT_BITS) == 0ull; }
+    __device__ __forceinline__ void release() const { __stcg(word, 0ull); }      // one thread, when the scratch has been read
+};
+
 // The largest of every share of SEL_HELD candidates, to scratch[request][share].  Share t of 16 384 candidates has its members at
 // place_of(m, t, 1024); a CTA finds 64 shares' largest, four members per thread, so that the loads spread over all SMs.
 constexpr int SHARE_THREADS = 256, SHARES_PER_CTA = 64;
 __global__ void __launch_bounds__(SHARE_THREADS) spread_shares_kernel(const float* __restrict__ beam_scores, const float* __restrict__ cand_logp, int W_prev, int C,
-                                                                      uint32_t magic, int shift, unsigned long long* __restrict__ scratch) {
+                                                                      uint32_t magic, int shift, int k, unsigned long long* __restrict__ scratch,
+                                                                      unsigned long long* claims, const int32_t* parents) {
     constexpr int MEMBERS = SEL_HELD * SHARES_PER_CTA / SHARE_THREADS;
     static_assert(SEL_THREADS % SHARES_PER_CTA == 0 && SHARES_PER_CTA % 32 == 0 && MEMBERS * SHARE_THREADS == SEL_HELD * SHARES_PER_CTA, "shares of a CTA");
     __shared__ unsigned long long part[SHARE_THREADS];
+    __shared__ bool s_mine;
     const int tid = threadIdx.x, req = blockIdx.y;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const Claim claim(claims, req, parents + (long long)req * k);
+    const unsigned long long answer = tid == 0 ? claim.ask() : 0ull;      // (comes while the candidates do)
     const uint32_t N = (uint32_t)W_prev * (uint32_t)C, share = blockIdx.x * SHARES_PER_CTA + (tid & (SHARES_PER_CTA - 1));
     const uint32_t first = share / SEL_THREADS * (SEL_HELD * SEL_THREADS);
     const ScoreSource src{beam_scores + (long long)req * W_prev, cand_logp + (long long)req * N, magic, shift, C};
@@ -468,8 +498,9 @@ __global__ void __launch_bounds__(SHARE_THREADS) spread_shares_kernel(const floa
         if (i < N) best.take(src.score(i), i);
     }
     part[tid] = best.composite(src);
+    if (tid == 0) s_mine = claim.settle(answer);
     __syncthreads();
-    if (tid < SHARES_PER_CTA) {
+    if (s_mine && tid < SHARES_PER_CTA) {
         unsigned long long x = part[tid];
 #pragma unroll
         for (int j = SHARES_PER_CTA; j < SHARE_THREADS; j += SHARES_PER_CTA) x = max(x, part[j + tid]);
@@ -481,10 +512,14 @@ __global__ void __launch_bounds__(SHARE_THREADS) spread_shares_kernel(const floa
 // largest of sixteen threads' by shuffles; a CTA takes 1024 candidates, so that the loads spread over all SMs.
 template <int V>
 __global__ void __launch_bounds__(SHARE_THREADS) select_shares_kernel(const float* __restrict__ beam_scores, const float* __restrict__ cand_logp, int W_prev, int C,
-                                                                      uint32_t magic, int shift, unsigned long long* __restrict__ scratch) {
+                                                                      uint32_t magic, int shift, int k, unsigned long long* __restrict__ scratch,
+                                                                      unsigned long long* claims, const int32_t* parents) {
+    __shared__ bool s_mine;
     const int tid = threadIdx.x, req = blockIdx.y;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const Claim claim(claims, req, parents + (long long)req * k);
+    const unsigned long long answer = tid == 0 ? claim.ask() : 0ull;      // (comes while the candidates do)
     const uint32_t N = (uint32_t)W_prev * (uint32_t)C;
     const ScoreSource src{beam_scores + (long long)req * W_prev, cand_logp + (long long)req * N, magic, shift, C};
     scratch += (long long)req * (ONELA_SELECT_PARTS * SEL_CAP);
@@ -498,6 +533,9 @@ __global__ void __launch_bounds__(SHARE_THREADS) select_shares_kernel(const floa
             if (i < N) best[j] = max(best[j], src(i));
         }
     }
+    if (tid == 0) s_mine = claim.settle(answer);
+    __syncthreads();
+    if (!s_mine) return;
 #pragma unroll
     for (int j = 0; j < 4 / V; ++j) {
 #pragma unroll
@@ -511,7 +549,8 @@ __global__ void __launch_bounds__(SHARE_THREADS) select_shares_kernel(const floa
 // candidates of those shares that reach it, their order.  (A cluster that shared this work out spent 4 us of 14 in its barriers.)
 __global__ void __launch_bounds__(SEL_THREADS) select_of_shares_kernel(const float* __restrict__ beam_scores, const float* __restrict__ cand_logp, int W_prev, int C,
                                                                        uint32_t magic, int shift, int k, int log2_share, unsigned long long* __restrict__ scratch,
-                                                                       int32_t* __restrict__ parents, int32_t* __restrict__ codes, float* __restrict__ scores) {
+                                                                       unsigned long long* claims, unsigned parts, int32_t* __restrict__ parents,
+                                                                       int32_t* __restrict__ codes, float* __restrict__ scores) {
     extern __shared__ unsigned long long room[];             // [2][SEL_LIST]: list and sort buffer; the shares that reach the bound
     __shared__ SelectShared sh;
     __shared__ unsigned n_list, n_hits;
@@ -525,50 +564,61 @@ __global__ void __launch_bounds__(SEL_THREADS) select_of_shares_kernel(const flo
     codes += (long long)req * k;
     scores += (long long)req * k;
     scratch += (long long)req * (ONELA_SELECT_PARTS * SEL_CAP);
+    const Claim claim(claims, req, parents);
+    const unsigned long long state = claim.state();
     unsigned long long held[SEL_HELD];
 #pragma unroll
     for (int j = 0; j < SEL_HELD; ++j) {
         const uint32_t i = (uint32_t)j * SEL_THREADS + tid;
         held[j] = i < shares ? __ldcg(scratch + i) : 0ull;
     }
-    const unsigned long long bound = bound_of(held, k, sh);
-    uint16_t* hits = reinterpret_cast<uint16_t*>(room + 2 * SEL_LIST);
+    unsigned n = N;                                          // candidates that the exhaustive selection has to look at: all of them
+    const unsigned long long* list = nullptr;                // ... or those of a list
+    if (state == claim.token + parts) {
+        const unsigned long long bound = bound_of(held, k, sh);
+        uint16_t* hits = reinterpret_cast<uint16_t*>(room + 2 * SEL_LIST);
 #pragma unroll
-    for (int j = 0; j < SEL_HELD; ++j)
-        if (held[j] >= bound) hits[atomicAdd(&n_hits, 1u)] = (uint16_t)(j * SEL_THREADS + tid);
-    __syncthreads();
-    auto each = [&](auto&& put) {
-        const uint32_t todo = n_hits << log2_share;
+        for (int j = 0; j < SEL_HELD; ++j)
+            if (held[j] >= bound) hits[atomicAdd(&n_hits, 1u)] = (uint16_t)(j * SEL_THREADS + tid);
+        __syncthreads();
+        auto each = [&](auto&& put) {
+            const uint32_t todo = n_hits << log2_share;
 #pragma unroll 4
-        for (uint32_t x = tid; x < todo; x += SEL_THREADS) {
-            const uint32_t i = ((uint32_t)hits[x >> log2_share] << log2_share) + (x & ((1u << log2_share) - 1u));
-            if (i < N) {
-                const unsigned long long c = src(i);
-                if (c >= bound) put(c);
+            for (uint32_t x = tid; x < todo; x += SEL_THREADS) {
+                const uint32_t i = ((uint32_t)hits[x >> log2_share] << log2_share) + (x & ((1u << log2_share) - 1u));
+                if (i < N) {
+                    const unsigned long long c = src(i);
+                    if (c >= bound) put(c);
+                }
             }
+        };
+        each([&](unsigned long long c) {
+            const unsigned at = atomicAdd(&n_list, 1u);
+            if (at < SEL_LIST) room[at] = c;
+        });
+        __syncthreads();
+        n = n_list;
+        if (n <= SEL_LIST) {
+            if (tid == 0) claim.release();
+            order_and_emit(room, (int)n, k, sh, src, parents, codes, scores);
+            return;
         }
-    };
-    each([&](unsigned long long c) {
-        const unsigned at = atomicAdd(&n_list, 1u);
-        if (at < SEL_LIST) room[at] = c;
-    });
-    __syncthreads();
-    const unsigned n = n_list;
-    if (n <= SEL_LIST) {
-        order_and_emit(room, (int)n, k, sh, src, parents, codes, scores);
-        return;
+        // too many for shared memory (candidates that gather in few shares): the list again, to global memory
+        __syncthreads();
+        if (tid == 0) n_list = 0u;
+        __syncthreads();
+        unsigned long long* out = scratch + SEL_SHARES;
+        each([&](unsigned long long c) { out[atomicAdd(&n_list, 1u)] = c; });
+        __threadfence_block();
+        list = out;
     }
-    // too many for shared memory (candidates that gather in few shares): the list again, to global memory
     __syncthreads();
-    if (tid == 0) n_list = 0u;
-    __syncthreads();
-    unsigned long long* list = scratch + SEL_SHARES;
-    each([&](unsigned long long c) { list[atomicAdd(&n_list, 1u)] = c; });
-    __threadfence_block();
-    __syncthreads();
-    select_topk<SEL_HELD>([&](uint32_t i) { return __ldcg(list + i); }, n, k, sh);
+    select_topk<SEL_HELD>([&](uint32_t i) { return list ? __ldcg(list + i) : src(i); }, n, k, sh);
+    if (tid == 0 && claim.mine(state)) claim.release();      // (select_topk ends with a barrier; a claim that not all CTAs got ends too)
     sort_and_emit<1>(sh.sel, room, k, k, sh, src, parents, codes, scores);
 }
+
+constexpr unsigned N_ALL = 0xffffffffu;       // no list of those that reach the bound
 
 // grid (CTAs of a cluster, requests).  SHARES: the shares' largest come from scratch (spread_shares_kernel),
 // and only the shares that reach the bound are looked into.  `scratch` ([request][ONELA_SELECT_PARTS * SEL_CAP], or null): also
@@ -576,10 +626,11 @@ __global__ void __launch_bounds__(SEL_THREADS) select_of_shares_kernel(const flo
 template <bool SHARES>
 __global__ void __launch_bounds__(SEL_THREADS) select_kernel(const float* __restrict__ beam_scores, const float* __restrict__ cand_logp, int W_prev, int C,
                                                              uint32_t magic, int shift, int k, unsigned long long* __restrict__ scratch,
-                                                             int32_t* __restrict__ parents, int32_t* __restrict__ codes, float* __restrict__ scores) {
+                                                             unsigned long long* claims, unsigned parts, int32_t* __restrict__ parents,
+                                                             int32_t* __restrict__ codes, float* __restrict__ scores) {
     extern __shared__ unsigned long long room[];             // [8][1024]: the threads' largest; later list and sort
     __shared__ SelectShared sh;
-    __shared__ unsigned n_list, n_mine, n_hits, s_at;
+    __shared__ unsigned n_list, n_mine, n_hits, s_at, s_claimed;
     __shared__ unsigned long long s_bound;
     const int tid = threadIdx.x;
     const int ctas = gridDim.x, rank = blockIdx.x, req = blockIdx.y;
@@ -595,6 +646,10 @@ __global__ void __launch_bounds__(SEL_THREADS) select_kernel(const float* __rest
     const uint32_t span = (uint32_t)ctas * SEL_THREADS, me = (uint32_t)rank * SEL_THREADS + tid;
     const uint32_t items = SHARES ? (N + SEL_HELD * SEL_THREADS - 1) / (SEL_HELD * SEL_THREADS) * SEL_THREADS : N;     // candidates, or shares
     const int stripes = (int)((items + span - 1) / span);
+    const Claim claim(claims, req, parents);
+    unsigned long long state = 0ull;
+    if constexpr (SHARES) state = claim.state();
+    const bool shared = !SHARES || state == claim.token + parts;      // (the same for the whole cluster: only its first CTA ends its claim)
     // 1. this thread's candidates (shares)
     unsigned long long best = 0ull;
     if constexpr (SHARES) {
@@ -612,100 +667,112 @@ __global__ void __launch_bounds__(SEL_THREADS) select_kernel(const float* __rest
         }
         best = top.composite(src);
     }
-    // 2. the bound
-    unsigned long long bound = 1ull;                         // (a composite is never 0: the index word of a candidate is not)
-    if (ctas > 1) {
-        st_cluster64(in_first_cta(room + rank * SEL_THREADS + tid), best);
-        cluster_barrier();
-        if (rank == 0) {
-            unsigned long long mine[SEL_CTAS];
+    unsigned n = N_ALL;
+    bool listed = false;
+    if (shared) {
+        // 2. the bound
+        unsigned long long bound = 1ull;                         // (a composite is never 0: the index word of a candidate is not)
+        if (ctas > 1) {
+            st_cluster64(in_first_cta(room + rank * SEL_THREADS + tid), best);
+            cluster_barrier();
+            if (rank == 0) {
+                unsigned long long mine[SEL_CTAS];
 #pragma unroll
-            for (int c = 0; c < SEL_CTAS; ++c) mine[c] = c < ctas ? room[c * SEL_THREADS + tid] : 0ull;
-            bound = bound_of(mine, k, sh);
-            if (tid == 0) { s_bound = bound; n_list = 0u; }
+                for (int c = 0; c < SEL_CTAS; ++c) mine[c] = c < ctas ? room[c * SEL_THREADS + tid] : 0ull;
+                bound = bound_of(mine, k, sh);
+                if (tid == 0) { s_bound = bound; n_list = 0u; }
+            }
+            cluster_barrier();
+            if (rank != 0) bound = ld_cluster64(in_first_cta(&s_bound));
+        } else {
+            if (stripes > 1) {
+                const unsigned long long mine[1] = {best};
+                bound = bound_of(mine, k, sh);
+            }
+            if (tid == 0) n_list = 0u;
+            __syncthreads();
         }
-        cluster_barrier();
-        if (rank != 0) bound = ld_cluster64(in_first_cta(&s_bound));
-    } else {
-        if (stripes > 1) {
-            const unsigned long long mine[1] = {best};
-            bound = bound_of(mine, k, sh);
+        // 3. the candidates that reach it: the shares whose largest does are listed, then all threads look into their members;
+        // what they find goes to a list of this CTA's, which is then appended to the first CTA's
+        uint16_t* hits = reinterpret_cast<uint16_t*>(room + 2 * SEL_LIST);      // thread (+ 1024 x stripe: share), of this CTA
+        if constexpr (SHARES) {
+            if (best >= bound)
+                for (int j = 0; j < stripes; ++j) {
+                    const uint32_t i = place_of(j, me, span);
+                    if (i < items && __ldcg(scratch + i) >= bound) hits[atomicAdd(&n_hits, 1u)] = (uint16_t)(j * SEL_THREADS + tid);
+                }
+        } else if (best >= bound) {
+            hits[atomicAdd(&n_hits, 1u)] = (uint16_t)tid;
         }
-        if (tid == 0) n_list = 0u;
         __syncthreads();
-    }
-    // 3. the candidates that reach it: the shares whose largest does are listed, then all threads look into their members;
-    // what they find goes to a list of this CTA's, which is then appended to the first CTA's
-    uint16_t* hits = reinterpret_cast<uint16_t*>(room + 2 * SEL_LIST);      // thread (+ 1024 x stripe: share), of this CTA
-    if constexpr (SHARES) {
-        if (best >= bound)
-            for (int j = 0; j < stripes; ++j) {
-                const uint32_t i = place_of(j, me, span);
-                if (i < items && __ldcg(scratch + i) >= bound) hits[atomicAdd(&n_hits, 1u)] = (uint16_t)(j * SEL_THREADS + tid);
-            }
-    } else if (best >= bound) {
-        hits[atomicAdd(&n_hits, 1u)] = (uint16_t)tid;
-    }
-    __syncthreads();
-    const int members = SHARES ? SEL_HELD : stripes;
-    auto each = [&](auto&& put) {
-        const int todo = (int)n_hits * members;
+        const int members = SHARES ? SEL_HELD : stripes;
+        auto each = [&](auto&& put) {
+            const int todo = (int)n_hits * members;
 #pragma unroll 2
-        for (int x = tid; x < todo; x += SEL_THREADS) {
-            const int q = x / members, m = x - q * members;
-            uint32_t i = hits[q];
-            if constexpr (SHARES) {                          // share i of stripe j: member m among the 16 384 candidates it lies in
-                i = place_of((int)(i / SEL_THREADS), (uint32_t)rank * SEL_THREADS + (i & (SEL_THREADS - 1)), span);
-                i = i / SEL_THREADS * (SEL_HELD * SEL_THREADS) + place_of(m, i & (SEL_THREADS - 1), SEL_THREADS);
-            } else {
-                i = place_of(m, (uint32_t)rank * SEL_THREADS + i, span);
+            for (int x = tid; x < todo; x += SEL_THREADS) {
+                const int q = x / members, m = x - q * members;
+                uint32_t i = hits[q];
+                if constexpr (SHARES) {                          // share i of stripe j: member m among the 16 384 candidates it lies in
+                    i = place_of((int)(i / SEL_THREADS), (uint32_t)rank * SEL_THREADS + (i & (SEL_THREADS - 1)), span);
+                    i = i / SEL_THREADS * (SEL_HELD * SEL_THREADS) + place_of(m, i & (SEL_THREADS - 1), SEL_THREADS);
+                } else {
+                    i = place_of(m, (uint32_t)rank * SEL_THREADS + i, span);
+                }
+                if (i < N) {
+                    const unsigned long long c = src(i);
+                    if (c >= bound) put(c);
+                }
             }
-            if (i < N) {
-                const unsigned long long c = src(i);
-                if (c >= bound) put(c);
-            }
+        };
+        unsigned long long* mine = room + SEL_LIST;              // (beside the first CTA's list)
+        each([&](unsigned long long c) {
+            const unsigned at = atomicAdd(&n_mine, 1u);
+            if (at < SEL_LIST) mine[at] = c;
+        });
+        __syncthreads();
+        const unsigned cnt = n_mine;
+        if (tid == 0) s_at = add_cluster(in_first_cta(&n_list), cnt);
+        __syncthreads();
+        {
+            const unsigned at = s_at;
+            const uint32_t list_at = in_first_cta(room);
+            for (unsigned i = tid; i < min(cnt, (unsigned)SEL_LIST); i += SEL_THREADS)
+                if (at + i < SEL_LIST) st_cluster64(list_at + (at + i) * 8, mine[i]);
         }
-    };
-    unsigned long long* mine = room + SEL_LIST;              // (beside the first CTA's list)
-    each([&](unsigned long long c) {
-        const unsigned at = atomicAdd(&n_mine, 1u);
-        if (at < SEL_LIST) mine[at] = c;
-    });
-    __syncthreads();
-    const unsigned cnt = n_mine;
-    if (tid == 0) s_at = add_cluster(in_first_cta(&n_list), cnt);
-    __syncthreads();
-    {
-        const unsigned at = s_at;
-        const uint32_t list_at = in_first_cta(room);
-        for (unsigned i = tid; i < min(cnt, (unsigned)SEL_LIST); i += SEL_THREADS)
-            if (at + i < SEL_LIST) st_cluster64(list_at + (at + i) * 8, mine[i]);
-    }
-    cluster_barrier();
-    unsigned n;
-    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(n) : "r"(in_first_cta(&n_list)) : "memory");
-    asm volatile("barrier.cluster.arrive.release;" ::: "memory");       // this thread has read the first CTA's memory
-    if (n > SEL_LIST && scratch) {
-        // too many for shared memory (candidates that gather in few threads' shares): the list again, to global memory
-        asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-        if (rank == 0 && tid == 0) n_list = 0u;
         cluster_barrier();
-        unsigned long long* out = scratch + SEL_SHARES;
-        each([&](unsigned long long c) { out[add_cluster(in_first_cta(&n_list), 1u)] = c; });
-        __threadfence();
-        asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+        asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(n) : "r"(in_first_cta(&n_list)) : "memory");
+        asm volatile("barrier.cluster.arrive.release;" ::: "memory");       // this thread has read the first CTA's memory
+        if (n > SEL_LIST && scratch) {
+            // too many for shared memory (candidates that gather in few threads' shares): the list again, to global memory
+            asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+            if (rank == 0 && tid == 0) {
+                n_list = 0u;
+                s_claimed = SHARES || claim.settle(claim.ask());
+            }
+            cluster_barrier();
+            unsigned claimed;
+            asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(claimed) : "r"(in_first_cta(&s_claimed)) : "memory");
+            listed = claimed != 0u;
+            unsigned long long* out = scratch + SEL_SHARES;
+            if (listed) each([&](unsigned long long c) { out[add_cluster(in_first_cta(&n_list), 1u)] = c; });
+            __threadfence();
+            asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+        }
+        asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
     }
-    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
     if (rank != 0) return;
     if (n <= SEL_LIST) {
+        if (SHARES && tid == 0) claim.release();             // (the cluster is through with the shares)
         order_and_emit(room, (int)n, k, sh, src, parents, codes, scores);
     } else {                                                 // exhaustively, over the list or over all candidates
-        if (scratch) {
+        if (listed) {
             const unsigned long long* list = scratch + SEL_SHARES;
             select_topk<SEL_HELD>([&](uint32_t i) { return __ldcg(list + i); }, n, k, sh);
         } else {
+            __syncthreads();
             select_topk<SEL_HELD>(src, N, k, sh);
         }
+        if (tid == 0 && (SHARES ? claim.mine(state) : listed)) claim.release();      // (select_topk ends with a barrier)
         sort_and_emit<1>(sh.sel, room, k, k, sh, src, parents, codes, scores);
     }
 }
@@ -724,8 +791,8 @@ bool from_shares(long long candidates, int k) { return candidates > (k <= ONE_CT
 int select_launches(long long candidates, int32_t W_new) { return from_shares(candidates, W_new) ? 2 : 1; }
 
 cudaError_t launch_select(const float* beam_scores, const float* cand_logp, int32_t req_count, int32_t W_prev, int32_t C,
-                          int32_t W_new, unsigned long long* scratch, int32_t* parents, int32_t* codes, float* scores,
-                          cudaStream_t stream) {
+                          int32_t W_new, unsigned long long* scratch, unsigned long long* claims, int32_t* parents, int32_t* codes,
+                          float* scores, cudaStream_t stream) {
     const long long N = (long long)W_prev * C;
     if (N > (long long)ONELA_SELECT_PARTS * 4096) return cudaErrorInvalidValue;
     // CTAs per request: one while the candidates are at most four per thread (the exchange between CTAs costs more than the
@@ -758,19 +825,22 @@ cudaError_t launch_select(const float* beam_scores, const float* cand_logp, int3
     uint32_t magic;
     int shift;
     divide_by(C, magic, shift);
+    unsigned parts = 0;                  // CTAs per request of the launch of shares
     if (shares) {
         cudaError_t e;
         if (W_new <= ONE_CTA_TO) {       // shares of 16 candidates; of 64 where the CTA's threads would not hold that many
             const bool wide = N > 1ll * SEL_SHARE * SEL_HELD * SEL_THREADS;
             static_assert(4ll * SEL_SHARE * SEL_HELD * SEL_THREADS >= (long long)ONELA_SELECT_PARTS * 4096, "the shares of the largest request");
-            e = launch_dependent(wide ? select_shares_kernel<4> : select_shares_kernel<1>, dim3((unsigned)((N + 1023) / 1024), req_count), dim3(SHARE_THREADS), 0,
-                                 stream, beam_scores, cand_logp, W_prev, C, magic, shift, scratch);
+            parts = (unsigned)((N + 1023) / 1024);
+            e = launch_dependent(wide ? select_shares_kernel<4> : select_shares_kernel<1>, dim3(parts, req_count), dim3(SHARE_THREADS), 0, stream, beam_scores, cand_logp,
+                                 W_prev, C, magic, shift, W_new, scratch, claims, parents);
             if (e != cudaSuccess) return e;
             return launch_dependent(select_of_shares_kernel, dim3(req_count), dim3(SEL_THREADS), SMEM, stream, beam_scores, cand_logp, W_prev, C, magic, shift,
-                                    W_new, wide ? 6 : 4, scratch, parents, codes, scores);
+                                    W_new, wide ? 6 : 4, scratch, claims, parts, parents, codes, scores);
         }
-        e = launch_dependent(spread_shares_kernel, dim3((unsigned)(blocks * (SEL_THREADS / SHARES_PER_CTA)), req_count), dim3(SHARE_THREADS), 0, stream, beam_scores,
-                             cand_logp, W_prev, C, magic, shift, scratch);
+        parts = (unsigned)(blocks * (SEL_THREADS / SHARES_PER_CTA));
+        e = launch_dependent(spread_shares_kernel, dim3(parts, req_count), dim3(SHARE_THREADS), 0, stream, beam_scores, cand_logp, W_prev, C, magic, shift, W_new,
+                             scratch, claims, parents);
         if (e != cudaSuccess) return e;
     }
     cudaLaunchConfig_t cfg = {};
@@ -786,7 +856,8 @@ cudaError_t launch_select(const float* beam_scores, const float* cand_logp, int3
     attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, shares ? select_kernel<true> : select_kernel<false>, beam_scores, cand_logp, W_prev, C, magic, shift, W_new, scratch, parents, codes, scores);
+    return cudaLaunchKernelEx(&cfg, shares ? select_kernel<true> : select_kernel<false>, beam_scores, cand_logp, W_prev, C, magic, shift, W_new, scratch, claims, parts, parents,
+                              codes, scores);
 }
 
 }  // namespace onela
@@ -806,7 +877,7 @@ extern "C" onela_status onela_select_beams_static(const float* beam_scores_dev, 
     if (req_count > STATIC_REQUESTS) return ONELA_E_CAPACITY;
     if ((int64_t)W_prev * C > (int64_t)ONELA_SELECT_PARTS * 4096) return ONELA_E_CAPACITY;
     if (W_new > ONELA_SELECT_CAP || W_new > (int64_t)W_prev * C) return ONELA_E_CAPACITY;
-    if (launch_select(beam_scores_dev, cand_logp_dev, req_count, W_prev, C, W_new, nullptr, parents_out_dev, codes_out_dev,
+    if (launch_select(beam_scores_dev, cand_logp_dev, req_count, W_prev, C, W_new, nullptr, nullptr, parents_out_dev, codes_out_dev,
                       scores_out_dev, static_cast<cudaStream_t>(stream)) != cudaSuccess)
         return ONELA_E_CUDA;
     return ONELA_OK;
