@@ -38,10 +38,10 @@ __global__ void __launch_bounds__(256) append_kernel(const char* __restrict__ k,
 
 // Copy of one (request, layer)'s states out of the store, 16 bytes per thread and step (a prefill has just left them in L2: the
 // launch is what it costs).
-__global__ void __launch_bounds__(256) export_state_kernel(const float4* __restrict__ slot, float4* __restrict__ out, int32_t n) {
+__global__ void __launch_bounds__(256) export_state_kernel(const float4* __restrict__ slot, float4* __restrict__ out, long long n) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    for (int32_t i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) out[i] = slot[i];
+    for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < n; i += (long long)gridDim.x * 256) out[i] = slot[i];
 }
 
 // The operand scale of a head (Layout::s0_scale) from the largest magnitude of its state.
@@ -175,16 +175,19 @@ cudaError_t launch_store_state(const float* S0_in, float* slot, float* scale_out
 cudaError_t launch_export_state(const float* slot, float* S0_out, int32_t H, int32_t dk, int32_t dv, cudaStream_t stream) {
     // A kernel of our own is a dependent launch, a copy by the runtime is not.  (Together with the prefill's own dependent
     // launch, us a pass of prefill + export: 3 x 100 tokens x 32 heads of 64 x 64 bf16 62 -> 45, 2 x 1021 tokens x 16 heads
-    // fp32 82 -> 74.5, 3 x 900 tokens x 16 heads of 128 x 128 160 -> 147, 16 384 tokens 450 -> 445.)  Memory of another device,
-    // which a kernel may not reach, is the runtime's.
+    // fp32 82 -> 74.5, 3 x 900 tokens x 16 heads of 128 x 128 160 -> 147, 16 384 tokens 450 -> 445.)  Where the store or the destination
+    // is not the current device's own memory (another device's, managed, the host's), which a kernel may not reach, and where the
+    // stream is another device's, which takes no kernel from here, the copy is the runtime's.
     cudaPointerAttributes at;
     int dev = 0;
-    const bool here = cudaGetDevice(&dev) == cudaSuccess && cudaPointerGetAttributes(&at, S0_out) == cudaSuccess && at.type == cudaMemoryTypeDevice && at.device == dev;
-    const long long n = (long long)H * dk * dv / 4;
-    if (here && n <= 0x7fffffff) {
+    auto here = [&](const void* p) { return cudaPointerGetAttributes(&at, p) == cudaSuccess && at.type == cudaMemoryTypeDevice && at.device == dev; };
+    if (cudaGetDevice(&dev) == cudaSuccess && here(S0_out) && here(slot)) {
+        const long long n = (long long)H * dk * dv / 4;
         const unsigned blocks = (unsigned)(n / 256 < 1184 ? (n + 255) / 256 : 1184);      // eight per SM at most
-        return launch_dependent(export_state_kernel, dim3(blocks), dim3(256), 0, stream, reinterpret_cast<const float4*>(slot),
-                                reinterpret_cast<float4*>(S0_out), (int32_t)n);
+        const cudaError_t e = launch_dependent(export_state_kernel, dim3(blocks), dim3(256), 0, stream, reinterpret_cast<const float4*>(slot),
+                                               reinterpret_cast<float4*>(S0_out), n);
+        if (e != cudaErrorInvalidResourceHandle) return e;
+        cudaGetLastError();
     }
     return cudaMemcpyAsync(S0_out, slot, (size_t)H * dk * dv * sizeof(float), cudaMemcpyDeviceToDevice, stream);
 }
