@@ -23,6 +23,7 @@
 // loop over the tiles of beams spills (the invariants of every pointer stay live): 64 x 64 40 us.
 // The only wait is for the MMAs' completion; it is bounded, and all threads agree on its outcome before going on
 // (ONELA_E_TIMEOUT in the status word otherwise).
+#include <atomic>
 #include <mutex>
 
 #include "onela_internal.h"
@@ -580,19 +581,40 @@ cudaError_t launch_lanes(const TiledArgs& a, cudaStream_t stream) {
     return launch_dependent(kern, grid, dim3(THREADS), smem, stream, a);
 }
 
+// SMs of the current device, 0 if there is none to ask.
+int sm_count() {
+    constexpr int MAX_DEVICES = 64;
+    static std::atomic<int> count_of[MAX_DEVICES] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEVICES) return 0;
+    int n = count_of[dev].load(std::memory_order_relaxed);
+    if (n == 0 && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess) count_of[dev].store(n, std::memory_order_relaxed);
+    return n;
+}
+
 // 64 x 64 bf16: four lanes per unit take a quarter fewer instructions per fold and leave room for six CTAs of 128 threads per SM
 // (five with delta records), 192 units in flight instead of 160; but a warp's chain is longer.  Eight / four lanes, us a
-// generation: 4 x 512 beams x 32 heads, 8 calls 384 / 375; 8 x 777, 4 calls 458 / 420; 2 x 400, 4 calls (832 tiles: two waves
-// of five CTAs, one of six) 90.6 / 74.4; 3 x 333 grouped heads 124.6 / 121.1; delta records 4 x 512 506 / 493, 4 x 300 182 /
-// 175.  Below one wave of five the longer chain shows: 2 x 300 beams x 16 heads (320 tiles) 74.3 / 75.5, 1 x 100 beams x 32
-// heads 33.3 / 33.5.  So the line lies at one wave of five CTAs on 148 SMs.  (Seven or eight CTAs spill; 64 beams per CTA 377
-// on the first, 13 % slower on the last; fp32 records 5 % slower and more.)
-constexpr int FOUR_LANES_FROM = 740;
+// generation on 148 SMs, tiles in brackets.
+// Raw records: 1 x 400 beams x 16 heads (208) 27.9 / 27.9, 2 x 320 x 16 (320) 29.0 / 29.4, 4 x 300 x 16 (640) 61.7 / 60.2, 4 x 384 x 16 (768:
+// two waves of five CTAs, one of six) 107.2 / 90.4, 3 x 500 x 24 (1152) 58.1 / 56.4, 4 x 512 x 32 (2048) 191.0 / 183.6.  So the line lies at
+// one wave of eight lanes' CTAs.  (Seven or eight CTAs spill; 64 beams per CTA 377 against 375, 13 % slower on narrow beams; fp32
+// records 5 % slower and more.)
+// Delta records: five CTAs of four lanes spill (104 bytes), four of eight do not, and the spills cost what the fold saves: what is
+// gained is a wave.  4 x 150 x 16 (640) 67.8 / 59.8, 3 x 224 x 16 (672) 39.9 / 37.3, 4 x 192 x 16 (768) 103.6 / 107.7, 1 x 500 x 32 (1024)
+// 55.1 / 55.3, 3 x 250 x 24 (1152) 58.3 / 59.4, 4 x 256 x 32 (2048) 196.7 / 188.9.  So four lanes where their waves are fewer.  (Four CTAs of
+// four lanes, without spills: 68.3, 40.1, 103.2, 53.4, 56.6, 193.1.)
+template <int KD, int VD, typename T, bool DELTA>
+bool four_lanes(const TiledArgs& a) {
+    constexpr int BPT = tiled_beams<KD, VD>() / (DELTA ? 2 : 1);
+    const long long tiles = (long long)((a.W + BPT - 1) / BPT) * a.Hk * a.g * a.req_count;
+    const long long eight = (long long)sm_count() * tiled_min_ctas<KD, VD, T, DELTA, 8>(), four = (long long)sm_count() * tiled_min_ctas<KD, VD, T, DELTA, 4>();
+    if (eight == 0) return false;
+    return DELTA ? (tiles + four - 1) / four < (tiles + eight - 1) / eight : tiles > eight;
+}
 template <int KD, int VD, typename T, typename OutT, bool DELTA>
 cudaError_t launch_one(const TiledArgs& a, cudaStream_t stream) {
     if constexpr (KD + VD <= 128 && sizeof(T) == 2) {
-        constexpr int BPT = tiled_beams<KD, VD>() / (DELTA ? 2 : 1);
-        if ((long long)((a.W + BPT - 1) / BPT) * a.Hk * a.g * a.req_count > FOUR_LANES_FROM) return launch_lanes<KD, VD, T, OutT, DELTA, 4>(a, stream);
+        if (four_lanes<KD, VD, T, DELTA>(a)) return launch_lanes<KD, VD, T, OutT, DELTA, 4>(a, stream);
     }
     return launch_lanes<KD, VD, T, OutT, DELTA, 8>(a, stream);
 }
