@@ -505,6 +505,11 @@ onela_status launch_decode(onela_ctx* ctx, int32_t req_begin, int32_t req_count,
         ta.depth = depth;
         ta.max_beam = c.max_beam;
         ta.delta = ctx->gtr() ? 1 : 0;
+        {
+            const long long es = ctx->elem_bytes, eo = c.out_dtype == ONELA_DTYPE_BF16 ? 2 : 4, Hv = ctx->Hv();
+            const long long beam = c.num_heads * 3 * c.dk * es + Hv * c.dv * (2 * es + eo);      // q, k, v, record (k | v), output
+            ta.call_bytes = (long long)c.num_layers * req_count * (Hv * (long long)s0_f16_head_bytes(c.dk, c.dv) + W * beam);
+        }
         for (int i = 0; i < req_count; ++i) ta.bases.base[i] = ctx->req[req_begin + i].step_base.back();
         if (launch_decode_tiled(ta, c.dk, c.dv, c.rec_dtype, c.out_dtype, s) != cudaSuccess) return ONELA_E_CUDA;
         ctx->launches++;

@@ -84,10 +84,10 @@ __host__ __device__ constexpr int tiled_min_ctas() { return KD + VD <= 128 ? (G 
 // replay leaving x unchanged - and after the contraction delta_t = beta_t (v_t - alpha_t S_{t-1} k_t) and
 // o_t = alpha_t S_{t-1} q_t + delta_t (k_t . q_t) are formed from the two rows and the record is written; always with
 // the append fused in, dk = dv <= 128.
-// G: lanes per unit, 8 or (64 x 64 bf16 in large launches) 4.  Four lanes add up what eight do, in eight lanes' order: lane g holds
+// REQUEST: an older record's lines are requested into L2 a level ahead (see launch_one).  G: lanes per unit, 8 or (64 x 64 bf16 in large launches) 4.  Four lanes add up what eight do, in eight lanes' order: lane g holds
 // the chunks of lanes g and g + 4, sums each by itself and adds the two, which is what the first exchange among eight lanes does.  So
 // a request's results do not depend on how many others share its launch.
-template <int KD, int VD, typename T, typename OutT, bool DELTA, int G>
+template <int KD, int VD, typename T, typename OutT, bool DELTA, int G, bool REQUEST>
 __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, VD, T, DELTA, G>()) decode_tiled_kernel(const TiledArgs a) {
     constexpr int NB = tiled_beams<KD, VD>(), CP = tile_pitch<VD>();
     constexpr int THREADS = NB * G, BPT = DELTA ? NB / 2 : NB;          // beams per tile
@@ -218,11 +218,6 @@ __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, 
         x.gate = __ldg(gates + slot);
         return x;
     };
-    // Where an older record does not fit in the registers beside the one at hand, its lines are requested into L2 a level ahead (a
-    // hint: they may come from HBM, and nothing else is in flight under the fold).  4 x 512 beams x 32 heads of 256 x 256 bf16, 4
-    // calls 584 -> 558 us, 2 x 300 beams with uniform parents 165 -> 156, fp32 298 -> 292; at 256 x 512, where the fold spills, 11 %
-    // slower; 128 x 256 fp32 the same.
-    constexpr bool REQUEST = KD == 256 && VD == 256;
     auto request_slot = [&](long long slot) {
         const char *kp = reinterpret_cast<const char*>(kplane + slot * a.k_stride), *vp = reinterpret_cast<const char*>(vplane + slot * a.v_stride);
         constexpr int KL = KD * (int)sizeof(T) / 128, VL = VD * (int)sizeof(T) / 128;      // lines
@@ -553,9 +548,9 @@ __global__ void __launch_bounds__(tiled_beams<KD, VD>() * G, tiled_min_ctas<KD, 
     }
 }
 
-template <int KD, int VD, typename T, typename OutT, bool DELTA, int G>
+template <int KD, int VD, typename T, typename OutT, bool DELTA, int G, bool REQUEST = false>
 cudaError_t launch_lanes(const TiledArgs& a, cudaStream_t stream) {
-    auto kern = decode_tiled_kernel<KD, VD, T, OutT, DELTA, G>;
+    auto kern = decode_tiled_kernel<KD, VD, T, OutT, DELTA, G, REQUEST>;
     constexpr int NB = tiled_beams<KD, VD>(), THREADS = NB * G, BPT = DELTA ? NB / 2 : NB;
     constexpr size_t smem = tiled_smem_bytes<KD, VD>();
     static_assert(smem <= 232448, "shared memory per CTA");
@@ -611,8 +606,24 @@ bool four_lanes(const TiledArgs& a) {
     if (eight == 0) return false;
     return DELTA ? (tiles + four - 1) / four < (tiles + eight - 1) / eight : tiles > eight;
 }
+
+// 256 x 256: an older record does not fit in the registers beside the one at hand, so where it comes from HBM its lines are requested
+// into L2 a level ahead (nothing else is in flight under the fold); where it is still in L2 the requests only cost issue slots.
+// What decides is what one decode call of all layers touches (TiledArgs::call_bytes): by the next call the L2 of 126 MB has seen that
+// much since the record was written.  Without / with requests, us a generation (4 or 8 calls, Zipf or uniform parents), MB a call in
+// brackets - bf16: 4 x 100 beams x 16 heads (28) 54.9 / 55.6, 109.6 / 111.9; 2 x 300 x 8 heads, 2 layers (33) 86.2 / 87.1, 185.6 / 188.0; 3
+// layers (50) 121.2 / 121.9, 269.7 / 267.1, uniform 124.6 / 122.9; 4 x 100 x 16, 2 layers (56) 100.7 / 99.7, 211.9 / 203.5; 2 x 300 x 8, 4 layers (67)
+// 371 / 351, 6 layers (101) 588 / 525.  fp32, two lines a lane: 2 x 300 x 8 (31) 130.9 / 134.5; 4 x 100 x 16 (47) 142.0 / 145.0; 1 x 128 x
+// 32, 2 layers (58) 108.6 / 109.9, 236.7 / 238.4; 3 layers (88) 166.5 / 164.9, 375.4 / 364.3; 4 x 100 x 16, 2 layers (95) 290.9 / 280.2.
+// (At 256 x 512, where the fold spills, requests were 11 % slower; 128 x 256 fp32 the same.)
+template <typename T>
+constexpr long long REQUEST_FROM = (sizeof(T) == 2 ? 48ll : 80ll) << 20;
+
 template <int KD, int VD, typename T, typename OutT, bool DELTA>
 cudaError_t launch_one(const TiledArgs& a, cudaStream_t stream) {
+    if constexpr (KD == 256 && VD == 256) {
+        if (a.call_bytes > REQUEST_FROM<T>) return launch_lanes<KD, VD, T, OutT, DELTA, 8, true>(a, stream);
+    }
     if constexpr (KD + VD <= 128 && sizeof(T) == 2) {
         if (four_lanes<KD, VD, T, DELTA>(a)) return launch_lanes<KD, VD, T, OutT, DELTA, 4>(a, stream);
     }

@@ -131,6 +131,7 @@ struct TiledArgs {
     long long s0_req_stride, s0_scale_req_stride, table_req_stride, arena_slots, k_stride, v_stride;
     int32_t req_count, W, Hk, g, depth, max_beam;
     int32_t delta;          // 1: the arena keeps (alpha, delta, k) records and the launch replays both projections forward
+    long long call_bytes;   // what a decode call of these requests touches in all layers: operand copies, tokens, records written, outputs
     BatchBases bases;
 };
 bool decode_tiled_supported(int32_t dk, int32_t dv);
