@@ -4,7 +4,7 @@
 // the contraction with S_0, which dominates these shapes (dv x dk multiply-adds per unit against 3 dk per record).
 //
 // One CTA = (request, value head, tile of 32 beams - 64 from 128 x 128 up), 8 lanes per (beam, head) unit (4 in large launches of
-// 64 x 64 bf16: see launch_one).
+// 64 x 64 bf16: see four_lanes).
 //   1. Every unit folds its query through its records, newest first:  c = k.r ; corr += beta c v ; r -= beta c k,
 //      the decay a running scalar.  corr stays in registers.  With the append fused in, the newest record comes from
 //      the caller's tensors and the unit also writes it to its arena slot.
@@ -74,7 +74,7 @@ __host__ __device__ constexpr size_t tiled_smem_bytes() {
 // CTAs per SM the registers are capped for: small CTAs are latency-bound (a string of dependent loads per level, one MMA
 // round trip), so the narrowest shape gets four, with bf16 records - half the registers - five (64 x 64 on the beam-512
 // stack: 30 -> 27 us; six: 28.5; fp32 records, five: 16 -> 17 us, three: 4 - 7 % slower at 65 536 units), unless a beam has two
-// rows, where five spill (4 x 300 beams x 16 heads, 6 calls, a generation: 185 -> 177 us).  (64 beams of 256 threads at two per
+// rows, where five of eight lanes spill (4 x 300 beams x 16 heads, 6 calls, a generation: 185 -> 177 us; four lanes: see four_lanes).  (64 beams of 256 threads at two per
 // SM, or 16 lanes per unit, were 5 - 10 % slower at 256 x 256.)
 template <int KD, int VD, typename T, bool DELTA, int G>
 __host__ __device__ constexpr int tiled_min_ctas() { return KD + VD <= 128 ? (G == 4 ? (DELTA ? 5 : 6) : sizeof(T) == 4 || DELTA ? 4 : 5) : tiled_beams<KD, VD>() == 64 ? 1 : 2; }
@@ -595,9 +595,10 @@ int sm_count() {
 // one wave of eight lanes' CTAs.  (Seven or eight CTAs spill; 64 beams per CTA 377 against 375, 13 % slower on narrow beams; fp32
 // records 5 % slower and more.)
 // Delta records: five CTAs of four lanes spill (104 bytes), four of eight do not, and the spills cost what the fold saves: what is
-// gained is a wave.  4 x 150 x 16 (640) 67.8 / 59.8, 3 x 224 x 16 (672) 39.9 / 37.3, 4 x 192 x 16 (768) 103.6 / 107.7, 1 x 500 x 32 (1024)
-// 55.1 / 55.3, 3 x 250 x 24 (1152) 58.3 / 59.4, 4 x 256 x 32 (2048) 196.7 / 188.9.  So four lanes where their waves are fewer.  (Four CTAs of
-// four lanes, without spills: 68.3, 40.1, 103.2, 53.4, 56.6, 193.1.)
+// gained is a wave.  4 x 150 x 16 (640) 67.4 / 60.5, 3 x 224 x 16 (672) 41.6 / 38.5, 4 x 192 x 16 (768) 103.6 / 109.1, 1 x 500 x 32 (1024)
+// 55.1 / 56.1, 3 x 250 x 24 (1152) 58.3 / 60.4, 3 x 200 x 32 (1248) 64.8 / 62.4, 4 x 256 x 32 (2048) 195.8 / 190.2, 4 x 512 x 32 (4096) 348.7 /
+// 340.6.  So four lanes where their waves are fewer.  (Four CTAs of four lanes, without spills, on the first, third, fourth, fifth and
+// seventh: 68.3, 103.2, 53.4, 56.6, 193.1.)
 template <int KD, int VD, typename T, bool DELTA>
 bool four_lanes(const TiledArgs& a) {
     constexpr int BPT = tiled_beams<KD, VD>() / (DELTA ? 2 : 1);
@@ -615,7 +616,8 @@ bool four_lanes(const TiledArgs& a) {
 // layers (50) 121.2 / 121.9, 269.7 / 267.1, uniform 124.6 / 122.9; 4 x 100 x 16, 2 layers (56) 100.7 / 99.7, 211.9 / 203.5; 2 x 300 x 8, 4 layers (67)
 // 371 / 351, 6 layers (101) 588 / 525.  fp32, two lines a lane: 2 x 300 x 8 (31) 130.9 / 134.5; 4 x 100 x 16 (47) 142.0 / 145.0; 1 x 128 x
 // 32, 2 layers (58) 108.6 / 109.9, 236.7 / 238.4; 3 layers (88) 166.5 / 164.9, 375.4 / 364.3; 4 x 100 x 16, 2 layers (95) 290.9 / 280.2.
-// (At 256 x 512, where the fold spills, requests were 11 % slower; 128 x 256 fp32 the same.)
+// (The bf16 instantiation with requests spills 4 bytes.  At 256 x 512, where the fold spills, requests were 11 % slower; 128 x 256 fp32
+// the same.)
 template <typename T>
 constexpr long long REQUEST_FROM = (sizeof(T) == 2 ? 48ll : 80ll) << 20;
 

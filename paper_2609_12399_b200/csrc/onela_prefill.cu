@@ -197,9 +197,10 @@ __device__ __forceinline__ void split_to_tmem(uint32_t taddr, const float* x, fl
 }
 
 // acc[r] = sum over l < N of rows[r][l] cols[l]: eight rows (pitch AP, read as broadcast vectors) times this lane's column, the
-// even and the odd l in the two halves of packed multiply-adds.  UNROLL steps of four l at a time: all of them where the code has
-// room for it (dk <= 64: 5000 tokens x 16 heads of 32 x 32 fp32 83.2 -> 79.5 us, 6000 x 32 heads of 64 x 64 124.0 -> 119.5), two at
-// dk = 128, whose roles miss the instruction cache (16 384 tokens 434.7 -> 429.5; four 439.6, eight 454.2).  Error against 64
+// even and the odd l in the two halves of packed multiply-adds.  UNROLL steps of four l at a time: all of them at dk <= 64 (5000
+// tokens x 16 heads of 32 x 32 fp32 83.2 -> 79.5 us, 6000 x 32 heads of 64 x 64 bf16 124.0 -> 119.5, although that one then spills 12
+// bytes: four steps, which do not, 1 - 2 % slower from 1021 to 16 384 tokens), two at dk = 128, whose roles miss the instruction cache
+// (16 384 tokens 434.7 -> 429.5; four 439.6, eight 454.2).  Error against 64
 // bits: 0.3 % smaller on the mean of fourteen shapes, none more than 0.5 % larger.
 template <int N, int UNROLL>
 __device__ __forceinline__ void rows8(float* acc, const float* rows, const float* cols, int pitch) {

@@ -9,9 +9,10 @@
 //
 // The candidates are cut into shares, the shares' largest give a bound that at least k of them reach - so at least k candidates
 // reach it, and hardly more do (1094 expected for k = 1024 of a million) - and only the shares that reach it are looked into:
-//   * up to 16 384 candidates (32 768 where many survive), or without scratch, a share is a thread's, in a cluster of up to eight CTAs of 1024 threads per
-//     request (`select_kernel`): the first CTA finds the bound, what reaches it is gathered in its shared memory (distributed
-//     shared memory, one remote atomic per CTA), ordered through a histogram of the scores and written out best first;
+//   * up to 16 384 candidates (32 768 where more than 256 survive), fewer than 48 per survivor, or without scratch, a share is a
+//     thread's, in a cluster of up to eight CTAs of 1024 threads per request (`select_kernel`): the first CTA finds the bound, what
+//     reaches it is gathered in its shared memory (distributed shared memory, one remote atomic per CTA), ordered through a histogram
+//     of the scores and written out best first;
 //   * beyond, shares of sixteen are spread over all SMs by a launch of their own (`spread_shares_kernel`), and the cluster goes on
 //     from their largest (`select_kernel<true>`).  A cluster alone waited 7.7 us for 512 x 256 candidates out of HBM;
 //   * where few survive (k <= 256), one CTA does the rest without a cluster's barriers, from shares of neighbours, whose members
@@ -784,8 +785,11 @@ __global__ void __launch_bounds__(SEL_THREADS) select_kernel(const float* __rest
 // generations (select, index, decode; us, one cluster reading all candidates / from shares): one CTA for the rest - 128 x 1000 ->
 // 128 115 / 101, 4 x 200 x 512 -> 200 98.5 / 94.2; a cluster for the rest - 2 x 512 x 128 -> 512 127.5 / 121.4, 8 x 512 x 512 -> 512
 // 215 / 193, 3 x 333 x 512 -> 333 281 / 250.  One CTA at 512 survivors of 8 x 512 x 512 198, at 1000 of 4 x 1000 x 1000 194 against the
-// cluster's 152: it then fetches 16 000 candidates by itself.  Below 16 384 candidates the second launch is not worth its host time:
-// 100 x 128 -> 100 66.8 / 64.0 as a graph, but 7 x 10 x 1000 -> 10, issued eagerly, 95.1 / 95.8.
+// cluster's 152: it then fetches 16 000 candidates by itself.  (Before the scratch was claimed, 0.5 us a selection.)
+// Between 12 800 and 16 384 candidates it depends on how many survive (as a graph, one cluster / from shares): 8 x 60 x 256 -> 60 51.8 /
+// 50.0, 1 x 16 x 1000 -> 16 49.2 / 47.1, 4 x 13 x 1000 -> 13 50.2 / 49.1; 1 x 100 x 160 -> 100 49.2 / 50.2, 4 x 128 x 100 -> 128 63.5 / 64.9, 2 x
+// 200 x 65 -> 200 49.1 / 51.2; issued eagerly the first three gain less, the last three lose up to 6 %.  Below, from shares is slower even
+// where few survive (8 x 16 x 512 -> 16 63.7 / 65.5, 4 x 60 x 100 -> 60 61.4 / 64.5, both eagerly).
 constexpr int SHARES_FROM = 16384, ONE_CTA_TO = 256;
 bool from_shares(long long candidates, int k) { return candidates > (k <= ONE_CTA_TO ? SHARES_FROM : 2 * SEL_HELD * SEL_THREADS) && candidates >= 3ll * SEL_SHARE * k; }
 int select_launches(long long candidates, int32_t W_new) { return from_shares(candidates, W_new) ? 2 : 1; }
