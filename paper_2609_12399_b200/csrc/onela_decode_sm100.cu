@@ -760,15 +760,17 @@ __global__ void __launch_bounds__(THREADS, 1) decode_ws_kernel(const __grid_cons
                 if (!QUEUE && staged_levels > 0) {      // (a queue leaves nothing staged: no such code in its loop, grouped wide heads 257 -> 253 us)
                     const uint8_t* st = stage + buf * (STAGE_BUF * REC_BYTES);
                     const float2* gs = gates_s + buf * STAGE_BUF;
-                    if constexpr (GROUPED) {
+                    if constexpr (GROUPED || (FUSED && sizeof(OutT) == 4)) {
                         const RecT newest = L::load_shared(st, gs, staged_idx_of(staged_levels - 1), g);
                         L::template fold_chain_simple<DELTA>(newest, staged_levels - 2, 0,
                                       [&](int level) { return L::load_shared(st, gs, staged_idx_of(level), g); }, r, corr, decay);
                     } else {
                         // Keys and gates a level ahead of their fold: a level's index shuffle and key loads are off its chain.  (Ten
                         // more registers; whole records ahead, or the loop unrolled, spill: 27 % slower.  Beam-512 stack, 4
-                        // layers, 8 calls 1069 -> 1046 us; 5 x 77 beams 251.4 -> 247.9; delta records 4 x 512 680 -> 673; the
-                        // grouped instantiation does not have the registers.)
+                        // layers, 8 calls 1069 -> 1046 us; 5 x 77 beams 251.4 -> 247.9; delta records 4 x 512 680 -> 673; fp32 outputs,
+                        // separate append, 4 x 512 851 -> 843.  The grouped instantiation does not have the registers; with fp32
+                        // outputs and the append fused in it loses: delta records 8 heads x 40 beams 36.9 -> 37.7, 2 x 200 207.6 -> 210.2,
+                        // 4 x 512 517 -> 524; raw 16 heads x 128 beams 35.3 -> 35.6, 5 x 77 128.2 -> 128.7, 4 x 512 588 -> 586.)
                         auto load_key = [&](RecT& x, int at) {
                             const uint4* p = reinterpret_cast<const uint4*>(st + at * REC_BYTES) + g;
 #pragma unroll
